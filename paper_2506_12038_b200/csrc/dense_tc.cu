@@ -20,6 +20,7 @@
 
 #include "common.h"
 #include "device_util.h"
+#include "selectors.cuh"
 
 namespace lcd {
 
@@ -746,26 +747,14 @@ dense_i8_kernel(const __grid_constant__ CUtensorMap tmap_act, const DenseParams 
 #pragma unroll
         for (int xq = 0; xq < 2; ++xq) {
           uint32_t sel[8], pick[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-          if (BITS == 4) {                  // natural order; pick = byte choice between entries 0..7 and 8..15
+          if constexpr (BITS == 4) {
 #pragma unroll
-            for (int wd = 0; wd < 4; ++wd) {
-              const uint32_t raw = cur[xq][NW > 3 ? wd : 0];
-              const uint32_t s7 = raw & 0x77777777u, pk = ((raw >> 1) & 0x44444444u) | 0x32103210u;
-              sel[2 * wd] = s7; sel[2 * wd + 1] = s7 >> 16; pick[2 * wd] = pk; pick[2 * wd + 1] = pk >> 16;
-            }
-          } else if (BITS == 2) {
+            for (int wd = 0; wd < 4; ++wd) selectors_4bit(cur[xq][wd], sel + 2 * wd, pick + 2 * wd);
+          } else if constexpr (BITS == 2) {
 #pragma unroll
-            for (int wd = 0; wd < 2; ++wd) {
-              const uint32_t raw = cur[xq][wd];
-              const uint32_t s0 = raw & 0x33333333u, s1 = (raw >> 2) & 0x33333333u;
-              sel[4 * wd] = s0; sel[4 * wd + 1] = s0 >> 16; sel[4 * wd + 2] = s1; sel[4 * wd + 3] = s1 >> 16;
-            }
+            for (int wd = 0; wd < 2; ++wd) selectors_2bit(cur[xq][wd], sel + 4 * wd);
           } else {
-            const uint32_t r0 = cur[xq][0], r1 = cur[xq][1], r2 = cur[xq][2];
-            const uint32_t ex = (((r0 >> 3) & 0x11111111u) | ((r1 >> 2) & 0x22222222u)) | ((r2 >> 1) & 0x44444444u);
-            const uint32_t d0 = r0 & 0x77777777u, d1 = r1 & 0x77777777u, d2 = r2 & 0x77777777u;
-            sel[0] = d0; sel[1] = d0 >> 16; sel[2] = d1; sel[3] = d1 >> 16;
-            sel[4] = d2; sel[5] = d2 >> 16; sel[6] = ex; sel[7] = ex >> 16;
+            selectors_3bit(cur[xq][0], cur[xq][1], cur[xq][2], sel);
           }
 #pragma unroll
           for (int c = 0; c < 2; ++c)

@@ -31,6 +31,7 @@
 
 #include "common.h"
 #include "device_util.h"
+#include "selectors.cuh"
 
 namespace lcd {
 
@@ -434,38 +435,21 @@ __device__ __forceinline__ void process_item(const uint8_t* item, const uint8_t*
   for (int h = 0; h < 2; ++h) {
     uint32_t sel_a[8], sel_b[8];    // selector words of rows g and g + 8: lookup l uses the low 16 bits of sel[l]
     uint32_t pick_a[8] = {0, 0, 0, 0, 0, 0, 0, 0}, pick_b[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    if (BITS == 4) {
+    if constexpr (BITS == 4) {
 #pragma unroll
-      for (int w = 0; w < 4; ++w) {     // word w: eight indices in natural order
-        const uint32_t ua = raw_a[(BITS == 4 ? 4 : 0) * h + (BITS == 4 ? w : 0)], ub = raw_b[(BITS == 4 ? 4 : 0) * h + (BITS == 4 ? w : 0)];
-        const uint32_t a7 = ua & 0x77777777u, b7 = ub & 0x77777777u;
-        const uint32_t ap = ((ua >> 1) & 0x44444444u) | 0x32103210u, bp = ((ub >> 1) & 0x44444444u) | 0x32103210u;
-        sel_a[2 * w] = a7; sel_a[2 * w + 1] = a7 >> 16; pick_a[2 * w] = ap; pick_a[2 * w + 1] = ap >> 16;
-        sel_b[2 * w] = b7; sel_b[2 * w + 1] = b7 >> 16; pick_b[2 * w] = bp; pick_b[2 * w + 1] = bp >> 16;
+      for (int w = 0; w < 4; ++w) {
+        selectors_4bit(raw_a[4 * h + w], sel_a + 2 * w, pick_a + 2 * w);
+        selectors_4bit(raw_b[4 * h + w], sel_b + 2 * w, pick_b + 2 * w);
       }
-    } else if (BITS == 2) {
+    } else if constexpr (BITS == 2) {
 #pragma unroll
       for (int w = 0; w < 2; ++w) {
-        const uint32_t ua = raw_a[2 * h + w], ub = raw_b[2 * h + w];
-        const uint32_t a0 = ua & 0x33333333u, a1 = (ua >> 2) & 0x33333333u;
-        const uint32_t b0 = ub & 0x33333333u, b1 = (ub >> 2) & 0x33333333u;
-        sel_a[4 * w] = a0; sel_a[4 * w + 1] = a0 >> 16; sel_a[4 * w + 2] = a1; sel_a[4 * w + 3] = a1 >> 16;
-        sel_b[4 * w] = b0; sel_b[4 * w + 1] = b0 >> 16; sel_b[4 * w + 2] = b1; sel_b[4 * w + 3] = b1 >> 16;
+        selectors_2bit(raw_a[2 * h + w], sel_a + 4 * w);
+        selectors_2bit(raw_b[2 * h + w], sel_b + 4 * w);
       }
     } else {
-      const uint32_t* ra = raw_a + 3 * h;
-      const uint32_t* rb = raw_b + 3 * h;
-      // bit b of columns 24..31 sits at bit 3 of the nibbles of word b: gather them into nibbles
-      const uint32_t xa = (((ra[0] >> 3) & 0x11111111u) | ((ra[1] >> 2) & 0x22222222u)) | ((ra[2] >> 1) & 0x44444444u);
-      const uint32_t xb = (((rb[0] >> 3) & 0x11111111u) | ((rb[1] >> 2) & 0x22222222u)) | ((rb[2] >> 1) & 0x44444444u);
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        const uint32_t da = ra[b] & 0x77777777u, db = rb[b] & 0x77777777u;
-        sel_a[2 * b] = da; sel_a[2 * b + 1] = da >> 16;
-        sel_b[2 * b] = db; sel_b[2 * b + 1] = db >> 16;
-      }
-      sel_a[6] = xa; sel_a[7] = xa >> 16;
-      sel_b[6] = xb; sel_b[7] = xb >> 16;
+      selectors_3bit(raw_a[3 * h], raw_a[3 * h + 1], raw_a[3 * h + 2], sel_a);
+      selectors_3bit(raw_b[3 * h], raw_b[3 * h + 1], raw_b[3 * h + 2], sel_b);
     }
     // four MMAs per plane: MMA j takes lookups 2j and 2j + 1 and staged words 2j, 2j + 1
 #pragma unroll
