@@ -21,15 +21,6 @@ static lcd_algo resolve_algo(const Problem& p, lcd_algo algo) {
   return kHaveDenseTc ? LCD_ALGO_DENSE_TC : LCD_ALGO_REFERENCE;
 }
 
-// LCD_ALGO_AUTO between 17 and 32 tokens on long rows: two launches of the register-table kernel (16 tokens, then
-// the rest) beat the tensor-core kernel, whose 128-token tile is mostly empty there and whose time grows with the
-// row length (measured on 4096 x 11008: 31.5 vs 41.0 us at M = 17, 46 vs 41 at M = 32 with 2-bit indices, 28.5 vs
-// 49 and 39 vs 49 with 3-bit ones; on rows of 4096 columns the two are within 5 % at M = 17 and the tensor-core
-// kernel wins from M = 24 on; from M = 64 it wins everywhere by 2 to 8 times).
-static bool two_chunks(const Problem& p, lcd_algo algo) {
-  return algo == LCD_ALGO_AUTO && p.act_bits == 4 && p.M > 16 && p.M <= 32 && p.K_pad >= 8192;
-}
-
 static bool small_m_family(lcd_algo a) {
   return a == LCD_ALGO_REGISTER_LUT || a == LCD_ALGO_BUCKET_LUT || a == LCD_ALGO_TC_LUT || a == LCD_ALGO_SHARED_BUCKET;
 }
@@ -79,12 +70,6 @@ static bool shape_problem(const void* header_host, int64_t M, Problem* p) {
 }
 
 static lcd_status workspace_for(const Problem& p, lcd_algo algo, size_t* bytes) {
-  if (two_chunks(p, algo)) {
-    Problem first = p;
-    first.M = 16;
-    *bytes = lut_gemv_workspace_bytes(&first, 1, LCD_ALGO_REGISTER_LUT);
-    return LCD_OK;
-  }
   const lcd_algo resolved = resolve_algo(p, algo);
   switch (resolved) {
     case LCD_ALGO_REFERENCE:
@@ -100,7 +85,7 @@ static lcd_status workspace_for(const Problem& p, lcd_algo algo, size_t* bytes) 
       return LCD_OK;
     case LCD_ALGO_DENSE_TC:
     case LCD_ALGO_DENSE_F16:
-      *bytes = dense_tc_workspace_bytes(p.M, p.K_pad);
+      *bytes = dense_tc_workspace_bytes(p);
       return LCD_OK;
     default:
       return LCD_ERR_INVALID_ARG;
@@ -176,18 +161,6 @@ extern "C" lcd_status lcd_lut_linear(const void* packed_weights_dev, const void*
   if (st != LCD_OK) return st;
   if (need > 0 && (!workspace || workspace_bytes < need)) return LCD_ERR_BUFFER_TOO_SMALL;
   if (need > 0 && !aligned(workspace, 256)) return LCD_ERR_INVALID_ARG;
-  if (two_chunks(p, algo)) {
-    // the second launch touches the scratch only after the first one has finished (stream order, dependency wait)
-    Problem part = p;
-    part.M = 16;
-    st = launch_lut_gemv(&part, 1, LCD_ALGO_REGISTER_LUT, workspace, workspace_bytes, status_word_dev, cuda_stream);
-    if (st != LCD_OK) return st;
-    part.M = p.M - 16;
-    part.act_idx = p.act_idx + 16 * (p.K_pad / 2);
-    part.act_scale = p.act_scale + 16;
-    part.y = p.y + 16 * p.ldy;
-    return launch_lut_gemv(&part, 1, LCD_ALGO_REGISTER_LUT, workspace, workspace_bytes, status_word_dev, cuda_stream);
-  }
   const lcd_algo resolved = resolve_algo(p, algo);
   switch (resolved) {
     case LCD_ALGO_REFERENCE:
@@ -336,6 +309,12 @@ static size_t fused_dense_bytes(const Problem& p) {
   return fused_dense_levels_bytes(p) + (size_t)round_up_u64((uint64_t)p.M * sizeof(float), 256);
 }
 
+static size_t fused_dense_total(const Problem* p, int count) {
+  size_t total = dense_takes_tensor_memory(p, count) ? lut_gemv_tc_workspace_bytes(p, count) : 0;
+  for (int i = 0; i < count; ++i) total += fused_dense_bytes(p[i]);
+  return total;
+}
+
 static lcd_status fused_problems(const lcd_fused_problem* problems, int count, lcd_algo algo, bool pointers,
                                  Problem* p, lcd_algo* resolved) {
   if (!problems || count < 1 || count > LCD_MAX_BATCH) return LCD_ERR_INVALID_ARG;
@@ -386,9 +365,7 @@ extern "C" lcd_status lcd_linear_fused_batch_workspace_bytes(const lcd_fused_pro
   if (st != LCD_OK) return st;
   if (!bytes) return LCD_ERR_INVALID_ARG;
   if (resolved == LCD_ALGO_DENSE_TC) {
-    size_t total = 0;
-    for (int i = 0; i < count; ++i) total += fused_dense_bytes(p[i]);
-    *bytes = total;
+    *bytes = fused_dense_total(p, count);
     return LCD_OK;
   }
   *bytes = lut_gemv_workspace_bytes(p, count, resolved);
@@ -406,30 +383,45 @@ extern "C" lcd_status lcd_linear_fused_batch(const lcd_fused_problem* problems, 
     // Many tokens: ONE launch transforms the inputs of all problems (Section 4.1, the operation sequence of
     // lcd_smooth_quantize_act) and writes the levels as the signed bytes the tensor-core kernel reads, in its order:
     // no packed 4-bit copy, no expansion pass.  Then that kernel, once per problem.
-    size_t need = 0;
-    for (int i = 0; i < count; ++i) need += fused_dense_bytes(p[i]);
+    // Projections of one call that share their input (q, k, v; gate, up) share its levels.  One launch of the
+    // tensor-memory kernel for all problems where it takes them.
+    const size_t need = fused_dense_total(p, count);
     if (!workspace || workspace_bytes < need) return LCD_ERR_BUFFER_TOO_SMALL;
     if (!aligned(workspace, 256)) return LCD_ERR_INVALID_ARG;
+    const bool tensor_memory = dense_takes_tensor_memory(p, count);
     lcd_act_problem acts[LCD_MAX_BATCH];
+    int n_acts = 0, act_of[LCD_MAX_BATCH];
     uint8_t* at = static_cast<uint8_t*>(workspace);
     for (int i = 0; i < count; ++i) {
-      acts[i].x_fp16 = p[i].x_fp16;
-      acts[i].M = p[i].M;
-      acts[i].K = p[i].K;
-      acts[i].ldx = p[i].ldx;
-      acts[i].inv_smooth = p[i].inv_smooth;
-      acts[i].static_scale = nullptr;
-      acts[i].act_idx = at;
-      acts[i].act_scale = reinterpret_cast<float*>(at + fused_dense_levels_bytes(p[i]));
+      act_of[i] = -1;
+      for (int j = 0; j < i; ++j)
+        if (p[j].x_fp16 == p[i].x_fp16 && p[j].M == p[i].M && p[j].K == p[i].K && p[j].ldx == p[i].ldx &&
+            p[j].inv_smooth == p[i].inv_smooth)
+          act_of[i] = act_of[j];
+      if (act_of[i] >= 0) continue;
+      lcd_act_problem& a = acts[n_acts];
+      a.x_fp16 = p[i].x_fp16;
+      a.M = p[i].M;
+      a.K = p[i].K;
+      a.ldx = p[i].ldx;
+      a.inv_smooth = p[i].inv_smooth;
+      a.static_scale = nullptr;
+      a.act_idx = at;
+      a.act_scale = reinterpret_cast<float*>(at + fused_dense_levels_bytes(p[i]));
       at += fused_dense_bytes(p[i]);
+      act_of[i] = n_acts++;
     }
-    st = launch_smooth_quantize_dense_levels(acts, count, p[0].bits, cuda_stream);
+    st = launch_smooth_quantize_dense_levels(acts, n_acts, p[0].bits, tensor_memory, cuda_stream);
     if (st != LCD_OK) return st;
     for (int i = 0; i < count; ++i) {
       p[i].act_bits = 4;
-      p[i].act_idx = acts[i].act_idx;
-      p[i].act_scale = acts[i].act_scale;
+      p[i].act_idx = acts[act_of[i]].act_idx;
+      p[i].act_scale = acts[act_of[i]].act_scale;
       p[i].dense_levels = true;
+    }
+    if (tensor_memory)
+      return launch_lut_gemv_tc(p, count, at, workspace_bytes - (size_t)(at - static_cast<uint8_t*>(workspace)), status_word_dev, cuda_stream);
+    for (int i = 0; i < count; ++i) {
       st = launch_dense_tc(p[i], false, nullptr, 0, status_word_dev, cuda_stream);
       if (st != LCD_OK) return st;
     }

@@ -42,7 +42,7 @@ struct Problem {
   int bits, C;
   const uint8_t* act_idx;   // device [M][K_pad/2] (4-bit levels + 8) or [M][K_pad] signed bytes (act_bits == 8)
   int act_bits = 4;         // 4 or 8; 16 = not quantised yet: the lookup kernel does Section 4.1 itself from x
-  bool dense_levels = false;          // act_idx already holds the signed bytes the int8 tensor-core kernel reads
+  bool dense_levels = false;          // act_idx already holds the signed bytes in the order of the kernel that takes the problem
   const void* x_fp16 = nullptr;       // act_bits == 16: device fp16 [M][ldx]
   int64_t ldx = 0;
   const float* inv_smooth = nullptr;  // act_bits == 16: device fp32 [K] or null
@@ -71,8 +71,8 @@ lcd_status launch_dbci(const float* weights, int64_t n, void* workspace, float* 
 lcd_status launch_reference(const Problem& p, void* stream);
 lcd_status launch_smooth_quantize_batch(const lcd_act_problem* probs, int count, void* stream);
 // The same transformation with the levels written as signed bytes [M][K_pad] in the order the int8 tensor-core kernel
-// reads them for this index width (act_idx of the problems points to that buffer)
-lcd_status launch_smooth_quantize_dense_levels(const lcd_act_problem* probs, int count, int bits, void* stream);
+// (tensor_memory: the tensor-memory kernel) reads them for this index width (act_idx of the problems points to that buffer)
+lcd_status launch_smooth_quantize_dense_levels(const lcd_act_problem* probs, int count, int bits, bool tensor_memory, void* stream);
 // LCD_ALGO_REGISTER_LUT / LCD_ALGO_BUCKET_LUT for up to LCD_MAX_BATCH problems of equal index width in one launch
 size_t lut_gemv_workspace_bytes(const Problem* probs, int count, lcd_algo algo);
 lcd_status launch_lut_gemv(const Problem* probs, int count, lcd_algo algo, void* workspace, size_t workspace_bytes,
@@ -84,11 +84,18 @@ lcd_status launch_lut_smem(const Problem* probs, int count, void* workspace, siz
                            int32_t* status_word, void* stream);
 // The family LCD_ALGO_AUTO stands for when every problem has at most 16 tokens.
 lcd_algo resolve_small_m(const Problem* probs, int count, lcd_algo algo);
-// LCD_ALGO_TC_LUT: the same arithmetic for up to 16 tokens with the looked-up bytes fed to tcgen05.mma kind::i8
+// LCD_ALGO_TC_LUT: the same arithmetic with the looked-up bytes fed to tcgen05.mma kind::i8 through tensor memory: stored
+// levels up to 32 tokens, any number of tokens with dense_levels (signed bytes written by launch_ready_levels).  Outside
+// that the register tables stand in.
+bool lut_gemv_tc_supported(const Problem* probs, int count);
+double lut_gemv_tc_estimate_us(const Problem* probs, int count);
+lcd_status launch_ready_levels(const Problem& p, void* out /* device [M][K_pad] */, void* stream);
 size_t lut_gemv_tc_workspace_bytes(const Problem* probs, int count);
 lcd_status launch_lut_gemv_tc(const Problem* probs, int count, void* workspace, size_t workspace_bytes,
                               int32_t* status_word, void* stream);
-size_t dense_tc_workspace_bytes(int64_t M, int64_t K_pad);
+// LCD_ALGO_DENSE_TC for several problems: whether the tensor-memory kernel (one launch for all of them) takes them
+bool dense_takes_tensor_memory(const Problem* probs, int count);
+size_t dense_tc_workspace_bytes(const Problem& p);
 lcd_status launch_dense_tc(const Problem& p, bool fp16_operands, void* workspace, size_t workspace_bytes,
                            int32_t* status_word, void* stream);
 

@@ -799,23 +799,6 @@ dense_i8_kernel(const __grid_constant__ CUtensorMap tmap_act, const DenseParams 
   if (threadIdx.x == 0 && *abort_flag && P.status) atomicExch(P.status, (int)LCD_ERR_TIMEOUT);
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_tiled() {
-  static EncodeTiledFn fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess)
-      return nullptr;
-    fn = reinterpret_cast<EncodeTiledFn>(p);
-  }
-  return fn;
-}
-
 int dense_sm_count() { return current_sm_count(); }
 
 template <int BITS, int BN>
@@ -924,7 +907,7 @@ lcd_status launch_dense_i8(const Problem& p, int8_t* levels, int32_t* status_wor
 struct TileShape { int bn, stage_clks, epilogue_clks; };
 constexpr TileShape kShapes[3] = {{128, 425, 0}, {192, 400, 6500}, {256, 535, 7500}};
 
-int pick_shape(int64_t M, int64_t N_pad, int64_t n_ks) {
+int pick_shape(int64_t M, int64_t N_pad, int64_t n_ks, int64_t* clocks = nullptr) {
   const int n_sm = dense_sm_count();
   int best = 0;
   int64_t best_cost = -1;
@@ -934,16 +917,58 @@ int pick_shape(int64_t M, int64_t N_pad, int64_t n_ks) {
     const int64_t cost = ((tiles + n_sm - 1) / n_sm) * (n_ks * t.stage_clks + t.epilogue_clks);
     if (best_cost < 0 || cost < best_cost) { best = i; best_cost = cost; }
   }
+  if (clocks) *clocks = best_cost;
   return best;
+}
+// Duration of one launch: the stage table at 1.9 GHz, 3 us before the first stage and after the last.
+double dense_estimate_us(const Problem& p) {
+  int64_t clocks = 0;
+  (void)pick_shape(p.M, p.N_pad, p.K_pad / kBK, &clocks);
+  return 3.0 + (double)clocks / 1900.0;
 }
 
 }  // namespace
 
-size_t dense_tc_workspace_bytes(int64_t M, int64_t K_pad) { return (size_t)round_up_u64((uint64_t)M * K_pad * 2, 256); }
+// The tensor-memory kernel is faster where this one's tiles, at least 128 tokens wide and a whole row long, leave SMs idle:
+// by the two kernels' estimates, and always up to 32 tokens.
+bool dense_takes_tensor_memory(const Problem* probs, int count) {
+  Problem ready[LCD_MAX_BATCH];
+  int64_t m = 0;
+  double dense_us = 0.0;
+  for (int i = 0; i < count; ++i) {
+    ready[i] = probs[i];
+    ready[i].act_bits = 4;
+    ready[i].dense_levels = true;
+    m = probs[i].M > m ? probs[i].M : m;
+    dense_us += dense_estimate_us(probs[i]);
+  }
+  if (!lut_gemv_tc_supported(ready, count)) return false;
+  return m <= 32 || lut_gemv_tc_estimate_us(ready, count) < dense_us;
+}
+
+namespace {
+size_t dense_levels_bytes(const Problem& p) { return (size_t)round_up_u64((uint64_t)p.M * p.K_pad * 2, 256); }
+}  // namespace
+
+// Expanded levels (fp16 at most), and behind them what the tensor-memory kernel needs where it takes the problem.
+size_t dense_tc_workspace_bytes(const Problem& p) {
+  return dense_levels_bytes(p) + (dense_takes_tensor_memory(&p, 1) ? lut_gemv_tc_workspace_bytes(&p, 1) : 0);
+}
 
 lcd_status launch_dense_tc(const Problem& p, bool fp16_operands, void* workspace, size_t workspace_bytes,
                            int32_t* status_word, void* stream) {
-  if (!p.dense_levels && (!workspace || workspace_bytes < dense_tc_workspace_bytes(p.M, p.K_pad))) return LCD_ERR_BUFFER_TOO_SMALL;
+  if (!p.dense_levels && (!workspace || workspace_bytes < dense_tc_workspace_bytes(p))) return LCD_ERR_BUFFER_TOO_SMALL;
+  if (!fp16_operands && !p.dense_levels && dense_takes_tensor_memory(&p, 1)) {
+    uint8_t* scratch = static_cast<uint8_t*>(workspace) + dense_levels_bytes(p);
+    Problem q = p;
+    if (!lut_gemv_tc_supported(&p, 1)) {       // too many tokens for the kernel to place the stored levels itself
+      const lcd_status st = launch_ready_levels(p, workspace, stream);
+      if (st != LCD_OK) return st;
+      q.act_idx = static_cast<const uint8_t*>(workspace);
+      q.dense_levels = true;
+    }
+    return launch_lut_gemv_tc(&q, 1, scratch, workspace_bytes - dense_levels_bytes(p), status_word, stream);
+  }
   if (p.M > 0x7fffffffLL / 2 || p.N > 0x7fffffffLL / 2) return LCD_ERR_UNSUPPORTED;
   if (p.bits == 4 && fp16_operands) return LCD_ERR_UNSUPPORTED;    // 4-bit indices: the int8 kernel only
   cudaStream_t s = static_cast<cudaStream_t>(stream);

@@ -978,6 +978,14 @@ int sm_count() { return current_sm_count(); }
 // LLaMA-70B-shaped MLP 46 vs 59.
 constexpr long long kSharedBucketMinItems = 32768;
 
+// From nine tokens on a warp-level MMA serves half as many rows, and the register tables are bound by that pipe; the
+// tensor-memory kernel is not, but pays about 2 us more per launch (tensor memory, the split tiles' second pass).
+// Measured at 16 tokens, 2 / 3 / 4 bit, register tables against tensor memory: 4096 x 4096 (4096 items) 8.0 / 8.2 / 10.9
+// vs 8.2 / 8.5 / 10.0 us, 4096 x 11008 (11008 items) 14.4 / 14.2 / 20.8 vs 10.3 / 10.9 / 14.7, LLaMA-7B-shaped layer
+// 28.3 / 28.8 / 44.2 vs 22.1 / 25.0 / 40.8, LLaMA-70B-shaped MLP 75.6 / 103 / 158 vs 59.5 / 68.6 / 120.  At 8 tokens the
+// register tables win on all but single matrices with long rows (7B layer 19.5 / 23.4 / 34.3 vs 21 / 24 / 41).
+constexpr long long kTensorMemoryMinItems = 8192;
+
 int planes_of(int bits, int kind) { return kind == kFixed16 ? 2 : (1 << bits); }
 
 struct ScratchLayout {
@@ -1024,14 +1032,19 @@ lcd_status launch_t(const GemvBatch& batch, int grid, size_t smem, int32_t* stat
 // and the launch has enough rows per CTA to pay for building them, else the register tables.
 lcd_algo resolve_small_m(const Problem* probs, int count, lcd_algo algo) {
   if (algo != LCD_ALGO_AUTO) return algo;
-  if (!lut_smem_supported(probs, count)) return LCD_ALGO_REGISTER_LUT;
   long long items = 0;
-  for (int i = 0; i < count; ++i) items += (probs[i].N_pad / kPairRows) * (probs[i].K_pad / kTileK);
-  return items >= kSharedBucketMinItems ? LCD_ALGO_SHARED_BUCKET : LCD_ALGO_REGISTER_LUT;
+  int64_t m = 0;
+  for (int i = 0; i < count; ++i) {
+    items += (probs[i].N_pad / kPairRows) * (probs[i].K_pad / kTileK);
+    m = probs[i].M > m ? probs[i].M : m;
+  }
+  if (items >= kSharedBucketMinItems && lut_smem_supported(probs, count)) return LCD_ALGO_SHARED_BUCKET;
+  if (m > 8 && items >= kTensorMemoryMinItems && lut_gemv_tc_supported(probs, count)) return LCD_ALGO_TC_LUT;
+  return LCD_ALGO_REGISTER_LUT;
 }
 
 size_t lut_gemv_workspace_bytes(const Problem* probs, int count, lcd_algo algo) {
-  if (algo == LCD_ALGO_TC_LUT) return lut_gemv_tc_workspace_bytes(probs, count);
+  if (algo == LCD_ALGO_TC_LUT && lut_gemv_tc_supported(probs, count)) return lut_gemv_tc_workspace_bytes(probs, count);
   if (algo == LCD_ALGO_SHARED_BUCKET) return lut_smem_workspace_bytes(probs, count);
   const int kind = algo == LCD_ALGO_BUCKET_LUT ? kBuckets : kFixed16;
   int64_t max_m = 1;
@@ -1046,7 +1059,8 @@ size_t lut_gemv_workspace_bytes(const Problem* probs, int count, lcd_algo algo) 
 lcd_status launch_lut_gemv(const Problem* probs, int count, lcd_algo algo, void* workspace, size_t workspace_bytes,
                            int32_t* status_word, void* stream) {
   if (count < 1 || count > LCD_MAX_BATCH) return LCD_ERR_INVALID_ARG;
-  if (algo == LCD_ALGO_TC_LUT) return launch_lut_gemv_tc(probs, count, workspace, workspace_bytes, status_word, stream);
+  if (algo == LCD_ALGO_TC_LUT && lut_gemv_tc_supported(probs, count))
+    return launch_lut_gemv_tc(probs, count, workspace, workspace_bytes, status_word, stream);
   if (algo == LCD_ALGO_SHARED_BUCKET) return launch_lut_smem(probs, count, workspace, workspace_bytes, status_word, stream);
   const int kind = algo == LCD_ALGO_BUCKET_LUT ? kBuckets : kFixed16;
   const int bits = probs[0].bits;

@@ -27,8 +27,21 @@ __device__ __forceinline__ uint32_t quant_nibble(float v) {
 // lcd_smooth_quantize_act returns).  kOutBytes / kOutBytes2: the levels q as signed bytes, [K_pad] per token, for
 // the tensor-core kernel that follows in the same call: in column order, or in the order in which the 2-bit
 // decoder lists the weights of a 32-column quarter (position 16*(c>>4) + 8*(c&1) + 4*((c>>3)&1) + ((c>>1)&3)
-// holds column c).
-constexpr int kOutNibbles = 0, kOutBytes = 1, kOutBytes2 = 2;
+// holds column c).  kOutTc / kOutTc2: the same bytes in the operand order of the tensor-memory kernel for 3- and 4-bit / for
+// 2-bit indices (tc_word below).
+constexpr int kOutNibbles = 0, kOutBytes = 1, kOutBytes2 = 2, kOutTc = 3, kOutTc2 = 4;
+
+// Operand order of the tensor-memory kernel: in a 128-column block, word t of 16-byte chunk c holds four columns of quarter
+// t.  The eight columns from k on (a multiple of 8) are two such words, tc_second words apart: 3 and 4 bit the first and
+// the last four columns, 2 bit the even and the odd ones.
+template <int OUT, typename Index>
+__device__ __forceinline__ uint32_t* tc_word(uint8_t* row, Index k) {
+  const int t = (int)(k >> 5) & 3, jj = (int)(k >> 3) & 3;
+  const int c = OUT == kOutTc2 ? 4 * (jj >> 1) + (jj & 1) : 2 * jj;
+  return reinterpret_cast<uint32_t*>(row + (k & ~(Index)127) + 16 * c + 4 * t);
+}
+template <int OUT>
+__host__ __device__ constexpr int tc_second() { return OUT == kOutTc2 ? 8 : 4; }
 
 __device__ __forceinline__ uint32_t prmt_q(uint32_t a, uint32_t b, uint32_t sel) {
   uint32_t d;
@@ -47,6 +60,10 @@ __device__ __forceinline__ void store_levels8(uint8_t* row, Index k, uint32_t pa
   o = (o + 0x78787878u) ^ 0x80808080u;
   if (OUT == kOutBytes) {
     *reinterpret_cast<uint2*>(row + k) = make_uint2(prmt_q(e, o, 0x5140u), prmt_q(e, o, 0x7362u));
+  } else if (OUT == kOutTc || OUT == kOutTc2) {
+    uint32_t* w = tc_word<OUT>(row, k);
+    w[0] = OUT == kOutTc2 ? e : prmt_q(e, o, 0x5140u);
+    w[tc_second<OUT>()] = OUT == kOutTc2 ? o : prmt_q(e, o, 0x7362u);
   } else {
     const Index quarter = k & ~(Index)31;
     const int c8 = (int)(k & 31) >> 3;                  // which eight columns of the quarter
@@ -60,6 +77,8 @@ template <int OUT>
 __device__ __forceinline__ void store_level1(uint8_t* row, int64_t k, uint32_t a) {
   const uint8_t q = (uint8_t)((a - 8u) & 0xffu);
   if (OUT == kOutBytes) row[k] = q;
+  else if (OUT == kOutTc) reinterpret_cast<uint8_t*>(tc_word<OUT>(row, k) + ((k >> 2) & 1) * tc_second<OUT>())[k & 3] = q;
+  else if (OUT == kOutTc2) reinterpret_cast<uint8_t*>(tc_word<OUT>(row, k) + (k & 1) * tc_second<OUT>())[(k >> 1) & 3] = q;
   else {
     const int c = (int)(k & 31);
     row[(k & ~(int64_t)31) + 16 * (c >> 4) + 8 * (c & 1) + 4 * ((c >> 3) & 1) + ((c >> 1) & 3)] = q;
@@ -370,6 +389,10 @@ __device__ __forceinline__ void smooth_quantize_token_words(const __half* __rest
         *reinterpret_cast<uint32_t*>(out + k / 2) = (e & 0x0f0f0f0fu) | ((o & 0x0f0f0f0fu) << 4);
       } else if (OUT == kOutBytes) {
         *reinterpret_cast<uint2*>(out + k) = make_uint2(prmt_q(e, o, 0x5140u), prmt_q(e, o, 0x7362u));
+      } else if (OUT == kOutTc || OUT == kOutTc2) {
+        uint32_t* w = tc_word<OUT>(out, k);
+        w[0] = OUT == kOutTc2 ? e : prmt_q(e, o, 0x5140u);
+        w[tc_second<OUT>()] = OUT == kOutTc2 ? o : prmt_q(e, o, 0x7362u);
       } else {
         const int c8 = (k & 31) >> 3;                  // which eight columns of the 32-column quarter
         uint8_t* dst = out + (k & ~31) + 16 * (c8 >> 1) + 4 * (c8 & 1);
@@ -441,7 +464,7 @@ cudaError_t launch_small_ctas(const cudaLaunchConfig_t& cfg, long long chunks, c
 }
 
 // out_form: kOutNibbles (act_idx = [M][K_pad / 2]) or signed bytes for the tensor-core kernel (act_idx = [M][K_pad],
-// kOutBytes in column order, kOutBytes2 in the 2-bit decoder's order).
+// kOutBytes in column order, kOutBytes2 in the 2-bit decoder's order, kOutTc / kOutTc2 for the tensor-memory kernel).
 lcd_status launch_quantize_form(const lcd_act_problem* probs, int count, int out_form, void* stream) {
   QuantProblem all[LCD_MAX_BATCH];
   long long tokens = 0;
@@ -459,7 +482,7 @@ lcd_status launch_quantize_form(const lcd_act_problem* probs, int count, int out
     q.cta0 = (int)a.M;          // (the token count until the launches are formed below)
     q.vec = (reinterpret_cast<uintptr_t>(a.x_fp16) % 16 == 0) && (a.ldx % 8 == 0) && (a.K % 8 == 0) &&
             (a.inv_smooth == nullptr || reinterpret_cast<uintptr_t>(a.inv_smooth) % 16 == 0) &&
-            (reinterpret_cast<uintptr_t>(a.act_idx) % (out_form == kOutNibbles ? 4 : 8) == 0);
+            (reinterpret_cast<uintptr_t>(a.act_idx) % (out_form == kOutNibbles ? 4 : 16) == 0);
     tokens += a.M;
     if (tokens > 0x7fffffffLL) return LCD_ERR_INVALID_ARG;
   }
@@ -508,6 +531,8 @@ lcd_status launch_quantize_form(const lcd_act_problem* probs, int count, int out
                : cudaLaunchKernelEx(&cfg, smooth_quantize_kernel<kQThreads, 0>, batch);
     else if (out_form == kOutBytes) e = launch_small_ctas<kOutBytes>(cfg, inst, batch);
     else if (out_form == kOutBytes2) e = launch_small_ctas<kOutBytes2>(cfg, inst, batch);
+    else if (out_form == kOutTc) e = launch_small_ctas<kOutTc>(cfg, inst, batch);
+    else if (out_form == kOutTc2) e = launch_small_ctas<kOutTc2>(cfg, inst, batch);
     else e = launch_small_ctas<kOutNibbles>(cfg, inst, batch);
     if (e != cudaSuccess) {
       set_cuda_error((int)e);
@@ -523,8 +548,8 @@ lcd_status launch_smooth_quantize_batch(const lcd_act_problem* probs, int count,
   return launch_quantize_form(probs, count, kOutNibbles, stream);
 }
 
-lcd_status launch_smooth_quantize_dense_levels(const lcd_act_problem* probs, int count, int bits, void* stream) {
-  return launch_quantize_form(probs, count, bits == 2 ? kOutBytes2 : kOutBytes, stream);
+lcd_status launch_smooth_quantize_dense_levels(const lcd_act_problem* probs, int count, int bits, bool tensor_memory, void* stream) {
+  return launch_quantize_form(probs, count, tensor_memory ? (bits == 2 ? kOutTc2 : kOutTc) : bits == 2 ? kOutBytes2 : kOutBytes, stream);
 }
 
 lcd_status launch_smooth_quantize(const void* x, int64_t M, int64_t K, int64_t ldx, const float* inv_smooth,
