@@ -905,10 +905,13 @@ struct TcPlan {
   size_t parts_bytes, flags_bytes;
   double us;                 // estimated duration
 };
-// One token width: the grid with the shortest estimate.  Measured on B200 (microseconds): a unit 0.33 / 0.35 / 0.57 at
-// up to 32 / 64 / 128 tokens, 2 bit (3 bit 5 % more; 4 bit 0.68 at any width: its lookups); 3 before the first unit and
-// after the last store; a tile's drain 0.016 a token; a cut tile 2.5 for the hand-over, and 512 bytes a token and part at
-// 20 GB/s per SM to read the parts back.  Candidates: all SMs (least work per CTA, most tiles cut), and, where the rows are
+// One token width: the grid with the shortest estimate.  Measured on B200 (microseconds): a unit 0.33 / 0.35 / 0.68 at
+// up to 32 / 64 / 128 tokens, 2 bit (3 bit 5 % more; 4 bit 0.68 / 0.68 / 0.88: its lookups; 128 tokens take 0.57 in a launch
+// of a few units per SM, 0.83 in one of a millisecond, as the dense kernel's stages lengthen too); 3 before the first unit
+// and after the last store; a tile's drain 0.016 a token; a cut tile 2.5 for the hand-over, and 512 bytes a token and part
+// at 20 GB/s per SM to read the parts back.  Against the dense kernel this chooses right to a few percent (2 bit, one call
+// from x to y, tensor memory / dense): 13B layer 127 / 224 at 256 tokens, 254 / 299 at 512, 500 / 544 at 1024, 1060 / 975 at
+// 2048; 7B layer 57 / 179 at 128, 320 / 348 at 1024, 684 / 637 at 2048; layer of 1024 columns 79 / 100 at 2048.  Candidates: all SMs (least work per CTA, most tiles cut), and, where the rows are
 // of one length, one to four CTAs per tile (no tile cut with one).
 TcPlan tc_plan_width(const Problem* probs, int count, int nt) {
   TcPlan q = {};
@@ -931,7 +934,7 @@ TcPlan tc_plan_width(const Problem* probs, int count, int nt) {
   const unsigned long long piece = (unsigned long long)(max_kt + 15) / 16, n_sm = (unsigned long long)tc_sm_count();
   unsigned long long most = n_sm < q.units ? n_sm : q.units;
   if (most > q.units / piece) most = q.units / piece;
-  const double unit_us = probs[0].bits == 4 ? 0.68 : (nt <= 32 ? 0.33 : nt == 64 ? 0.35 : 0.57) * (probs[0].bits == 3 ? 1.05 : 1.0);
+  const double unit_us = probs[0].bits == 4 ? (nt == 128 ? 0.88 : 0.68) : (nt <= 32 ? 0.33 : nt == 64 ? 0.35 : 0.68) * (probs[0].bits == 3 ? 1.05 : 1.0);
   const double tokens = (double)(max_m < nt ? max_m : nt);
   for (int s = 0; s <= 4; ++s) {
     unsigned long long grid = most;
