@@ -24,12 +24,16 @@ struct PerDeviceFlag {
   }
 };
 
-// Multiprocessors of the current device (148 if it cannot be asked).
+// Multiprocessors of the current device (148 if it cannot be asked).  Asked of the runtime once per device: the query costs
+// as much as a tenth of a launch and every call needs the number.
 inline int current_sm_count() {
+  static std::atomic<int> known[64];
   int dev = 0, n = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
-    n = 148;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 148;
+  const bool slot = dev >= 0 && dev < 64;
+  if (slot && (n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) return 148;
+  if (slot) known[dev].store(n, std::memory_order_relaxed);
   return n;
 }
 
