@@ -380,7 +380,8 @@ lcd_status lcd_linear_host(const void* packed_weights_dev, const void* header_ho
                            size_t scratch_bytes, int32_t* status_word_dev, void* cuda_stream);
 
 /* The same for up to LCD_MAX_BATCH independent problems with M <= 16 and equal index width (the projections of
- * a decoder layer): ONE host-to-device copy of all inputs, one grouped quantise launch, one grouped lookup
+ * a decoder layer): ONE host-to-device copy of all inputs (by a kernel
+ * that reads x_host_all itself up to 512 KB of pinned memory), one grouped quantise launch, one grouped lookup
  * launch (a single launch that does both when every problem has one token), ONE device-to-host copy of all
  * outputs (none when the outputs total at most 512 KB and y_host_all is pinned memory the device can address: the
  * kernels then store y into it directly).  The host staging buffers are laid out by the library:

@@ -484,6 +484,48 @@ extern "C" lcd_status lcd_dbci(const float* weights, int64_t n, void* workspace,
 
 // ---- host-buffer path -------------------------------------------------------------------------------
 namespace {
+// A small input is read by a kernel straight from the caller's pinned buffer: a copy on the copy engine takes 6 us from
+// its start to the kernel that follows it, whatever its size, this one 2.5 (7B layer, one token, 71 KB: 46 -> 36 us end
+// to end).  Above kGatherBytes the copy engine's rate wins.
+constexpr size_t kGatherBytes = 512 << 10;
+__global__ void __launch_bounds__(256) gather_host_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, unsigned n) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const unsigned i = blockIdx.x * 256 + threadIdx.x;
+  // dst may still be read, and the host buffer still be written (as another call's output), by the kernels before this one
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (i >= n) return;
+  uint4 v;
+  asm volatile("ld.volatile.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(src + i));
+  dst[i] = v;
+}
+// The device's address of pinned host memory, or null.
+void* mapped_host(const void* p) {
+  cudaPointerAttributes attr;
+  if (cudaPointerGetAttributes(&attr, p) == cudaSuccess && attr.type == cudaMemoryTypeHost) return attr.devicePointer;
+  (void)cudaGetLastError();
+  return nullptr;
+}
+lcd_status copy_in(void* dst, const void* src_host, size_t bytes, cudaStream_t stream) {
+  const void* mapped = bytes <= kGatherBytes && bytes % 16 == 0 && aligned(src_host, 16) ? mapped_host(src_host) : nullptr;
+  cudaError_t e;
+  if (mapped) {
+    const unsigned n = (unsigned)(bytes / 16);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((n + 255) / 256);
+    cfg.blockDim = dim3(256);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, gather_host_kernel, static_cast<const uint4*>(mapped), static_cast<uint4*>(dst), n);
+  } else {
+    e = cudaMemcpyAsync(dst, src_host, bytes, cudaMemcpyHostToDevice, stream);
+  }
+  if (e != cudaSuccess) { set_cuda_error((int)e); return LCD_ERR_CUDA; }
+  return LCD_OK;
+}
 struct HostScratch {
   size_t x_off, idx_off, scale_off, y_off, ws_off, ws_bytes, total;
 };
@@ -530,8 +572,8 @@ extern "C" lcd_status lcd_linear_host(const void* packed_weights_dev, const void
   if (!aligned(scratch, 256)) return LCD_ERR_INVALID_ARG;
   uint8_t* base = static_cast<uint8_t*>(scratch);
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-  cudaError_t e = cudaMemcpyAsync(base + s.x_off, x_host_fp16, (size_t)M * h.K * 2, cudaMemcpyHostToDevice, stream);
-  if (e != cudaSuccess) { set_cuda_error((int)e); return LCD_ERR_CUDA; }
+  st = copy_in(base + s.x_off, x_host_fp16, (size_t)M * h.K * 2, stream);
+  if (st != LCD_OK) return st;
   uint8_t* idx = base + s.idx_off;
   float* scale = reinterpret_cast<float*>(base + s.scale_off);
   float* y = reinterpret_cast<float*>(base + s.y_off);
@@ -542,7 +584,7 @@ extern "C" lcd_status lcd_linear_host(const void* packed_weights_dev, const void
   st = lcd_lut_linear(packed_weights_dev, header_host, idx, scale, M, y, (int64_t)h.N, LCD_ALGO_AUTO,
                       s.ws_bytes ? base + s.ws_off : nullptr, s.ws_bytes, status_word_dev, cuda_stream);
   if (st != LCD_OK) return st;
-  e = cudaMemcpyAsync(y_host, y, (size_t)M * h.N * 4, cudaMemcpyDeviceToHost, stream);
+  const cudaError_t e = cudaMemcpyAsync(y_host, y, (size_t)M * h.N * 4, cudaMemcpyDeviceToHost, stream);
   if (e != cudaSuccess) { set_cuda_error((int)e); return LCD_ERR_CUDA; }
   return LCD_OK;
 }
@@ -612,8 +654,8 @@ extern "C" lcd_status lcd_linear_host_batch(const lcd_host_problem* problems, in
   if (!aligned(scratch, 256)) return LCD_ERR_INVALID_ARG;
   uint8_t* base = static_cast<uint8_t*>(scratch);
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-  cudaError_t e = cudaMemcpyAsync(base, x_host_all, L.x_bytes, cudaMemcpyHostToDevice, stream);   // one copy in
-  if (e != cudaSuccess) { set_cuda_error((int)e); return LCD_ERR_CUDA; }
+  st = copy_in(base, x_host_all, L.x_bytes, stream);
+  if (st != LCD_OK) return st;
   // A small y goes straight into the caller's buffer when the device can address it (pinned, mapped host memory): the
   // kernels' stores cross the bus themselves and there is no copy out (7B layer, one token, 170 KB: 46 instead of
   // 59 us end to end).  Larger outputs are copied: the kernels store 32-byte pieces, which the bus takes badly
@@ -621,11 +663,7 @@ extern "C" lcd_status lcd_linear_host_batch(const lcd_host_problem* problems, in
   constexpr size_t kDirectOutputBytes = 512 << 10;
   uint8_t* y_direct = nullptr;
   if (L.y_bytes <= kDirectOutputBytes) {
-    cudaPointerAttributes attr;
-    if (cudaPointerGetAttributes(&attr, y_host_all) == cudaSuccess && attr.type == cudaMemoryTypeHost && attr.devicePointer)
-      y_direct = static_cast<uint8_t*>(attr.devicePointer);
-    else
-      (void)cudaGetLastError();
+    y_direct = static_cast<uint8_t*>(mapped_host(y_host_all));
   }
   lcd_act_problem acts[LCD_MAX_BATCH];
   Problem p[LCD_MAX_BATCH];
@@ -665,7 +703,7 @@ extern "C" lcd_status lcd_linear_host_batch(const lcd_host_problem* problems, in
                        cuda_stream);
   if (st != LCD_OK) return st;
   if (!y_direct) {
-    e = cudaMemcpyAsync(y_host_all, base + L.y_off[0], L.y_bytes, cudaMemcpyDeviceToHost, stream);   // one copy out
+    const cudaError_t e = cudaMemcpyAsync(y_host_all, base + L.y_off[0], L.y_bytes, cudaMemcpyDeviceToHost, stream);   // one copy out
     if (e != cudaSuccess) { set_cuda_error((int)e); return LCD_ERR_CUDA; }
   }
   return LCD_OK;
