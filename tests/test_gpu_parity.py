@@ -759,3 +759,24 @@ def test_dbci_matches_oracle(case):
     assert np.array_equal(r["labels"].cpu().numpy().astype(np.int64), ref["labels"])
     assert r["n_noise"] == int((ref["labels"] < 0).sum())
     assert np.array_equal(r["centroids"].cpu().numpy().astype(np.float64), ref["centroids"])
+
+
+@pytest.mark.parametrize("n", [4095, 4096, 4097, 8193, 20000])
+@pytest.mark.parametrize("outliers", [2, 70, 200])
+def test_dbci_clusters_across_tile_edges(n, outliers):
+    # clumps of many sizes, duplicates and isolated weights between them; the seed clusters' size sets MinPts on both
+    # sides of the clump sizes, so that core, border and noise points lie next to each other all along the array
+    rng = np.random.default_rng(n + outliers)
+    centres = np.sort(rng.uniform(-0.1, 0.1, 40))
+    sizes = rng.integers(1, 400, 40)
+    body = np.concatenate([c + np.round(rng.normal(0, 2e-4, s), 5) for c, s in zip(centres, sizes)])
+    body = np.resize(body, n - 2 * outliers)
+    w = np.concatenate([body, 0.5 + rng.normal(0, 1e-4, outliers), -0.5 + rng.normal(0, 1e-4, outliers)]).astype(np.float32)
+    r = lcd.dbci(torch.from_numpy(w).cuda(), max_centroids=4096)
+    torch.cuda.synchronize()
+    ref = O.dbci_scan(w)
+    assert np.array_equal(r["sorted"].cpu().numpy(), ref["sorted"])
+    assert (r["sigma"], r["eps"], r["min_pts"]) == (ref["sigma"], ref["eps"], ref["min_pts"])
+    assert np.array_equal(r["labels"].cpu().numpy().astype(np.int64), ref["labels"])
+    assert r["n_noise"] == int((ref["labels"] < 0).sum())
+    assert np.array_equal(r["centroids"].cpu().numpy().astype(np.float64), ref["centroids"])
