@@ -3,7 +3,7 @@
 //   a weight of cluster i with update dw moves to i - 1 when dw < -(C_i - C_{i-1}) / 2, to i + 1 when
 //   dw > (C_{i+1} - C_i) / 2 (binary32: one subtraction, one halving; edge clusters have one side);
 //   dC_j = sum over the weights that end up in j of (dw + (C_old - C_j)), counts alongside.
-// One CTA per row; per-thread compensated sums, combined in binary64 in a fixed order: results are reproducible.
+// One CTA per row; per-thread binary64 sums, combined in a fixed order: results are reproducible.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -23,9 +23,12 @@ __global__ void __launch_bounds__(kRcThreads) reclassify_kernel(const uint8_t* _
                                                                 uint8_t* __restrict__ new_idx, double* __restrict__ delta_c,
                                                                 int32_t* __restrict__ counts, const bool vec) {
   __shared__ float s_c[CMAX];
+  __shared__ double2 s_step[CMAX];          // C_i - C_{i-1} and C_i - C_{i+1}: what a weight of cluster i that moves brings along
+  __shared__ int s_total[3][4];             // packed counts of the CTA
   __shared__ float2 s_gap[CMAX];            // half-gaps (C_i - C_{i-1}) / 2 and (C_{i+1} - C_i) / 2, infinite at the edges
   const int64_t n = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid < 12) s_total[tid >> 2][tid & 3] = 0;
   if (tid < C) s_c[tid] = __half2float(__ushort_as_half(codebook[n * C + tid]));
   __syncthreads();
   if (tid < CMAX) {
@@ -33,54 +36,88 @@ __global__ void __launch_bounds__(kRcThreads) reclassify_kernel(const uint8_t* _
     s_gap[tid] = make_float2((tid > 0 && tid < C) ? __fmul_rn(__fsub_rn(s_c[tid], s_c[tid - 1]), 0.5f) : inf,
                              (tid < C - 1) ? __fmul_rn(__fsub_rn(s_c[tid + 1], s_c[tid]), 0.5f) : inf);
   }
-  __syncthreads();
-  // Per thread and cluster, in the thread's own column of shared memory (indexed by the data-dependent cluster; a
-  // register array would need one predicated copy of every operation per cluster): the sum of the arriving updates
-  // as an unevaluated pair of binary32 numbers (error-free two-sum: binary64 adds are scarce on this part) and
-  // integer counts of members and of arrivals from either side; the centroid differences of the arrivals are
-  // added at the end from the counts.
-  extern __shared__ uint4 s_dyn[];
-  // one 16-byte slot per thread and cluster: (hi, lo, counts low word, counts high word); the 64-bit count word is
-  // members | arrivals from the left << 21 | arrivals from the right << 42.  One load and one store per weight: the
-  // load/store unit's queue is what bounds this kernel.
-  uint4* s_slot = s_dyn;                                                  // [CMAX][kRcThreads]
+  // Per thread and cluster, in the thread's own column of shared memory (indexed by the data-dependent cluster; a register
+  // array would need one predicated copy of every operation per cluster): the binary64 sum of the arriving updates.  Members
+  // and arrivals from either side are counted, the arrivals' centroid differences added at the end from the counts: up to
+  // four clusters in bytes of three registers, emptied in time into a count per lane (4 bits of cluster and kind), up to
+  // eight in shared memory.  With more the counts' space would halve the CTAs on an SM: there the differences are added
+  // weight by weight and only the members are counted.  The shared-memory pipe bounds the kernel: a weight takes six passes
+  // through it here (thirteen when a slot of sixteen bytes held an error-free binary32 pair and the counts).  4096 x 4096,
+  // 4 / 8 / 16 clusters: 31 / 45 / 58 us (43 / 56 / 89 then).
+  extern __shared__ double s_sum[];                                             // [CMAX][kRcThreads]
+  constexpr bool kPacked = CMAX <= 4, kSteps = CMAX > 8;
+  int* s_count = reinterpret_cast<int*>(s_sum + CMAX * kRcThreads);             // [1 or 3][CMAX][kRcThreads]: members, from left, from right
 #pragma unroll
-  for (int c = 0; c < CMAX; ++c) s_slot[c * kRcThreads + tid] = make_uint4(0u, 0u, 0u, 0u);
+  for (int c = 0; c < CMAX; ++c) {
+    s_sum[c * kRcThreads + tid] = 0.0;
+    if (!kPacked) {
+#pragma unroll
+      for (int f = 0; f < (kSteps ? 1 : 3); ++f) s_count[(f * CMAX + c) * kRcThreads + tid] = 0;
+    }
+  }
+  if (kSteps && tid < CMAX)
+    s_step[tid] = make_double2((tid > 0 && tid < C) ? (double)s_c[tid] - (double)s_c[tid - 1] : 0.0,
+                               (tid < C - 1) ? (double)s_c[tid] - (double)s_c[tid + 1] : 0.0);
+  __syncthreads();
   const uint8_t* ir = idx + n * K;
   const float* dr = delta_w + n * ldw;
   uint8_t* outr = new_idx + n * K;
-  // branch-free: s_gap[i] = (half-gap to the left, half-gap to the right) of cluster i, infinite at the edges.
+  uint32_t members = 0, from_left = 0, from_right = 0;
   // An index is reduced to the table size CMAX before it addresses shared memory, so a byte >= C (the caller's
   // error) cannot reach outside the slots: such a weight keeps its reduced index and is counted in no cluster.
   auto one = [&](int i, float dw) {
     const float2 gap = s_gap[i];
-    const int left = dw < -gap.x ? 1 : 0;
-    const int right = (dw > gap.y ? 1 : 0) & (left ^ 1);
-    const int j = i - left + right;
-    const int slot = j * kRcThreads + tid;
-    uint4 v = s_slot[slot];
-    const float h = __uint_as_float(v.x), l = __uint_as_float(v.y);
-    const float t = __fadd_rn(h, dw);                            // two-sum of (hi, dw)
-    const float bb = __fsub_rn(t, h);
-    const float err = __fadd_rn(__fsub_rn(h, __fsub_rn(t, bb)), __fsub_rn(dw, bb));
-    unsigned long long cnt = ((unsigned long long)v.w << 32) | v.z;
-    cnt += 1ull + ((unsigned long long)right << 21) + ((unsigned long long)left << 42);
-    v.x = __float_as_uint(t);
-    v.y = __float_as_uint(__fadd_rn(l, err));
-    v.z = (uint32_t)cnt;
-    v.w = (uint32_t)(cnt >> 32);
-    s_slot[slot] = v;
+    const bool left = dw < -gap.x, right = !left && dw > gap.y;
+    const int j = i - (left ? 1 : 0) + (right ? 1 : 0);
+    double d = (double)dw;
+    if (kSteps && (left || right)) {
+      const double2 step = s_step[i];
+      d += left ? step.x : step.y;
+    }
+    s_sum[j * kRcThreads + tid] += d;
+    if (kPacked) {
+      const uint32_t one_j = 1u << (8 * j);
+      members += one_j;
+      from_left += right ? one_j : 0u;
+      from_right += left ? one_j : 0u;
+    } else {
+      int* at = s_count + j * kRcThreads + tid;
+      atomicAdd(at, 1);
+      if (!kSteps) {
+        if (right) atomicAdd(at + CMAX * kRcThreads, 1);
+        if (left) atomicAdd(at + 2 * CMAX * kRcThreads, 1);
+      }
+    }
     return (uint32_t)j;
   };
+  int total = 0;      // packed: lane 4 f + c: this warp's members (f = 0) of cluster c, arrivals from the left, from the right
+  auto empty = [&]() {
+    if (kPacked) {
+      const uint32_t w[3] = {members, from_left, from_right};
+#pragma unroll
+      for (int f = 0; f < 3; ++f) {
+        // bytes of the lanes' words, at most 255 each, summed in 16-bit fields
+        const uint32_t even = __reduce_add_sync(0xffffffffu, w[f] & 0x00ff00ffu), odd = __reduce_add_sync(0xffffffffu, (w[f] >> 8) & 0x00ff00ffu);
+        if ((lane >> 2) == f) total += (int)((((lane & 1) ? odd : even) >> ((lane & 2) ? 16 : 0)) & 0xffffu);
+      }
+      members = from_left = from_right = 0;
+    }
+  };
+  int step = 0;
   if (vec) {      // 16 weights per thread and step: one 16-byte index load, four 16-byte update loads, one 16-byte store
-    for (int64_t k = (int64_t)tid * 16; k < K; k += (int64_t)kRcThreads * 16) {
+    for (int64_t k0 = 0; k0 < K; k0 += (int64_t)kRcThreads * 16) {
+      if (kPacked && ++step == 16) { empty(); step = 1; }           // 240 weights since: no byte has overflowed
+      const int64_t k = k0 + (int64_t)tid * 16;
+      if (k >= K) continue;
       const uint4 iv = __ldg(reinterpret_cast<const uint4*>(ir + k));
       const uint32_t iw[4] = {iv.x, iv.y, iv.z, iv.w};
+      float4 d[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) d[q] = __ldg(reinterpret_cast<const float4*>(dr + k + 4 * q));
       uint32_t ow[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const float4 d = __ldg(reinterpret_cast<const float4*>(dr + k + 4 * q));
-        const float dv[4] = {d.x, d.y, d.z, d.w};
+        const float dv[4] = {d[q].x, d[q].y, d[q].z, d[q].w};
         uint32_t o = 0;
 #pragma unroll
         for (int e = 0; e < 4; ++e) o |= one((int)((iw[q] >> (8 * e)) & (uint32_t)(CMAX - 1)), dv[e]) << (8 * e);
@@ -89,50 +126,71 @@ __global__ void __launch_bounds__(kRcThreads) reclassify_kernel(const uint8_t* _
       *reinterpret_cast<uint4*>(outr + k) = make_uint4(ow[0], ow[1], ow[2], ow[3]);
     }
   } else {
-    for (int64_t k = tid; k < K; k += kRcThreads) outr[k] = (uint8_t)one(ir[k] & (CMAX - 1), dr[k]);
+    for (int64_t k0 = 0; k0 < K; k0 += kRcThreads) {
+      if (kPacked && ++step == 256) { empty(); step = 1; }
+      const int64_t k = k0 + tid;
+      if (k < K) outr[k] = (uint8_t)one(ir[k] & (CMAX - 1), dr[k]);
+    }
   }
-  // Block reduction of the pairs and counts, still in binary32 pairs (binary64 operations only on the C final values
-  // of the row: they are slow enough here that a few dozen per thread dominated the kernel), fixed order.
-  auto two_sum = [](float& h, float& l, float h2, float l2) {
-    const float t = __fadd_rn(h, h2);
-    const float bb = __fsub_rn(t, h);
-    const float err = __fadd_rn(__fsub_rn(h, __fsub_rn(t, bb)), __fsub_rn(h2, bb));
-    h = t;
-    l = __fadd_rn(__fadd_rn(l, l2), err);
-  };
-  // One warp folds the 256 columns of slots: every lane adds its eight columns, then a butterfly over the lanes.
-  // (A butterfly in every warp made this reduction as expensive as the 16 weights a thread handles per 4096 columns.)
+  empty();
+  if (kPacked && lane < 12) atomicAdd(&s_total[lane >> 2][lane & 3], total);
+  // A warp folds the 256 columns of slots of every eighth cluster: each lane adds its eight columns, then a butterfly over
+  // the lanes (a butterfly in every warp over its own columns costs as much as the row's weights).
   __syncthreads();
-  if (warp == 0) {
+  for (int c = warp; c < C; c += kRcThreads / 32) {
+    double sum = 0.0;
+    int q = 0, fl = 0, fr = 0;
 #pragma unroll
-    for (int c = 0; c < CMAX; ++c) {
-      float h = 0.0f, l = 0.0f;
-      unsigned long long c3 = 0ull;
-#pragma unroll
-      for (int w = 0; w < kRcThreads / 32; ++w) {
-        const uint4 sv = s_slot[c * kRcThreads + w * 32 + lane];
-        two_sum(h, l, __uint_as_float(sv.x), __uint_as_float(sv.y));
-        c3 += ((unsigned long long)sv.w << 32) | sv.z;          // K <= 2^25: a thread counts at most 2^17, eight of them 2^20 < 2^21
+    for (int w = 0; w < kRcThreads / 32; ++w) {
+      const int at = c * kRcThreads + w * 32 + lane;
+      sum += s_sum[at];
+      if (!kPacked) q += s_count[at];
+      if (!kPacked && !kSteps) {
+        fl += s_count[CMAX * kRcThreads + at];
+        fr += s_count[2 * CMAX * kRcThreads + at];
       }
-      // fields of the packed count word may carry into each other once summed over threads: unpack before the lanes meet
-      int q = (int)(c3 & 0x1fffffull), fl = (int)((c3 >> 21) & 0x1fffffull), fr = (int)((c3 >> 42) & 0x1fffffull);
+    }
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float h2 = __shfl_xor_sync(0xffffffffu, h, o), l2 = __shfl_xor_sync(0xffffffffu, l, o);
-        two_sum(h, l, h2, l2);
-        q += __shfl_xor_sync(0xffffffffu, q, o);
+    for (int o = 16; o > 0; o >>= 1) {
+      sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      if (!kPacked) q += __shfl_xor_sync(0xffffffffu, q, o);
+      if (!kPacked && !kSteps) {
         fl += __shfl_xor_sync(0xffffffffu, fl, o);
         fr += __shfl_xor_sync(0xffffffffu, fr, o);
       }
-      if (lane == 0 && c < C) {
-        double v = (double)h + (double)l;
-        if (c > 0) v += (double)fl * ((double)s_c[c - 1] - (double)s_c[c]);
-        if (c < C - 1) v += (double)fr * ((double)s_c[c + 1] - (double)s_c[c]);
-        delta_c[n * C + c] = v;
-        counts[n * C + c] = q;
-      }
+    }
+    if (kPacked) {
+      q = s_total[0][c & 3];
+      fl = s_total[1][c & 3];
+      fr = s_total[2][c & 3];
+    }
+    if (lane == 0) {
+      if (c > 0) sum += (double)fl * ((double)s_c[c - 1] - (double)s_c[c]);
+      if (c < C - 1) sum += (double)fr * ((double)s_c[c + 1] - (double)s_c[c]);
+      delta_c[n * C + c] = sum;
+      counts[n * C + c] = q;
     }
   }
+}
+
+template <int CMAX>
+lcd_status launch_rows(const uint8_t* idx, const uint16_t* codebook, const float* delta_w, int64_t N, int64_t K, int64_t ldw, int C,
+                       uint8_t* new_idx, double* delta_c, int32_t* counts, bool vec, cudaStream_t s) {
+  auto kern = reclassify_kernel<CMAX>;
+  constexpr int smem = CMAX * kRcThreads * (CMAX <= 4 ? 8 : CMAX <= 8 ? 20 : 12);
+  if (smem > 40 * 1024) {             // (with the static tables more than the 48 KB that need no opt-in)
+    static PerDeviceFlag attr_set;    // needs the opt-in, on every device
+    int dev;
+    if (attr_set.first(&dev)) {
+      const cudaError_t ea = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      if (ea != cudaSuccess) { set_cuda_error((int)ea); return LCD_ERR_CUDA; }
+      attr_set.done(dev);
+    }
+  }
+  kern<<<(unsigned)N, kRcThreads, smem, s>>>(idx, codebook, delta_w, K, ldw, C, new_idx, delta_c, counts, vec);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) { set_cuda_error((int)e); return LCD_ERR_CUDA; }
+  return LCD_OK;
 }
 
 }  // namespace
@@ -142,22 +200,9 @@ lcd_status launch_reclassify(const uint8_t* idx, const uint16_t* codebook, const
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
   const bool vec = K % 16 == 0 && ldw % 4 == 0 && al16(idx) && al16(delta_w) && al16(new_idx);
-  if (C <= 4) reclassify_kernel<4><<<(unsigned)N, kRcThreads, 4 * kRcThreads * 16, s>>>(idx, codebook, delta_w, K, ldw, C, new_idx, delta_c, counts, vec);
-  else if (C <= 8) reclassify_kernel<8><<<(unsigned)N, kRcThreads, 8 * kRcThreads * 16, s>>>(idx, codebook, delta_w, K, ldw, C, new_idx, delta_c, counts, vec);
-  else {
-    static PerDeviceFlag attr_set;    // 80 KB of dynamic shared memory needs the opt-in, on every device
-    int dev;
-    if (attr_set.first(&dev)) {
-      const cudaError_t ea = cudaFuncSetAttribute(reclassify_kernel<kRcMaxC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                  kRcMaxC * kRcThreads * 16);
-      if (ea != cudaSuccess) { set_cuda_error((int)ea); return LCD_ERR_CUDA; }
-      attr_set.done(dev);
-    }
-    reclassify_kernel<kRcMaxC><<<(unsigned)N, kRcThreads, kRcMaxC * kRcThreads * 16, s>>>(idx, codebook, delta_w, K, ldw, C, new_idx, delta_c, counts, vec);
-  }
-  const cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) { set_cuda_error((int)e); return LCD_ERR_CUDA; }
-  return LCD_OK;
+  if (C <= 4) return launch_rows<4>(idx, codebook, delta_w, N, K, ldw, C, new_idx, delta_c, counts, vec, s);
+  if (C <= 8) return launch_rows<8>(idx, codebook, delta_w, N, K, ldw, C, new_idx, delta_c, counts, vec, s);
+  return launch_rows<kRcMaxC>(idx, codebook, delta_w, N, K, ldw, C, new_idx, delta_c, counts, vec, s);
 }
 
 }  // namespace lcd
