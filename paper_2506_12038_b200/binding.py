@@ -7,7 +7,9 @@ library is missing, importing this module raises.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
+from array import array
 from ctypes import c_char_p, c_int, c_int64, c_size_t, c_void_p, POINTER, Structure, byref
 
 import numpy as np
@@ -287,6 +289,21 @@ class ActBatch:
                "lcd_smooth_quantize_act_batch")
 
 
+# Workspace sizes are functions of the sizes alone; asking costs as much as a launch.
+@functools.lru_cache(maxsize=64)
+def _dbci_workspace_bytes(n: int, max_centroids: int) -> int:
+    need = c_size_t(0)
+    _check(lib.lcd_dbci_workspace_bytes(n, max_centroids, byref(need)), "lcd_dbci_workspace_bytes")
+    return need.value
+
+
+@functools.lru_cache(maxsize=64)
+def _smoothing_workspace_bytes(T: int, K: int, G: int) -> int:
+    need = c_size_t(0)
+    _check(lib.lcd_smoothing_search_workspace_bytes(T, K, G, byref(need)), "lcd_smoothing_search_workspace_bytes")
+    return need.value
+
+
 def dbci(weights, max_centroids: int = 4096, want_labels: bool = True, stream=None):
     """Section 3.1 on a flat CUDA fp32 tensor.  Returns a dict: sigma, eps, min_pts, left, right, n_noise,
     n_clusters_found, centroids (CUDA fp32, ascending), sorted (CUDA fp32) and labels (CUDA int32, in sorted order)."""
@@ -294,14 +311,13 @@ def dbci(weights, max_centroids: int = 4096, want_labels: bool = True, stream=No
     w = weights.reshape(-1)
     assert w.is_cuda and w.dtype == torch.float32 and w.is_contiguous()
     n = w.numel()
-    need = c_size_t(0)
-    _check(lib.lcd_dbci_workspace_bytes(n, max_centroids, byref(need)), "lcd_dbci_workspace_bytes")
-    ws = torch.empty(need.value, dtype=torch.uint8, device=w.device)
+    need = _dbci_workspace_bytes(n, max_centroids)
+    ws = torch.empty(need, dtype=torch.uint8, device=w.device)
     cents = torch.empty((max_centroids,), dtype=torch.float32, device=w.device)
     labels = torch.empty((n,), dtype=torch.int32, device=w.device) if want_labels else None
     srt = torch.empty((n,), dtype=torch.float32, device=w.device)
     res = torch.zeros((ctypes.sizeof(DbciResult),), dtype=torch.uint8, device=w.device)
-    _check(lib.lcd_dbci(c_void_p(w.data_ptr()), n, c_void_p(ws.data_ptr()), need.value, c_void_p(cents.data_ptr()),
+    _check(lib.lcd_dbci(c_void_p(w.data_ptr()), n, c_void_p(ws.data_ptr()), need, c_void_p(cents.data_ptr()),
                         max_centroids, c_void_p(labels.data_ptr()) if labels is not None else None,
                         c_void_p(srt.data_ptr()), c_void_p(res.data_ptr()), _stream_ptr(stream)), "lcd_dbci")
     r = DbciResult.from_buffer_copy(res.cpu().numpy().tobytes())
@@ -327,9 +343,8 @@ def reclassify(idx, codebook, delta_w, stream=None, out=None):
         new_idx, delta_c, counts = out
         assert new_idx.dtype == torch.uint8 and delta_c.dtype == torch.float64 and counts.dtype == torch.int32
         assert new_idx.shape == idx.shape and delta_c.shape == (N, C) and counts.shape == (N, C)
-    _check(lib.lcd_reclassify(c_void_p(idx.data_ptr()), c_void_p(codebook.data_ptr()), c_void_p(delta_w.data_ptr()), N, K,
-                              delta_w.stride(0), C, c_void_p(new_idx.data_ptr()), c_void_p(delta_c.data_ptr()),
-                              c_void_p(counts.data_ptr()), _stream_ptr(stream)), "lcd_reclassify")
+    _check(lib.lcd_reclassify(idx.data_ptr(), codebook.data_ptr(), delta_w.data_ptr(), N, K, delta_w.stride(0), C,
+                              new_idx.data_ptr(), delta_c.data_ptr(), counts.data_ptr(), _stream_ptr(stream)), "lcd_reclassify")
     return new_idx, delta_c, counts
 
 
@@ -340,17 +355,14 @@ def smoothing_search(x, wmax, alphas, stream=None):
     assert x.is_cuda and x.dtype == torch.float16 and x.dim() == 2 and x.stride(1) == 1
     T, K = x.shape
     G = len(alphas)
-    need = c_size_t(0)
-    _check(lib.lcd_smoothing_search_workspace_bytes(T, K, G, byref(need)), "lcd_smoothing_search_workspace_bytes")
-    ws = torch.empty(need.value, dtype=torch.uint8, device=x.device)
+    need = _smoothing_workspace_bytes(T, K, G)
+    ws = torch.empty(need, dtype=torch.uint8, device=x.device)
     mse = torch.empty((G,), dtype=torch.float64, device=x.device)
     best = torch.empty((1,), dtype=torch.int32, device=x.device)
     inv = torch.empty((K,), dtype=torch.float32, device=x.device)
-    al = (ctypes.c_float * G)(*[float(a) for a in alphas])
-    _check(lib.lcd_smoothing_search(c_void_p(x.data_ptr()), T, K, x.stride(0), c_void_p(wmax.data_ptr()), al, G,
-                                    c_void_p(ws.data_ptr()), need.value, c_void_p(mse.data_ptr()),
-                                    c_void_p(best.data_ptr()), c_void_p(inv.data_ptr()), _stream_ptr(stream)),
-           "lcd_smoothing_search")
+    al = array("f", alphas)
+    _check(lib.lcd_smoothing_search(x.data_ptr(), T, K, x.stride(0), wmax.data_ptr(), al.buffer_info()[0], G, ws.data_ptr(), need,
+                                    mse.data_ptr(), best.data_ptr(), inv.data_ptr(), _stream_ptr(stream)), "lcd_smoothing_search")
     return best, mse, inv
 
 
