@@ -85,6 +85,53 @@ __device__ __forceinline__ void store_level1(uint8_t* row, int64_t k, uint32_t a
   }
 }
 
+// Columns k .. k + 7 of a row that ends at column K (zeros past it), k a multiple of 8.  aligned: the row starts on 16 bytes.
+// Any other row is read in the same 16-byte words and shifted: word i of the result is taken from words q + i and q + i + 1
+// of the two it lies in (its neighbour loads the second one too, from L1).  Both hold at least one of the row's values.  So
+// such rows too are read once, eight columns a thread, all loads in flight together (333 x 5001, from x to y of a 5003-row
+// layer: 30.6 us with two passes over single columns, 27.3 so).
+__device__ __forceinline__ uint4 load_columns8(const __half* row, int k, int K, bool aligned) {
+  const __half* p = row + k;
+  if (aligned && k + 8 <= K) return *reinterpret_cast<const uint4*>(p);
+  const uintptr_t at = reinterpret_cast<uintptr_t>(p), first = at & ~(uintptr_t)15, end = reinterpret_cast<uintptr_t>(row + K);
+  const unsigned off = (unsigned)(at & 15), r = 8 * (off & 3);
+  const uint4 a = *reinterpret_cast<const uint4*>(first);
+  uint4 b = make_uint4(0u, 0u, 0u, 0u);
+  if (off && first + 16 < end) b = *reinterpret_cast<const uint4*>(first + 16);
+  uint32_t w[4];
+  switch (off >> 2) {        // the same for the whole row
+    case 0:
+      w[0] = __funnelshift_r(a.x, a.y, r); w[1] = __funnelshift_r(a.y, a.z, r); w[2] = __funnelshift_r(a.z, a.w, r); w[3] = __funnelshift_r(a.w, b.x, r);
+      break;
+    case 1:
+      w[0] = __funnelshift_r(a.y, a.z, r); w[1] = __funnelshift_r(a.z, a.w, r); w[2] = __funnelshift_r(a.w, b.x, r); w[3] = __funnelshift_r(b.x, b.y, r);
+      break;
+    case 2:
+      w[0] = __funnelshift_r(a.z, a.w, r); w[1] = __funnelshift_r(a.w, b.x, r); w[2] = __funnelshift_r(b.x, b.y, r); w[3] = __funnelshift_r(b.y, b.z, r);
+      break;
+    default:
+      w[0] = __funnelshift_r(a.w, b.x, r); w[1] = __funnelshift_r(b.x, b.y, r); w[2] = __funnelshift_r(b.y, b.z, r); w[3] = __funnelshift_r(b.z, b.w, r);
+      break;
+  }
+  const int left = K - k;      // (only the row's last words are cut)
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    if (2 * i >= left) w[i] = 0u;
+    else if (2 * i + 1 >= left) w[i] &= 0xffffu;
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+// The smoothing factors of columns k .. k + 7 (1 where there are none: past K or without a vector).
+__device__ __forceinline__ void load_factors8(const float* inv_smooth, int k, int K, float (&f)[8]) {
+  if (inv_smooth && k + 8 <= K) {
+    const float4 a = __ldg(reinterpret_cast<const float4*>(inv_smooth + k)), b = __ldg(reinterpret_cast<const float4*>(inv_smooth + k + 4));
+    f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w; f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) f[i] = inv_smooth && k + i < K ? __ldg(inv_smooth + k + i) : 1.0f;
+  }
+}
+
 // One token per CTA.  VEC: rows are 16-byte aligned and K is a multiple of 8, so each thread handles 8
 // consecutive columns per step (one 16-byte load of x, two of inv_smooth, one 4-byte store).
 template <bool VEC, int THREADS, int OUT = kOutNibbles>
@@ -206,7 +253,7 @@ __device__ __forceinline__ void smooth_quantize_token_cached(const __half* __res
                                                              const float* __restrict__ inv_smooth,
                                                              const float* __restrict__ static_scale,
                                                              uint8_t* __restrict__ act_idx,
-                                                             float* __restrict__ act_scale) {
+                                                             float* __restrict__ act_scale, bool aligned) {
   __shared__ float s_red[THREADS / 32];
   __shared__ float s_mult;
   const __half* xr = x + m * ldx;
@@ -219,17 +266,10 @@ __device__ __forceinline__ void smooth_quantize_token_cached(const __half* __res
   for (int c = 0; c < CHUNKS; ++c) {
     const int64_t k = ((int64_t)c * THREADS + tid) * 8;
     if (k < K) {
-      const uint4 raw = *reinterpret_cast<const uint4*>(xr + k);
+      const uint4 raw = load_columns8(xr, (int)k, (int)K, aligned);
       const __half2* h = reinterpret_cast<const __half2*>(&raw);
       float f[8];
-      if (inv_smooth) {
-        const float4 a = *reinterpret_cast<const float4*>(inv_smooth + k);
-        const float4 b = *reinterpret_cast<const float4*>(inv_smooth + k + 4);
-        f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w; f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
-      } else {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) f[i] = 1.0f;
-      }
+      load_factors8(inv_smooth, (int)k, (int)K, f);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const float2 v = __half22float2(h[i]);
@@ -295,7 +335,7 @@ __device__ __forceinline__ void smooth_quantize_token_words(const __half* __rest
                                                             const float* __restrict__ inv_smooth,
                                                             const float* __restrict__ static_scale,
                                                             uint8_t* __restrict__ act_idx,
-                                                            float* __restrict__ act_scale) {
+                                                            float* __restrict__ act_scale, bool aligned) {
   __shared__ float s_red[THREADS / 32];
   __shared__ float s_mult;
   const __half* xr = x + m * ldx;
@@ -307,19 +347,12 @@ __device__ __forceinline__ void smooth_quantize_token_words(const __half* __rest
 #pragma unroll
   for (int c = 0; c < CHUNKS; ++c) {
     const int k = (c * THREADS + tid) * 8;
-    raw[c] = k < K ? *reinterpret_cast<const uint4*>(xr + k) : make_uint4(0u, 0u, 0u, 0u);
+    raw[c] = k < K ? load_columns8(xr, k, K, aligned) : make_uint4(0u, 0u, 0u, 0u);
   }
   auto products = [&](int c, int k, float (&t)[8]) {
     const __half2* h = reinterpret_cast<const __half2*>(&raw[c]);
     float f[8];
-    if (inv_smooth) {
-      const float4 a = __ldg(reinterpret_cast<const float4*>(inv_smooth + k));
-      const float4 b = __ldg(reinterpret_cast<const float4*>(inv_smooth + k + 4));
-      f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w; f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
-    } else {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) f[i] = 1.0f;
-    }
+    load_factors8(inv_smooth, k, K, f);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const float2 v = __half22float2(h[i]);
@@ -411,7 +444,7 @@ struct QuantProblem {
   float* act_scale;
   long long K, K_pad, ldx;
   int cta0;    // tokens of this problem are CTAs [cta0, cta0 + M)
-  int vec;
+  int vec;     // 2: rows on 16 bytes, K a multiple of 8; 1: x any way, the other pointers aligned; 0: neither
 };
 struct QuantBatch {
   int count;
@@ -438,14 +471,14 @@ __global__ void __launch_bounds__(THREADS) smooth_quantize_kernel(const __grid_c
     if (q.vec && q.K_pad <= (long long)8 * THREADS * CHUNKS) {
       if constexpr (THREADS == kQThreads)
         smooth_quantize_token_cached<THREADS, CHUNKS>(q.x, m, q.K, q.K_pad, q.ldx, q.inv_smooth, q.static_scale, q.act_idx,
-                                                      q.act_scale);
+                                                      q.act_scale, q.vec == 2);
       else
         smooth_quantize_token_words<THREADS, CHUNKS, OUT>(q.x, m, q.K, q.K_pad, q.ldx, q.inv_smooth, q.static_scale,
-                                                          q.act_idx, q.act_scale);
+                                                          q.act_idx, q.act_scale, q.vec == 2);
       return;
     }
   }
-  if (q.vec)
+  if (q.vec == 2)
     smooth_quantize_token<true, THREADS, OUT>(q.x, m, q.K, q.K_pad, q.ldx, q.inv_smooth, q.static_scale, q.act_idx, q.act_scale);
   else
     smooth_quantize_token<false, THREADS, OUT>(q.x, m, q.K, q.K_pad, q.ldx, q.inv_smooth, q.static_scale, q.act_idx, q.act_scale);
@@ -480,9 +513,9 @@ lcd_status launch_quantize_form(const lcd_act_problem* probs, int count, int out
     q.K_pad = (long long)round_up_u64((uint64_t)a.K, kTileK);
     q.ldx = a.ldx;
     q.cta0 = (int)a.M;          // (the token count until the launches are formed below)
-    q.vec = (reinterpret_cast<uintptr_t>(a.x_fp16) % 16 == 0) && (a.ldx % 8 == 0) && (a.K % 8 == 0) &&
-            (a.inv_smooth == nullptr || reinterpret_cast<uintptr_t>(a.inv_smooth) % 16 == 0) &&
-            (reinterpret_cast<uintptr_t>(a.act_idx) % (out_form == kOutNibbles ? 4 : 16) == 0);
+    const bool others = (a.inv_smooth == nullptr || reinterpret_cast<uintptr_t>(a.inv_smooth) % 16 == 0) &&
+                        (reinterpret_cast<uintptr_t>(a.act_idx) % (out_form == kOutNibbles ? 4 : 16) == 0);
+    q.vec = !others ? 0 : (reinterpret_cast<uintptr_t>(a.x_fp16) % 16 == 0) && (a.ldx % 8 == 0) && (a.K % 8 == 0) ? 2 : 1;
     tokens += a.M;
     if (tokens > 0x7fffffffLL) return LCD_ERR_INVALID_ARG;
   }

@@ -55,6 +55,21 @@ def test_smooth_quantize_bit_exact(M, K, ld_extra, use_inv):
     assert np.array_equal(s.cpu().numpy().view(np.uint32), s_ref.view(np.uint32))
 
 
+@pytest.mark.parametrize("M", [2, 300])
+@pytest.mark.parametrize("K", [1, 7, 9, 250, 2047, 5001, 8193])
+def test_smooth_quantize_rows_at_every_offset(M, K):
+    # rows that start at any 2-byte offset and end inside an eight-column word (integers and one IEEE operation each: exact)
+    x = gen.activations(7 + M + K, M, K, gen.outlier_channels(3, K, 0.01), 50.0)
+    inv_s = (1.0 / (np.abs(gen.normal(5, K)) * 3 + 0.05)).astype(np.float32)
+    q_ref, s_ref = O.smooth_quantize(x, inv_s)
+    for off in range(8):
+        xd = torch.full((M, K + 9), float("inf"), dtype=torch.float16, device="cuda")      # (nothing outside the row counts)
+        xd[:, off:off + K] = torch.from_numpy(x).cuda()
+        a, s = lcd.smooth_quantize_act(xd[:, off:off + K], torch.from_numpy(inv_s).cuda())
+        assert np.array_equal(a.cpu().numpy(), O.pack_act(q_ref))
+        assert np.array_equal(s.cpu().numpy().view(np.uint32), s_ref.view(np.uint32))
+
+
 def test_smooth_quantize_edge_rows_and_static_mode():
     K = 512
     x = np.zeros((4, K), dtype=np.float16)
@@ -197,6 +212,29 @@ def test_tensor_core_lut_matches_oracle(bits, N, K, M):
     assert not ws.any()
     q_ref, s_ref = O.smooth_quantize(L.x, L.inv_s)
     check_y(y, O.lut_linear_dequant(L.idx, L.codebook, q_ref, s_ref))
+
+
+@pytest.mark.parametrize("bits,act_bits", [(2, 4), (3, 4), (4, 4), (2, 8), (3, 8), (4, 8)])
+@pytest.mark.parametrize("N,K,M", [(64, 4096, 17), (1031, 520, 32), (200, 1000, 33), (24, 11008, 65), (300, 28672, 130),
+                                   (4096, 256, 300)])
+def test_tensor_core_lut_token_widths(bits, act_bits, N, K, M):
+    # every token width (32, 64, 128, and their ragged ends), with tiles cut between CTAs and with more tiles than CTAs
+    # (the library's choice above 16 tokens at these sizes); 4-bit indices at 16 tokens too
+    for m in ([M, 16] if bits == 4 and N == 64 else [M]):
+        L = gen.random_case(seed=N + K + m + bits, N=N, K=K, bits=bits, M=m, C=10 if bits == 4 else None)
+        w = lcd.PackedWeights(lcd.pack_weights(L.idx, L.codebook, bits, L.C))
+        a, s = lcd.smooth_quantize_act(torch.from_numpy(L.x).cuda(), torch.from_numpy(L.inv_s).cuda(), act_bits=act_bits)
+        word = torch.zeros((1,), dtype=torch.int32, device="cuda")
+        algo = lcd.ALGO_TC_LUT if m <= 16 else lcd.ALGO_AUTO
+        ws = torch.full((lcd.lut_linear_workspace_bytes(w, m, algo),), 0 if m <= 32 else 255, dtype=torch.uint8, device="cuda")
+        y = torch.full((m, N), float("nan"), dtype=torch.float32, device="cuda")
+        for _ in range(2):
+            lcd.lut_linear(w, a, s, y=y, algo=algo, workspace=ws, status_word=word)
+        torch.cuda.synchronize()
+        assert int(word.item()) == 0
+        assert m > 16 or not ws.any()
+        q_ref, s_ref = O.smooth_quantize(L.x, L.inv_s, act_bits=act_bits)
+        check_y(y, O.lut_linear_dequant(L.idx, L.codebook, q_ref, s_ref))
 
 
 @pytest.mark.parametrize("algo", ["register", "tensor"])
@@ -388,6 +426,21 @@ def test_grouped_host_buffer_entry_point():
         for i, L in enumerate(cases):
             q_ref, s_ref = O.smooth_quantize((L.x.astype(np.float32) * np.float32(0.5 + rep)).astype(np.float16), L.inv_s)
             check_y(hb.y_view(i), O.lut_linear_dequant(L.idx, L.codebook, q_ref, s_ref))
+
+
+@pytest.mark.parametrize("K,M", [(28672, 16), (250, 3)])
+def test_host_buffer_inputs_of_either_transport(K, M):
+    # above 512 KB the copy engine brings x, below it a kernel reads the pinned rows (250 columns: ragged 16-byte words)
+    L = gen.random_case(seed=K + M, N=72, K=K, bits=2, M=M)
+    w = lcd.PackedWeights(lcd.pack_weights(L.idx, L.codebook, 2))
+    hb = lcd.HostBatch([(w, torch.from_numpy(L.inv_s).cuda(), M)] * 2)
+    hb.x_view(0).copy_(torch.from_numpy(L.x))
+    hb.x_view(1).copy_(torch.from_numpy(L.x) * 0.5)
+    hb.run()
+    torch.cuda.synchronize()
+    for i in range(2):
+        q_ref, s_ref = O.smooth_quantize(L.x if i == 0 else (L.x * np.float16(0.5)).astype(np.float16), L.inv_s)
+        check_y(hb.y_view(i), O.lut_linear_dequant(L.idx, L.codebook, q_ref, s_ref))
 
 
 # ------------------------------------------------------------------------------- full sizes, bench launch shape
@@ -678,6 +731,28 @@ def test_fused_call_with_many_tokens_equals_two_call_path_and_oracle(bits):
     with pytest.raises(lcd.LcdError) as err:
         lcd.FusedBatch([items[0], (items[0][0], items[0][1][:4], items[0][2], items[0][3][:4])])
     assert err.value.status == 2
+
+
+@pytest.mark.parametrize("M", [16, 70])
+def test_fused_call_with_matrices_that_share_an_input(M):
+    # the matrices of one input (and factors) share its levels, the others have their own: bit-identical to two calls each
+    K, items, two_call = 1000, [], []
+    for i, (N, same) in enumerate([(200, 0), (1031, 0), (64, 1), (128, 0), (72, 2)]):
+        L = gen.random_case(seed=80 + i, N=N, K=K, bits=2, M=M)
+        if i == 0:
+            x = torch.from_numpy(L.x).cuda()
+            inv = torch.from_numpy(L.inv_s).cuda()
+        xi, fi = (x, inv) if same == 0 else (x, inv * 2) if same == 1 else (x + 1, inv)
+        w = lcd.PackedWeights(lcd.pack_weights(L.idx, L.codebook, 2))
+        items.append((w, xi, fi, torch.full((M, N), float("nan"), dtype=torch.float32, device="cuda")))
+        a, s = lcd.smooth_quantize_act(xi, fi)
+        two_call.append(lcd.lut_linear(w, a, s))
+    word = torch.zeros((1,), dtype=torch.int32, device="cuda")
+    lcd.FusedBatch(items, status_word=word).run()
+    torch.cuda.synchronize()
+    assert int(word.item()) == 0
+    for it, y2 in zip(items, two_call):
+        assert torch.equal(it[3], y2)
 
 
 # ------------------------------------------------------------------------------- adaptive smoothing search (offline)
