@@ -1,4 +1,5 @@
-"""Thin ctypes binding of the C ABI in include/lcd.h: argument marshalling only.
+"""Thin binding of the C ABI in include/lcd.h: argument marshalling only.  What a running program calls again and again goes
+through the module _host_calls (csrc/host_calls.cpp), the rest through ctypes.
 
 Every step of the path (index packing, input transformation, table lookup and accumulation) runs inside
 liblcd_b200.so; torch is used for device memory and streams.  There is no CPU fallback: if the shared
@@ -9,7 +10,6 @@ from __future__ import annotations
 import ctypes
 import functools
 import os
-from array import array
 from ctypes import c_char_p, c_int, c_int64, c_size_t, c_void_p, POINTER, Structure, byref
 
 import numpy as np
@@ -129,6 +129,19 @@ def _check(st: int, where: str):
         raise LcdError(st, where, detail)
 
 
+_host_calls = None
+
+
+def _calls():
+    """The module of the repeated calls, loaded at the first of them (it needs torch's libraries)."""
+    global _host_calls
+    if _host_calls is None:
+        import torch  # noqa: F401
+        from . import _host_calls as module
+        _host_calls = module
+    return _host_calls
+
+
 def _np_ptr(a: np.ndarray) -> c_void_p:
     return c_void_p(a.ctypes.data)
 
@@ -187,6 +200,7 @@ class PackedWeights:
         import torch
         self.header = bytes(blob[:HEADER_BYTES])
         self._hdr_buf = ctypes.create_string_buffer(self.header, HEADER_BYTES)
+        self._hdr_addr = ctypes.addressof(self._hdr_buf)
         f = np.frombuffer(self.header, dtype="<u8")
         self.N, self.K, self.K_pad = int(f[1]), int(f[2]), int(f[3])
         u = np.frombuffer(self.header, dtype="<u4")
@@ -198,30 +212,17 @@ class PackedWeights:
 
     @property
     def header_ptr(self) -> c_void_p:
-        return c_void_p(ctypes.addressof(self._hdr_buf))
+        return c_void_p(self._hdr_addr)
 
 
 def smooth_quantize_act(x, inv_smooth=None, static_scale=None, act_idx=None, act_scale=None, stream=None,
                         act_bits: int = 4):
     """x: CUDA fp16 [M,K] (row stride may exceed K) -> (act_idx uint8 [M,K_pad/2], act_scale fp32 [M]); with
     act_bits = 8 the levels come back as int8 [M,K_pad]."""
-    import torch
-    assert x.is_cuda and x.dtype == torch.float16 and x.dim() == 2 and x.stride(1) == 1
-    M, K = x.shape
-    K_pad = (K + 255) // 256 * 256
-    assert act_bits in (4, 8)
-    if act_idx is None:
-        act_idx = (torch.empty((M, K_pad // 2), dtype=torch.uint8, device=x.device) if act_bits == 4 else
-                   torch.empty((M, K_pad), dtype=torch.int8, device=x.device))
-    assert act_idx.dtype == (torch.uint8 if act_bits == 4 else torch.int8)
-    if act_scale is None:
-        act_scale = torch.empty((M,), dtype=torch.float32, device=x.device)
-    st = lib.lcd_smooth_quantize_act(x.data_ptr(), M, K, x.stride(0),
-                                     inv_smooth.data_ptr() if inv_smooth is not None else None,
-                                     static_scale.data_ptr() if static_scale is not None else None,
-                                     act_bits, act_idx.data_ptr(), act_scale.data_ptr(), _stream_ptr(stream))
-    _check(st, "lcd_smooth_quantize_act")
-    return act_idx, act_scale
+    out = (_host_calls or _calls()).smooth_quantize_act(x, inv_smooth, static_scale, act_idx, act_scale, act_bits, stream)
+    if out.__class__ is int:
+        _check(out, "lcd_smooth_quantize_act")
+    return out
 
 
 def lut_linear_workspace_bytes(w: PackedWeights, M: int, algo: int = ALGO_AUTO) -> int:
@@ -237,21 +238,14 @@ def lut_linear(w: PackedWeights, act_idx, act_scale, y=None, algo: int = ALGO_AU
                status_word=None, stream=None):
     """y[m][n] = s_q[m] * sum_k q[m][k] * cb[n][idx[n][k]]  (CUDA fp32 [M,N]).  act_idx: uint8 packed 4-bit
     levels, or int8 8-bit levels (as smooth_quantize_act returns them for act_bits = 8)."""
-    import torch
-    M = act_idx.shape[0]
-    fn, name = ((lib.lcd_lut_linear_act8, "lcd_lut_linear_act8") if act_idx.dtype == torch.int8 else
-                (lib.lcd_lut_linear, "lcd_lut_linear"))
-    if y is None:
-        y = torch.empty((M, w.N), dtype=torch.float32, device=act_idx.device)
-    need = lut_linear_workspace_bytes(w, M, algo)
-    have = workspace.numel() * workspace.element_size() if workspace is not None else 0
-    if have < need:
-        workspace, have = torch.zeros(need, dtype=torch.uint8, device=act_idx.device), need   # must start zero-filled
-    st = fn(w.dev.data_ptr(), w.header_ptr, act_idx.data_ptr(), act_scale.data_ptr(), M, y.data_ptr(), y.stride(0), algo,
-            workspace.data_ptr() if workspace is not None else None, have,
-            status_word.data_ptr() if status_word is not None else None, _stream_ptr(stream))
-    _check(st, name)
-    return y
+    fn = (_host_calls or _calls()).lut_linear
+    y_out = fn(w.dev, w._hdr_addr, w.N, w._workspace_bytes, act_idx, act_scale, y, algo, workspace, status_word, stream)
+    if y_out is None:                # the first call at this number of tokens
+        lut_linear_workspace_bytes(w, act_idx.shape[0], algo)
+        y_out = fn(w.dev, w._hdr_addr, w.N, w._workspace_bytes, act_idx, act_scale, y, algo, workspace, status_word, stream)
+    if y_out.__class__ is int:
+        _check(y_out, "lcd_lut_linear")
+    return y_out
 
 
 def lut_linear_static(w: PackedWeights, act_idx, act_scale, y, algo: int = ALGO_AUTO, status_word=None, stream=None):
@@ -283,24 +277,19 @@ class ActBatch:
             a.inv_smooth = inv_s.data_ptr() if inv_s is not None else None
             a.static_scale = None
             a.act_idx, a.act_scale = idx.data_ptr(), scale.data_ptr()
+        self._arr_addr = ctypes.addressof(self.arr)
 
     def run(self, stream=None):
-        _check(lib.lcd_smooth_quantize_act_batch(self.arr, self.count, self.act_bits, _stream_ptr(stream)),
-               "lcd_smooth_quantize_act_batch")
+        st = (_host_calls or _calls()).act_batch(self._arr_addr, self.count, self.act_bits, stream)
+        if st:
+            _check(st, "lcd_smooth_quantize_act_batch")
 
 
-# Workspace sizes are functions of the sizes alone; asking costs as much as a launch.
+# A function of the sizes alone; asking costs as much as a launch.
 @functools.lru_cache(maxsize=64)
 def _dbci_workspace_bytes(n: int, max_centroids: int) -> int:
     need = c_size_t(0)
     _check(lib.lcd_dbci_workspace_bytes(n, max_centroids, byref(need)), "lcd_dbci_workspace_bytes")
-    return need.value
-
-
-@functools.lru_cache(maxsize=64)
-def _smoothing_workspace_bytes(T: int, K: int, G: int) -> int:
-    need = c_size_t(0)
-    _check(lib.lcd_smoothing_search_workspace_bytes(T, K, G, byref(need)), "lcd_smoothing_search_workspace_bytes")
     return need.value
 
 
@@ -330,40 +319,20 @@ def reclassify(idx, codebook, delta_w, stream=None, out=None):
     """Section 3.2 bookkeeping.  idx: CUDA uint8 [N,K]; codebook: CUDA fp16 [N,C] rows ascending; delta_w: CUDA fp32
     [N,K].  Returns (new_idx uint8 [N,K], delta_c fp64 [N,C], counts int32 [N,C]); `out` may give those three
     tensors to write into."""
-    import torch
-    assert idx.dtype == torch.uint8 and codebook.dtype == torch.float16 and delta_w.dtype == torch.float32
-    assert idx.is_contiguous() and codebook.is_contiguous() and delta_w.stride(1) == 1
-    N, K = idx.shape
-    C = codebook.shape[1]
-    if out is None:
-        new_idx = torch.empty_like(idx)
-        delta_c = torch.empty((N, C), dtype=torch.float64, device=idx.device)
-        counts = torch.empty((N, C), dtype=torch.int32, device=idx.device)
-    else:
-        new_idx, delta_c, counts = out
-        assert new_idx.dtype == torch.uint8 and delta_c.dtype == torch.float64 and counts.dtype == torch.int32
-        assert new_idx.shape == idx.shape and delta_c.shape == (N, C) and counts.shape == (N, C)
-    _check(lib.lcd_reclassify(idx.data_ptr(), codebook.data_ptr(), delta_w.data_ptr(), N, K, delta_w.stride(0), C,
-                              new_idx.data_ptr(), delta_c.data_ptr(), counts.data_ptr(), _stream_ptr(stream)), "lcd_reclassify")
-    return new_idx, delta_c, counts
+    new_idx, delta_c, counts = out if out is not None else (None, None, None)
+    r = (_host_calls or _calls()).reclassify(idx, codebook, delta_w, new_idx, delta_c, counts, stream)
+    if r.__class__ is int:
+        _check(r, "lcd_reclassify")
+    return r
 
 
 def smoothing_search(x, wmax, alphas, stream=None):
     """Section 3.4 grid search on a calibration batch.  x: CUDA fp16 [T,K]; wmax: CUDA fp32 [K]; alphas: list of
     floats.  Returns (best index tensor int32 [1], mse fp64 [G], inv_smooth fp32 [K]) on the device."""
-    import torch
-    assert x.is_cuda and x.dtype == torch.float16 and x.dim() == 2 and x.stride(1) == 1
-    T, K = x.shape
-    G = len(alphas)
-    need = _smoothing_workspace_bytes(T, K, G)
-    ws = torch.empty(need, dtype=torch.uint8, device=x.device)
-    mse = torch.empty((G,), dtype=torch.float64, device=x.device)
-    best = torch.empty((1,), dtype=torch.int32, device=x.device)
-    inv = torch.empty((K,), dtype=torch.float32, device=x.device)
-    al = array("f", alphas)
-    _check(lib.lcd_smoothing_search(x.data_ptr(), T, K, x.stride(0), wmax.data_ptr(), al.buffer_info()[0], G, ws.data_ptr(), need,
-                                    mse.data_ptr(), best.data_ptr(), inv.data_ptr(), _stream_ptr(stream)), "lcd_smoothing_search")
-    return best, mse, inv
+    r = (_host_calls or _calls()).smoothing_search(x, wmax, alphas, stream)
+    if r.__class__ is int:
+        _check(r, "lcd_smoothing_search")
+    return r
 
 
 def resolve_batch_algo(weights_and_tokens, algo: int = ALGO_AUTO) -> int:
@@ -400,10 +369,12 @@ class FusedBatch:
         self.workspace = torch.zeros(max(need.value, 256), dtype=torch.uint8, device=self._keep[0][1].device)
         self.status_word = status_word
 
+        self._arr_addr = ctypes.addressof(self.arr)
+
     def run(self, stream=None):
-        _check(lib.lcd_linear_fused_batch(self.arr, self.count, self.algo, self.workspace.data_ptr(), self.workspace.numel(),
-                                          self.status_word.data_ptr() if self.status_word is not None else None,
-                                          _stream_ptr(stream)), "lcd_linear_fused_batch")
+        st = (_host_calls or _calls()).linear_batch(0, self._arr_addr, self.count, self.algo, self.workspace, self.status_word, stream)
+        if st:
+            _check(st, "lcd_linear_fused_batch")
 
 
 class LinearBatch:
@@ -429,11 +400,13 @@ class LinearBatch:
         self.workspace = torch.zeros(max(need.value, 256), dtype=torch.uint8, device=self._keep[0][1].device)
         self.status_word = status_word
 
+        self._arr_addr = ctypes.addressof(self.arr)
+
     def run(self, stream=None):
-        fn = lib.lcd_lut_linear_batch_act8 if self.act8 else lib.lcd_lut_linear_batch
-        _check(fn(self.arr, self.count, self.algo, self.workspace.data_ptr(), self.workspace.numel(),
-                  self.status_word.data_ptr() if self.status_word is not None else None,
-                  _stream_ptr(stream)), "lcd_lut_linear_batch")
+        st = (_host_calls or _calls()).linear_batch(2 if self.act8 else 1, self._arr_addr, self.count, self.algo, self.workspace,
+                                                    self.status_word, stream)
+        if st:
+            _check(st, "lcd_lut_linear_batch")
 
 
 class HostBatch:

@@ -1,14 +1,17 @@
-"""Builds the C-ABI shared library (liblcd_b200.so) in-tree with nvcc for sm_100a."""
+"""Builds the C-ABI shared library (liblcd_b200.so) in-tree with nvcc for sm_100a, and the Python module of the repeated calls
+(_host_calls.so, g++ against the installed torch's headers)."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "liblcd_b200.so")
+CALLS = os.path.join(HERE, "_host_calls.so")
 SOURCES = ["api.cu", "pack.cpp", "quantize.cu", "quantize8.cu", "smoothing.cu", "reclassify.cu", "dbci.cu", "reference.cu", "lut_gemv.cu", "lut_smem.cu", "lut_gemv_tc.cu", "dense_tc.cu", "static_scratch.cu"]
 
 
@@ -20,9 +23,9 @@ def nvcc_path() -> str:
 
 
 def needs_build() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(CALLS):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(CALLS))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "lcd.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
@@ -52,7 +55,20 @@ def build(force: bool = False, verbose: bool = False) -> str:
         raise RuntimeError("nvcc failed")
     subprocess.check_call([nvcc_path(), "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-o", LIB] + objs +
                           ["-cudart", "static"])
+    build_calls()
     return LIB
+
+
+def build_calls() -> None:
+    import importlib.util
+    torch_dir = os.path.dirname(importlib.util.find_spec("torch").origin)
+    cuda = os.path.dirname(os.path.dirname(nvcc_path())) if os.path.isabs(nvcc_path()) else "/usr/local/cuda"
+    include = [os.path.join(torch_dir, "include"), os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"),
+               sysconfig.get_paths()["include"], os.path.join(cuda, "include"), os.path.join(ROOT, "include")]
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", *(f"-I{d}" for d in include),
+                           os.path.join(CSRC, "host_calls.cpp"), "-o", CALLS, f"-L{HERE}", "-l:" + os.path.basename(LIB),
+                           f"-L{os.path.join(torch_dir, 'lib')}", "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10",
+                           "-Wl,-rpath,$ORIGIN"])
 
 
 if __name__ == "__main__":
