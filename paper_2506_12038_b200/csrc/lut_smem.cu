@@ -26,10 +26,15 @@
 // warps takes every 16th row group of a piece and streams its index bytes through its own ring of bulk copies.
 // Per slice a row's four bucket sums are added to zero-filled scratch [row][4] as fp32 (integers below 2^24, so
 // the additions are exact and their order does not matter: one vector reduction per row).  When every CTA of the
-// launch has added its last sum (a counter in the scratch that all CTAs wait for, bounded; the launch is
-// cooperative, so all of them are resident), the rows of all problems are dealt to all threads of the grid: each
-// takes a row's totals back, leaves zeros, forms s_q * sum_w cb[w] * S_w and writes y.  Results are bit-identical
-// from run to run.
+// launch has added its last sum (a counter in the scratch, the gate), the rows of all problems are dealt to all threads of
+// the grid: each takes a row's totals back, leaves zeros, forms s_q * sum_w cb[w] * S_w and writes y.  Results are
+// bit-identical from run to run.
+//
+// Gate.  A CTA waits for the others only for kGateNs; then it leaves its rows to the CTA that arrives last, which never
+// waits.  So the launch ends whatever is resident beside it and need not be cooperative: a cooperative launch does not
+// overlap with the kernel before it in its stream (call after call in a stream: 7B layer 21.0 us, 18.9 so; 70B gate and up
+// 34.5, 31.9; 70B down 25.8, 21.4).  Counting the row groups per 512 rows and letting who completes them finish them needs
+// no waiting at all, but one SM then finishes up to 13 such chunks, 250 KB (70B gate and up 33.7).
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -46,6 +51,8 @@ constexpr int kItemBytes = 1024;            // one 16-row x 256-column item at 2
 constexpr int kMiscBytes = 512;             // mbarriers, partial maxima
 constexpr int kMaxCta = 304;
 constexpr unsigned long long kTimeoutNs = 2000000000ull;
+constexpr unsigned long long kGateNs = 50000ull;      // CTAs of an undisturbed launch arrive within 5 us of one another
+constexpr int kGateLeft = 1 << 16;                    // the gate counts arrivals below, CTAs that have left their rows above
 
 // Shape of one kernel instance: W table blocks per slice, DEPTH ring slots per warp, WARPS warps per CTA.
 // Shared memory: [window start, +kMiscBytes) barriers and maxima | ring | (gap) | tables at the FIXED window address
@@ -76,7 +83,8 @@ struct SbProblem {
 struct SbBatch {
   int count, n_cta;
   float* sq;          // scratch [LCD_MAX_BATCH]: s_q of the fused problems, zero on entry and on exit
-  int* gate;          // scratch [2]: CTAs that have added all their sums / that have written their rows; zero on entry and exit
+  int* gate;          // scratch [2]: CTAs that have added all their sums (and that left their rows) / that are through; zero on entry and exit
+  int* left;          // scratch [kMaxCta]: 1 = this CTA's rows are left to the last one; zero on entry and exit
   int row0[LCD_MAX_BATCH + 1];   // first row of every problem in the launch-wide row numbering (N_pad rows each)
   SbProblem p[LCD_MAX_BATCH];
   uint2 start[kMaxCta + 1];   // x = problem << 16 | slice, y = row group; entry n_cta is the end
@@ -495,41 +503,84 @@ lut_smem_kernel(const __grid_constant__ SbBatch batch, int32_t* __restrict__ sta
     p_cur = locate(r, &n_cur);
     c_cur = __ldg(reinterpret_cast<const uint2*>(batch.p[p_cur].codebook + (size_t)n_cur * 4));
   }
-  int& s_go = *reinterpret_cast<int*>(smem + WARPS * DEPTH * 8 + WARPS * 4);   // in the misc area: no static shared memory
+  // what a CTA does after the gate, in the misc area (no static shared memory): -1 nothing, else its rows and those of that
+  // many CTAs that have left theirs
+  int& s_others = *reinterpret_cast<int*>(smem + WARPS * DEPTH * 8 + WARPS * 4);
   __threadfence();                       // this thread's reductions are performed
   __syncthreads();
   if (tid == 0) {
-    int go = 1;
-    atomicAdd(batch.gate, 1);
-    const unsigned long long t0 = globaltimer();
-    for (uint32_t it = 0;; ++it) {
-      int seen;
-      asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(seen) : "l"(batch.gate) : "memory");
-      if (seen >= (int)gridDim.x) break;
-      if ((it & 63u) == 63u && globaltimer() - t0 > kTimeoutNs) { go = 0; break; }
-      __nanosleep(32);
+    const int n = (int)gridDim.x, before = atomicAdd(batch.gate, 1);
+    int others = 0;
+    if ((before & (kGateLeft - 1)) == n - 1) {
+      others = before / kGateLeft;
+      __threadfence();
+    } else {
+      const unsigned long long t0 = globaltimer();
+      for (uint32_t it = 0;; ++it) {
+        int seen;
+        asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(seen) : "l"(batch.gate) : "memory");
+        if ((seen & (kGateLeft - 1)) == n) break;
+        if ((it & 63u) == 63u && globaltimer() - t0 > kGateNs) {
+          // counted before the last CTA arrives: that one will look for this word; after: all sums are there, the rows are
+          // finished here
+          if ((atomicAdd(batch.gate, kGateLeft) & (kGateLeft - 1)) < n) {
+            others = -1;
+            asm volatile("st.release.gpu.global.s32 [%0], 1;" ::"l"(batch.left + blockIdx.x) : "memory");
+          }
+          __threadfence();
+          break;
+        }
+        __nanosleep(32);
+      }
     }
-    s_go = go;
+    s_others = others;
   }
   __syncthreads();
-  if (!s_go) {
-    if (tid == 0 && status) atomicExch(status, (int)LCD_ERR_TIMEOUT);
-    return;
-  }
-  for (; r < total_rows; r += (int)gridDim.x * kThreads) {
-    const SbProblem& P = batch.p[p_cur];
-    float4* src = reinterpret_cast<float4*>(P.sums) + n_cur;
-    const float4 Sw = __ldcg(src);
-    const float sq = P.act_bits == 16 ? __ldcg(batch.sq + p_cur) : __ldg(P.act_scale);
-    __stcg(src, make_float4(0.0f, 0.0f, 0.0f, 0.0f));          // handed on zero-filled
-    const float2 c01 = __half22float2(*reinterpret_cast<const __half2*>(&c_cur.x));
-    const float2 c23 = __half22float2(*reinterpret_cast<const __half2*>(&c_cur.y));
-    const float v = (c01.x * Sw.x + c01.y * Sw.y) + (c23.x * Sw.z + c23.y * Sw.w);
-    if (n_cur < P.N) P.y[n_cur] = v * sq;
-    const int r_next = r + (int)gridDim.x * kThreads;
-    if (r_next < total_rows) {
-      p_cur = locate(r_next, &n_cur);
-      c_cur = __ldg(reinterpret_cast<const uint2*>(batch.p[p_cur].codebook + (size_t)n_cur * 4));
+  const int others = s_others;
+  auto finish_rows = [&]() {
+    for (; r < total_rows; r += (int)gridDim.x * kThreads) {
+      const SbProblem& P = batch.p[p_cur];
+      float4* src = reinterpret_cast<float4*>(P.sums) + n_cur;
+      const float4 Sw = __ldcg(src);
+      const float sq = P.act_bits == 16 ? __ldcg(batch.sq + p_cur) : __ldg(P.act_scale);
+      __stcg(src, make_float4(0.0f, 0.0f, 0.0f, 0.0f));          // handed on zero-filled
+      const float2 c01 = __half22float2(*reinterpret_cast<const __half2*>(&c_cur.x));
+      const float2 c23 = __half22float2(*reinterpret_cast<const __half2*>(&c_cur.y));
+      const float v = (c01.x * Sw.x + c01.y * Sw.y) + (c23.x * Sw.z + c23.y * Sw.w);
+      if (n_cur < P.N) P.y[n_cur] = v * sq;
+      const int r_next = r + (int)gridDim.x * kThreads;
+      if (r_next < total_rows) {
+        p_cur = locate(r_next, &n_cur);
+        c_cur = __ldg(reinterpret_cast<const uint2*>(batch.p[p_cur].codebook + (size_t)n_cur * 4));
+      }
+    }
+  };
+  if (others >= 0) finish_rows();
+  if (others > 0) {
+    const unsigned long long t0 = globaltimer();
+    for (int found = 0, cta = 0; found < others; cta = cta + 1 == (int)gridDim.x ? 0 : cta + 1) {
+      __syncthreads();
+      if (tid == 0) {
+        int seen;
+        asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(seen) : "l"(batch.left + cta) : "memory");
+        if (seen) __stcg(batch.left + cta, 0);
+        else if (cta == 0 && globaltimer() - t0 > kTimeoutNs) seen = -1;
+        s_others = seen;
+      }
+      __syncthreads();
+      const int seen = s_others;
+      if (seen < 0) {
+        if (tid == 0 && status) atomicExch(status, (int)LCD_ERR_TIMEOUT);
+        break;
+      }
+      if (seen == 0) continue;
+      ++found;
+      r = cta * kThreads + tid;
+      if (r < total_rows) {
+        p_cur = locate(r, &n_cur);
+        c_cur = __ldg(reinterpret_cast<const uint2*>(batch.p[p_cur].codebook + (size_t)n_cur * 4));
+      }
+      finish_rows();
     }
   }
   // the CTA that leaves last clears the counters and the scales
@@ -551,8 +602,8 @@ using LaunchShape = Shape<kSliceBlocks, kDepth, kWarps>;
 
 int slices_of(int64_t n_kt) { return (int)((n_kt + kSliceBlocks - 1) / kSliceBlocks); }
 
-// Scratch of a launch: 256 bytes of counters and scales, then every problem's bucket sums.
-constexpr size_t kGateBytes = 256;
+// Scratch of a launch: 256 bytes of counters and scales, a word per CTA, then every problem's bucket sums.
+constexpr size_t kGateBytes = (256 + kMaxCta * sizeof(int) + 255) / 256 * 256;
 size_t sums_bytes(const Problem& p) { return (size_t)round_up_u64((uint64_t)p.N_pad * 4 * sizeof(float), 256); }
 
 }  // namespace
@@ -582,6 +633,7 @@ lcd_status launch_lut_smem(const Problem* probs, int count, void* workspace, siz
   batch.count = count;
   batch.gate = reinterpret_cast<int*>(workspace);
   batch.sq = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + 64);
+  batch.left = reinterpret_cast<int*>(static_cast<uint8_t*>(workspace) + 256);
   batch.row0[0] = 0;
   size_t off = kGateBytes;
   for (int i = 0; i < count; ++i) {
@@ -727,14 +779,11 @@ lcd_status launch_lut_smem(const Problem* probs, int count, void* workspace, siz
   cfg.blockDim = dim3(LaunchShape::kThreads);
   cfg.dynamicSmemBytes = LaunchShape::kSmemBytes;
   cfg.stream = static_cast<cudaStream_t>(stream);
-  // cooperative: all CTAs wait for one another before the rows are finished, so all of them must be resident
-  cudaLaunchAttribute attr[2];
+  cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeCooperative;
-  attr[1].val.cooperative = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 2;
+  cfg.numAttrs = 1;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, batch, status_word);
   if (e != cudaSuccess) { set_cuda_error((int)e); return LCD_ERR_CUDA; }
   return LCD_OK;

@@ -146,6 +146,31 @@ def test_shared_bucket_matches_oracle(N, K, fused):
     check_y(y, O.lut_linear_dequant(L.idx, L.codebook, q_ref, s_ref))
 
 
+def test_shared_bucket_beside_a_long_kernel_of_another_stream():
+    # the other kernel holds SMs for longer than the CTAs of a launch wait for one another: those that arrive last finish
+    # the rows of those that have left; the same sums in the same order, so y is the undisturbed launch's
+    L = gen.random_case(seed=8, N=4096, K=8192, bits=2, M=1)
+    w = lcd.PackedWeights(lcd.pack_weights(L.idx, L.codebook, 2))
+    x, inv_s = torch.from_numpy(L.x).cuda(), torch.from_numpy(L.inv_s).cuda()
+    y = torch.empty((1, 4096), dtype=torch.float32, device="cuda")
+    word = torch.zeros((1,), dtype=torch.int32, device="cuda")
+    fb = lcd.FusedBatch([(w, x, inv_s, y)], algo=lcd.ALGO_SHARED_BUCKET, status_word=word)
+    fb.run()
+    expected = y.clone()
+    a = torch.randn(6144, 6144, device="cuda")
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    for _ in range(5):
+        with torch.cuda.stream(side):
+            b = a @ a                       # fp32: milliseconds, every SM
+        for _ in range(3):
+            y.fill_(float("nan"))
+            fb.run()
+            assert torch.equal(y, expected)
+        side.synchronize()
+    assert torch.isfinite(b).all() and int(word.item()) == 0 and not fb.workspace.any()
+
+
 def test_shared_bucket_grouped_fewer_centroids_and_refusals():
     shapes = [(200, 1000, 4), (4096, 512, 3), (24, 11008, 4), (1031, 520, 1), (8, 256, 2)]
     cases = [gen.random_case(seed=61 * i + 5, N=N, K=K, bits=2, M=1, C=C) for i, (N, K, C) in enumerate(shapes)]
