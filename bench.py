@@ -282,9 +282,10 @@ def measure_config(args, cfg_id, M, dev, world, local, primary):
     algo = {"auto": lcd.ALGO_AUTO, "register": lcd.ALGO_REGISTER_LUT, "bucket": lcd.ALGO_BUCKET_LUT,
             "tensor": lcd.ALGO_TC_LUT, "shared": lcd.ALGO_SHARED_BUCKET}[args.algo]
     # which lookup kernel the library runs for this launch shape (its own answer, not a guess made here)
-    shared_bucket = grouped and lcd.resolve_batch_algo([(mt["w"][0], M) for mt in mats], algo) == lcd.ALGO_SHARED_BUCKET \
-        and args.act_bits == 4
-    lookup_kernel = "lut_smem_kernel" if shared_bucket else "lut_gemv_kernel"
+    resolved = lcd.resolve_batch_algo([(mt["w"][0], M) for mt in mats], algo) if grouped else None
+    shared_bucket = resolved == lcd.ALGO_SHARED_BUCKET and args.act_bits == 4
+    lookup_kernel = ("lut_smem_kernel" if shared_bucket else
+                     "lut_gemv_tc_kernel" if resolved == lcd.ALGO_TC_LUT else "lut_gemv_kernel")
     # every kernel that can give up on a bounded wait reports it here; a non-zero word voids the run
     status = torch.zeros((1,), dtype=torch.int32, device=dev)
     if grouped:

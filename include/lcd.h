@@ -43,8 +43,8 @@ typedef enum {
 /* Which kernel family lcd_lut_linear uses.  Every family computes the same y. */
 typedef enum {
   LCD_ALGO_AUTO = 0,        /* M <= 16: SHARED_BUCKET where it applies and the layer is large enough to pay    */
-                            /* for its tables, else REGISTER_LUT; DENSE_TC above (17..32 tokens on rows of at   */
-                            /* least 8192 columns: REGISTER_LUT in two launches, measured faster there)         */
+                            /* for its tables, TC_LUT from 9 tokens on unless the call is small, else            */
+                            /* REGISTER_LUT; above 16 tokens DENSE_TC                                            */
   LCD_ALGO_REFERENCE = 1,   /* plain per-weight lookup cb[n][idx] and multiply-accumulate; any M, slow        */
   LCD_ALGO_BUCKET_LUT = 2,  /* Section 4.2 centroid-stationary buckets: per output and per centroid w the exact */
                             /* integer sum S_w of the activation levels whose weight index is w (one-hot byte   */
@@ -55,11 +55,12 @@ typedef enum {
                             /* accumulated by int8 tensor-core MMAs against the activation levels.  M <= 16.     */
   LCD_ALGO_DENSE_TC = 4,    /* batched prefill on tcgen05 tensor cores: the byte tables of REGISTER_LUT decode   */
                             /* the indices into two int8 planes in shared memory, int8 levels arrive by TMA,     */
-                            /* kind::i8 MMAs accumulate exact int32 sums in tensor memory.                      */
+                            /* kind::i8 MMAs accumulate exact int32 sums in tensor memory.  Below a few hundred  */
+                            /* tokens, where TC_LUT's kernel is estimated to be faster, that one runs.          */
   LCD_ALGO_DENSE_F16 = 5,   /* the same with fp16 operands: indices decoded through the codebook into fp16     */
                             /* shared-memory tiles, fp32 accumulators (no fixed-point step; slower).            */
   LCD_ALGO_TC_LUT = 6,      /* REGISTER_LUT's tables and sums, the looked-up bytes written to tensor memory as  */
-                            /* the A operand of tcgen05 kind::i8 MMAs over a 16-token tile.  M <= 16.            */
+                            /* the A operand of tcgen05 kind::i8 MMAs.  M <= 16.                                 */
   LCD_ALGO_SHARED_BUCKET = 7/* Section 4.2 centroid-stationary buckets with the tables in shared memory: for    */
                             /* every four columns a table indexed by the byte of their four weight indices      */
                             /* holds the four partial bucket sums of the token's levels, so one load looks four */
@@ -166,8 +167,8 @@ lcd_status lcd_smooth_quantize_act_batch(const lcd_act_problem* problems /* host
  *                       aligned (may be NULL when that size is 0).  REGISTER_LUT and BUCKET_LUT keep integer
  *                       partial sums and arrival counters there: the caller zero-fills it once before its
  *                       first use, every call that completes leaves it zero-filled again, and two calls that
- *                       may overlap on the device need separate workspaces.  The other families do not care
- *                       about its contents;
+ *                       may overlap on the device need separate workspaces.  SHARED_BUCKET and TC_LUT, and any
+ *                       call with at most 32 tokens, keep to the same rule.  Above, its contents do not matter;
  *   status_word_dev:    device int32 or NULL; receives LCD_ERR_TIMEOUT if a bounded device-side wait
  *                       expired (the output is then invalid and the workspace must be zero-filled again);
  *                       never written otherwise.
@@ -310,7 +311,8 @@ lcd_status lcd_reclassify(const uint8_t* idx, const uint16_t* codebook_fp16, con
  * LCD_ALGO_AUTO or LCD_ALGO_DENSE_TC and the call is: one launch that transforms the inputs of all problems (same
  * operation sequence, same levels) and writes them as the signed bytes the int8 tensor-core kernel reads, in its
  * order, into the workspace (per problem M * K_pad bytes and M scales; no zero-fill contract, the contents are
- * scratch), then that kernel once per problem: no packed 4-bit copy and no expansion pass in between.  y equals
+ * scratch; equal inputs are transformed once), then that kernel once per problem, or the one of TC_LUT once for all
+ * where it is estimated to be faster: no packed 4-bit copy and no expansion pass in between.  y equals
  * the two-call result of LCD_ALGO_DENSE_TC bit for bit.  A mix of problems with at most 16 and more than 16 tokens
  * gives LCD_ERR_UNSUPPORTED (use the two calls).
  * -------------------------------------------------------------------------------------------- */

@@ -1,4 +1,5 @@
-// Batched-prefill path (many tokens): the layer is a dense contraction y[M x N] = diag(s_q) * Q[M x K] * Wd[N x K]^T,
+// Batched-prefill path (many tokens; LCD_ALGO_DENSE_TC hands over to the tensor-memory kernel where that one's estimate is
+// lower, see dense_takes_tensor_memory): the layer is a dense contraction y[M x N] = diag(s_q) * Q[M x K] * Wd[N x K]^T,
 // where Wd[n][k] = cb[n][idx[n][k]] is what the lookup of Section 4.2 of the LCD paper returns and Q holds the
 // activation levels of Section 4.1.  Two kernels share one structure (one persistent CTA per SM, tiles of 128 weight
 // rows x BN tokens, every role a warp or a group of warps, mbarrier pipelines, accumulators in tensor memory):

@@ -972,19 +972,24 @@ namespace {
 int sm_count() { return current_sm_count(); }
 
 // items (16 rows x 256 columns) of a launch from which LCD_ALGO_AUTO takes the shared-memory bucket tables.  Their
-// launch costs about 7 us before and after the lookups (token maximum, tables, the grid-wide finish) against 3.5 us
-// of the register tables, and looks weights up 1.6 times as fast: measured per launch, 4096 x 4096 7.3 vs 5.7 us,
-// 11008 x 4096 9.3 vs 8.3, the seven matrices of a LLaMA-7B-shaped layer (49408 items) 20.0 vs 22.4, the three of a
-// LLaMA-70B-shaped MLP 46 vs 59.
+// launch costs about 7 us before and after the lookups (token maximum, tables, the rows' finish) against 3.5 us
+// of the register tables, and looks weights up 1.3 times as fast: measured per launch from x to y, gate and up of a 7B layer
+// (22016 items) 11.7 vs 11.5 us, the seven matrices of the layer (49408 items) 18.6 vs 19.4, of a 13B layer 24.8 vs 27.0,
+// 70B gate and up 31.4 vs 37.7; 5120 x 5120 8.5 vs 7.7.
 constexpr long long kSharedBucketMinItems = 32768;
 
 // From nine tokens on a warp-level MMA serves half as many rows, and the register tables are bound by that pipe; the
 // tensor-memory kernel is not, but pays about 2 us more per launch (tensor memory, the split tiles' second pass).
-// Measured at 16 tokens, 2 / 3 / 4 bit, register tables against tensor memory: 4096 x 4096 (4096 items) 8.0 / 8.2 / 10.9
-// vs 8.2 / 8.5 / 10.0 us, 4096 x 11008 (11008 items) 14.4 / 14.2 / 20.8 vs 10.3 / 10.9 / 14.7, LLaMA-7B-shaped layer
+// Measured with the input transformation before it, 9 and 16 tokens, 2 bit (3 and 4 bit alike), register tables against
+// tensor memory: seven matrices of 1024 columns (3040 items) 9.3 and 9.8 vs 11.4 and 11.7 us, 4096 x 4096 (4096 items) 9.6
+// and 10.3 vs 9.9 and 9.9, 4096 x 5120 (5120 items) 11.9 and 13.1 vs 10.2 and 10.5, 5120 x 5120 13.2 and 14.3 vs 10.7 and
+// 10.8; the lookup alone at 16 tokens, 2 / 3 / 4 bit: 4096 x 11008 14.4 / 14.2 / 20.8 vs 10.3 / 10.9 / 14.7, LLaMA-7B-shaped layer
 // 28.3 / 28.8 / 44.2 vs 22.1 / 25.0 / 40.8, LLaMA-70B-shaped MLP 75.6 / 103 / 158 vs 59.5 / 68.6 / 120.  At 8 tokens the
 // register tables win on all but single matrices with long rows (7B layer 19.5 / 23.4 / 34.3 vs 21 / 24 / 41).
-constexpr long long kTensorMemoryMinItems = 8192;
+constexpr long long kTensorMemoryMinItems = 5000;
+// Fewer items too where the matrices have a CTA or less per tile of 128 rows but many tiles, with short rows: no tile is cut
+// (8192 x 2048, 9 and 16 tokens: 9.8 and 10.5 vs 7.7 and 7.7 us; 14336 x 1024 9.7 and 10.3 vs 6.3 and 6.3).
+constexpr int kTensorMemoryShortRow = 8;          // 256-column blocks
 
 int planes_of(int bits, int kind) { return kind == kFixed16 ? 2 : (1 << bits); }
 
@@ -1033,13 +1038,17 @@ lcd_status launch_t(const GemvBatch& batch, int grid, size_t smem, int32_t* stat
 lcd_algo resolve_small_m(const Problem* probs, int count, lcd_algo algo) {
   if (algo != LCD_ALGO_AUTO) return algo;
   long long items = 0;
-  int64_t m = 0;
+  int64_t m = 0, tiles = 0, blocks = 0;
   for (int i = 0; i < count; ++i) {
     items += (probs[i].N_pad / kPairRows) * (probs[i].K_pad / kTileK);
     m = probs[i].M > m ? probs[i].M : m;
+    tiles += (probs[i].N_pad + 127) / 128;
+    blocks = probs[i].K_pad / kTileK > blocks ? probs[i].K_pad / kTileK : blocks;
   }
   if (items >= kSharedBucketMinItems && lut_smem_supported(probs, count)) return LCD_ALGO_SHARED_BUCKET;
-  if (m > 8 && items >= kTensorMemoryMinItems && lut_gemv_tc_supported(probs, count)) return LCD_ALGO_TC_LUT;
+  const int n_sm = current_sm_count();
+  const bool uncut = blocks <= kTensorMemoryShortRow && tiles <= n_sm && 3 * tiles >= n_sm;
+  if (m > 8 && (items >= kTensorMemoryMinItems || uncut) && lut_gemv_tc_supported(probs, count)) return LCD_ALGO_TC_LUT;
   return LCD_ALGO_REGISTER_LUT;
 }
 
