@@ -944,7 +944,12 @@ bool dense_takes_tensor_memory(const Problem* probs, int count) {
     dense_us += dense_estimate_us(probs[i]);
   }
   if (!lut_gemv_tc_supported(ready, count)) return false;
-  return m <= 32 || lut_gemv_tc_estimate_us(ready, count) < dense_us;
+  if (m <= 32) return true;
+  // Long launches run under the power cap, where the tensor-memory kernel's units lengthen more than the dense kernel's
+  // stages (7B layer at 1784 tokens: estimates 464 and 475 us, a call takes 615 and 557; 13B layer at 1024 tokens: 412 and
+  // 440, a call takes 500 and 544).
+  const double us = lut_gemv_tc_estimate_us(ready, count), over = us <= 300.0 ? 0.0 : us >= 600.0 ? 1.0 : (us - 300.0) / 300.0;
+  return us * (1.0 + 0.1 * over) < dense_us;
 }
 
 namespace {
