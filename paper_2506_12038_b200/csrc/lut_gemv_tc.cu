@@ -21,6 +21,13 @@
 // scratch (one int32 per output where pieces are short enough for the sum of both planes).  A CTA therefore only ever
 // waits for CTAs of smaller number, which were launched before it, and normally finds their part there already.
 //
+// Where there are few tiles and many tokens, that one CTA reads megabits while the others have nothing to do: then the CTAs
+// of a tile are a cluster (resident together, so they may wait for one another), every one stores its part of the tokens
+// that are not its own and, after the cluster's barrier, finishes its own from the other CTAs' parts (4096 x 11008, 2 bit,
+// 48 tokens, transformation to y: 16.9 us with one finisher, 15.1 so; 512 x 14336 at 16 tokens 13.2 and 11.0; 2048 x 11008
+// at 32 tokens 16.7 and 13.6).  With few
+// tokens the one finisher is as fast; the launcher's estimate decides (tc_plan_width).
+//
 // Layout.  An item of the index area (16 rows x 256 columns, lane 4g + t of a tile holds row g, column quarter t) is
 // loaded as it lies; the 16x128b form of tcgen05.st wants exactly that distribution: lane 4g + t writes word t of
 // every 4-word block of rows g and g + 8 (measured with 16 warps storing: 64 clocks per 2 KB, 16x256b takes 127,
@@ -82,6 +89,7 @@ struct TcBatch {
   int count;
   unsigned per, extra;       // units of the launch: grid * per + extra
   float ctas_per_unit;       // about grid / units
+  int share;                 // SHARE: CTAs per tile
   int words;                 // 1: parts are sums of both planes, 2: the planes apart
   int clean;                 // leave the scratch zero-filled
   unsigned long long nonce;  // marks a part as left by this launch; the reader puts zero back
@@ -245,6 +253,9 @@ struct Segments {
   __device__ __forceinline__ int row_tile(const TcProblem& P) const { return P.n_mt == 1 ? tile : tile / P.n_mt; }
 };
 
+// Tokens of a tile that each of its `share` CTAs finishes (a multiple of eight, what the epilogue stores at a time).
+__device__ __forceinline__ int share_tokens(int n_tok, int share) { return ((n_tok + 7) / 8 + share - 1) / share * 8; }
+
 // Byte tables of one row: entry i is byte i & 3 of word i >> 2.  2 bit: one word (used twice by the lookup).
 template <int BITS>
 struct RowTables {
@@ -306,7 +317,8 @@ __host__ __device__ constexpr int tc_smem_layout(int what) {
   return what == 0 ? kB : what == 1 ? kRingSlot : what == 2 ? kB + kRing : kB + kRing + 8 * kBars + 16;
 }
 
-template <int BITS, int NT, int ACT>
+// SHARE: the CTAs of a tile are a cluster and finish it together (its own instances: 0.2 us of a launch otherwise).
+template <int BITS, int NT, int ACT, bool SHARE>
 __global__ void __launch_bounds__(kTcThreads, 1)
 lut_gemv_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcBatch B, int* status) {
   extern __shared__ uint8_t tc_smem_raw[];
@@ -376,6 +388,113 @@ lut_gemv_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ 
   const uint32_t u0 = unit_begin(blockIdx.x, B), u1 = unit_begin(blockIdx.x + 1, B);      // not empty
   Segments sg;
   sg.first(u0, u1, B);
+
+  // The piece's first tile, reached last, has columns in other CTAs: the decoder warps finish it.  The other parts come by bulk
+  // copies into the shared memory that rings and levels have left (with plain loads, 32 KB in flight per SM, this took
+  // 12 us for 100 tokens and three parts), tokens in rounds of as many as fit.
+  auto finish = [&](uint32_t acc) {
+    const TcProblem& P = B.p[sg.p];
+    {
+      const uint32_t last = u1 - u0 - 1, tile0 = P.unit0 + (uint32_t)sg.tile * (uint32_t)P.n_kt, quad = warp & 3;
+      const int share = SHARE ? B.share : 0, rank = SHARE ? (int)(blockIdx.x % (uint32_t)share) : 0;
+      const int parts = SHARE ? share - 1 : (int)(blockIdx.x - unit_owner(tile0, B));      // at most kTcMaxParts (the launcher's grid)
+      auto part_block = [&](int i) { return SHARE ? blockIdx.x - rank + (i < rank ? i : i + 1) : blockIdx.x - 1 - i; };
+      const int rt = sg.row_tile(P), m0 = (sg.tile - rt * P.n_mt) * NT, all_tok = min(NT, P.M - m0);
+      // this CTA's tokens
+      const int own = SHARE ? share_tokens(all_tok, share) : NT, first_tok = rank * own, n_tok = min(all_tok, first_tok + own);
+      const int row = 32 * (int)quad + lane, out = rt * kTcRows + row, words = B.words;
+      const float row_scale = tc_row_scale<BITS>(P.codebook + (size_t)min(out, P.n_rp * 16 - 1) * (1 << BITS));
+      const int fit = (tc_smem_layout<BITS, NT>(2) / (parts * words * kTcRows * 4)) & ~3, step = fit < NT ? fit : NT;
+      const size_t part_ints = (size_t)words * NT * kTcRows;
+      asm volatile("griddepcontrol.wait;" ::: "memory");     // scales, scratch and y belong to earlier kernels until here
+      tc_wait(done(last % (2 * S)), (last / (2 * S)) & 1u, abort_flag);
+      __syncwarp();
+      tc_fence_after();
+      const uint32_t t_hi = tmem_base + ((32 * quad) << 16) + kAccCol0 + acc * (2 * NT);
+      uint32_t round = 0;
+#pragma unroll 1
+      for (int c0 = first_tok; c0 < n_tok; c0 += step, ++round) {
+        const int n_now = min(step, n_tok - c0);
+        if (warp == 0) {
+          if (lane == 0) tc_expect(part_bar, (uint32_t)(parts * words * n_now * kTcRows * 4));
+          __syncwarp();
+          if (lane < parts) {          // a lane per part: its copy starts as soon as it is there
+            const int* src = B.parts + (size_t)part_block(lane) * part_ints + c0 * kTcRows;
+            if (!SHARE && round == 0) {
+              unsigned long long* flag = B.flags + (blockIdx.x - 1 - lane);
+              const unsigned long long t0 = tc_timer();
+              unsigned long long seen = 0;
+#pragma unroll 1
+              for (uint32_t it = 1;; ++it) {
+                asm volatile("ld.acquire.gpu.global.b64 %0, [%1];" : "=l"(seen) : "l"(flag) : "memory");
+                if (seen == B.nonce) break;
+                if ((it & 63u) == 0 && (*abort_flag || tc_timer() - t0 > kTcWaitNs)) { *abort_flag = 1; break; }
+              }
+              *flag = 0ull;
+            }
+            asm volatile("fence.proxy.async;" ::: "memory");       // written by ordinary stores, read by copies
+            for (int w = 0; w < words; ++w)
+              tc_bulk(base + (uint32_t)((lane * words + w) * step * kTcRows * 4), src + w * NT * kTcRows,
+                      (uint32_t)(n_now * kTcRows * 4), part_bar);
+          }
+          __syncwarp();
+        }
+        const int* buf = reinterpret_cast<const int*>(gen_base) + row;
+        bool landed = false;
+#pragma unroll 1
+        for (int c = 4 * (warp >> 2); c < n_now; c += 16) {
+          uint32_t hi[4], lo[4];
+          tc_ld4(t_hi + c0 + c, hi);
+          tc_ld4(t_hi + NT + c0 + c, lo);
+          const int m = m0 + c0 + c;
+          const float sc = m + (lane & 3) < P.M ? __ldg(P.act_scale + m + (lane & 3)) : 0.0f;
+          if (!landed) tc_wait(part_bar, round & 1u, abort_flag);
+          landed = true;
+          __syncwarp();
+          tc_wait_ld4(hi, lo);
+          if (words == 1) {
+            long long sum[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              sum[j] = ACT == kActPacked4 ? (long long)((int)hi[j] >> 4) * 256 + ((int)lo[j] >> 4) : (long long)(int)hi[j] * 256 + (int)lo[j];
+            for (int p = 0; p < parts; ++p)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) sum[j] += buf[(p * step + c + j) * kTcRows];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const float s = __shfl_sync(0xffffffffu, sc, j) * row_scale;
+              if (c + j < n_now && out < P.N) P.y[(size_t)(m + j) * P.ldy + out] = __ll2float_rn(sum[j]) * s;
+            }
+          } else {
+            for (int p = 0; p < parts; ++p)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                hi[j] += (uint32_t)buf[(2 * p * step + c + j) * kTcRows];
+                lo[j] += (uint32_t)buf[((2 * p + 1) * step + c + j) * kTcRows];
+              }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const float s = __shfl_sync(0xffffffffu, sc, j) * (ACT == kActPacked4 ? row_scale * 0.0625f : row_scale);
+              if (c + j < n_now && out < P.N) P.y[(size_t)(m + j) * P.ldy + out] = ((float)(int)hi[j] * 256.0f + (float)(int)lo[j]) * s;
+            }
+          }
+          if (B.clean)
+            for (int p = 0; p < parts; ++p) {
+              int* at = B.parts + (size_t)part_block(p) * part_ints + (c0 + c) * kTcRows + row;
+#pragma unroll
+              for (int j = 0; j < 4; ++j)
+                if (c + j < n_now) {
+                  __stcg(at + j * kTcRows, 0);
+                  if (words == 2) __stcg(at + (NT + j) * kTcRows, 0);
+                }
+            }
+        }
+        if (!landed) tc_wait(part_bar, round & 1u, abort_flag);      // (the copies land before the CTA may exit)
+        asm volatile("bar.sync 2, 512;" ::: "memory");               // the buffer has been read
+      }
+      if (*abort_flag && round > 0) tc_drain(part_bar, (round - 1) & 1u);
+    }
+  };
 
   if (warp == kTcCopyWarp) {
     // ------------------------------------------------------------------ index copies
@@ -568,106 +687,7 @@ lut_gemv_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ 
       sg.next(B);
       ++n_seg;
     }
-    // The piece's first tile, reached last, has columns in other CTAs: these warps finish it.  The other parts come by bulk
-    // copies into the shared memory that rings and levels have left (with plain loads, 32 KB in flight per SM, this took
-    // 12 us for 100 tokens and three parts), tokens in rounds of as many as fit.
-    const TcProblem& P = B.p[sg.p];
-    if (sg.ka > 0 && sg.kb == P.n_kt - 1) {
-      const uint32_t last = u1 - u0 - 1, tile0 = P.unit0 + (uint32_t)sg.tile * (uint32_t)P.n_kt;
-      const int parts = (int)(blockIdx.x - unit_owner(tile0, B));          // 1..kTcMaxParts (ka > 0; the launcher's grid)
-      const int rt = sg.row_tile(P), m0 = (sg.tile - rt * P.n_mt) * NT, n_tok = min(NT, P.M - m0);
-      const int row = 32 * (int)quad + lane, out = rt * kTcRows + row, words = B.words;
-      const float row_scale = tc_row_scale<BITS>(P.codebook + (size_t)min(out, P.n_rp * 16 - 1) * (1 << BITS));
-      const int fit = (tc_smem_layout<BITS, NT>(2) / (parts * words * kTcRows * 4)) & ~3, step = fit < NT ? fit : NT;
-      const size_t part_ints = (size_t)words * NT * kTcRows;
-      asm volatile("griddepcontrol.wait;" ::: "memory");     // scales, scratch and y belong to earlier kernels until here
-      tc_wait(done(last % (2 * S)), (last / (2 * S)) & 1u, abort_flag);
-      __syncwarp();
-      tc_fence_after();
-      const uint32_t t_hi = tmem_base + ((32 * quad) << 16) + kAccCol0 + (n_seg % NBUF) * (2 * NT);
-      uint32_t round = 0;
-#pragma unroll 1
-      for (int c0 = 0; c0 < n_tok; c0 += step, ++round) {
-        const int n_now = min(step, n_tok - c0);
-        if (warp == 0) {
-          if (lane == 0) tc_expect(part_bar, (uint32_t)(parts * words * n_now * kTcRows * 4));
-          __syncwarp();
-          if (lane < parts) {          // a lane per part: its copy starts as soon as it is there
-            const int* src = B.parts + (size_t)(blockIdx.x - 1 - lane) * part_ints + c0 * kTcRows;
-            if (round == 0) {
-              unsigned long long* flag = B.flags + (blockIdx.x - 1 - lane);
-              const unsigned long long t0 = tc_timer();
-              unsigned long long seen = 0;
-#pragma unroll 1
-              for (uint32_t it = 1;; ++it) {
-                asm volatile("ld.acquire.gpu.global.b64 %0, [%1];" : "=l"(seen) : "l"(flag) : "memory");
-                if (seen == B.nonce) break;
-                if ((it & 63u) == 0 && (*abort_flag || tc_timer() - t0 > kTcWaitNs)) { *abort_flag = 1; break; }
-              }
-              *flag = 0ull;
-            }
-            asm volatile("fence.proxy.async;" ::: "memory");       // written by ordinary stores, read by copies
-            for (int w = 0; w < words; ++w)
-              tc_bulk(base + (uint32_t)((lane * words + w) * step * kTcRows * 4), src + w * NT * kTcRows,
-                      (uint32_t)(n_now * kTcRows * 4), part_bar);
-          }
-          __syncwarp();
-        }
-        const int* buf = reinterpret_cast<const int*>(gen_base) + row;
-        bool landed = false;
-#pragma unroll 1
-        for (int c = 4 * (warp >> 2); c < n_now; c += 16) {
-          uint32_t hi[4], lo[4];
-          tc_ld4(t_hi + c0 + c, hi);
-          tc_ld4(t_hi + NT + c0 + c, lo);
-          const int m = m0 + c0 + c;
-          const float sc = m + (lane & 3) < P.M ? __ldg(P.act_scale + m + (lane & 3)) : 0.0f;
-          if (!landed) tc_wait(part_bar, round & 1u, abort_flag);
-          landed = true;
-          __syncwarp();
-          tc_wait_ld4(hi, lo);
-          if (words == 1) {
-            long long sum[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-              sum[j] = ACT == kActPacked4 ? (long long)((int)hi[j] >> 4) * 256 + ((int)lo[j] >> 4) : (long long)(int)hi[j] * 256 + (int)lo[j];
-            for (int p = 0; p < parts; ++p)
-#pragma unroll
-              for (int j = 0; j < 4; ++j) sum[j] += buf[(p * step + c + j) * kTcRows];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const float s = __shfl_sync(0xffffffffu, sc, j) * row_scale;
-              if (c + j < n_now && out < P.N) P.y[(size_t)(m + j) * P.ldy + out] = __ll2float_rn(sum[j]) * s;
-            }
-          } else {
-            for (int p = 0; p < parts; ++p)
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                hi[j] += (uint32_t)buf[(2 * p * step + c + j) * kTcRows];
-                lo[j] += (uint32_t)buf[((2 * p + 1) * step + c + j) * kTcRows];
-              }
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const float s = __shfl_sync(0xffffffffu, sc, j) * (ACT == kActPacked4 ? row_scale * 0.0625f : row_scale);
-              if (c + j < n_now && out < P.N) P.y[(size_t)(m + j) * P.ldy + out] = ((float)(int)hi[j] * 256.0f + (float)(int)lo[j]) * s;
-            }
-          }
-          if (B.clean)
-            for (int p = 0; p < parts; ++p) {
-              int* at = B.parts + (size_t)(blockIdx.x - 1 - p) * part_ints + (c0 + c) * kTcRows + row;
-#pragma unroll
-              for (int j = 0; j < 4; ++j)
-                if (c + j < n_now) {
-                  __stcg(at + j * kTcRows, 0);
-                  if (words == 2) __stcg(at + (NT + j) * kTcRows, 0);
-                }
-            }
-        }
-        if (!landed) tc_wait(part_bar, round & 1u, abort_flag);      // (the copies land before the CTA may exit)
-        asm volatile("bar.sync 2, 512;" ::: "memory");               // the buffer has been read
-      }
-      if (*abort_flag) tc_drain(part_bar, (round - 1) & 1u);
-    }
+    if (!SHARE && sg.ka > 0 && sg.kb == B.p[sg.p].n_kt - 1) finish(n_seg % NBUF);
   } else if (warp < kTcFirstToken || (ACT == kActReady && warp < kTcCopyWarp)) {
     // ------------------------------------------------------------------ epilogue
     asm volatile("griddepcontrol.wait;" ::: "memory");     // scales, scratch and y belong to earlier kernels until here
@@ -677,15 +697,19 @@ lut_gemv_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ 
     do {
       const TcProblem& P = B.p[sg.p];
       const bool owner = sg.kb == P.n_kt - 1;
-      if (owner && sg.ka > 0) break;                       // the last one: finished by the decoder warps
+      if (!SHARE && owner && sg.ka > 0) break;       // the last one: finished by the decoder warps
+      const bool whole_tile = !SHARE && owner;
       const uint32_t buf = n_seg % NBUF;
       const int rt = sg.row_tile(P), m0 = (sg.tile - rt * P.n_mt) * NT, n_tok = min(NT, P.M - m0), out = rt * kTcRows + row;
+      // a shared tile: this CTA finishes these tokens itself
+      const int skip0 = SHARE ? (int)(blockIdx.x % (uint32_t)B.share) * share_tokens(n_tok, B.share) : 0;
+      const int skip1 = SHARE ? skip0 + share_tokens(n_tok, B.share) : 0;
       float row_scale = 0.0f;
-      if (owner) row_scale = tc_row_scale<BITS>(P.codebook + (size_t)min(out, P.n_rp * 16 - 1) * (1 << BITS)) * (ACT == kActPacked4 ? 0.0625f : 1.0f);
+      if (whole_tile) row_scale = tc_row_scale<BITS>(P.codebook + (size_t)min(out, P.n_rp * 16 - 1) * (1 << BITS)) * (ACT == kActPacked4 ? 0.0625f : 1.0f);
       int* part = B.parts + (size_t)blockIdx.x * words * NT * kTcRows + row;
       auto scales = [&](int c) {
         const int m = m0 + 8 * c + (lane & 7);
-        return owner && m < P.M ? __ldg(P.act_scale + m) : 0.0f;
+        return whole_tile && m < P.M ? __ldg(P.act_scale + m) : 0.0f;
       };
       float sc = scales(half);
       tc_wait(acc_full(buf), (n_seg / NBUF) & 1u, abort_flag);
@@ -710,7 +734,7 @@ lut_gemv_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ 
         }
         // (uniform) all eight tokens are inside: no test per token; these warps compete with the decoders for issue slots
         const bool whole = 8 * c + 8 <= n_tok;
-        if (owner) {
+        if (whole_tile) {
           float* y = P.y + (size_t)(m0 + 8 * c) * P.ldy + out;
           float v[8];
 #pragma unroll
@@ -728,7 +752,7 @@ lut_gemv_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ 
                 if (8 * c + j < n_tok) y[(size_t)j * P.ldy] = v[j];
             }
           }
-        } else {
+        } else if (!SHARE || 8 * c < skip0 || 8 * c >= skip1) {
           int* at = part + 8 * c * kTcRows;
           if (words == 1) {
             // (packed levels are held as 16 q: all sums are multiples of 16)
@@ -754,12 +778,12 @@ lut_gemv_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ 
       }
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");     // (n_tok <= 8 * half: the first loads are still out)
       tc_fence_before();
-      if (!owner) __threadfence();
+      if (!whole_tile) __threadfence();
       __syncwarp();
       if (lane == 0) {
         tc_arrive(acc_empty(buf));
         // the last of the warps says that the part is there (one flag: a reader's look at one takes it a microsecond)
-        if (!owner && atomicAdd(parts_stored, 1) == 4 * kEpiHalves - 1) {
+        if (!whole_tile && !SHARE && atomicAdd(parts_stored, 1) == 4 * kEpiHalves - 1) {
           __threadfence();
           asm volatile("st.release.gpu.global.b64 [%0], %1;" ::"l"(B.flags + blockIdx.x), "l"(B.nonce) : "memory");
         }
@@ -857,6 +881,14 @@ lut_gemv_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ 
     } while (sg.next(B));
   }
 
+  if constexpr (SHARE) {
+    // every CTA of the cluster has stored its part (its warps have left their roles: all their waits are bounded)
+    __threadfence();
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    if (warp < kTcDecoders) finish(0);
+  }
   tc_fence_before();
   __syncthreads();
   if (warp == kTcMmaWarp) {
@@ -899,20 +931,27 @@ __global__ void __launch_bounds__(256) ready_levels_kernel(const uint8_t* __rest
 int tc_sm_count() { return current_sm_count(); }
 
 // Shape of a launch.
+constexpr int kTcMaxShare = 8;                // CTAs of a portable cluster
+
+// Clusters of `size` CTAs with an SM each that are resident together (the graphics processing clusters' sizes decide).
+int tc_max_clusters(int size);
+
 struct TcPlan {
-  int act, nt, words, grid;
+  int act, nt, words, grid, share;
   unsigned long long units;
   size_t parts_bytes, flags_bytes;
   double us;                 // estimated duration
 };
 // One token width: the grid with the shortest estimate.  Measured on B200 (microseconds): a unit 0.33 / 0.35 / 0.68 at
 // up to 32 / 64 / 128 tokens, 2 bit (3 bit 5 % more; 4 bit 0.68 / 0.68 / 0.88: its lookups; 128 tokens take 0.57 in a launch
-// of a few units per SM, 0.83 in one of a millisecond, as the dense kernel's stages lengthen too); 3 before the first unit
-// and after the last store; a tile's drain 0.016 a token; a cut tile 2.5 for the hand-over, and 512 bytes a token and part
-// at 20 GB/s per SM to read the parts back.  Against the dense kernel this chooses right to a few percent (2 bit, one call
-// from x to y, tensor memory / dense): 13B layer 127 / 224 at 256 tokens, 254 / 299 at 512, 500 / 544 at 1024, 1060 / 975 at
-// 2048; 7B layer 57 / 179 at 128, 320 / 348 at 1024, 684 / 637 at 2048; layer of 1024 columns 79 / 100 at 2048.  Candidates: all SMs (least work per CTA, most tiles cut), and, where the rows are
-// of one length, one to four CTAs per tile (no tile cut with one).
+// of a few units per SM, 0.83 in one of a millisecond, as the dense kernel's stages lengthen too); 3 before the
+// first unit and after the last store; a tile's drain 0.016 a token; a cut tile 2.5 for the hand-over, and 512 bytes a token
+// and part at 20 GB/s per SM to read the parts back; a tile shared in a cluster 3.6, each CTA reading its tokens only.
+// Against the dense kernel this chooses right to a few percent (2 bit, one call from x to y, tensor memory / dense): 13B
+// layer 127 / 224 at 256 tokens, 254 / 299 at 512, 500 / 544 at 1024, 1060 / 975 at 2048; 7B layer 57 / 179 at 128, 320 /
+// 348 at 1024, 684 / 637 at 2048; layer of 1024 columns 79 / 100 at 2048.  Candidates: all SMs (least work per CTA, most
+// tiles cut), and, where the rows are of one length, one CTA per tile (none cut), two to four with the last one finishing,
+// two to eight as a cluster that finishes together.
 TcPlan tc_plan_width(const Problem* probs, int count, int nt) {
   TcPlan q = {};
   q.act = probs[0].dense_levels ? kActReady : probs[0].act_bits == 8 ? kActBytes : kActPacked4;
@@ -936,21 +975,22 @@ TcPlan tc_plan_width(const Problem* probs, int count, int nt) {
   if (most > q.units / piece) most = q.units / piece;
   const double unit_us = probs[0].bits == 4 ? (nt == 128 ? 0.88 : 0.68) : (nt <= 32 ? 0.33 : nt == 64 ? 0.35 : 0.68) * (probs[0].bits == 3 ? 1.05 : 1.0);
   const double tokens = (double)(max_m < nt ? max_m : nt);
-  for (int s = 0; s <= 4; ++s) {
-    unsigned long long grid = most;
-    if (s > 0) {
-      if (min_kt != max_kt || tiles * s > most) break;
-      grid = tiles * s;
-    }
-    const double parts = s > 0 ? s - 1 : (double)grid / tiles + 0.5;
-    const double drains = nt > 32 && s != 1 ? 1.0 + (double)tiles / grid : 1.0;        // tiles drained one after the other
-    const double us = 3.0 + (double)((q.units + grid - 1) / grid) * unit_us + drains * tokens * 0.016 +
-                      (parts > 0 ? 2.5 + parts * tokens * 512 / 20000 : 0.0);
-    if (s == 0 || us < q.us) {
+  auto consider = [&](unsigned long long grid, int share, double parts, double fixed, double read_tokens, double drains) {
+    const double us = fixed + (double)((q.units + grid - 1) / grid) * unit_us + drains * tokens * 0.016 + parts * read_tokens * 512 / 20000;
+    if (q.grid == 0 || us < q.us) {
       q.us = us;
       q.grid = (int)grid;
+      q.share = share;
     }
-  }
+  };
+  const double drains = nt > 32 ? 1.0 + (double)tiles / most : 1.0;        // tiles drained one after the other
+  consider(most, 0, (double)most / tiles + 0.5, 5.5, tokens, drains);
+  if (min_kt == max_kt)
+    for (int s = 1; s <= kTcMaxShare && s <= min_kt && tiles * s <= n_sm; ++s) {
+      if (s == 1) consider(tiles, 0, 0.0, 3.0, 0.0, 1.0);
+      else if (s <= 4 && tiles * s <= most) consider(tiles * s, 0, s - 1, 5.5, tokens, nt > 32 ? 1.0 + 1.0 / s : 1.0);
+      if (s > 1 && tiles <= (unsigned long long)tc_max_clusters(s)) consider(tiles * s, s, s - 1, 6.6, (double)(((int64_t)tokens + 8 * s - 1) / (8 * s) * 8), 1.0);
+    }
   q.words = probs[0].act_bits == 4 && (q.units + q.grid - 1) / q.grid <= kTcWordUnits ? 1 : 2;
   q.parts_bytes = (size_t)q.grid * q.words * q.nt * kTcRows * sizeof(int);
   q.flags_bytes = (size_t)round_up_u64((uint64_t)q.grid * sizeof(unsigned long long), 256);
@@ -979,26 +1019,29 @@ unsigned long long tc_nonce() {
 }
 
 template <typename... Params, typename... Args>
-lcd_status tc_launch(void (*kern)(Params...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream, Args&&... args) {
+lcd_status tc_launch(void (*kern)(Params...), unsigned grid, unsigned cluster, unsigned block, size_t smem, cudaStream_t stream, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, args...);
   if (e != cudaSuccess) { set_cuda_error((int)e); return LCD_ERR_CUDA; }
   return LCD_OK;
 }
 
 // Weights are streamed before griddepcontrol.wait; levels, scales, scratch and y are touched after it.
-template <int BITS, int NT, int ACT>
-lcd_status tc_launch_t(const TcMaps& maps, const TcBatch& batch, int grid, int32_t* status, cudaStream_t stream) {
-  auto kern = lut_gemv_tc_kernel<BITS, NT, ACT>;
+template <int BITS, int NT, int ACT, bool SHARE>
+lcd_status tc_launch_instance(const TcMaps& maps, const TcBatch& batch, int grid, int32_t* status, cudaStream_t stream) {
+  auto kern = lut_gemv_tc_kernel<BITS, NT, ACT, SHARE>;
   constexpr size_t smem = 1024 + (size_t)tc_smem_layout<BITS, NT>(3);
   static_assert(smem <= 227 * 1024, "shared memory of one CTA");
   static PerDeviceFlag attr_set;   // per template instance and device
@@ -1008,7 +1051,42 @@ lcd_status tc_launch_t(const TcMaps& maps, const TcBatch& batch, int grid, int32
     if (e != cudaSuccess) { set_cuda_error((int)e); return LCD_ERR_CUDA; }
     attr_set.done(dev);
   }
-  return tc_launch(kern, (unsigned)grid, kTcThreads, smem, stream, maps, batch, status);
+  return tc_launch(kern, (unsigned)grid, (unsigned)(SHARE ? batch.share : 1), kTcThreads, smem, stream, maps, batch, status);
+}
+template <int BITS, int NT, int ACT>
+lcd_status tc_launch_t(const TcMaps& maps, const TcBatch& batch, int grid, int32_t* status, cudaStream_t stream) {
+  return batch.share > 0 ? tc_launch_instance<BITS, NT, ACT, true>(maps, batch, grid, status, stream)
+                         : tc_launch_instance<BITS, NT, ACT, false>(maps, batch, grid, status, stream);
+}
+
+int tc_max_clusters(int size) {
+  static std::atomic<int> known[64][kTcMaxShare + 1];         // + 1; a property of the device
+  int dev = 0;
+  const bool have = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64;
+  if (have) {
+    const int v = known[dev][size].load(std::memory_order_relaxed);
+    if (v > 0) return v - 1;
+  }
+  auto kern = lut_gemv_tc_kernel<2, 16, kActPacked4, true>;                  // (every instance takes an SM to itself)
+  constexpr size_t smem = 1024 + (size_t)tc_smem_layout<2, 16>(3);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)size);
+  cfg.blockDim = dim3(kTcThreads);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)size;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (!have || cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return 0;                    // (no device: no shares)
+  }
+  known[dev][size].store(n + 1, std::memory_order_relaxed);
+  return n;
 }
 
 template <int BITS>
@@ -1056,10 +1134,10 @@ lcd_status launch_ready_levels(const Problem& p, void* out, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   // (4-bit indices: the order of 3-bit ones)
   if (p.bits == 2)
-    return p.act_bits == 8 ? tc_launch(ready_levels_kernel<2, true>, blocks, 256, 0, s, p.act_idx, n, o)
-                           : tc_launch(ready_levels_kernel<2, false>, blocks, 256, 0, s, p.act_idx, n, o);
-  return p.act_bits == 8 ? tc_launch(ready_levels_kernel<3, true>, blocks, 256, 0, s, p.act_idx, n, o)
-                         : tc_launch(ready_levels_kernel<3, false>, blocks, 256, 0, s, p.act_idx, n, o);
+    return p.act_bits == 8 ? tc_launch(ready_levels_kernel<2, true>, blocks, 1, 256, 0, s, p.act_idx, n, o)
+                           : tc_launch(ready_levels_kernel<2, false>, blocks, 1, 256, 0, s, p.act_idx, n, o);
+  return p.act_bits == 8 ? tc_launch(ready_levels_kernel<3, true>, blocks, 1, 256, 0, s, p.act_idx, n, o)
+                         : tc_launch(ready_levels_kernel<3, false>, blocks, 1, 256, 0, s, p.act_idx, n, o);
 }
 
 lcd_status launch_lut_gemv_tc(const Problem* probs, int count, void* workspace, size_t workspace_bytes,
@@ -1120,6 +1198,7 @@ lcd_status launch_lut_gemv_tc(const Problem* probs, int count, void* workspace, 
   batch.per = (unsigned)(total / q.grid);
   batch.extra = (unsigned)(total % q.grid);
   batch.ctas_per_unit = (float)((double)q.grid / (double)total);
+  batch.share = q.share;
   batch.words = q.words;
   batch.clean = max_m <= 32;       // few tokens: the scratch, zero-filled by the caller, is left zero-filled
   batch.nonce = tc_nonce();
