@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include "common.h"
+#include "device_util.h"
 
 namespace lcd {
 
@@ -54,11 +55,15 @@ __global__ void __launch_bounds__(256) smoothing_factors_kernel(const __half* __
 // partial[g][t] = sum_k (x - level * s_q * s)^2 of token t under candidate g, kTokens tokens a CTA (a factor is loaded and
 // widened once for all of them); the CTA that arrives last averages, picks the first smallest candidate and writes its
 // factors.  Bound by instruction issue: per element and candidate two multiplications, clip, rounding by one addition, one
-// conversion and four binary64 operations (11 M elements of 4096 columns, 128 tokens, 21 candidates: 26 us for the
+// conversion and four binary64 operations (11 M elements of 4096 columns, 128 tokens, 21 candidates: 24.5 us for the
 // whole search; 56 with a division per element and pass, three conversions and a kernel each for maxima, factors and pick).
 constexpr int kTokens = 4;
-template <bool VEC>
-__global__ void __launch_bounds__(256) smoothing_error_kernel(const __half* __restrict__ x, int64_t T, int64_t K, int64_t ldx, int G,
+// PER_SM: CTAs that an SM must hold.  Four leave all the registers the compiler wants (56); a grid that does not fit four times
+// into the SMs is 10 % faster with five (512 tokens x 14336 columns x 33 candidates 262 -> 237 us), a smaller one 8 % slower
+// (128 x 4096 x 9: 15.0, 16.3).  Single columns a step (rows at odd addresses) want 79 registers (200 x 5003 x 11: 35.7 us,
+// 38.3 with four CTAs).
+template <bool VEC, int PER_SM>
+__global__ void __launch_bounds__(256, PER_SM) smoothing_error_kernel(const __half* __restrict__ x, int64_t T, int64_t K, int64_t ldx, int G,
                                                               const float* __restrict__ s, const float* __restrict__ inv,
                                                               double* __restrict__ partial, unsigned* __restrict__ arrived,
                                                               double* __restrict__ mse, int32_t* __restrict__ best, float* __restrict__ inv_smooth) {
@@ -238,8 +243,9 @@ lcd_status launch_smoothing_search(const void* x, int64_t T, int64_t K, int64_t 
     // rows of x start on 16 bytes (the rows of the factors do where K is a multiple of four)
     const bool vec = K % 8 == 0 && ldx % 8 == 0 && reinterpret_cast<uintptr_t>(x) % 16 == 0;
     cfg.gridDim = dim3((unsigned)((T + kTokens - 1) / kTokens), (unsigned)G);
-    e = vec ? cudaLaunchKernelEx(&cfg, smoothing_error_kernel<true>, xh, T, K, ldx, G, (const float*)s, (const float*)inv, partial, arrived, mse, best, inv_smooth)
-            : cudaLaunchKernelEx(&cfg, smoothing_error_kernel<false>, xh, T, K, ldx, G, (const float*)s, (const float*)inv, partial, arrived, mse, best, inv_smooth);
+    const bool many = (uint64_t)cfg.gridDim.x * cfg.gridDim.y > 4ull * (uint64_t)current_sm_count();
+    auto kern = !vec ? smoothing_error_kernel<false, 1> : many ? smoothing_error_kernel<true, 5> : smoothing_error_kernel<true, 4>;
+    e = cudaLaunchKernelEx(&cfg, kern, xh, T, K, ldx, G, (const float*)s, (const float*)inv, partial, arrived, mse, best, inv_smooth);
   }
   if (e != cudaSuccess) { set_cuda_error((int)e); return LCD_ERR_CUDA; }
   return LCD_OK;
