@@ -2,9 +2,11 @@
 // sort; sigma from six nearest-rank percentiles; two seed clusters around the extreme weights; MinPts and eps from
 // them; DBSCAN on the rest; lower medians.  On sorted one-dimensional data DBSCAN is local: a point's neighbours are its
 // neighbours in the array, core points chain into one cluster while the gap to the core point before is at most eps, and
-// another point looks for a core point within eps on either side.  So two passes over the sorted array do it: one marks
+// another point needs the nearest core point on either side.  So two passes over the sorted array do it: one marks
 // the core points and sums up every tile (first and last core point, gaps between), one writes the labels, with a scan
-// over the tiles between them.  A tile without gaps or non-core points, nearly every one, is written without being read
+// over the tiles in either direction between them: what lies before a word of 32 points and the first core point after it
+// are then known, and no point looks at another one, however many share its value (walking out to the core points takes up
+// to MinPts steps a point: 400 K weights on eight values 107 ms, 0.2 so).  A tile without gaps or non-core points, nearly every one, is written without being read
 // again, and where 4096 weights span less than eps two of them tell so: little more than the labels' 4 bytes a weight is
 // moved (45 M weights: 130 us after the sort; with a thread a point, two max-scans and a sum-scan over the whole
 // array 2600).
@@ -108,6 +110,11 @@ struct Chain {
   float first, last;
   int any, gaps;
 };
+// The first core point after a tile, if there is one.
+struct Next {
+  float v;
+  int any;
+};
 __device__ __forceinline__ bool gap_after(float before, float at, double eps) { return (double)at - (double)before > eps; }
 __device__ __forceinline__ Chain join(const Chain& a, const Chain& b, double eps) {
   if (!a.any) return b;
@@ -205,16 +212,34 @@ __global__ void __launch_bounds__(32 * kTileWarps) dbci_mark_kernel(const float*
   }
 }
 
-// Exclusive scan of the tiles' chains in place: chains[t] becomes the chain of all tiles before t.  One CTA; a thread joins
-// its run of tiles, the threads' runs are scanned, then it walks its run again.
-__global__ void __launch_bounds__(1024) dbci_scan_kernel(DbciParams* __restrict__ P, Chain* __restrict__ chains, int n_tiles) {
+// Exclusive scan of the tiles' chains in place: chains[t] becomes the chain of all tiles before t; next[t] the first core
+// point of all tiles after t.  One CTA; a thread joins its run of tiles, the threads' runs are scanned, then it walks its run
+// again, backwards and forwards.
+__global__ void __launch_bounds__(1024) dbci_scan_kernel(DbciParams* __restrict__ P, Chain* __restrict__ chains, Next* __restrict__ next, int n_tiles) {
   __shared__ Chain part[1024];
+  __shared__ float first_of[1024];
+  __shared__ unsigned any_of[32];          // threads whose runs have core points, a word per warp
   const double eps = P->eps;
   const int per = (n_tiles + 1023) / 1024, t0 = threadIdx.x * per, t1 = min(t0 + per, n_tiles);
   Chain mine = {0.0f, 0.0f, 0, 0};
   for (int t = t0; t < t1; ++t) mine = join(mine, chains[t], eps);
   part[threadIdx.x] = mine;
+  first_of[threadIdx.x] = mine.first;
+  const unsigned any_word = __ballot_sync(0xffffffffu, mine.any != 0);
+  if ((threadIdx.x & 31) == 0) any_of[threadIdx.x >> 5] = any_word;
   __syncthreads();
+  Next after = {0.0f, 0};
+  {
+    int w = threadIdx.x >> 5;
+    unsigned word = any_of[w] & ~(0xffffffffu >> (31 - (threadIdx.x & 31)));        // the threads after this one
+    while (word == 0 && ++w < 32) word = any_of[w];
+    if (word) after = {first_of[32 * w + __ffs(word) - 1], 1};
+  }
+  for (int t = t1 - 1; t >= t0; --t) {
+    next[t] = after;
+    const Chain c = chains[t];
+    if (c.any) after = {c.first, 1};
+  }
   for (int o = 1; o < 1024; o <<= 1) {
     Chain v = part[threadIdx.x];
     if ((int)threadIdx.x >= o) v = join(part[threadIdx.x - o], v, eps);
@@ -236,7 +261,7 @@ __global__ void __launch_bounds__(1024) dbci_scan_kernel(DbciParams* __restrict_
 // first / last member of every cluster
 __global__ void __launch_bounds__(32 * kTileWarps) dbci_label_kernel(const float* __restrict__ x, long long n, DbciParams* __restrict__ P,
                                                                      const unsigned* __restrict__ core, const Chain* __restrict__ chains,
-                                                                     const unsigned char* __restrict__ plain, int* __restrict__ labels,
+                                                                     const Next* __restrict__ next, const unsigned char* __restrict__ plain, int* __restrict__ labels,
                                                                      int* __restrict__ first, int* __restrict__ last, int max_clusters) {
   __shared__ Chain part[kTileWarps];
   const long long L = P->L, R = P->R, tile0 = (long long)blockIdx.x * kTile;
@@ -277,13 +302,25 @@ __global__ void __launch_bounds__(32 * kTileWarps) dbci_label_kernel(const float
   __syncthreads();
   Chain run = before;
   for (int w = 0; w < warp; ++w) run = join(run, part[w], eps);
+  // the first core point after every word: of the warp's later words, of the later warps, of the later tiles
+  Next after = next[blockIdx.x];
+  for (int w = kTileWarps - 1; w > warp; --w)
+    if (part[w].any) after = {part[w].first, 1};
+  float next_v[kWarpSteps];
+  unsigned has_next = 0;
+  int noise = 0;
+#pragma unroll
+  for (int i = kWarpSteps - 1; i >= 0; --i) {
+    next_v[i] = after.v;
+    has_next |= after.any ? 1u << i : 0u;
+    if (words[i]) after = {__shfl_sync(0xffffffffu, vs[i], __ffs(words[i]) - 1), 1};
+  }
 #pragma unroll
   for (int i = 0; i < kWarpSteps; ++i) {
     const long long g0 = w0 + 32 * i, g = g0 + lane;
-    const unsigned word = words[i], below = word & ((1u << lane) - 1u);
+    const unsigned word = words[i], below = word & ((1u << lane) - 1u), above = word & ~(0xffffffffu >> (31 - lane));
     const float v = vs[i];
-    const int src = below ? 31 - __clz(below) : lane;
-    const float vb = __shfl_sync(0xffffffffu, v, src);
+    const float vb = __shfl_sync(0xffffffffu, v, below ? 31 - __clz(below) : lane), va = __shfl_sync(0xffffffffu, v, above ? __ffs(above) - 1 : lane);
     const bool is = (word >> lane) & 1u;
     // the core point before this one: in this word, or the last of the run so far
     const bool starts = is && (below ? (double)v - (double)vb > eps : !run.any || gap_after(run.last, v, eps));
@@ -296,23 +333,17 @@ __global__ void __launch_bounds__(32 * kTileWarps) dbci_label_kernel(const float
       else if (g >= R) lab = n_mid + 1;
       else if (is) lab = upto;
       else {
-        // nearest core point on either side, as far as eps reaches; no core point lies between the two found
-        double dl = 1e300, dr = 1e300;
-        long long pc = -1;
-        for (long long j = g - 1; j >= L && (double)v - (double)x[j] <= eps; --j)
-          if ((core[j >> 5] >> (j & 31)) & 1u) { pc = j; dl = (double)v - (double)x[j]; break; }
-        long long nx = -1;
-        for (long long j = g + 1; j < R && (double)x[j] - (double)v <= eps; ++j)
-          if ((core[j >> 5] >> (j & 31)) & 1u) { nx = j; dr = (double)x[j] - (double)v; break; }
-        if (pc >= 0 && dl <= dr) lab = upto;
-        else if (nx >= 0) lab = upto + ((pc < 0 || gap_after(x[pc], x[nx], eps)) ? 1 : 0);
+        const bool has_left = below || run.any, has_right = above || ((has_next >> i) & 1u);
+        const float left = below ? vb : run.last, right = above ? va : next_v[i];
+        const double dl = has_left ? (double)v - (double)left : 1e300, dr = has_right ? (double)right - (double)v : 1e300;
+        if (dl <= eps && dl <= dr) lab = upto;
+        else if (dr <= eps) lab = upto + (!has_left || gap_after(left, right, eps) ? 1 : 0);
         else lab = -1;
       }
       if (labels) labels[g] = lab;
     }
-    // First and last member of every cluster, and the noise count: a warp whose lanes agree sends one pair.
-    const unsigned noise = __ballot_sync(0xffffffffu, lab == -1);
-    if (lane == 0 && noise) atomicAdd(&P->n_noise, __popc(noise));
+    noise += __popc(__ballot_sync(0xffffffffu, lab == -1));
+    // First and last member of every cluster: a warp whose lanes agree sends one pair.
     const int lab0 = __shfl_sync(0xffffffffu, lab, 0);
     if (__all_sync(0xffffffffu, lab == lab0)) {
       if (lab0 >= 0 && lab0 < max_clusters) {
@@ -325,6 +356,7 @@ __global__ void __launch_bounds__(32 * kTileWarps) dbci_label_kernel(const float
     }
     run = join(run, word_chain(word, v, eps), eps);
   }
+  if (lane == 0 && noise) atomicAdd(&P->n_noise, noise);
 }
 
 // lower medians of the clusters in ascending order; result scalars
@@ -362,7 +394,7 @@ __global__ void __launch_bounds__(256) dbci_centroid_kernel(const float* __restr
 size_t al256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 struct DbciLayout {
-  size_t sorted, core, chains, plain, first, last, params, cub, total, cub_bytes;
+  size_t sorted, core, chains, next, plain, first, last, params, cub, total, cub_bytes;
 };
 DbciLayout dbci_layout(int64_t n, int max_clusters) {
   DbciLayout l;
@@ -371,6 +403,7 @@ DbciLayout dbci_layout(int64_t n, int max_clusters) {
   l.sorted = off; off += al256((size_t)n * sizeof(float));
   l.core = off; off += al256(((size_t)n + 31) / 32 * sizeof(unsigned));
   l.chains = off; off += al256(tiles * sizeof(Chain));
+  l.next = off; off += al256(tiles * sizeof(Next));
   l.plain = off; off += al256(tiles);
   l.first = off; off += al256((size_t)max_clusters * sizeof(int));
   l.last = off; off += al256((size_t)max_clusters * sizeof(int));
@@ -396,6 +429,7 @@ lcd_status launch_dbci(const float* weights, int64_t n, void* workspace, float* 
   float* x = apart ? sorted_out : reinterpret_cast<float*>(base + l.sorted);
   unsigned* core = reinterpret_cast<unsigned*>(base + l.core);
   Chain* chains = reinterpret_cast<Chain*>(base + l.chains);
+  Next* next = reinterpret_cast<Next*>(base + l.next);
   unsigned char* plain = base + l.plain;
   int* first = reinterpret_cast<int*>(base + l.first);
   int* last = reinterpret_cast<int*>(base + l.last);
@@ -407,8 +441,8 @@ lcd_status launch_dbci(const float* weights, int64_t n, void* workspace, float* 
   if (e != cudaSuccess) { set_cuda_error((int)e); return LCD_ERR_CUDA; }
   dbci_params_kernel<<<1, 256, 0, s>>>(x, n, P, first, last, max_clusters);
   dbci_mark_kernel<<<tiles, 32 * kTileWarps, 0, s>>>(x, n, P, core, chains, plain);
-  dbci_scan_kernel<<<1, 1024, 0, s>>>(P, chains, (int)tiles);
-  dbci_label_kernel<<<tiles, 32 * kTileWarps, 0, s>>>(x, n, P, core, chains, plain, labels, first, last, max_clusters);
+  dbci_scan_kernel<<<1, 1024, 0, s>>>(P, chains, next, (int)tiles);
+  dbci_label_kernel<<<tiles, 32 * kTileWarps, 0, s>>>(x, n, P, core, chains, next, plain, labels, first, last, max_clusters);
   dbci_centroid_kernel<<<1, 256, 0, s>>>(x, n, P, first, last, max_clusters, centroids, max_centroids, result);
   if (sorted_out && !apart) {
     e = cudaMemcpyAsync(sorted_out, x, (size_t)n * sizeof(float), cudaMemcpyDeviceToDevice, s);

@@ -880,3 +880,39 @@ def test_dbci_clusters_across_tile_edges(n, outliers):
     assert np.array_equal(r["labels"].cpu().numpy().astype(np.int64), ref["labels"])
     assert r["n_noise"] == int((ref["labels"] < 0).sum())
     assert np.array_equal(r["centroids"].cpu().numpy().astype(np.float64), ref["centroids"])
+
+
+def _milliseconds(call, passes=3):
+    best = float("inf")
+    for _ in range(passes):
+        start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        start.record()
+        call()
+        end.record()
+        end.synchronize()
+        best = min(best, start.elapsed_time(end))
+    return best
+
+
+@pytest.mark.parametrize("kind", ["levels", "clipped", "uniform"])
+def test_dbci_repeated_values(kind):
+    # many copies of few values and seed clusters that are a large part of n: most points are no core points and MinPts is in
+    # the tens of thousands; the work per point must not grow with it (the Gaussian array of the same size, all core points,
+    # is the measure; a walk over the copies is 7 to 500 times as long at this size)
+    n = 400_000
+    rng = np.random.default_rng(5)
+    if kind == "levels":
+        w = np.repeat(np.linspace(-0.07, 0.07, 8), n // 8)
+    elif kind == "clipped":
+        w = np.clip(rng.normal(0, 0.02, n), -0.05, 0.05)
+    else:
+        w = rng.uniform(-0.05, 0.05, n)
+    w = torch.from_numpy(w.astype(np.float32)).bfloat16().float()
+    r = lcd.dbci(w.cuda(), max_centroids=4096)
+    ref = O.dbci_scan(w.numpy())
+    assert (r["sigma"], r["eps"], r["min_pts"]) == (ref["sigma"], ref["eps"], ref["min_pts"]) and ref["min_pts"] > 20000
+    assert np.array_equal(r["labels"].cpu().numpy().astype(np.int64), ref["labels"])
+    assert r["n_noise"] == int((ref["labels"] < 0).sum())
+    assert np.array_equal(r["centroids"].cpu().numpy().astype(np.float64), ref["centroids"])
+    repeated, plain = w.cuda(), torch.from_numpy(rng.normal(0, 0.02, n).astype(np.float32)).cuda()
+    assert _milliseconds(lambda: lcd.dbci(repeated)) < 3 * _milliseconds(lambda: lcd.dbci(plain))
