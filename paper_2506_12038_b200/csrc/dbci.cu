@@ -38,7 +38,8 @@ __device__ long long warp_bound(const float* x, long long lo, long long hi, doub
     const long long step = (hi - lo + 31) / 32, at = lo + lane * step;
     bool before = false;
     if (at < hi) before = STRICT ? (double)x[at] <= v : (double)x[at] < v;
-    const int n = __popc(__ballot_sync(0xffffffffu, before));      // probes 0 .. n - 1 lie before the bound
+    // probes 0 .. n - 1 lie before the bound (the last that says so counts: NaNs sorted to the front compare false)
+    const int n = 32 - __clz(__ballot_sync(0xffffffffu, before));
     if (n == 0) return lo;
     lo += (n - 1) * step + 1;
     const long long end = lo + step - 1;
@@ -125,6 +126,7 @@ __device__ __forceinline__ Chain join(const Chain& a, const Chain& b, double eps
 // Whether the middle point at g is a core point: at least k points y of the middle with v - eps <= y <= v + eps (binary64).
 // A binary32 y is >= a binary64 bound exactly if it is >= the bound rounded up to binary32, and likewise on the other side.
 __device__ __forceinline__ bool is_core(const float* __restrict__ x, long long L, long long R, long long g, float v, double eps, long long k) {
+  if (k <= 1) return true;                                   // itself (and k = 0: an empty seed cluster, left by a NaN weight)
   const float a = __double2float_ru((double)v - eps), b = __double2float_rd((double)v + eps);
   const long long left = g - (k - 1), right = g + (k - 1);
   if (left >= L && x[left] >= a) return true;                // k - 1 neighbours on one side, the usual case

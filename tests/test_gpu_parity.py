@@ -916,3 +916,21 @@ def test_dbci_repeated_values(kind):
     assert np.array_equal(r["centroids"].cpu().numpy().astype(np.float64), ref["centroids"])
     repeated, plain = w.cuda(), torch.from_numpy(rng.normal(0, 0.02, n).astype(np.float32)).cuda()
     assert _milliseconds(lambda: lcd.dbci(repeated)) < 3 * _milliseconds(lambda: lcd.dbci(plain))
+
+
+@pytest.mark.parametrize("n", [1000, 5000])
+def test_dbci_with_a_negative_nan(n):
+    # sorted to the front; nothing lies within sigma of it, so the left seed cluster and MinPts are empty, every middle weight
+    # is a core point and eps is infinite: one middle cluster.  sigma and the right seed cluster are the others' own
+    w = np.random.default_rng(n).normal(0, 0.02, n).astype(np.float32)
+    w[n // 3] = np.array([0xffc00000], dtype=np.uint32).view(np.float32)[0]
+    r = lcd.dbci(torch.from_numpy(w).cuda())
+    x = np.concatenate([[w[n // 3]], np.sort(np.delete(w, n // 3))])
+    xd = x.astype(np.float64)
+    pos, neg = xd[1:][xd[1:] > 0], np.append(-xd[1:][xd[1:] < 0][::-1], np.nan)
+    sigma = sum(v[int(np.ceil(p * v.size)) - 1] for p in (0.6827, 0.9544, 0.9974) for v in (pos, neg)) / 12
+    R = 1 + int((xd[1:] < xd[-1] - sigma).sum())
+    assert r["sigma"] == pytest.approx(sigma, rel=1e-15)
+    assert (r["eps"], r["min_pts"], r["left"], r["right"], r["n_noise"]) == (np.inf, 0, 0, n - R, 0)
+    assert np.array_equal(r["sorted"].cpu().numpy(), x, equal_nan=True)
+    assert np.array_equal(r["labels"].cpu().numpy(), np.where(np.arange(n) < R, 1, 2))
