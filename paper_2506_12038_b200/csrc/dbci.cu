@@ -48,14 +48,14 @@ __device__ long long warp_bound(const float* x, long long lo, long long hi, doub
   return lo;
 }
 
-// Two warps; the other threads clear the clusters' first and last members.
+// All CTAs clear the clusters' first and last members (a list as long as the caller wants), two warps of CTA 0 do the rest.
 __global__ void __launch_bounds__(256) dbci_params_kernel(const float* __restrict__ x, long long n, DbciParams* __restrict__ P,
                                                           int* __restrict__ first, int* __restrict__ last, int max_clusters) {
   __shared__ long long found[2];
   __shared__ double sigma_s;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int i = threadIdx.x - 64; i < max_clusters; i += 192)
-    if (i >= 0) { first[i] = 0x7fffffff; last[i] = -1; }
+  for (int i = blockIdx.x * 256 + threadIdx.x; i < max_clusters; i += gridDim.x * 256) { first[i] = 0x7fffffff; last[i] = -1; }
+  if (blockIdx.x != 0) return;
   if (warp < 2) {
     const long long at = warp == 0 ? warp_bound<true>(x, 0, n, 0.0) : warp_bound<false>(x, 0, n, 0.0);
     if (lane == 0) found[warp] = at;
@@ -441,7 +441,8 @@ lcd_status launch_dbci(const float* weights, int64_t n, void* workspace, float* 
   size_t tmp_bytes = l.cub_bytes;
   cudaError_t e = cub::DeviceRadixSort::SortKeys(base + l.cub, tmp_bytes, weights, x, (int)n, 0, 32, s);
   if (e != cudaSuccess) { set_cuda_error((int)e); return LCD_ERR_CUDA; }
-  dbci_params_kernel<<<1, 256, 0, s>>>(x, n, P, first, last, max_clusters);
+  const unsigned fill = (unsigned)((max_clusters + 255) / 256);
+  dbci_params_kernel<<<fill < 1024 ? fill : 1024, 256, 0, s>>>(x, n, P, first, last, max_clusters);
   dbci_mark_kernel<<<tiles, 32 * kTileWarps, 0, s>>>(x, n, P, core, chains, plain);
   dbci_scan_kernel<<<1, 1024, 0, s>>>(P, chains, next, (int)tiles);
   dbci_label_kernel<<<tiles, 32 * kTileWarps, 0, s>>>(x, n, P, core, chains, next, plain, labels, first, last, max_clusters);

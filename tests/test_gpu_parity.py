@@ -934,3 +934,11 @@ def test_dbci_with_a_negative_nan(n):
     assert (r["eps"], r["min_pts"], r["left"], r["right"], r["n_noise"]) == (np.inf, 0, 0, n - R, 0)
     assert np.array_equal(r["sorted"].cpu().numpy(), x, equal_nan=True)
     assert np.array_equal(r["labels"].cpu().numpy(), np.where(np.arange(n) < R, 1, 2))
+
+
+def test_dbci_long_centroid_list():
+    # clearing the list's bookkeeping takes the GPU's bandwidth, not one SM's (128 MB: 2.6 ms by one CTA)
+    w = torch.from_numpy(np.random.default_rng(2).normal(0, 0.02, 4096).astype(np.float32)).cuda()
+    short, long = lcd.dbci(w, max_centroids=4096), lcd.dbci(w, max_centroids=1 << 24)
+    assert short["n_noise"] == long["n_noise"] and torch.equal(short["labels"], long["labels"]) and torch.equal(short["centroids"], long["centroids"])
+    assert _milliseconds(lambda: lcd.dbci(w, max_centroids=1 << 24)) < _milliseconds(lambda: lcd.dbci(w, max_centroids=4096)) + 1.0
