@@ -21,6 +21,14 @@ static lcd_algo resolve_algo(const Problem& p, lcd_algo algo) {
   return kHaveDenseTc ? LCD_ALGO_DENSE_TC : LCD_ALGO_REFERENCE;
 }
 
+// LCD_ALGO_AUTO between 17 and 32 tokens of 4-bit levels on rows that the tensor-memory kernel does not take (more than 65536
+// columns): two launches of the register tables (16 tokens, then the rest).  The tensor-core kernel's 128-token tile is mostly
+// empty there, its time grows with the row length, and the workspace is left zero-filled, as up to 16 tokens
+// (4096 x 73728, 3 bit, 17 / 32 tokens: 77 / 86 us, the tensor-core kernel 312 / 313).
+static bool two_chunks(const Problem& p, lcd_algo algo) {
+  return algo == LCD_ALGO_AUTO && p.act_bits == 4 && p.M > 16 && p.M <= 32 && !lut_gemv_tc_supported(&p, 1);
+}
+
 static bool small_m_family(lcd_algo a) {
   return a == LCD_ALGO_REGISTER_LUT || a == LCD_ALGO_BUCKET_LUT || a == LCD_ALGO_TC_LUT || a == LCD_ALGO_SHARED_BUCKET;
 }
@@ -70,6 +78,14 @@ static bool shape_problem(const void* header_host, int64_t M, Problem* p) {
 }
 
 static lcd_status workspace_for(const Problem& p, lcd_algo algo, size_t* bytes) {
+  if (two_chunks(p, algo)) {
+    // enough for 8-bit levels too, which take the tensor-core kernel: who asks does not say which levels there will be
+    Problem first = p;
+    first.M = 16;
+    const size_t tables = lut_gemv_workspace_bytes(&first, 1, LCD_ALGO_REGISTER_LUT), dense = dense_tc_workspace_bytes(p);
+    *bytes = tables > dense ? tables : dense;
+    return LCD_OK;
+  }
   const lcd_algo resolved = resolve_algo(p, algo);
   switch (resolved) {
     case LCD_ALGO_REFERENCE:
@@ -161,6 +177,18 @@ extern "C" lcd_status lcd_lut_linear(const void* packed_weights_dev, const void*
   if (st != LCD_OK) return st;
   if (need > 0 && (!workspace || workspace_bytes < need)) return LCD_ERR_BUFFER_TOO_SMALL;
   if (need > 0 && !aligned(workspace, 256)) return LCD_ERR_INVALID_ARG;
+  if (two_chunks(p, algo)) {
+    // the second launch touches the scratch only after the first one has finished (stream order, dependency wait)
+    Problem part = p;
+    part.M = 16;
+    st = launch_lut_gemv(&part, 1, LCD_ALGO_REGISTER_LUT, workspace, workspace_bytes, status_word_dev, cuda_stream);
+    if (st != LCD_OK) return st;
+    part.M = p.M - 16;
+    part.act_idx = p.act_idx + 16 * (p.K_pad / 2);
+    part.act_scale = p.act_scale + 16;
+    part.y = p.y + 16 * p.ldy;
+    return launch_lut_gemv(&part, 1, LCD_ALGO_REGISTER_LUT, workspace, workspace_bytes, status_word_dev, cuda_stream);
+  }
   const lcd_algo resolved = resolve_algo(p, algo);
   switch (resolved) {
     case LCD_ALGO_REFERENCE:

@@ -942,3 +942,18 @@ def test_dbci_long_centroid_list():
     short, long = lcd.dbci(w, max_centroids=4096), lcd.dbci(w, max_centroids=1 << 24)
     assert short["n_noise"] == long["n_noise"] and torch.equal(short["labels"], long["labels"]) and torch.equal(short["centroids"], long["centroids"])
     assert _milliseconds(lambda: lcd.dbci(w, max_centroids=1 << 24)) < _milliseconds(lambda: lcd.dbci(w, max_centroids=4096)) + 1.0
+
+
+@pytest.mark.parametrize("act_bits", [4, 8])
+@pytest.mark.parametrize("M", [17, 32])
+def test_up_to_32_tokens_on_rows_beyond_the_tensor_memory_kernel(M, act_bits):
+    # more than 65536 columns; with 4-bit levels the workspace keeps to the zero-fill rule, as everywhere up to 32 tokens
+    L = gen.random_case(seed=M, N=40, K=70000, bits=3, M=M)
+    w = lcd.PackedWeights(lcd.pack_weights(L.idx, L.codebook, 3))
+    a, s = lcd.smooth_quantize_act(torch.from_numpy(L.x).cuda(), torch.from_numpy(L.inv_s).cuda(), act_bits=act_bits)
+    ws = torch.zeros(lcd.lut_linear_workspace_bytes(w, M), dtype=torch.uint8, device="cuda")
+    q_ref, s_ref = O.smooth_quantize(L.x, L.inv_s, act_bits=act_bits)
+    for _ in range(2):
+        y = lcd.lut_linear(w, a, s, workspace=ws)
+        check_y(y, O.lut_linear_dequant(L.idx, L.codebook, q_ref, s_ref))
+        assert act_bits == 8 or not ws.any()
