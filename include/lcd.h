@@ -164,11 +164,14 @@ lcd_status lcd_smooth_quantize_act_batch(const lcd_act_problem* problems /* host
  *   algo:               LCD_ALGO_AUTO: see lcd_algo; a family asked for
  *                       outside its range => LCD_ERR_UNSUPPORTED;
  *   workspace:          device scratch of at least lcd_lut_linear_workspace_bytes(...) bytes, 256-byte
- *                       aligned (may be NULL when that size is 0).  REGISTER_LUT and BUCKET_LUT keep integer
- *                       partial sums and arrival counters there: the caller zero-fills it once before its
- *                       first use, every call that completes leaves it zero-filled again, and two calls that
- *                       may overlap on the device need separate workspaces.  SHARED_BUCKET and TC_LUT, and any
- *                       call with at most 32 tokens, keep to the same rule.  Above, its contents do not matter;
+ *                       aligned (may be NULL when that size is 0).  Two calls that may overlap on the device need
+ *                       separate workspaces.  REGISTER_LUT, BUCKET_LUT and SHARED_BUCKET keep partial sums and
+ *                       arrival counters there: the caller zero-fills it once before its first use, and every call
+ *                       that completes leaves it zero-filled again.  So does any call of at most 32 tokens that finds
+ *                       it zero-filled, except DENSE_F16, and beyond 65536 columns DENSE_TC and 8-bit levels of 17 to
+ *                       32 tokens.  Those and all calls of more than 32 tokens do not care about its contents and
+ *                       leave their own: zero-fill it before it is handed to a call of the first kind.  (AUTO up to
+ *                       32 tokens may be one; TC_LUT and DENSE_TC up to 65536 columns do not care at any number);
  *   status_word_dev:    device int32 or NULL; receives LCD_ERR_TIMEOUT if a bounded device-side wait
  *                       expired (the output is then invalid and the workspace must be zero-filled again);
  *                       never written otherwise.

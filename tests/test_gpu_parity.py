@@ -257,7 +257,7 @@ def test_tensor_core_lut_token_widths(bits, act_bits, N, K, M):
             lcd.lut_linear(w, a, s, y=y, algo=algo, workspace=ws, status_word=word)
         torch.cuda.synchronize()
         assert int(word.item()) == 0
-        assert m > 16 or not ws.any()
+        assert m > 32 or not ws.any()
         q_ref, s_ref = O.smooth_quantize(L.x, L.inv_s, act_bits=act_bits)
         check_y(y, O.lut_linear_dequant(L.idx, L.codebook, q_ref, s_ref))
 
@@ -957,3 +957,30 @@ def test_up_to_32_tokens_on_rows_beyond_the_tensor_memory_kernel(M, act_bits):
         y = lcd.lut_linear(w, a, s, workspace=ws)
         check_y(y, O.lut_linear_dequant(L.idx, L.codebook, q_ref, s_ref))
         assert act_bits == 8 or not ws.any()
+
+
+def test_workspace_rules():
+    # include/lcd.h: who wants the workspace zero-filled, who leaves it so, and who does not care
+    L = gen.random_case(seed=4, N=300, K=4096, bits=2, M=24)
+    w = lcd.PackedWeights(lcd.pack_weights(L.idx, L.codebook, 2))
+    a, s = lcd.smooth_quantize_act(torch.from_numpy(L.x).cuda(), torch.from_numpy(L.inv_s).cuda())
+    q_ref, s_ref = O.smooth_quantize(L.x, L.inv_s)
+    y_ref = O.lut_linear_dequant(L.idx, L.codebook, q_ref, s_ref)
+    calls = [(1, lcd.ALGO_SHARED_BUCKET), (8, lcd.ALGO_REGISTER_LUT), (8, lcd.ALGO_BUCKET_LUT), (12, lcd.ALGO_TC_LUT), (1, lcd.ALGO_AUTO),
+             (16, lcd.ALGO_AUTO), (24, lcd.ALGO_AUTO), (5, lcd.ALGO_DENSE_TC), (24, lcd.ALGO_DENSE_TC), (24, lcd.ALGO_DENSE_F16)]
+    ws = torch.zeros(max(lcd.lut_linear_workspace_bytes(w, m, algo) for m, algo in calls), dtype=torch.uint8, device="cuda")
+
+    def run(m, algo):
+        y = lcd.lut_linear(w, a[:m], s[:m], algo=algo, workspace=ws)
+        check_y(y, y_ref[:m], tight=algo != lcd.ALGO_DENSE_F16)
+
+    for m, algo in calls[:-1]:
+        run(m, algo)
+        assert not ws.any()
+    run(*calls[-1])                                     # leaves its levels, which the next ones do not mind
+    assert ws.any()
+    for m, algo in ((12, lcd.ALGO_TC_LUT), (24, lcd.ALGO_AUTO), (24, lcd.ALGO_DENSE_TC), (5, lcd.ALGO_DENSE_TC)):
+        ws.fill_(255)
+        run(m, algo)
+    ws.zero_()
+    run(8, lcd.ALGO_REGISTER_LUT)
