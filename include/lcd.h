@@ -60,7 +60,8 @@ typedef enum {
   LCD_ALGO_DENSE_F16 = 5,   /* the same with fp16 operands: indices decoded through the codebook into fp16     */
                             /* shared-memory tiles, fp32 accumulators (no fixed-point step; slower).            */
   LCD_ALGO_TC_LUT = 6,      /* REGISTER_LUT's tables and sums, the looked-up bytes written to tensor memory as  */
-                            /* the A operand of tcgen05 kind::i8 MMAs.  M <= 16.                                 */
+                            /* the A operand of tcgen05 kind::i8 MMAs.  M <= 16.  Rows of more than 65536        */
+                            /* columns run REGISTER_LUT, workspace rule included (the same y).                   */
   LCD_ALGO_SHARED_BUCKET = 7/* Section 4.2 centroid-stationary buckets with the tables in shared memory: for    */
                             /* every four columns a table indexed by the byte of their four weight indices      */
                             /* holds the four partial bucket sums of the token's levels, so one load looks four */
@@ -162,7 +163,7 @@ lcd_status lcd_smooth_quantize_act_batch(const lcd_act_problem* problems /* host
  *   act_idx, act_scale: device, as written by lcd_smooth_quantize_act for the same K;
  *   y:                  device out, fp32 [M][ldy], ldy >= N;
  *   algo:               LCD_ALGO_AUTO: see lcd_algo; a family asked for
- *                       outside its range => LCD_ERR_UNSUPPORTED;
+ *                       outside its range => LCD_ERR_UNSUPPORTED (but see TC_LUT);
  *   workspace:          device scratch of at least lcd_lut_linear_workspace_bytes(...) bytes, 256-byte
  *                       aligned (may be NULL when that size is 0).  Two calls that may overlap on the device need
  *                       separate workspaces.  REGISTER_LUT, BUCKET_LUT and SHARED_BUCKET keep partial sums and
@@ -220,8 +221,9 @@ lcd_status lcd_lut_linear_batch(const lcd_linear_problem* problems /* host */, i
                                 void* workspace, size_t workspace_bytes, int32_t* status_word_dev,
                                 void* cuda_stream);
 
-/* Which family a grouped call with these shapes and this `algo` runs (what LCD_ALGO_AUTO stands for): only the
- * header_host and M fields of the problems are read.  The fused call (lcd_linear_fused_batch) chooses the same way. */
+/* Which family a grouped call with these shapes and this `algo` runs (what LCD_ALGO_AUTO stands for, REGISTER_LUT for a
+ * TC_LUT whose rows it does not take): only the header_host and M fields of the problems are read.  The fused call
+ * (lcd_linear_fused_batch) chooses the same way, with REGISTER_LUT in place of TC_LUT. */
 lcd_status lcd_lut_linear_batch_resolve(const lcd_linear_problem* problems /* host */, int count, lcd_algo algo,
                                         lcd_algo* resolved);
 

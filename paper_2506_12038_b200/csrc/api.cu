@@ -213,9 +213,11 @@ static lcd_status batch_algo(const lcd_linear_problem* problems, int count, lcd_
     if (problems[i].M < 1 || problems[i].M > 16) return problems[i].M < 1 ? LCD_ERR_INVALID_ARG : LCD_ERR_UNSUPPORTED;
   return LCD_OK;
 }
-// The family a grouped call runs: the caller's, or the library's choice for these shapes.
+// The family a grouped call runs: the caller's, or the library's choice for these shapes (the register tables, of the same
+// arithmetic, in place of a tensor-memory kernel that does not take the rows).
 static lcd_status batch_family(const Problem* p, int count, lcd_algo algo, lcd_algo* resolved) {
   *resolved = resolve_small_m(p, count, algo);
+  if (*resolved == LCD_ALGO_TC_LUT && !lut_gemv_tc_supported(p, count)) *resolved = LCD_ALGO_REGISTER_LUT;
   if (*resolved == LCD_ALGO_SHARED_BUCKET && !lut_smem_supported(p, count)) return LCD_ERR_UNSUPPORTED;
   return LCD_OK;
 }

@@ -110,3 +110,17 @@ def test_every_export_declares_its_argument_types():
     for name in binding.EXPORTS:
         if name != "lcd_last_cuda_error":
             assert getattr(binding.lib, name).argtypes, name
+
+
+@pytest.mark.parametrize("K,family", [(65536, lcd.ALGO_TC_LUT), (65537, lcd.ALGO_REGISTER_LUT)])
+def test_resolve_names_the_family_that_runs(K, family):
+    # rows that the tensor-memory kernel does not take run the register tables, also in a group with shorter ones
+    class Weights:
+        def __init__(self, K):
+            blob = lcd.pack_weights(np.zeros((1, K), dtype=np.uint8), np.ones((1, 4), dtype=np.float16), 2)
+            self.buf = ctypes.create_string_buffer(bytes(blob[:64]), 64)
+            self.header_ptr = ctypes.cast(self.buf, ctypes.c_void_p)
+    short, row = Weights(300), Weights(K)
+    assert lcd.resolve_batch_algo([(row, 12)], lcd.ALGO_TC_LUT) == family
+    assert lcd.resolve_batch_algo([(short, 12), (row, 3)], lcd.ALGO_TC_LUT) == family
+    assert lcd.resolve_batch_algo([(short, 12)], lcd.ALGO_TC_LUT) == lcd.ALGO_TC_LUT
