@@ -111,7 +111,7 @@ struct Chain {
   float first, last;
   int any, gaps;
 };
-// The first core point after a tile, if there is one.
+// The first core point of a tile, later the first one after it; whether there is one.
 struct Next {
   float v;
   int any;
@@ -160,7 +160,7 @@ __device__ __forceinline__ Chain word_chain(unsigned word, float v, double eps) 
 
 __global__ void __launch_bounds__(32 * kTileWarps) dbci_mark_kernel(const float* __restrict__ x, long long n, const DbciParams* __restrict__ P,
                                                                     unsigned* __restrict__ core, Chain* __restrict__ chains,
-                                                                    unsigned char* __restrict__ plain) {
+                                                                    Next* __restrict__ next, unsigned char* __restrict__ plain) {
   __shared__ Chain part[kTileWarps];
   __shared__ int all[kTileWarps];
   const long long L = P->L, R = P->R, k = P->min_pts, tile0 = (long long)blockIdx.x * kTile;
@@ -174,6 +174,7 @@ __global__ void __launch_bounds__(32 * kTileWarps) dbci_mark_kernel(const float*
       if (threadIdx.x < kTile / 32) core[(tile0 >> 5) + threadIdx.x] = 0xffffffffu;
       if (threadIdx.x == 0) {
         chains[blockIdx.x] = {x[tile0], high, 1, 0};
+        next[blockIdx.x] = {x[tile0], 1};
         plain[blockIdx.x] = 1;
       }
       return;
@@ -210,38 +211,44 @@ __global__ void __launch_bounds__(32 * kTileWarps) dbci_mark_kernel(const float*
       e = e && all[w];
     }
     chains[blockIdx.x] = t;
+    next[blockIdx.x] = {t.first, t.any};
     plain[blockIdx.x] = (unsigned char)(e && t.gaps == 0);
   }
 }
 
-// Exclusive scan of the tiles' chains in place: chains[t] becomes the chain of all tiles before t; next[t] the first core
-// point of all tiles after t.  One CTA; a thread joins its run of tiles, the threads' runs are scanned, then it walks its run
-// again, backwards and forwards.
+// Exclusive scans over the tiles in place, by one CTA each.  CTA 0: chains[t] becomes the chain of all tiles before t; a thread
+// joins its run of tiles, the threads' runs are scanned, then it walks its run again.  CTA 1: next[t] becomes the first core
+// point of all tiles after t.
 __global__ void __launch_bounds__(1024) dbci_scan_kernel(DbciParams* __restrict__ P, Chain* __restrict__ chains, Next* __restrict__ next, int n_tiles) {
   __shared__ Chain part[1024];
-  __shared__ float first_of[1024];
-  __shared__ unsigned any_of[32];          // threads whose runs have core points, a word per warp
+  __shared__ unsigned any_of[32];          // CTA 1: threads whose runs have core points, a word per warp
   const double eps = P->eps;
-  const int per = (n_tiles + 1023) / 1024, t0 = threadIdx.x * per, t1 = min(t0 + per, n_tiles);
-  Chain mine = {0.0f, 0.0f, 0, 0};
-  for (int t = t0; t < t1; ++t) mine = join(mine, chains[t], eps);
-  part[threadIdx.x] = mine;
-  first_of[threadIdx.x] = mine.first;
-  const unsigned any_word = __ballot_sync(0xffffffffu, mine.any != 0);
-  if ((threadIdx.x & 31) == 0) any_of[threadIdx.x >> 5] = any_word;
-  __syncthreads();
-  Next after = {0.0f, 0};
-  {
+  const int per = (n_tiles + 1023) / 1024, t0 = min((int)threadIdx.x * per, n_tiles), t1 = min(t0 + per, n_tiles);
+  if (blockIdx.x == 1) {
+    Next after = {0.0f, 0};
+    for (int t = t1 - 1; t >= t0; --t) {
+      const Next c = next[t];
+      if (c.any) after = c;
+    }
+    part[threadIdx.x].first = after.v;
+    const unsigned any_word = __ballot_sync(0xffffffffu, after.any != 0);
+    if ((threadIdx.x & 31) == 0) any_of[threadIdx.x >> 5] = any_word;
+    __syncthreads();
     int w = threadIdx.x >> 5;
     unsigned word = any_of[w] & ~(0xffffffffu >> (31 - (threadIdx.x & 31)));        // the threads after this one
     while (word == 0 && ++w < 32) word = any_of[w];
-    if (word) after = {first_of[32 * w + __ffs(word) - 1], 1};
+    after = {word ? part[32 * w + __ffs(word) - 1].first : 0.0f, word != 0};
+    for (int t = t1 - 1; t >= t0; --t) {
+      const Next c = next[t];
+      next[t] = after;
+      if (c.any) after = c;
+    }
+    return;
   }
-  for (int t = t1 - 1; t >= t0; --t) {
-    next[t] = after;
-    const Chain c = chains[t];
-    if (c.any) after = {c.first, 1};
-  }
+  Chain mine = {0.0f, 0.0f, 0, 0};
+  for (int t = t0; t < t1; ++t) mine = join(mine, chains[t], eps);
+  part[threadIdx.x] = mine;
+  __syncthreads();
   for (int o = 1; o < 1024; o <<= 1) {
     Chain v = part[threadIdx.x];
     if ((int)threadIdx.x >= o) v = join(part[threadIdx.x - o], v, eps);
@@ -261,11 +268,12 @@ __global__ void __launch_bounds__(1024) dbci_scan_kernel(DbciParams* __restrict_
 
 // labels of all sorted points (0 left cluster, 1.. middle clusters in order, last = right cluster, -1 noise) and the
 // first / last member of every cluster
-__global__ void __launch_bounds__(32 * kTileWarps) dbci_label_kernel(const float* __restrict__ x, long long n, DbciParams* __restrict__ P,
+__global__ void __launch_bounds__(32 * kTileWarps, 4) dbci_label_kernel(const float* __restrict__ x, long long n, DbciParams* __restrict__ P,
                                                                      const unsigned* __restrict__ core, const Chain* __restrict__ chains,
                                                                      const Next* __restrict__ next, const unsigned char* __restrict__ plain, int* __restrict__ labels,
                                                                      int* __restrict__ first, int* __restrict__ last, int max_clusters) {
   __shared__ Chain part[kTileWarps];
+  __shared__ Next next_of[kTileWarps][kWarpSteps];          // the first core point after every word
   const long long L = P->L, R = P->R, tile0 = (long long)blockIdx.x * kTile;
   const double eps = P->eps;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_mid = P->n_mid;
@@ -304,19 +312,17 @@ __global__ void __launch_bounds__(32 * kTileWarps) dbci_label_kernel(const float
   __syncthreads();
   Chain run = before;
   for (int w = 0; w < warp; ++w) run = join(run, part[w], eps);
-  // the first core point after every word: of the warp's later words, of the later warps, of the later tiles
+  // of the warp's later words, of the later warps, of the later tiles
   Next after = next[blockIdx.x];
   for (int w = kTileWarps - 1; w > warp; --w)
     if (part[w].any) after = {part[w].first, 1};
-  float next_v[kWarpSteps];
-  unsigned has_next = 0;
   int noise = 0;
 #pragma unroll
   for (int i = kWarpSteps - 1; i >= 0; --i) {
-    next_v[i] = after.v;
-    has_next |= after.any ? 1u << i : 0u;
+    if (lane == 0) next_of[warp][i] = after;
     if (words[i]) after = {__shfl_sync(0xffffffffu, vs[i], __ffs(words[i]) - 1), 1};
   }
+  __syncwarp();
 #pragma unroll
   for (int i = 0; i < kWarpSteps; ++i) {
     const long long g0 = w0 + 32 * i, g = g0 + lane;
@@ -335,8 +341,9 @@ __global__ void __launch_bounds__(32 * kTileWarps) dbci_label_kernel(const float
       else if (g >= R) lab = n_mid + 1;
       else if (is) lab = upto;
       else {
-        const bool has_left = below || run.any, has_right = above || ((has_next >> i) & 1u);
-        const float left = below ? vb : run.last, right = above ? va : next_v[i];
+        const Next after_word = next_of[warp][i];
+        const bool has_left = below || run.any, has_right = above || after_word.any;
+        const float left = below ? vb : run.last, right = above ? va : after_word.v;
         const double dl = has_left ? (double)v - (double)left : 1e300, dr = has_right ? (double)right - (double)v : 1e300;
         if (dl <= eps && dl <= dr) lab = upto;
         else if (dr <= eps) lab = upto + (!has_left || gap_after(left, right, eps) ? 1 : 0);
@@ -443,8 +450,8 @@ lcd_status launch_dbci(const float* weights, int64_t n, void* workspace, float* 
   if (e != cudaSuccess) { set_cuda_error((int)e); return LCD_ERR_CUDA; }
   const unsigned fill = (unsigned)((max_clusters + 255) / 256);
   dbci_params_kernel<<<fill < 1024 ? fill : 1024, 256, 0, s>>>(x, n, P, first, last, max_clusters);
-  dbci_mark_kernel<<<tiles, 32 * kTileWarps, 0, s>>>(x, n, P, core, chains, plain);
-  dbci_scan_kernel<<<1, 1024, 0, s>>>(P, chains, next, (int)tiles);
+  dbci_mark_kernel<<<tiles, 32 * kTileWarps, 0, s>>>(x, n, P, core, chains, next, plain);
+  dbci_scan_kernel<<<2, 1024, 0, s>>>(P, chains, next, (int)tiles);
   dbci_label_kernel<<<tiles, 32 * kTileWarps, 0, s>>>(x, n, P, core, chains, next, plain, labels, first, last, max_clusters);
   dbci_centroid_kernel<<<1, 256, 0, s>>>(x, n, P, first, last, max_clusters, centroids, max_centroids, result);
   if (sorted_out && !apart) {
