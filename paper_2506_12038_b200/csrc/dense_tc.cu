@@ -284,7 +284,7 @@ dense_tc_kernel(const __grid_constant__ CUtensorMap tmap_act, const DenseParams 
         tmem_ld32(tmem_base + ((uint32_t)(32 * quad) << 16) + buf * BN + 32 * c, v);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
         const int mc = m0 + 32 * c;
-        const float my_scale = mc + lane < P.M ? __ldg(P.act_scale + mc + lane) : 0.0f;
+        const float my_scale = mc + lane < P.M ? ld_global(P.act_scale + mc + lane) : 0.0f;
 #pragma unroll
         for (int j = 0; j < 32; ++j) {
           const float s = __shfl_sync(0xffffffffu, my_scale, j);
@@ -635,7 +635,7 @@ dense_i8_kernel(const __grid_constant__ CUtensorMap tmap_act, const DenseParams 
       static_assert(kMyChunks % 2 == 0, "an even number of 16-token chunks per epilogue warp");
       auto pair_scales = [&](int r) {
         const int m = m0 + 16 * (half + (kI8EpiWarps / 4) * (2 * r + (lane >> 4))) + (lane & 15);
-        return m < P.M ? __ldg(P.act_scale + m) : 0.0f;
+        return m < P.M ? ld_global(P.act_scale + m) : 0.0f;
       };
       float sc_cur = pair_scales(0), sc_next = 0.0f;
       ok = __all_sync(0xffffffffu, bar_wait(tmem_full(buf), (tl / NBUF) & 1u, abort_flag));

@@ -37,6 +37,27 @@ inline int current_sm_count() {
   return n;
 }
 
+#ifdef __CUDACC__
+// Loads of what an earlier kernel of the stream writes, behind griddepcontrol.wait.  A kernel launched with programmatic
+// stream serialization may be running while that one still writes, and __ldg (ld.global.nc, what loads through const
+// __restrict__ pointers become too) is only for data that nobody writes while the reading kernel runs.
+__device__ __forceinline__ float ld_global(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ unsigned short ld_global(const unsigned short* p) {
+  unsigned short v;
+  asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint4 ld_global(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+#endif
+
 // cuTensorMapEncodeTiled, asked of the driver (the library does not link against it); null if there is none.
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,

@@ -737,7 +737,7 @@ lut_gemv_kernel(const __grid_constant__ GemvBatch batch, int32_t* __restrict__ s
           const float A = s_amax[m];
           sq_tok[G][e] = A > 0.0f ? __fdiv_rn(A, 7.0f) : 1.0f;
         } else {
-          sq_tok[G][e] = __ldg(P.act_scale + m);
+          sq_tok[G][e] = ld_global(P.act_scale + m);
         }
       }
     }

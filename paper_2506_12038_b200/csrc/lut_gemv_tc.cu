@@ -447,7 +447,7 @@ lut_gemv_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ 
           tc_ld4(t_hi + c0 + c, hi);
           tc_ld4(t_hi + NT + c0 + c, lo);
           const int m = m0 + c0 + c;
-          const float sc = m + (lane & 3) < P.M ? __ldg(P.act_scale + m + (lane & 3)) : 0.0f;
+          const float sc = m + (lane & 3) < P.M ? ld_global(P.act_scale + m + (lane & 3)) : 0.0f;
           if (!landed) tc_wait(part_bar, round & 1u, abort_flag);
           landed = true;
           __syncwarp();
@@ -709,7 +709,7 @@ lut_gemv_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ 
       int* part = B.parts + (size_t)blockIdx.x * words * NT * kTcRows + row;
       auto scales = [&](int c) {
         const int m = m0 + 8 * c + (lane & 7);
-        return whole_tile && m < P.M ? __ldg(P.act_scale + m) : 0.0f;
+        return whole_tile && m < P.M ? ld_global(P.act_scale + m) : 0.0f;
       };
       float sc = scales(half);
       tc_wait(acc_full(buf), (n_seg / NBUF) & 1u, abort_flag);
@@ -813,7 +813,7 @@ lut_gemv_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ 
           const uint4* src = reinterpret_cast<const uint4*>(P.act + (size_t)tok * row + (size_t)kt * (ACT == kActBytes ? 256 : 128)) +
                              (lane & 7) * kVec;
 #pragma unroll
-          for (int v = 0; v < kVec; ++v) cur[it][v] = __ldg(src + v);
+          for (int v = 0; v < kVec; ++v) cur[it][v] = ld_global(src + v);
         }
       }
     };

@@ -333,7 +333,7 @@ lut_smem_kernel(const __grid_constant__ SbBatch batch, int32_t* __restrict__ sta
           }
         }
       } else {
-        lv = __ldg(reinterpret_cast<const unsigned short*>(P.act_idx + (k >> 1)));
+        lv = ld_global(reinterpret_cast<const unsigned short*>(P.act_idx + (k >> 1)));
       }
     };
     if (warp < width * 8) load_columns(task_column(warp));
@@ -542,7 +542,7 @@ lut_smem_kernel(const __grid_constant__ SbBatch batch, int32_t* __restrict__ sta
       const SbProblem& P = batch.p[p_cur];
       float4* src = reinterpret_cast<float4*>(P.sums) + n_cur;
       const float4 Sw = __ldcg(src);
-      const float sq = P.act_bits == 16 ? __ldcg(batch.sq + p_cur) : __ldg(P.act_scale);
+      const float sq = P.act_bits == 16 ? __ldcg(batch.sq + p_cur) : ld_global(P.act_scale);
       __stcg(src, make_float4(0.0f, 0.0f, 0.0f, 0.0f));          // handed on zero-filled
       const float2 c01 = __half22float2(*reinterpret_cast<const __half2*>(&c_cur.x));
       const float2 c23 = __half22float2(*reinterpret_cast<const __half2*>(&c_cur.y));

@@ -21,13 +21,15 @@ struct AlphaList {
 
 // For 32 columns a CTA: xmax_k = max over the batch of |x[t][k]|, then for every candidate s[g][k] (binary64 powers, one
 // rounding to binary32; zero maxima leave the channel alone; clamp to [1e-5, 1e5]) and 1 / s[g][k], which the error kernel
-// would otherwise divide out once per token.  CTA 0 clears the error kernel's arrival counter.
-__global__ void __launch_bounds__(256) smoothing_factors_kernel(const __half* __restrict__ x, int64_t T, int64_t K, int64_t ldx,
-                                                                const float* __restrict__ wmax, const AlphaList alphas,
+// would otherwise divide out once per token.  CTA 0 clears the error kernel's arrival counter.  x and wmax are read with
+// ordinary loads (no __restrict__): this kernel may be running while an earlier one still writes them.  It does not let the next
+// one in early, which reads the factors with __ldg, for data that nobody writes while the reading kernel runs (an early
+// start gains nothing, 24.3 us either way; ordinary loads there take 26.2, __ldcg 28.0).
+__global__ void __launch_bounds__(256) smoothing_factors_kernel(const __half* x, int64_t T, int64_t K, int64_t ldx,
+                                                                const float* wmax, const AlphaList alphas,
                                                                 float* __restrict__ s, float* __restrict__ inv, unsigned* __restrict__ arrived) {
   __shared__ float part[8][32];
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
   const int64_t k = (int64_t)blockIdx.x * 32 + lane;
   if (blockIdx.x == 0 && threadIdx.x == 0) *arrived = 0u;

@@ -984,3 +984,19 @@ def test_workspace_rules():
         run(m, algo)
     ws.zero_()
     run(8, lcd.ALGO_REGISTER_LUT)
+
+
+@pytest.mark.parametrize("K", [4096, 1001])
+def test_smoothing_searches_one_after_another(K):
+    # two inputs in turn with nothing between the calls, whose kernels overlap and whose workspaces the allocator hands on:
+    # every search reads its own factors (the sums run in a fixed order: bit-identical to the undisturbed search)
+    xs = [torch.from_numpy(gen.activations(i, 64, K, gen.outlier_channels(i, K, 0.01), 50.0)).cuda() for i in (1, 2)]
+    wmax = [torch.from_numpy((np.abs(gen.normal(i, K)) + 0.1).astype(np.float32)).cuda() for i in (3, 4)]
+    alphas = [i / 20 for i in range(21)]
+    alone = []
+    for x, w in zip(xs, wmax):
+        alone.append(lcd.smoothing_search(x, w, alphas))
+        torch.cuda.synchronize()
+    results = [lcd.smoothing_search(xs[i % 2], wmax[i % 2], alphas) for i in range(40)]
+    for i, r in enumerate(results):
+        assert all(torch.equal(a, b) for a, b in zip(r, alone[i % 2]))
