@@ -297,6 +297,16 @@ def dbci(weights, max_centroids: int = 4096, want_labels: bool = True, stream=No
     """Section 3.1 on a flat CUDA fp32 tensor.  Returns a dict: sigma, eps, min_pts, left, right, n_noise,
     n_clusters_found, centroids (CUDA fp32, ascending), sorted (CUDA fp32) and labels (CUDA int32, in sorted order)."""
     import torch
+    if stream is not None and stream.cuda_stream != _stream_ptr():
+        # everything below allocates, clears and reads back on the current stream: make it the given one
+        caller = torch.cuda.current_stream()
+        given = stream if isinstance(stream, torch.cuda.Stream) or not stream.cuda_stream else torch.cuda.ExternalStream(stream.cuda_stream)
+        with torch.cuda.stream(given):
+            out = dbci(weights, max_centroids, want_labels)
+        for t in (out["centroids"], out["sorted"], out["labels"]):
+            if t is not None:
+                t.record_stream(caller)
+        return out
     w = weights.reshape(-1)
     assert w.is_cuda and w.dtype == torch.float32 and w.is_contiguous()
     n = w.numel()
@@ -308,7 +318,7 @@ def dbci(weights, max_centroids: int = 4096, want_labels: bool = True, stream=No
     res = torch.zeros((ctypes.sizeof(DbciResult),), dtype=torch.uint8, device=w.device)
     _check(lib.lcd_dbci(c_void_p(w.data_ptr()), n, c_void_p(ws.data_ptr()), need, c_void_p(cents.data_ptr()),
                         max_centroids, c_void_p(labels.data_ptr()) if labels is not None else None,
-                        c_void_p(srt.data_ptr()), c_void_p(res.data_ptr()), _stream_ptr(stream)), "lcd_dbci")
+                        c_void_p(srt.data_ptr()), c_void_p(res.data_ptr()), _stream_ptr()), "lcd_dbci")
     r = DbciResult.from_buffer_copy(res.cpu().numpy().tobytes())
     return {"sigma": r.sigma, "eps": r.eps, "min_pts": r.min_pts, "left": r.left, "right": r.right,
             "n_noise": r.n_noise, "n_clusters_found": r.n_clusters_found,

@@ -10,6 +10,7 @@
 #include <ATen/ops/empty.h>
 #include <ATen/ops/empty_like.h>
 #include <ATen/ops/zeros.h>
+#include <c10/cuda/CUDACachingAllocator.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
@@ -38,18 +39,39 @@ bool require(bool ok, const char* what) {
   if (!ok) PyErr_SetString(PyExc_AssertionError, what);
   return ok;
 }
-// The raw handle of a torch stream object, or of the current stream of the current device.
-bool stream_of(PyObject* o, void** out) {
-  if (o == Py_None) {
-    *out = c10::cuda::getCurrentCUDAStream().stream();
-    return true;
+// The stream of a call: a torch stream object's, or the current one of the current device.  For its life a given stream is the
+// current one, so that what the call allocates belongs to the stream that its kernels run on and is cleared there; outputs are
+// recorded for the caller's stream as well, whose kernels will read them.
+class CallStream {
+ public:
+  explicit CallStream(PyObject* o) : caller_(c10::cuda::getCurrentCUDAStream()), raw_(caller_.stream()) {
+    if (o == Py_None) return;
+    PyObject* h = PyObject_GetAttrString(o, "cuda_stream");
+    void* given = h ? PyLong_AsVoidPtr(h) : nullptr;
+    Py_XDECREF(h);
+    failed_ = PyErr_Occurred() != nullptr;
+    if (failed_ || given == raw_) return;
+    raw_ = static_cast<cudaStream_t>(given);
+    c10::cuda::setCurrentCUDAStream(c10::cuda::getStreamFromExternal(raw_, caller_.device_index()));
+    other_ = true;
   }
-  PyObject* h = PyObject_GetAttrString(o, "cuda_stream");
-  if (!h) return false;
-  *out = PyLong_AsVoidPtr(h);
-  Py_DECREF(h);
-  return !PyErr_Occurred();
-}
+  ~CallStream() {
+    if (other_) c10::cuda::setCurrentCUDAStream(caller_);
+  }
+  CallStream(const CallStream&) = delete;
+  CallStream& operator=(const CallStream&) = delete;
+  bool ok() const { return !failed_; }
+  void* raw() const { return raw_; }
+  PyObject* output(const at::Tensor& t) const {
+    if (other_) c10::cuda::CUDACachingAllocator::recordStream(t.storage().data_ptr(), caller_);
+    return THPVariable_Wrap(t);
+  }
+
+ private:
+  c10::cuda::CUDAStream caller_;
+  cudaStream_t raw_;
+  bool failed_ = false, other_ = false;
+};
 bool count_args(Py_ssize_t have, Py_ssize_t want) {
   if (have != want) PyErr_Format(PyExc_TypeError, "%zd arguments expected, %zd given", want, have);
   return have == want;
@@ -75,6 +97,8 @@ PyObject* smooth_quantize_act(PyObject*, PyObject* const* a, Py_ssize_t n) {
   const long bits = PyLong_AsLong(a[5]);
   if ((bits == -1 && PyErr_Occurred()) || !require(bits == 4 || bits == 8, "act_bits: 4 or 8")) return nullptr;
   const at::ScalarType type = bits == 4 ? at::kByte : at::kChar;
+  const CallStream stream(a[6]);
+  if (!stream.ok()) return nullptr;
   at::Tensor idx, scale;
   if (a[3] == Py_None) idx = at::empty({M, bits == 4 ? K_pad / 2 : K_pad}, x->options().dtype(type));
   else if (const at::Tensor* t = tensor_of(a[3], "act_idx")) idx = *t;
@@ -83,15 +107,15 @@ PyObject* smooth_quantize_act(PyObject*, PyObject* const* a, Py_ssize_t n) {
   if (a[4] == Py_None) scale = at::empty({M}, x->options().dtype(at::kFloat));
   else if (const at::Tensor* t = tensor_of(a[4], "act_scale")) scale = *t;
   else return nullptr;
-  void *inv, *fixed, *stream;
-  if (!address_of(a[1], "inv_smooth", &inv) || !address_of(a[2], "static_scale", &fixed) || !stream_of(a[6], &stream)) return nullptr;
+  void *inv, *fixed;
+  if (!address_of(a[1], "inv_smooth", &inv) || !address_of(a[2], "static_scale", &fixed)) return nullptr;
   const lcd_status st = without_gil([&] {
     return lcd_smooth_quantize_act(x->data_ptr(), M, K, x->stride(0), static_cast<float*>(inv), static_cast<float*>(fixed),
-                                   (int)bits, static_cast<uint8_t*>(idx.data_ptr()), static_cast<float*>(scale.data_ptr()), stream);
+                                   (int)bits, static_cast<uint8_t*>(idx.data_ptr()), static_cast<float*>(scale.data_ptr()), stream.raw());
   });
   if (st != LCD_OK) return PyLong_FromLong((long)st);
-  PyObject* o0 = a[3] == Py_None ? THPVariable_Wrap(idx) : Py_NewRef(a[3]);
-  PyObject* o1 = a[4] == Py_None ? THPVariable_Wrap(scale) : Py_NewRef(a[4]);
+  PyObject* o0 = a[3] == Py_None ? stream.output(idx) : Py_NewRef(a[3]);
+  PyObject* o1 = a[4] == Py_None ? stream.output(scale) : Py_NewRef(a[4]);
   PyObject* out = o0 && o1 ? PyTuple_Pack(2, o0, o1) : nullptr;
   Py_XDECREF(o0);
   Py_XDECREF(o1);
@@ -126,6 +150,8 @@ PyObject* lut_linear(PyObject*, PyObject* const* a, Py_ssize_t n) {
     need = PyLong_AsSize_t(bytes);
     if (PyErr_Occurred()) return nullptr;
   }
+  const CallStream stream(a[10]);
+  if (!stream.ok()) return nullptr;
   at::Tensor y, ws;
   if (a[6] == Py_None) y = at::empty({M, N}, idx->options().dtype(at::kFloat));
   else if (const at::Tensor* t = tensor_of(a[6], "y")) y = *t;
@@ -140,8 +166,8 @@ PyObject* lut_linear(PyObject*, PyObject* const* a, Py_ssize_t n) {
     ws = at::zeros({(int64_t)need}, idx->options().dtype(at::kByte));      // must start zero-filled
     have = need;
   }
-  void *word, *stream;
-  if (!address_of(a[9], "status_word", &word) || !stream_of(a[10], &stream)) return nullptr;
+  void* word;
+  if (!address_of(a[9], "status_word", &word)) return nullptr;
   void* scratch = ws.defined() ? ws.data_ptr() : nullptr;
   const lcd_status st = without_gil([&] {
     const float* s = static_cast<const float*>(scale->data_ptr());
@@ -149,12 +175,12 @@ PyObject* lut_linear(PyObject*, PyObject* const* a, Py_ssize_t n) {
     int32_t* flag = static_cast<int32_t*>(word);
     return idx->scalar_type() == at::kChar
                ? lcd_lut_linear_act8(w->data_ptr(), header, static_cast<const int8_t*>(idx->data_ptr()), s, M, out, y.stride(0),
-                                     (lcd_algo)algo, scratch, have, flag, stream)
+                                     (lcd_algo)algo, scratch, have, flag, stream.raw())
                : lcd_lut_linear(w->data_ptr(), header, static_cast<const uint8_t*>(idx->data_ptr()), s, M, out, y.stride(0),
-                                (lcd_algo)algo, scratch, have, flag, stream);
+                                (lcd_algo)algo, scratch, have, flag, stream.raw());
   });
   if (st != LCD_OK) return PyLong_FromLong((long)st);
-  return a[6] == Py_None ? THPVariable_Wrap(y) : Py_NewRef(a[6]);
+  return a[6] == Py_None ? stream.output(y) : Py_NewRef(a[6]);
   END_HANDLE_TH_ERRORS
 }
 
@@ -162,11 +188,13 @@ PyObject* lut_linear(PyObject*, PyObject* const* a, Py_ssize_t n) {
 PyObject* act_batch(PyObject*, PyObject* const* a, Py_ssize_t n) {
   HANDLE_TH_ERRORS
   if (!count_args(n, 4)) return nullptr;
-  void *arr = PyLong_AsVoidPtr(a[0]), *stream;
+  void* arr = PyLong_AsVoidPtr(a[0]);
   const int count = (int)PyLong_AsLong(a[1]), bits = (int)PyLong_AsLong(a[2]);
-  if (PyErr_Occurred() || !stream_of(a[3], &stream)) return nullptr;
+  if (PyErr_Occurred()) return nullptr;
+  const CallStream stream(a[3]);
+  if (!stream.ok()) return nullptr;
   return PyLong_FromLong((long)without_gil(
-      [&] { return lcd_smooth_quantize_act_batch(static_cast<const lcd_act_problem*>(arr), count, bits, stream); }));
+      [&] { return lcd_smooth_quantize_act_batch(static_cast<const lcd_act_problem*>(arr), count, bits, stream.raw()); }));
   END_HANDLE_TH_ERRORS
 }
 
@@ -176,20 +204,22 @@ PyObject* linear_batch(PyObject*, PyObject* const* a, Py_ssize_t n) {
   HANDLE_TH_ERRORS
   if (!count_args(n, 7)) return nullptr;
   const long form = PyLong_AsLong(a[0]);
-  void *arr = PyLong_AsVoidPtr(a[1]), *word, *stream;
+  void *arr = PyLong_AsVoidPtr(a[1]), *word;
   const int count = (int)PyLong_AsLong(a[2]);
   const lcd_algo algo = (lcd_algo)PyLong_AsLong(a[3]);
   if (PyErr_Occurred()) return nullptr;
   const at::Tensor* ws = tensor_of(a[4], "workspace");
-  if (!ws || !address_of(a[5], "status_word", &word) || !stream_of(a[6], &stream)) return nullptr;
+  if (!ws || !address_of(a[5], "status_word", &word)) return nullptr;
+  const CallStream stream(a[6]);
+  if (!stream.ok()) return nullptr;
   void* scratch = ws->data_ptr();
   const size_t bytes = (size_t)ws->numel();
   return PyLong_FromLong((long)without_gil([&] {
     int32_t* flag = static_cast<int32_t*>(word);
-    if (form == 0) return lcd_linear_fused_batch(static_cast<const lcd_fused_problem*>(arr), count, algo, scratch, bytes, flag, stream);
+    if (form == 0) return lcd_linear_fused_batch(static_cast<const lcd_fused_problem*>(arr), count, algo, scratch, bytes, flag, stream.raw());
     const lcd_linear_problem* p = static_cast<const lcd_linear_problem*>(arr);
-    return form == 1 ? lcd_lut_linear_batch(p, count, algo, scratch, bytes, flag, stream)
-                     : lcd_lut_linear_batch_act8(p, count, algo, scratch, bytes, flag, stream);
+    return form == 1 ? lcd_lut_linear_batch(p, count, algo, scratch, bytes, flag, stream.raw())
+                     : lcd_lut_linear_batch_act8(p, count, algo, scratch, bytes, flag, stream.raw());
   }));
   END_HANDLE_TH_ERRORS
 }
@@ -206,6 +236,8 @@ PyObject* reclassify(PyObject*, PyObject* const* a, Py_ssize_t n) {
                    dw->stride(1) == 1, "contiguous [N, K], [N, C] and rows of delta_w"))
     return nullptr;
   const int64_t N = idx->size(0), K = idx->size(1), C = cb->size(1);
+  const CallStream stream(a[6]);
+  if (!stream.ok()) return nullptr;
   at::Tensor out[3];
   if (a[3] == Py_None) {
     out[0] = at::empty_like(*idx);
@@ -223,19 +255,17 @@ PyObject* reclassify(PyObject*, PyObject* const* a, Py_ssize_t n) {
                  "out: [N, K], [N, C], [N, C]"))
       return nullptr;
   }
-  void* stream;
-  if (!stream_of(a[6], &stream)) return nullptr;
   const lcd_status st = without_gil([&] {
     return lcd_reclassify(static_cast<const uint8_t*>(idx->data_ptr()), static_cast<const uint16_t*>(cb->data_ptr()),
                           static_cast<const float*>(dw->data_ptr()), N, K, dw->stride(0), (int)C,
                           static_cast<uint8_t*>(out[0].data_ptr()), static_cast<double*>(out[1].data_ptr()),
-                          static_cast<int32_t*>(out[2].data_ptr()), stream);
+                          static_cast<int32_t*>(out[2].data_ptr()), stream.raw());
   });
   if (st != LCD_OK) return PyLong_FromLong((long)st);
   if (a[3] != Py_None) return PyTuple_Pack(3, a[3], a[4], a[5]);
   PyObject* r = PyTuple_New(3);
   for (int i = 0; r && i < 3; ++i) {
-    PyObject* o = THPVariable_Wrap(out[i]);
+    PyObject* o = stream.output(out[i]);
     if (!o) Py_CLEAR(r);
     else PyTuple_SET_ITEM(r, i, o);
   }
@@ -262,18 +292,18 @@ PyObject* smoothing_search(PyObject*, PyObject* const* a, Py_ssize_t n) {
   size_t need = 0;
   const lcd_status sized = lcd_smoothing_search_workspace_bytes(T, K, G, &need);
   if (sized != LCD_OK) return PyLong_FromLong((long)sized);
+  const CallStream stream(a[3]);
+  if (!stream.ok()) return nullptr;
   const at::Tensor ws = at::empty({(int64_t)need}, x->options().dtype(at::kByte));
   const at::Tensor mse = at::empty({G}, x->options().dtype(at::kDouble)), best = at::empty({1}, x->options().dtype(at::kInt)),
                    inv = at::empty({K}, x->options().dtype(at::kFloat));
-  void* stream;
-  if (!stream_of(a[3], &stream)) return nullptr;
   const lcd_status st = without_gil([&] {
     return lcd_smoothing_search(x->data_ptr(), T, K, x->stride(0), static_cast<const float*>(wmax->data_ptr()), alphas.data(), G,
                                 ws.data_ptr(), need, static_cast<double*>(mse.data_ptr()), static_cast<int32_t*>(best.data_ptr()),
-                                static_cast<float*>(inv.data_ptr()), stream);
+                                static_cast<float*>(inv.data_ptr()), stream.raw());
   });
   if (st != LCD_OK) return PyLong_FromLong((long)st);
-  PyObject *o0 = THPVariable_Wrap(best), *o1 = THPVariable_Wrap(mse), *o2 = THPVariable_Wrap(inv);
+  PyObject *o0 = stream.output(best), *o1 = stream.output(mse), *o2 = stream.output(inv);
   PyObject* out = o0 && o1 && o2 ? PyTuple_Pack(3, o0, o1, o2) : nullptr;
   Py_XDECREF(o0);
   Py_XDECREF(o1);

@@ -1000,3 +1000,44 @@ def test_smoothing_searches_one_after_another(K):
     results = [lcd.smoothing_search(xs[i % 2], wmax[i % 2], alphas) for i in range(40)]
     for i, r in enumerate(results):
         assert all(torch.equal(a, b) for a, b in zip(r, alone[i % 2]))
+
+
+def test_calls_on_a_given_stream_while_the_current_one_is_busy():
+    # what a call allocates for itself is cleared on the stream its kernels run on: behind milliseconds of other work on the
+    # current stream it would still hold what its block held before
+    L = gen.random_case(seed=6, N=4096, K=4096, bits=3, M=8)
+    w = lcd.PackedWeights(lcd.pack_weights(L.idx, L.codebook, 3))
+    x, inv_s = torch.from_numpy(L.x).cuda(), torch.from_numpy(L.inv_s).cuda()
+    wmax = torch.rand(4096, device="cuda") + 0.1
+    weights = torch.from_numpy(np.random.default_rng(1).normal(0, 0.02, 50_000).astype(np.float32)).cuda()
+    idx = torch.randint(0, 4, (64, 1000), dtype=torch.uint8, device="cuda")
+    cb, dw = torch.randn(64, 4, device="cuda").sort(dim=1).values.half(), torch.randn(64, 1000, device="cuda")
+
+    def calls(stream=None):
+        a, s = lcd.smooth_quantize_act(x, inv_s, stream=stream)
+        y = lcd.lut_linear(w, a, s, algo=lcd.ALGO_REGISTER_LUT, stream=stream)
+        r = lcd.dbci(weights, stream=stream)
+        return [a, s, y, r["centroids"], r["labels"], r["sorted"], torch.tensor([r["sigma"], r["eps"]]),
+                *lcd.reclassify(idx, cb, dw, stream=stream), *lcd.smoothing_search(x, wmax, [0.0, 0.5, 1.0], stream=stream)]
+
+    expected = calls()
+    q_ref, s_ref = O.smooth_quantize(L.x, L.inv_s)
+    check_y(expected[2], O.lut_linear_dequant(L.idx, L.codebook, q_ref, s_ref))
+    busy = torch.randn(8192, 8192, device="cuda")
+    product = busy @ busy
+    side = torch.cuda.Stream()
+    calls(side)                                             # (its blocks come from the device, which may wait for it)
+    need = lcd.lut_linear_workspace_bytes(w, 8, lcd.ALGO_REGISTER_LUT)
+    for stream, current in ((side, torch.cuda.current_stream()), (torch.cuda.default_stream(), torch.cuda.Stream())):
+        for _ in range(3):
+            with torch.cuda.stream(current):
+                dirty = [torch.full((n,), 255, dtype=torch.uint8, device="cuda") for n in (need, 64, 512, 1 << 16, 1 << 20)]
+                torch.cuda.synchronize()
+                del dirty
+                for _ in range(3):
+                    torch.mm(busy, busy, out=product)       # fp32: tens of milliseconds
+                got = calls(stream)
+                assert not current.query()                  # (still busy: nothing waited for it)
+                stream.synchronize()
+            assert all(torch.equal(g, e) for g, e in zip(got, expected))
+            torch.cuda.synchronize()
