@@ -199,8 +199,7 @@ class PackedWeights:
     def __init__(self, blob: np.ndarray, device="cuda"):
         import torch
         self.header = bytes(blob[:HEADER_BYTES])
-        self._hdr_buf = ctypes.create_string_buffer(self.header, HEADER_BYTES)
-        self._hdr_addr = ctypes.addressof(self._hdr_buf)
+        self._place_header()
         f = np.frombuffer(self.header, dtype="<u8")
         self.N, self.K, self.K_pad = int(f[1]), int(f[2]), int(f[3])
         u = np.frombuffer(self.header, dtype="<u4")
@@ -208,7 +207,19 @@ class PackedWeights:
         self.nbytes = int(blob.size)
         self.dev = torch.from_numpy(np.ascontiguousarray(blob)).to(device)
         assert self.dev.data_ptr() % 256 == 0
-        self._workspace_bytes = {}      # (tokens, algo) -> bytes: a function of the header
+
+    def _place_header(self):
+        self._workspace_bytes = {}      # (tokens, algo) -> bytes: a function of the header and the GPU's number of SMs
+        self._hdr_buf = ctypes.create_string_buffer(self.header, HEADER_BYTES)
+        self._hdr_addr = ctypes.addressof(self._hdr_buf)
+
+    # a copy's header lies elsewhere, and it may be used on another GPU
+    def __getstate__(self):
+        return {k: v for k, v in self.__dict__.items() if k not in ("_hdr_buf", "_hdr_addr", "_workspace_bytes")}
+
+    def __setstate__(self, state):
+        self.__dict__.update(state)
+        self._place_header()
 
     @property
     def header_ptr(self) -> c_void_p:

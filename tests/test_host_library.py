@@ -124,3 +124,23 @@ def test_resolve_names_the_family_that_runs(K, family):
     assert lcd.resolve_batch_algo([(row, 12)], lcd.ALGO_TC_LUT) == family
     assert lcd.resolve_batch_algo([(short, 12), (row, 3)], lcd.ALGO_TC_LUT) == family
     assert lcd.resolve_batch_algo([(short, 12)], lcd.ALGO_TC_LUT) == lcd.ALGO_TC_LUT
+
+
+@pytest.mark.parametrize("how", ["deepcopy", "pickle", "copy"])
+def test_copies_of_packed_weights_have_their_own_header(how):
+    import copy
+    import gc
+    import pickle
+    blob = lcd.pack_weights(np.zeros((5, 300), dtype=np.uint8), np.ones((5, 4), dtype=np.float16), 2)
+    room = np.empty(blob.size + 256, dtype=np.uint8)
+    at = -room.ctypes.data % 256
+    room[at:at + blob.size] = blob
+    w = lcd.PackedWeights(room[at:at + blob.size], device="cpu")
+    assert lcd.lut_linear_workspace_bytes(w, 3) >= 0
+    c = copy.deepcopy(w) if how == "deepcopy" else pickle.loads(pickle.dumps(w)) if how == "pickle" else copy.copy(w)
+    assert c.header_ptr.value == c._hdr_addr == ctypes.addressof(c._hdr_buf)
+    assert how == "copy" or c._hdr_addr != w._hdr_addr
+    del w
+    gc.collect()
+    assert ctypes.string_at(c._hdr_addr, 64) == c.header == bytes(blob[:64])
+    assert (c.N, c.K, c.bits, c.C) == (5, 300, 2, 4) and lcd.lut_linear_workspace_bytes(c, 4) >= 0
