@@ -319,6 +319,8 @@ __device__ __forceinline__ void smooth_quantize_token_cached(const __half* __res
           const float u = is_static ? t[c][i] : __fmul_rn(t[c][i], r);
           packed |= quant_nibble(u) << (4 * i);
         }
+        // past the row's end level 0: 0 * r is none where r is infinite (a token whose maximum is below 7 / FLT_MAX)
+        if (k + 8 > K) packed = (packed & (0xffffffffu >> (4 * (k + 8 - K)))) | (0x88888888u << (4 * (K - k)));
       }
       *reinterpret_cast<uint32_t*>(out + k / 2) = packed;
     }
@@ -414,6 +416,10 @@ __device__ __forceinline__ void smooth_quantize_token_words(const __half* __rest
           const float u = fminf(fmaxf(is_static ? t[i] : __fmul_rn(t[i], r_eff), -8.0f), 7.0f);
           // clipped, then rounded to an integer (ties to even) by one addition: the low byte of the sum is the level
           b[i] = __float_as_uint(__fadd_rn(u, OUT == kOutNibbles ? 12582920.0f : 12582912.0f));
+        }
+        if (k + 8 > K) {               // past the row's end level 0, as above
+#pragma unroll
+          for (int i = 1; i < 8; ++i) b[i] = k + i < K ? b[i] : (OUT == kOutNibbles ? 8u : 0u);
         }
         e = prmt_q(prmt_q(b[0], b[2], 0x0040u), prmt_q(b[4], b[6], 0x0040u), 0x5410u);
         o = prmt_q(prmt_q(b[1], b[3], 0x0040u), prmt_q(b[5], b[7], 0x0040u), 0x5410u);

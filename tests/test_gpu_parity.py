@@ -1041,3 +1041,19 @@ def test_calls_on_a_given_stream_while_the_current_one_is_busy():
                 stream.synchronize()
             assert all(torch.equal(g, e) for g, e in zip(got, expected))
             torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("M", [2, 300])
+@pytest.mark.parametrize("K", [1, 250, 2043, 8191])
+def test_padding_levels_of_tokens_whose_scale_overflows(M, K):
+    # 7 / max is infinite: every non-zero product saturates, and the columns past the row still hold level 0
+    x, inv_s = torch.full((M, K), 2.0 ** -24, dtype=torch.float16, device="cuda"), torch.full((K,), 3.2e-31, device="cuda")
+    a, s = lcd.smooth_quantize_act(x, inv_s)
+    assert np.array_equal(a.cpu().numpy(), O.pack_act(np.full((M, K), 7, dtype=np.int8)))
+    # the forms that the many-token kernels read: a matrix of one value gives the sum of a row's levels, padding included
+    if M > 16:
+        w = lcd.PackedWeights(lcd.pack_weights(np.zeros((16, K), dtype=np.uint8), np.full((16, 4), 32768, dtype=np.float16), 2))
+        y = torch.empty((M, 16), device="cuda")
+        lcd.FusedBatch([(w, x, inv_s, y)]).run()
+        assert torch.equal(y, lcd.lut_linear(w, a, s))
+        assert torch.allclose(y.double(), 7 * K * 32768 * s.double()[:, None].expand(M, 16), rtol=1e-6, atol=0)
