@@ -85,13 +85,17 @@ __device__ __forceinline__ void store_level1(uint8_t* row, int64_t k, uint32_t a
   }
 }
 
-// Columns k .. k + 7 of a row that ends at column K (zeros past it), k a multiple of 8.  aligned: the row starts on 16 bytes.
+// Columns k .. k + 7 of a row that ends at column K (zeros past it), k a multiple of 8.  ALIGNED: all rows start on 16 bytes and
+// K is a multiple of 8 (instances of their own: with both ways in one kernel such rows took 4 to 20 % longer: 2048 x 5120
+// 9.05 us, 8.70 apart; 2048 x 11008 18.6 and 16.5; 1 x 4096 2.34 and 2.20).  aligned: the row starts on 16 bytes.
 // Any other row is read in the same 16-byte words and shifted: word i of the result is taken from words q + i and q + i + 1
 // of the two it lies in (its neighbour loads the second one too, from L1).  Both hold at least one of the row's values.  So
 // such rows too are read once, eight columns a thread, all loads in flight together (333 x 5001, from x to y of a 5003-row
 // layer: 30.6 us with two passes over single columns, 27.3 so).
+template <bool ALIGNED>
 __device__ __forceinline__ uint4 load_columns8(const __half* row, int k, int K, bool aligned) {
   const __half* p = row + k;
+  if constexpr (ALIGNED) return *reinterpret_cast<const uint4*>(p);
   if (aligned && k + 8 <= K) return *reinterpret_cast<const uint4*>(p);
   const uintptr_t at = reinterpret_cast<uintptr_t>(p), first = at & ~(uintptr_t)15, end = reinterpret_cast<uintptr_t>(row + K);
   const unsigned off = (unsigned)(at & 15), r = 8 * (off & 3);
@@ -122,13 +126,14 @@ __device__ __forceinline__ uint4 load_columns8(const __half* row, int k, int K, 
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 // The smoothing factors of columns k .. k + 7 (1 where there are none: past K or without a vector).
+template <bool ALIGNED>
 __device__ __forceinline__ void load_factors8(const float* inv_smooth, int k, int K, float (&f)[8]) {
-  if (inv_smooth && k + 8 <= K) {
+  if (inv_smooth && (ALIGNED || k + 8 <= K)) {
     const float4 a = __ldg(reinterpret_cast<const float4*>(inv_smooth + k)), b = __ldg(reinterpret_cast<const float4*>(inv_smooth + k + 4));
     f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w; f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
   } else {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) f[i] = inv_smooth && k + i < K ? __ldg(inv_smooth + k + i) : 1.0f;
+    for (int i = 0; i < 8; ++i) f[i] = !ALIGNED && inv_smooth && k + i < K ? __ldg(inv_smooth + k + i) : 1.0f;
   }
 }
 
@@ -247,7 +252,7 @@ __device__ __forceinline__ void smooth_quantize_token(const __half* __restrict__
 // Same result as smooth_quantize_token<true>, for rows of at most 8 * THREADS * CHUNKS columns: every thread
 // keeps its products t_k = x_k * inv_smooth_k in registers between the maximum search and the rounding, so x
 // and inv_smooth are read once and all loads are in flight together.
-template <int THREADS, int CHUNKS>
+template <int THREADS, int CHUNKS, bool ALIGNED>
 __device__ __forceinline__ void smooth_quantize_token_cached(const __half* __restrict__ x, int64_t m, int64_t K,
                                                              int64_t K_pad, int64_t ldx,
                                                              const float* __restrict__ inv_smooth,
@@ -266,10 +271,10 @@ __device__ __forceinline__ void smooth_quantize_token_cached(const __half* __res
   for (int c = 0; c < CHUNKS; ++c) {
     const int64_t k = ((int64_t)c * THREADS + tid) * 8;
     if (k < K) {
-      const uint4 raw = load_columns8(xr, (int)k, (int)K, aligned);
+      const uint4 raw = load_columns8<ALIGNED>(xr, (int)k, (int)K, aligned);
       const __half2* h = reinterpret_cast<const __half2*>(&raw);
       float f[8];
-      load_factors8(inv_smooth, (int)k, (int)K, f);
+      load_factors8<ALIGNED>(inv_smooth, (int)k, (int)K, f);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const float2 v = __half22float2(h[i]);
@@ -320,7 +325,7 @@ __device__ __forceinline__ void smooth_quantize_token_cached(const __half* __res
           packed |= quant_nibble(u) << (4 * i);
         }
         // past the row's end level 0: 0 * r is none where r is infinite (a token whose maximum is below 7 / FLT_MAX)
-        if (k + 8 > K) packed = (packed & (0xffffffffu >> (4 * (k + 8 - K)))) | (0x88888888u << (4 * (K - k)));
+        if (!ALIGNED && k + 8 > K) packed = (packed & (0xffffffffu >> (4 * (k + 8 - K)))) | (0x88888888u << (4 * (K - k)));
       }
       *reinterpret_cast<uint32_t*>(out + k / 2) = packed;
     }
@@ -331,7 +336,7 @@ __device__ __forceinline__ void smooth_quantize_token_cached(const __half* __res
 // loaded (four registers per eight columns, so that enough CTAs fit an SM to keep the memory system busy) and forms
 // the products x_k * inv_smooth_k twice, with the same single operations, once for the maximum and once for the
 // levels; inv_smooth comes from L1 the second time.  Rows of at most 8 * THREADS * CHUNKS columns.
-template <int THREADS, int CHUNKS, int OUT = kOutNibbles>
+template <int THREADS, int CHUNKS, int OUT, bool ALIGNED>
 __device__ __forceinline__ void smooth_quantize_token_words(const __half* __restrict__ x, int64_t m, int64_t K64,
                                                             int64_t K_pad64, int64_t ldx,
                                                             const float* __restrict__ inv_smooth,
@@ -349,12 +354,12 @@ __device__ __forceinline__ void smooth_quantize_token_words(const __half* __rest
 #pragma unroll
   for (int c = 0; c < CHUNKS; ++c) {
     const int k = (c * THREADS + tid) * 8;
-    raw[c] = k < K ? load_columns8(xr, k, K, aligned) : make_uint4(0u, 0u, 0u, 0u);
+    raw[c] = k < K ? load_columns8<ALIGNED>(xr, k, K, aligned) : make_uint4(0u, 0u, 0u, 0u);
   }
   auto products = [&](int c, int k, float (&t)[8]) {
     const __half2* h = reinterpret_cast<const __half2*>(&raw[c]);
     float f[8];
-    load_factors8(inv_smooth, k, K, f);
+    load_factors8<ALIGNED>(inv_smooth, k, K, f);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const float2 v = __half22float2(h[i]);
@@ -417,7 +422,7 @@ __device__ __forceinline__ void smooth_quantize_token_words(const __half* __rest
           // clipped, then rounded to an integer (ties to even) by one addition: the low byte of the sum is the level
           b[i] = __float_as_uint(__fadd_rn(u, OUT == kOutNibbles ? 12582920.0f : 12582912.0f));
         }
-        if (k + 8 > K) {               // past the row's end level 0, as above
+        if (!ALIGNED && k + 8 > K) {               // past the row's end level 0, as above
 #pragma unroll
           for (int i = 1; i < 8; ++i) b[i] = k + i < K ? b[i] : (OUT == kOutNibbles ? 8u : 0u);
         }
@@ -459,8 +464,8 @@ struct QuantBatch {
 
 // One CTA per token of every problem of the batch.  CHUNKS > 0: rows of at most 8 * THREADS * CHUNKS columns take the
 // register-resident path (the launcher picks the smallest instance that covers the batch's longest row, so that the
-// instance's register count, and with it the number of CTAs per SM, fits the rows at hand).
-template <int THREADS, int CHUNKS, int OUT = kOutNibbles>
+// instance's register count, and with it the number of CTAs per SM, fits the rows at hand).  ALIGNED: see load_columns8.
+template <int THREADS, int CHUNKS, int OUT, bool ALIGNED>
 __global__ void __launch_bounds__(THREADS) smooth_quantize_kernel(const __grid_constant__ QuantBatch batch) {
   // This kernel may itself have been started early (programmatic stream serialization): wait for the kernel
   // before it, then let the next one start its own prologue; that one still waits for this grid to finish
@@ -476,10 +481,10 @@ __global__ void __launch_bounds__(THREADS) smooth_quantize_kernel(const __grid_c
   if constexpr (CHUNKS > 0) {
     if (q.vec && q.K_pad <= (long long)8 * THREADS * CHUNKS) {
       if constexpr (THREADS == kQThreads)
-        smooth_quantize_token_cached<THREADS, CHUNKS>(q.x, m, q.K, q.K_pad, q.ldx, q.inv_smooth, q.static_scale, q.act_idx,
+        smooth_quantize_token_cached<THREADS, CHUNKS, ALIGNED>(q.x, m, q.K, q.K_pad, q.ldx, q.inv_smooth, q.static_scale, q.act_idx,
                                                       q.act_scale, q.vec == 2);
       else
-        smooth_quantize_token_words<THREADS, CHUNKS, OUT>(q.x, m, q.K, q.K_pad, q.ldx, q.inv_smooth, q.static_scale,
+        smooth_quantize_token_words<THREADS, CHUNKS, OUT, ALIGNED>(q.x, m, q.K, q.K_pad, q.ldx, q.inv_smooth, q.static_scale,
                                                           q.act_idx, q.act_scale, q.vec == 2);
       return;
     }
@@ -492,14 +497,19 @@ __global__ void __launch_bounds__(THREADS) smooth_quantize_kernel(const __grid_c
 
 namespace {
 
-template <int OUT>
+// (the two-pass kernel goes by each problem's own alignment)
+template <int OUT, bool ALIGNED>
 cudaError_t launch_small_ctas(const cudaLaunchConfig_t& cfg, long long chunks, const QuantBatch& batch) {
-  if (chunks < 1 || chunks > 8) return cudaLaunchKernelEx(&cfg, smooth_quantize_kernel<kQThreadsMany, 0, OUT>, batch);
-  if (chunks <= 2) return cudaLaunchKernelEx(&cfg, smooth_quantize_kernel<kQThreadsMany, 2, OUT>, batch);
-  if (chunks <= 3) return cudaLaunchKernelEx(&cfg, smooth_quantize_kernel<kQThreadsMany, 3, OUT>, batch);
-  if (chunks <= 4) return cudaLaunchKernelEx(&cfg, smooth_quantize_kernel<kQThreadsMany, 4, OUT>, batch);
-  if (chunks <= 6) return cudaLaunchKernelEx(&cfg, smooth_quantize_kernel<kQThreadsMany, 6, OUT>, batch);
-  return cudaLaunchKernelEx(&cfg, smooth_quantize_kernel<kQThreadsMany, 8, OUT>, batch);
+  if (chunks < 1 || chunks > 8) return cudaLaunchKernelEx(&cfg, smooth_quantize_kernel<kQThreadsMany, 0, OUT, false>, batch);
+  if (chunks <= 2) return cudaLaunchKernelEx(&cfg, smooth_quantize_kernel<kQThreadsMany, 2, OUT, ALIGNED>, batch);
+  if (chunks <= 3) return cudaLaunchKernelEx(&cfg, smooth_quantize_kernel<kQThreadsMany, 3, OUT, ALIGNED>, batch);
+  if (chunks <= 4) return cudaLaunchKernelEx(&cfg, smooth_quantize_kernel<kQThreadsMany, 4, OUT, ALIGNED>, batch);
+  if (chunks <= 6) return cudaLaunchKernelEx(&cfg, smooth_quantize_kernel<kQThreadsMany, 6, OUT, ALIGNED>, batch);
+  return cudaLaunchKernelEx(&cfg, smooth_quantize_kernel<kQThreadsMany, 8, OUT, ALIGNED>, batch);
+}
+template <int OUT>
+cudaError_t launch_small_ctas(const cudaLaunchConfig_t& cfg, long long chunks, const QuantBatch& batch, bool aligned) {
+  return aligned ? launch_small_ctas<OUT, true>(cfg, chunks, batch) : launch_small_ctas<OUT, false>(cfg, chunks, batch);
 }
 
 // out_form: kOutNibbles (act_idx = [M][K_pad / 2]) or signed bytes for the tensor-core kernel (act_idx = [M][K_pad],
@@ -543,6 +553,7 @@ lcd_status launch_quantize_form(const lcd_act_problem* probs, int count, int out
     QuantBatch batch;
     batch.count = 0;
     long long grid = 0;
+    bool aligned = true;                         // every problem of the launch
     for (int i = first; i < count; ++i) {
       if (done[i]) continue;
       const int mine = instance_of(all[i]);
@@ -551,6 +562,7 @@ lcd_status launch_quantize_form(const lcd_act_problem* probs, int count, int out
       QuantProblem& q = batch.p[batch.count++];
       q = all[i];
       q.cta0 = (int)grid;
+      aligned = aligned && q.vec == 2;
       grid += all[i].cta0;
       done[i] = true;
     }
@@ -566,13 +578,14 @@ lcd_status launch_quantize_form(const lcd_act_problem* probs, int count, int out
     cfg.numAttrs = 1;
     cudaError_t e;
     if (!many)
-      e = inst ? cudaLaunchKernelEx(&cfg, smooth_quantize_kernel<kQThreads, kQChunks>, batch)
-               : cudaLaunchKernelEx(&cfg, smooth_quantize_kernel<kQThreads, 0>, batch);
-    else if (out_form == kOutBytes) e = launch_small_ctas<kOutBytes>(cfg, inst, batch);
-    else if (out_form == kOutBytes2) e = launch_small_ctas<kOutBytes2>(cfg, inst, batch);
-    else if (out_form == kOutTc) e = launch_small_ctas<kOutTc>(cfg, inst, batch);
-    else if (out_form == kOutTc2) e = launch_small_ctas<kOutTc2>(cfg, inst, batch);
-    else e = launch_small_ctas<kOutNibbles>(cfg, inst, batch);
+      e = !inst     ? cudaLaunchKernelEx(&cfg, smooth_quantize_kernel<kQThreads, 0, kOutNibbles, false>, batch)
+          : aligned ? cudaLaunchKernelEx(&cfg, smooth_quantize_kernel<kQThreads, kQChunks, kOutNibbles, true>, batch)
+                    : cudaLaunchKernelEx(&cfg, smooth_quantize_kernel<kQThreads, kQChunks, kOutNibbles, false>, batch);
+    else if (out_form == kOutBytes) e = launch_small_ctas<kOutBytes>(cfg, inst, batch, aligned);
+    else if (out_form == kOutBytes2) e = launch_small_ctas<kOutBytes2>(cfg, inst, batch, aligned);
+    else if (out_form == kOutTc) e = launch_small_ctas<kOutTc>(cfg, inst, batch, aligned);
+    else if (out_form == kOutTc2) e = launch_small_ctas<kOutTc2>(cfg, inst, batch, aligned);
+    else e = launch_small_ctas<kOutNibbles>(cfg, inst, batch, aligned);
     if (e != cudaSuccess) {
       set_cuda_error((int)e);
       return LCD_ERR_CUDA;
