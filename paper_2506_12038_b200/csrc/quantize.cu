@@ -91,18 +91,30 @@ __device__ __forceinline__ void store_level1(uint8_t* row, int64_t k, uint32_t a
 // Any other row is read in the same 16-byte words and shifted: word i of the result is taken from words q + i and q + i + 1
 // of the two it lies in (its neighbour loads the second one too, from L1).  Both hold at least one of the row's values.  So
 // such rows too are read once, eight columns a thread, all loads in flight together (333 x 5001, from x to y of a 5003-row
-// layer: 30.6 us with two passes over single columns, 27.3 so).
+// layer: 30.6 us with two passes over single columns, 27.3 so).  The words hold columns of the neighbouring rows too.  edge:
+// they may also hold what lies before or behind the caller's x, at the first and the last row; there those columns are read one
+// by one.
+struct XBounds {
+  uintptr_t begin, end;
+};
 template <bool ALIGNED>
-__device__ __forceinline__ uint4 load_columns8(const __half* row, int k, int K, bool aligned) {
+__device__ __forceinline__ uint4 load_columns8(const __half* row, int k, int K, bool aligned, bool edge, const XBounds& x) {
   const __half* p = row + k;
   if constexpr (ALIGNED) return *reinterpret_cast<const uint4*>(p);
   if (aligned && k + 8 <= K) return *reinterpret_cast<const uint4*>(p);
   const uintptr_t at = reinterpret_cast<uintptr_t>(p), first = at & ~(uintptr_t)15, end = reinterpret_cast<uintptr_t>(row + K);
   const unsigned off = (unsigned)(at & 15), r = 8 * (off & 3);
+  const bool second = off && first + 16 < end;
+  uint32_t w[4];
+  if (edge && (first < x.begin || first + (second ? 32 : 16) > x.end)) {
+    const unsigned short* u = reinterpret_cast<const unsigned short*>(p);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[i] = (k + 2 * i < K ? (uint32_t)u[2 * i] : 0u) | (k + 2 * i + 1 < K ? (uint32_t)u[2 * i + 1] << 16 : 0u);
+    return make_uint4(w[0], w[1], w[2], w[3]);
+  }
   const uint4 a = *reinterpret_cast<const uint4*>(first);
   uint4 b = make_uint4(0u, 0u, 0u, 0u);
-  if (off && first + 16 < end) b = *reinterpret_cast<const uint4*>(first + 16);
-  uint32_t w[4];
+  if (second) b = *reinterpret_cast<const uint4*>(first + 16);
   switch (off >> 2) {        // the same for the whole row
     case 0:
       w[0] = __funnelshift_r(a.x, a.y, r); w[1] = __funnelshift_r(a.y, a.z, r); w[2] = __funnelshift_r(a.z, a.w, r); w[3] = __funnelshift_r(a.w, b.x, r);
@@ -258,7 +270,7 @@ __device__ __forceinline__ void smooth_quantize_token_cached(const __half* __res
                                                              const float* __restrict__ inv_smooth,
                                                              const float* __restrict__ static_scale,
                                                              uint8_t* __restrict__ act_idx,
-                                                             float* __restrict__ act_scale, bool aligned) {
+                                                             float* __restrict__ act_scale, bool aligned, bool edge, const XBounds& bounds) {
   __shared__ float s_red[THREADS / 32];
   __shared__ float s_mult;
   const __half* xr = x + m * ldx;
@@ -271,7 +283,7 @@ __device__ __forceinline__ void smooth_quantize_token_cached(const __half* __res
   for (int c = 0; c < CHUNKS; ++c) {
     const int64_t k = ((int64_t)c * THREADS + tid) * 8;
     if (k < K) {
-      const uint4 raw = load_columns8<ALIGNED>(xr, (int)k, (int)K, aligned);
+      const uint4 raw = load_columns8<ALIGNED>(xr, (int)k, (int)K, aligned, edge, bounds);
       const __half2* h = reinterpret_cast<const __half2*>(&raw);
       float f[8];
       load_factors8<ALIGNED>(inv_smooth, (int)k, (int)K, f);
@@ -342,7 +354,7 @@ __device__ __forceinline__ void smooth_quantize_token_words(const __half* __rest
                                                             const float* __restrict__ inv_smooth,
                                                             const float* __restrict__ static_scale,
                                                             uint8_t* __restrict__ act_idx,
-                                                            float* __restrict__ act_scale, bool aligned) {
+                                                            float* __restrict__ act_scale, bool aligned, bool edge, const XBounds& bounds) {
   __shared__ float s_red[THREADS / 32];
   __shared__ float s_mult;
   const __half* xr = x + m * ldx;
@@ -354,7 +366,7 @@ __device__ __forceinline__ void smooth_quantize_token_words(const __half* __rest
 #pragma unroll
   for (int c = 0; c < CHUNKS; ++c) {
     const int k = (c * THREADS + tid) * 8;
-    raw[c] = k < K ? load_columns8<ALIGNED>(xr, k, K, aligned) : make_uint4(0u, 0u, 0u, 0u);
+    raw[c] = k < K ? load_columns8<ALIGNED>(xr, k, K, aligned, edge, bounds) : make_uint4(0u, 0u, 0u, 0u);
   }
   auto products = [&](int c, int k, float (&t)[8]) {
     const __half2* h = reinterpret_cast<const __half2*>(&raw[c]);
@@ -455,6 +467,7 @@ struct QuantProblem {
   float* act_scale;
   long long K, K_pad, ldx;
   int cta0;    // tokens of this problem are CTAs [cta0, cta0 + M)
+  XBounds bounds;
   int vec;     // 2: rows on 16 bytes, K a multiple of 8; 1: x any way, the other pointers aligned; 0: neither
 };
 struct QuantBatch {
@@ -480,12 +493,14 @@ __global__ void __launch_bounds__(THREADS) smooth_quantize_kernel(const __grid_c
   const int64_t m = (int64_t)blockIdx.x - q.cta0;
   if constexpr (CHUNKS > 0) {
     if (q.vec && q.K_pad <= (long long)8 * THREADS * CHUNKS) {
+      const uintptr_t row = reinterpret_cast<uintptr_t>(q.x + m * q.ldx);
+      const bool edge = row < q.bounds.begin + 16 || row + 2 * q.K + 16 > q.bounds.end;
       if constexpr (THREADS == kQThreads)
         smooth_quantize_token_cached<THREADS, CHUNKS, ALIGNED>(q.x, m, q.K, q.K_pad, q.ldx, q.inv_smooth, q.static_scale, q.act_idx,
-                                                      q.act_scale, q.vec == 2);
+                                                      q.act_scale, q.vec == 2, edge, q.bounds);
       else
         smooth_quantize_token_words<THREADS, CHUNKS, OUT, ALIGNED>(q.x, m, q.K, q.K_pad, q.ldx, q.inv_smooth, q.static_scale,
-                                                          q.act_idx, q.act_scale, q.vec == 2);
+                                                          q.act_idx, q.act_scale, q.vec == 2, edge, q.bounds);
       return;
     }
   }
@@ -528,6 +543,7 @@ lcd_status launch_quantize_form(const lcd_act_problem* probs, int count, int out
     q.K = a.K;
     q.K_pad = (long long)round_up_u64((uint64_t)a.K, kTileK);
     q.ldx = a.ldx;
+    q.bounds = {reinterpret_cast<uintptr_t>(q.x), reinterpret_cast<uintptr_t>(q.x + (a.M - 1) * a.ldx + a.K)};
     q.cta0 = (int)a.M;          // (the token count until the launches are formed below)
     const bool others = (a.inv_smooth == nullptr || reinterpret_cast<uintptr_t>(a.inv_smooth) % 16 == 0) &&
                         (reinterpret_cast<uintptr_t>(a.act_idx) % (out_form == kOutNibbles ? 4 : 16) == 0);

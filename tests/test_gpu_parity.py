@@ -1057,3 +1057,20 @@ def test_padding_levels_of_tokens_whose_scale_overflows(M, K):
         lcd.FusedBatch([(w, x, inv_s, y)]).run()
         assert torch.equal(y, lcd.lut_linear(w, a, s))
         assert torch.allclose(y.double(), 7 * K * 32768 * s.double()[:, None].expand(M, 16), rtol=1e-6, atol=0)
+
+
+@pytest.mark.parametrize("M", [1, 3, 300])
+@pytest.mark.parametrize("K,ld_extra", [(5, 0), (17, 2), (250, 0), (2047, 1), (8193, 0)])
+def test_smooth_quantize_reads_x_only(M, K, ld_extra):
+    # the first and the last row begin and end inside a 16-byte word whose rest is not x: their columns are read one by one
+    # there (x begins at any 2-byte offset of its allocation and ends with the last row's last column)
+    x = gen.activations(3 + M + K, M, K, gen.outlier_channels(3, K, 0.01), 50.0)
+    inv_s = (1.0 / (np.abs(gen.normal(5, K)) * 3 + 0.05)).astype(np.float32)
+    q_ref, s_ref = O.smooth_quantize(x, inv_s)
+    for off in (0, 1, 3, 6, 7):
+        flat = torch.full((off + (M - 1) * (K + ld_extra) + K,), float("inf"), dtype=torch.float16, device="cuda")
+        rows = flat[off:].as_strided((M, K), (K + ld_extra, 1))
+        rows.copy_(torch.from_numpy(x))
+        a, s = lcd.smooth_quantize_act(rows, torch.from_numpy(inv_s).cuda())
+        assert np.array_equal(a.cpu().numpy(), O.pack_act(q_ref))
+        assert np.array_equal(s.cpu().numpy().view(np.uint32), s_ref.view(np.uint32))
