@@ -18,8 +18,8 @@
 // (problem, row tile, token tile, column unit), cut evenly over the CTAs, at most one per SM.  A CTA walks its piece from
 // the end to the beginning.  A tile that is cut between CTAs is finished by the CTA with the tile's last columns, which
 // reaches it last, with all its decoder warps; the others reach their part first and leave it in their slot of the
-// scratch (one int32 per output where pieces are short enough for the sum of both planes).  A CTA therefore only ever
-// waits for CTAs of smaller number, which were launched before it, and normally finds their part there already.
+// scratch (one int32 per output where rows and pieces are short enough for the sum of both planes, see tc_plan_width).  A CTA
+// therefore only ever waits for CTAs of smaller number, which were launched before it, and normally finds their part there.
 //
 // Where there are few tiles and many tokens, that one CTA reads megabits while the others have nothing to do: then the CTAs
 // of a tile are a cluster (resident together, so they may wait for one another), every one stores its part of the tokens
@@ -59,6 +59,7 @@ constexpr int kTcDecoders = 16, kTcFirstEpi = 16, kTcFirstToken = 20, kTcTokenWa
 constexpr int kTcCopyWarp = 24, kTcMmaWarp = 25, kTcLevelWarp = 26;
 constexpr int kTcThreads = 32 * 27;
 constexpr int kTcWordUnits = 32;              // column units whose sum of both planes fits one int32: 32752 * 8 * 8192 < 2^31
+constexpr int kTcExactUnits = 32;             // column units up to which either plane's sums of 4-bit levels fit 24 bits: 255 * 8 * 8192 < 2^24
 constexpr int kTcMaxParts = 17;               // CTAs that share a tile, its finisher not counted (see tc_plan_width)
 constexpr unsigned long long kTcWaitNs = 2000000000ull;
 
@@ -975,8 +976,10 @@ TcPlan tc_plan_width(const Problem* probs, int count, int nt) {
   if (most > q.units / piece) most = q.units / piece;
   const double unit_us = probs[0].bits == 4 ? (nt == 128 ? 0.88 : 0.68) : (nt <= 32 ? 0.33 : nt == 64 ? 0.35 : 0.68) * (probs[0].bits == 3 ? 1.05 : 1.0);
   const double tokens = (double)(max_m < nt ? max_m : nt);
+  const bool long_rows = max_kt > kTcExactUnits;
+  const double part_bytes = probs[0].act_bits == 4 && long_rows ? 768 : 512;      // (two planes: 5120 x 13824 at 100 tokens 25.8 -> 24.9 us)
   auto consider = [&](unsigned long long grid, int share, double parts, double fixed, double read_tokens, double drains) {
-    const double us = fixed + (double)((q.units + grid - 1) / grid) * unit_us + drains * tokens * 0.016 + parts * read_tokens * 512 / 20000;
+    const double us = fixed + (double)((q.units + grid - 1) / grid) * unit_us + drains * tokens * 0.016 + parts * read_tokens * part_bytes / 20000;
     if (q.grid == 0 || us < q.us) {
       q.us = us;
       q.grid = (int)grid;
@@ -991,7 +994,10 @@ TcPlan tc_plan_width(const Problem* probs, int count, int nt) {
       else if (s <= 4 && tiles * s <= most) consider(tiles * s, 0, s - 1, 5.5, tokens, nt > 32 ? 1.0 + 1.0 / s : 1.0);
       if (s > 1 && tiles <= (unsigned long long)tc_max_clusters(s)) consider(tiles * s, s, s - 1, 6.6, (double)(((int64_t)tokens + 8 * s - 1) / (8 * s) * 8), 1.0);
     }
-  q.words = probs[0].act_bits == 4 && (q.units + q.grid - 1) / q.grid <= kTcWordUnits ? 1 : 2;
+  // One number a part where the planes' sums fit 24 bits (255 * 8 * 8192 < 2^24): rounding their sum is then the same as rounding
+  // them apart, what whole tiles and the dense kernel do, and y does not depend on which tiles were cut.  On longer rows the
+  // planes stay apart (4096 x 11008, 2 bit, lookup alone at 48 / 16 tokens 12.5 / 10.5 us, 11.8 / 9.9 as one number).
+  q.words = probs[0].act_bits == 4 && !long_rows && (q.units + q.grid - 1) / q.grid <= kTcWordUnits ? 1 : 2;
   q.parts_bytes = (size_t)q.grid * q.words * q.nt * kTcRows * sizeof(int);
   q.flags_bytes = (size_t)round_up_u64((uint64_t)q.grid * sizeof(unsigned long long), 256);
   return q;

@@ -1074,3 +1074,40 @@ def test_smooth_quantize_reads_x_only(M, K, ld_extra):
         a, s = lcd.smooth_quantize_act(rows, torch.from_numpy(inv_s).cuda())
         assert np.array_equal(a.cpu().numpy(), O.pack_act(q_ref))
         assert np.array_equal(s.cpu().numpy().view(np.uint32), s_ref.view(np.uint32))
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("M,K,rows", [(1, 28672, (256, 72)), (12, 28672, (256, 200)), (24, 28672, (256, 200, 72)), (48, 28672, (4096,)),
+                                      (300, 28672, (256, 72)), (40, 66000, (72,)), (1100, 28672, (2048,)), (300, 8192, (256, 72))])
+def test_sums_beyond_24_bits_are_the_same_everywhere(bits, M, K, rows):
+    # one-signed levels and centroids near the top of their range: the planes' sums take more than 24 bits (up to 8192 columns they
+    # cannot), and every kernel and cut (register tables, tensor memory with tiles whole, shared and in parts, the dense kernel;
+    # alone and in a group) returns the same: each plane rounded, 256 times the one plus the other, times the scales
+    rng = np.random.default_rng(bits + M)
+    x = torch.from_numpy(rng.uniform(0.93, 1.0, (M, K)).astype(np.float16)).cuda()
+    a, s = lcd.smooth_quantize_act(x, None)
+    q = torch.from_numpy(O.unpack_act(a.cpu().numpy(), K)).cuda().double()
+    items, expected = [], []
+    for N in rows:
+        cb = np.sort(rng.uniform(0.8, 0.999, (N, 1 << bits)), axis=1).astype(np.float16)
+        idx = rng.integers(0, 1 << bits, (N, K), dtype=np.uint8)
+        w = lcd.PackedWeights(lcd.pack_weights(idx, cb, bits))
+        fixed = torch.from_numpy(np.rint(cb.astype(np.float64) * 2.0 ** 15)).cuda()        # 16-bit fixed point, all rows below 2^0
+        fixed = torch.gather(fixed, 1, torch.from_numpy(idx).cuda().long())
+        high = torch.floor(fixed / 256)
+        H, L = q @ high.T, q @ (fixed - 256 * high).T                                      # whole numbers below 2^53: exact
+        assert (H.max() > 2 ** 24) == (K > 8192)
+        expected.append((H.float() * 256 + L.float()) * (s[:, None] * 2.0 ** -15))
+        items.append((w, x, None, torch.empty((M, N), dtype=torch.float32, device="cuda")))
+    algos = [lcd.ALGO_REGISTER_LUT, lcd.ALGO_TC_LUT] if M <= 16 else [lcd.ALGO_AUTO, lcd.ALGO_DENSE_TC]
+    for (w, _, _, y), e in zip(items, expected):
+        for algo in algos:
+            assert torch.equal(lcd.lut_linear(w, a, s, algo=algo), e), algo
+    if M <= 16:
+        lcd.LinearBatch([(w, a, s, y) for w, _, _, y in items], algo=lcd.ALGO_TC_LUT).run()
+        for (_, _, _, y), e in zip(items, expected):
+            assert torch.equal(y, e)
+            y.fill_(0)
+    lcd.FusedBatch(items, algo=lcd.ALGO_REGISTER_LUT if M <= 16 else lcd.ALGO_AUTO).run()
+    for (_, _, _, y), e in zip(items, expected):
+        assert torch.equal(y, e)
