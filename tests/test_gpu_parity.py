@@ -1111,3 +1111,9 @@ def test_sums_beyond_24_bits_are_the_same_everywhere(bits, M, K, rows):
     lcd.FusedBatch(items, algo=lcd.ALGO_REGISTER_LUT if M <= 16 else lcd.ALGO_AUTO).run()
     for (_, _, _, y), e in zip(items, expected):
         assert torch.equal(y, e)
+
+
+@pytest.mark.parametrize("N,K,C,ld_extra", [(3, 1023, 4, 0), (3, 1025, 4, 1), (5, 2047, 8, 0), (4, 2049, 10, 0), (2, 20011, 2, 5), (2, 70001, 4, 0), (2, 65281, 3, 0)])
+def test_reclassify_rows_at_any_alignment(N, K, C, ld_extra):
+    # runs of weights a thread takes at once and their ends; more than 255 weights a thread, where the packed counts are emptied
+    test_reclassify_matches_oracle(N, K, C, ld_extra)
