@@ -24,9 +24,9 @@
 // Where there are few tiles and many tokens, that one CTA reads megabits while the others have nothing to do: then the CTAs
 // of a tile are a cluster (resident together, so they may wait for one another), every one stores its part of the tokens
 // that are not its own and, after the cluster's barrier, finishes its own from the other CTAs' parts (4096 x 11008, 2 bit,
-// 48 tokens, transformation to y: 16.9 us with one finisher, 15.1 so; 512 x 14336 at 16 tokens 13.2 and 11.0; 2048 x 11008
-// at 32 tokens 16.7 and 13.6).  With few
-// tokens the one finisher is as fast; the launcher's estimate decides (tc_plan_width).
+// 48 tokens, transformation to y: 16.9 us with one finisher, 15.1 so, parts of one number both; 512 x 14336 at 16 tokens
+// 13.2 and 11.0; 2048 x 11008 at 32 tokens 16.7 and 13.6).  With few tokens the one finisher is as fast; the launcher's
+// estimate decides (tc_plan_width).
 //
 // Layout.  An item of the index area (16 rows x 256 columns, lane 4g + t of a tile holds row g, column quarter t) is
 // loaded as it lies; the 16x128b form of tcgen05.st wants exactly that distribution: lane 4g + t writes word t of

@@ -86,12 +86,12 @@ __device__ __forceinline__ void store_level1(uint8_t* row, int64_t k, uint32_t a
 }
 
 // Columns k .. k + 7 of a row that ends at column K (zeros past it), k a multiple of 8.  ALIGNED: all rows start on 16 bytes and
-// K is a multiple of 8 (instances of their own: with both ways in one kernel such rows took 4 to 20 % longer: 2048 x 5120
+// K is a multiple of 8 (instances of their own: with both ways in one kernel such rows took 4 to 12 % longer: 2048 x 5120
 // 9.05 us, 8.70 apart; 2048 x 11008 18.6 and 16.5; 1 x 4096 2.34 and 2.20).  aligned: the row starts on 16 bytes.
 // Any other row is read in the same 16-byte words and shifted: word i of the result is taken from words q + i and q + i + 1
 // of the two it lies in (its neighbour loads the second one too, from L1).  Both hold at least one of the row's values.  So
 // such rows too are read once, eight columns a thread, all loads in flight together (333 x 5001, from x to y of a 5003-row
-// layer: 30.6 us with two passes over single columns, 27.3 so).  The words hold columns of the neighbouring rows too.  edge:
+// layer: 30.6 us with two passes over single columns, 27.6 so).  The words hold columns of the neighbouring rows too.  edge:
 // they may also hold what lies before or behind the caller's x, at the first and the last row; there those columns are read one
 // by one.
 struct XBounds {

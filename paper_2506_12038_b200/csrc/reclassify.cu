@@ -41,9 +41,9 @@ __global__ void __launch_bounds__(kRcThreads) reclassify_kernel(const uint8_t* _
   // and arrivals from either side are counted, the arrivals' centroid differences added at the end from the counts: up to
   // four clusters in bytes of three registers, emptied in time into a count per lane (4 bits of cluster and kind), up to
   // eight in shared memory.  With more the counts' space would halve the CTAs on an SM: there the differences are added
-  // weight by weight and only the members are counted.  The shared-memory pipe bounds the kernel: a weight takes six passes
-  // through it here (thirteen when a slot of sixteen bytes held an error-free binary32 pair and the counts).  4096 x 4096,
-  // 4 / 8 / 16 clusters: 31 / 45 / 58 us (43 / 56 / 89 then).
+  // weight by weight and only the members are counted.  The load/store data pipe is what the kernel fills most (70 % busy, 55 %
+  // of the warps resident at 42 registers): a weight takes six passes through it here (thirteen when a slot of sixteen bytes
+  // held an error-free binary32 pair and the counts).  4096 x 4096, 4 / 8 / 16 clusters: 32.5 / 47 / 58 us (43 / 56 / 89 then).
   extern __shared__ double s_sum[];                                             // [CMAX][kRcThreads]
   constexpr bool kPacked = CMAX <= 4, kSteps = CMAX > 8;
   int* s_count = reinterpret_cast<int*>(s_sum + CMAX * kRcThreads);             // [1 or 3][CMAX][kRcThreads]: members, from left, from right

@@ -56,9 +56,10 @@ __global__ void __launch_bounds__(256) smoothing_factors_kernel(const __half* x,
 
 // partial[g][t] = sum_k (x - level * s_q * s)^2 of token t under candidate g, kTokens tokens a CTA (a factor is loaded and
 // widened once for all of them); the CTA that arrives last averages, picks the first smallest candidate and writes its
-// factors.  Bound by instruction issue: per element and candidate two multiplications, clip, rounding by one addition, one
-// conversion and four binary64 operations (11 M elements of 4096 columns, 128 tokens, 21 candidates: 24.5 us for the
-// whole search; 56 with a division per element and pass, three conversions and a kernel each for maxima, factors and pick).
+// factors.  Per element and candidate two multiplications, clip, rounding by one addition, one conversion and four binary64
+// operations, 25 instructions in all.  128 tokens, 4096 columns, 21 candidates, 11 M of them: 8 us of issue, but 22 us alone
+// (issue 50 %, half of the warps resident, no pipe above 24 %: the loads' latency; 0.9 waves of CTAs), 24.2 for the whole
+// search (56 with a division per element and pass, three conversions and a kernel each for maxima, factors and pick).
 constexpr int kTokens = 4;
 // PER_SM: CTAs that an SM must hold.  Four leave all the registers the compiler wants (56); a grid that does not fit four times
 // into the SMs is 10 % faster with five (512 tokens x 14336 columns x 33 candidates 262 -> 237 us), a smaller one 8 % slower
