@@ -255,7 +255,7 @@ def lut_linear(w: PackedWeights, act_idx, act_scale, y=None, algo: int = ALGO_AU
         lut_linear_workspace_bytes(w, act_idx.shape[0], algo)
         y_out = fn(w.dev, w._hdr_addr, w.N, w._workspace_bytes, act_idx, act_scale, y, algo, workspace, status_word, stream)
     if y_out.__class__ is int:
-        _check(y_out, "lcd_lut_linear")
+        _check(y_out, "lcd_lut_linear_act8" if act_idx.dtype.is_signed else "lcd_lut_linear")
     return y_out
 
 

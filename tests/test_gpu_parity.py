@@ -1117,3 +1117,12 @@ def test_sums_beyond_24_bits_are_the_same_everywhere(bits, M, K, rows):
 def test_reclassify_rows_at_any_alignment(N, K, C, ld_extra):
     # runs of weights a thread takes at once and their ends; more than 255 weights a thread, where the packed counts are emptied
     test_reclassify_matches_oracle(N, K, C, ld_extra)
+
+
+@pytest.mark.parametrize("act_bits,name", [(4, "lcd_lut_linear:"), (8, "lcd_lut_linear_act8:")])
+def test_lookup_errors_name_the_call(act_bits, name):
+    L = gen.random_case(seed=1, N=16, K=300, bits=2, M=20)
+    w = lcd.PackedWeights(lcd.pack_weights(L.idx, L.codebook, 2))
+    a, s = lcd.smooth_quantize_act(torch.from_numpy(L.x).cuda(), None, act_bits=act_bits)
+    with pytest.raises(lcd.LcdError, match=name):
+        lcd.lut_linear(w, a, s, y=torch.empty((20, 8), device="cuda"))          # rows of y shorter than N
