@@ -326,7 +326,7 @@ def dbci(weights, max_centroids: int = 4096, want_labels: bool = True, stream=No
     cents = torch.empty((max_centroids,), dtype=torch.float32, device=w.device)
     labels = torch.empty((n,), dtype=torch.int32, device=w.device) if want_labels else None
     srt = torch.empty((n,), dtype=torch.float32, device=w.device)
-    res = torch.zeros((ctypes.sizeof(DbciResult),), dtype=torch.uint8, device=w.device)
+    res = torch.empty((ctypes.sizeof(DbciResult),), dtype=torch.uint8, device=w.device)
     _check(lib.lcd_dbci(c_void_p(w.data_ptr()), n, c_void_p(ws.data_ptr()), need, c_void_p(cents.data_ptr()),
                         max_centroids, c_void_p(labels.data_ptr()) if labels is not None else None,
                         c_void_p(srt.data_ptr()), c_void_p(res.data_ptr()), _stream_ptr()), "lcd_dbci")

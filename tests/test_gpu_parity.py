@@ -1126,3 +1126,42 @@ def test_lookup_errors_name_the_call(act_bits, name):
     a, s = lcd.smooth_quantize_act(torch.from_numpy(L.x).cuda(), None, act_bits=act_bits)
     with pytest.raises(lcd.LcdError, match=name):
         lcd.lut_linear(w, a, s, y=torch.empty((20, 8), device="cuda"))          # rows of y shorter than N
+
+
+def _sort_inputs(kind, n, rng):
+    w = rng.normal(0, 0.02, n)
+    if kind == "bf16":                       # few values, each many times
+        return torch.from_numpy(w.astype(np.float32)).bfloat16().float().numpy()
+    if kind == "levels":                     # buckets of one value
+        w = (np.arange(n) % 8 - 3.5) * 0.02
+    elif kind == "clumps":                   # many keys in few fine bins: the general sort
+        w = (np.arange(n) % 8 - 3.5) * 0.02 * (1 + 1e-4 * rng.normal(0, 1, n))
+    elif kind == "pruned":                   # zeros of either sign keep their order
+        w = w * (rng.uniform(0, 1, n) < 0.5)
+    elif kind == "infinite":                 # a bucket that spans every order of magnitude
+        w[::max(1, n // 100)] = np.inf
+        w[1::max(2, n // 50)] = -np.inf
+    elif kind == "wide":
+        w = np.exp(10 * rng.normal(0, 1, n)) * rng.choice([-1.0, 1.0], n)
+    elif kind == "constant":
+        w = np.full(n, 0.25)
+    return w.astype(np.float32)
+
+
+# one CTA's most keys and the first array of several buckets; a tile of the partition and one more
+@pytest.mark.parametrize("n", [2, 33, 16384, 16385, 20481, 300_007])
+@pytest.mark.parametrize("kind", ["gauss", "bf16", "levels", "clumps", "pruned", "infinite", "wide", "constant"])
+def test_dbci_sort_is_the_stable_sort_bit_for_bit(kind, n):
+    w = _sort_inputs(kind, n, np.random.default_rng(n))
+    r = lcd.dbci(torch.from_numpy(w).cuda())
+    want = np.sort(w, kind="stable")         # zeros of either sign are equal there too
+    assert np.array_equal(r["sorted"].cpu().numpy().view(np.int32), want.view(np.int32))
+
+
+@pytest.mark.parametrize("n", [4_000_003, 50_400_000])      # the partition's wide tiles; beyond what the own sort takes
+def test_dbci_sort_of_large_arrays(n):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    w = torch.randn(n, generator=g, device="cuda") * 0.02
+    r = lcd.dbci(w)
+    assert torch.equal(r["sorted"], torch.sort(w).values)
