@@ -6,6 +6,8 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "common.h"
 #include "device_util.h"
 
@@ -24,7 +26,7 @@ struct AlphaList {
 // would otherwise divide out once per token.  CTA 0 clears the error kernel's arrival counter.  x and wmax are read with
 // ordinary loads (no __restrict__): this kernel may be running while an earlier one still writes them.  It does not let the next
 // one in early, which reads the factors with __ldg, for data that nobody writes while the reading kernel runs (an early
-// start gains nothing, 24.3 us either way; ordinary loads there take 26.2, __ldcg 28.0).
+// start gains nothing; ordinary loads there cost 8 % of the search, __ldcg 15).
 __global__ void __launch_bounds__(256) smoothing_factors_kernel(const __half* x, int64_t T, int64_t K, int64_t ldx,
                                                                 const float* wmax, const AlphaList alphas,
                                                                 float* __restrict__ s, float* __restrict__ inv, unsigned* __restrict__ arrived) {
@@ -56,15 +58,15 @@ __global__ void __launch_bounds__(256) smoothing_factors_kernel(const __half* x,
 
 // partial[g][t] = sum_k (x - level * s_q * s)^2 of token t under candidate g, kTokens tokens a CTA (a factor is loaded and
 // widened once for all of them); the CTA that arrives last averages, picks the first smallest candidate and writes its
-// factors.  Per element and candidate two multiplications, clip, rounding by one addition, one conversion and four binary64
-// operations, 25 instructions in all.  128 tokens, 4096 columns, 21 candidates, 11 M of them: 8 us of issue, but 22 us alone
-// (issue 50 %, half of the warps resident, no pipe above 24 %: the loads' latency; 0.9 waves of CTAs), 24.2 for the whole
-// search (56 with a division per element and pass, three conversions and a kernel each for maxima, factors and pick).
+// factors.  Per element and candidate two multiplications, rounding by one addition, one conversion and four binary64
+// operations, 22 instructions in all with the pass that finds the tokens' maxima.  What bounds it is issue and the half-rate
+// integer and minimum pipe: 128 tokens, 4096 columns, 21 candidates, 11 M of them: 22.1 us for the whole search (24.1 with a clip, two
+// minimum operations, and an integer addition more; 512 x 14336 x 33: 205 and 236), of which the factors' kernel takes 6 and
+// starting, the last CTA's means and the copy of the winner's factors 5.
 constexpr int kTokens = 4;
-// PER_SM: CTAs that an SM must hold.  Four leave all the registers the compiler wants (56); a grid that does not fit four times
-// into the SMs is 10 % faster with five (512 tokens x 14336 columns x 33 candidates 262 -> 237 us), a smaller one 8 % slower
-// (128 x 4096 x 9: 15.0, 16.3).  Single columns a step (rows at odd addresses) want 79 registers (200 x 5003 x 11: 35.7 us,
-// 38.3 with four CTAs).
+// PER_SM: CTAs that an SM must hold.  Four leave all the registers the compiler wants; a grid that does not fit four times
+// into the SMs is faster with five (512 tokens x 14336 columns x 33 candidates 221 -> 205 us, six 208; 128 x 4096 x 21: 24.4, 22.1
+// and 22.9), a smaller one is not.  Single columns a step (rows at odd addresses) take what they want (200 x 5003 x 11: 31.7 us).
 template <bool VEC, int PER_SM>
 __global__ void __launch_bounds__(256, PER_SM) smoothing_error_kernel(const __half* __restrict__ x, int64_t T, int64_t K, int64_t ldx, int G,
                                                               const float* __restrict__ s, const float* __restrict__ inv,
@@ -125,38 +127,44 @@ __global__ void __launch_bounds__(256, PER_SM) smoothing_error_kernel(const __ha
   __syncthreads();
   float r[kTokens];
   double sq[kTokens], err[kTokens] = {};
+  bool finite = true;
 #pragma unroll
   for (int t = 0; t < kTokens; ++t) {
     float A = 0.0f;
 #pragma unroll
     for (int w = 0; w < 8; ++w) A = fmaxf(A, s_f[t][w]);
+    finite = finite && A < 3e38f;
     r[t] = A > 0.0f ? __fdiv_rn(127.0f, A) : 0.0f;
     sq[t] = A > 0.0f ? (double)__fdiv_rn(A, 127.0f) : 1.0;
   }
-  for (int64_t k = (int64_t)tid * W; k < K; k += 256 * W) {
-    float iv[W], sv[W];
-    columns(ig, k, iv);
-    columns(sg, k, sv);
-    double sd[W];
+  // |x / s| * (127 / A) is at most 127 and a rounding: clipping changes nothing where A is finite
+  auto errors = [&](auto clip) {
+    for (int64_t k = (int64_t)tid * W; k < K; k += 256 * W) {
+      float iv[W], sv[W];
+      columns(ig, k, iv);
+      columns(sg, k, sv);
+      double sd[W];
 #pragma unroll
-    for (int i = 0; i < W; ++i) sd[i] = (double)sv[i];
+      for (int i = 0; i < W; ++i) sd[i] = (double)sv[i];
 #pragma unroll
-    for (int t = 0; t < kTokens; ++t)
-      if (t < n_tok) {
-        float xv[W];
-        activations(t, k, xv);
+      for (int t = 0; t < kTokens; ++t)
+        if (t < n_tok) {
+          float xv[W];
+          activations(t, k, xv);
 #pragma unroll
-        for (int i = 0; i < W; ++i) {
-          // clipped first (the bounds are integers: the same level), then rounded half to even by one addition, which leaves
-          // the level in the sum's low bits; the same bits under the exponent of 2^52 are the level as a binary64 number
-          const float u = fminf(fmaxf(__fmul_rn(__fmul_rn(xv[i], iv[i]), r[t]), -128.0f), 127.0f);
-          const int bits = (int)(__float_as_uint(__fadd_rn(u, 12582912.0f)) + (0x80000000u - 0x4b400000u));      // level + 2^31
-          const double lev = __hiloint2double(0x43300000, bits) - 4503601774854144.0;                            // 2^52 + 2^31
-          const double d = (double)xv[i] - lev * sq[t] * sd[i];
-          err[t] += d * d;
+          for (int i = 0; i < W; ++i) {
+            // clipped first (the bounds are integers: the same level), then rounded half to even by one addition, which leaves
+            // the level in the sum's low bits; under the exponent of 2^52 the sum's bits are the level and a constant, binary64
+            const float v = __fmul_rn(__fmul_rn(xv[i], iv[i]), r[t]), u = decltype(clip)::value ? fminf(fmaxf(v, -128.0f), 127.0f) : v;
+            const int bits = (int)__float_as_uint(__fadd_rn(u, 12582912.0f));                 // 0x4b400000 + level
+            const double lev = __hiloint2double(0x43300000, bits) - (4503599627370496.0 + 1262485504.0);
+            const double d = (double)xv[i] - lev * sq[t] * sd[i];
+            err[t] += d * d;
+          }
         }
-      }
-  }
+    }
+  };
+  if (finite) errors(std::false_type()); else errors(std::true_type());
 #pragma unroll
   for (int t = 0; t < kTokens; ++t) {
 #pragma unroll

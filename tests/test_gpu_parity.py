@@ -811,6 +811,14 @@ def test_smoothing_search_matches_oracle(T, K, ld_extra):
     assert np.array_equal(a.cpu().numpy(), O.pad_act8(q_ref)) and np.array_equal(sc.cpu().numpy(), s_q_ref)
 
 
+def test_smoothing_search_with_an_infinite_activation():
+    # the token's maximum is infinite: no candidate has a finite error, the first one is taken
+    x = torch.randn(8, 512, device="cuda").half()
+    x[3, 100] = float("inf")
+    best, mse, inv = lcd.smoothing_search(x, torch.full((512,), 0.08, device="cuda"), [0.0, 0.5, 1.0])
+    assert not torch.isfinite(mse).any() and best.item() == 0
+
+
 # ------------------------------------------------------------------------------- reclassification (offline)
 @pytest.mark.parametrize("N,K,C,ld_extra", [(64, 4096, 4, 0), (33, 1000, 8, 8), (5, 250, 5, 3), (3, 7, 1, 0), (2, 300, 16, 0)])
 def test_reclassify_matches_oracle(N, K, C, ld_extra):
