@@ -28,6 +28,23 @@ __global__ void __launch_bounds__(kRcThreads) reclassify_kernel(const uint8_t* _
   __shared__ float2 s_gap[CMAX];            // half-gaps (C_i - C_{i-1}) / 2 and (C_{i+1} - C_i) / 2, infinite at the edges
   const int64_t n = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint8_t* ir = idx + n * K;
+  const float* dr = delta_w + n * ldw;
+  uint8_t* outr = new_idx + n * K;
+  // 16 weights per thread and step: one 16-byte index load, four 16-byte update loads, one 16-byte store.  Above eight clusters,
+  // where shared memory holds few CTAs an SM, the first step's loads are on their way before the thresholds are made (4096 x 4096,
+  // 10 / 16 clusters 55.0 / 59.4 -> 51.0 / 55.4 us, 777 x 8192, 10 clusters 24.7 -> 21.9); with fewer the registers that
+  // takes cost as much (8192 x 8192, 4 clusters 99.2 -> 102.5).
+  constexpr bool kAhead = CMAX > 8;
+  uint4 iv = make_uint4(0u, 0u, 0u, 0u);
+  float4 d[4];
+  auto load = [&](int64_t k) {
+    if (k >= K) return;
+    iv = __ldg(reinterpret_cast<const uint4*>(ir + k));
+#pragma unroll
+    for (int q = 0; q < 4; ++q) d[q] = __ldg(reinterpret_cast<const float4*>(dr + k + 4 * q));
+  };
+  if (kAhead && vec) load((int64_t)tid * 16);
   if (tid < 12) s_total[tid >> 2][tid & 3] = 0;
   if (tid < C) s_c[tid] = __half2float(__ushort_as_half(codebook[n * C + tid]));
   __syncthreads();
@@ -43,7 +60,7 @@ __global__ void __launch_bounds__(kRcThreads) reclassify_kernel(const uint8_t* _
   // eight in shared memory.  With more the counts' space would halve the CTAs on an SM: there the differences are added
   // weight by weight and only the members are counted.  The load/store data pipe is what the kernel fills most (70 % busy, 55 %
   // of the warps resident at 42 registers): a weight takes six passes through it here (thirteen when a slot of sixteen bytes
-  // held an error-free binary32 pair and the counts).  4096 x 4096, 4 / 8 / 16 clusters: 32.5 / 47 / 58 us (43 / 56 / 89 then).
+  // held an error-free binary32 pair and the counts).  4096 x 4096, 4 / 8 / 16 clusters: 32.8 / 47 / 55 us (43 / 56 / 89 then).
   extern __shared__ double s_sum[];                                             // [CMAX][kRcThreads]
   constexpr bool kPacked = CMAX <= 4, kSteps = CMAX > 8;
   int* s_count = reinterpret_cast<int*>(s_sum + CMAX * kRcThreads);             // [1 or 3][CMAX][kRcThreads]: members, from left, from right
@@ -59,9 +76,6 @@ __global__ void __launch_bounds__(kRcThreads) reclassify_kernel(const uint8_t* _
     s_step[tid] = make_double2((tid > 0 && tid < C) ? (double)s_c[tid] - (double)s_c[tid - 1] : 0.0,
                                (tid < C - 1) ? (double)s_c[tid] - (double)s_c[tid + 1] : 0.0);
   __syncthreads();
-  const uint8_t* ir = idx + n * K;
-  const float* dr = delta_w + n * ldw;
-  uint8_t* outr = new_idx + n * K;
   uint32_t members = 0, from_left = 0, from_right = 0;
   // An index is reduced to the table size CMAX before it addresses shared memory, so a byte >= C (the caller's
   // error) cannot reach outside the slots: such a weight keeps its reduced index and is counted in no cluster.
@@ -104,16 +118,13 @@ __global__ void __launch_bounds__(kRcThreads) reclassify_kernel(const uint8_t* _
     }
   };
   int step = 0;
-  if (vec) {      // 16 weights per thread and step: one 16-byte index load, four 16-byte update loads, one 16-byte store
+  if (vec) {
     for (int64_t k0 = 0; k0 < K; k0 += (int64_t)kRcThreads * 16) {
       if (kPacked && ++step == 16) { empty(); step = 1; }           // 240 weights since: no byte has overflowed
       const int64_t k = k0 + (int64_t)tid * 16;
       if (k >= K) continue;
-      const uint4 iv = __ldg(reinterpret_cast<const uint4*>(ir + k));
+      if (!kAhead || k0 > 0) load(k);
       const uint32_t iw[4] = {iv.x, iv.y, iv.z, iv.w};
-      float4 d[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) d[q] = __ldg(reinterpret_cast<const float4*>(dr + k + 4 * q));
       uint32_t ow[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
