@@ -294,27 +294,30 @@ __global__ void __launch_bounds__(kMapThreads) sort_map_kernel(long long n, int 
 }
 
 // A tile of 1024 * ITEMS keys at a time: its keys are put in bucket order in shared memory (a key's rank in its bucket is the
-// result of the atomic that counts it), one reservation per bucket in the output, and written out in runs.  The next tile's
-// keys are asked for before the writes.
+// result of the atomic that counts it), one reservation per bucket in the output, and written out in runs, whose beginnings are
+// bits of a map of the tile (a bucket's number beside every key would be a store and a load more).  The next tile's keys are
+// asked for before the writes.
 constexpr int kPartThreads = 1024;
 template <int ITEMS>
-constexpr int partition_smem() { return kBins * 4 + kFineMax / 4 + kMaxBuckets * 8 + kPartThreads * ITEMS * 6; }
+constexpr int partition_smem() { return kBins * 4 + kFineMax / 4 + kMaxBuckets * 8 + kPartThreads * ITEMS * 4 + kPartThreads * ITEMS / 32 * 8; }
 template <int ITEMS>
 __global__ void __launch_bounds__(kPartThreads, 1) sort_partition_kernel(const unsigned* __restrict__ in, long long n, const SortState* st,
                                                                          const unsigned* table_g, const unsigned* begins_g,
                                                                          unsigned* cursor, unsigned* __restrict__ out) {
-  constexpr int TILE = kPartThreads * ITEMS;
+  constexpr int TILE = kPartThreads * ITEMS, kLong = 128;
   extern __shared__ __align__(16) unsigned sm[];
   __shared__ unsigned part[kPartThreads / 32 + 1];
+  __shared__ uint2 long_runs[TILE / kLong];
+  __shared__ int n_long;
   wait_for_last_kernel();
   let_next_kernel_start();
   if (st->general) return;
   unsigned* at = sm;                                      // [kMaxBuckets] counts, then first place in the tile
-  unsigned* delta = at + kMaxBuckets;                     // [kMaxBuckets] place in the output - place in the tile
+  unsigned* delta = at + kMaxBuckets;                     // [kMaxBuckets] of the tile's runs: place in the output - place in the tile
   unsigned* table = delta + kMaxBuckets;                  // [kBins]
   unsigned* begins = table + kBins;                       // [kFineMax / 16]
   unsigned* keys = begins + kFineMax / 16;                // [TILE]
-  unsigned short* ids = reinterpret_cast<unsigned short*>(keys + TILE);               // [TILE]
+  uint2* runs = reinterpret_cast<uint2*>(keys + TILE);    // [TILE / 32] of 32 places: the first one's run, a bit for each place that begins one
   const int tid = threadIdx.x;
   const FineMap map(st);
   const bool many = st->n_buckets > kMaxBuckets / 2;
@@ -336,6 +339,8 @@ __global__ void __launch_bounds__(kPartThreads, 1) sort_partition_kernel(const u
     reinterpret_cast<uint4*>(at)[tid] = make_uint4(0u, 0u, 0u, 0u);
     if (many) reinterpret_cast<uint4*>(at)[kPartThreads + tid] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
+    if (tid < TILE / 32) runs[tid] = make_uint2(0u, 0u);          // (the last tile's have been read)
+    if (tid == 0) n_long = 0;
     unsigned place[ITEMS];                                // bucket << 16 | rank
     auto classify = [&](auto whole) {
 #pragma unroll
@@ -353,41 +358,65 @@ __global__ void __launch_bounds__(kPartThreads, 1) sort_partition_kernel(const u
     auto reserve = [&](auto bpt) {
       constexpr int BPT = decltype(bpt)::value;
       unsigned g[BPT], e = 0;
+      bool had[BPT];
 #pragma unroll
       for (int q = 0; q < BPT; ++q) {
         const unsigned c = at[q * kPartThreads + tid];
+        had[q] = c != 0;
         if (c) g[q] = atomicAdd(cursor + q * kPartThreads + tid, c);
       }
+      // (counts of at most TILE keys in the low half, buckets with keys in the upper one)
       uint4* mine = reinterpret_cast<uint4*>(at) + tid * (BPT / 4);
 #pragma unroll
       for (int q = 0; q < BPT / 4; ++q) {
         const uint4 w = mine[q];
-        e += w.x + w.y + w.z + w.w;
+        e += w.x + w.y + w.z + w.w + (((w.x != 0) + (w.y != 0) + (w.z != 0) + (w.w != 0)) << 16);
       }
       e = block_exclusive<kPartThreads / 32>(e, part);
 #pragma unroll
       for (int q = 0; q < BPT / 4; ++q) {
-        const uint4 w = mine[q];
-        mine[q] = make_uint4(e, e + w.x, e + w.x + w.y, e + w.x + w.y + w.z);
-        e += w.x + w.y + w.z + w.w;
+        uint4 w = mine[q];
+        // a bucket's first place in the tile and its run's number; the words of 32 places whose first one it has
+        auto place_run = [&](unsigned& w1) {
+          const unsigned first = e & 0xffffu, run = e >> 16, c = w1;
+          w1 = e;
+          if (c) {
+            atomicOr(&runs[first >> 5].y, 1u << (first & 31u));
+            if (c >= kLong) long_runs[atomicAdd(&n_long, 1)] = make_uint2(first | c << 16, run);
+            else
+              for (unsigned word = (first + 31u) >> 5; 32u * word < first + c; ++word) runs[word].x = run;
+            e += c + 0x10000u;
+          }
+        };
+        place_run(w.x); place_run(w.y); place_run(w.z); place_run(w.w);
+        mine[q] = w;
       }
       __syncthreads();
 #pragma unroll
-      for (int q = 0; q < BPT; ++q) delta[q * kPartThreads + tid] = g[q] - at[q * kPartThreads + tid];      // (of a bucket without keys: not read)
+      for (int q = 0; q < BPT; ++q) {
+        const unsigned w = at[q * kPartThreads + tid];
+        if (had[q]) delta[w >> 16] = g[q] - (w & 0xffffu);
+      }
+      for (int i = tid >> 5; i < n_long; i += kPartThreads / 32) {        // a warp for each (sorted inputs have nothing else)
+        const unsigned first = long_runs[i].x & 0xffffu, end = first + (long_runs[i].x >> 16);
+        for (unsigned word = ((first + 31u) >> 5) + (tid & 31u); 32u * word < end; word += 32u) runs[word].x = long_runs[i].y;
+      }
     };
     if (many) reserve(std::integral_constant<int, kMaxBuckets / kPartThreads>());
     else reserve(std::integral_constant<int, kMaxBuckets / 2 / kPartThreads>());
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j)
       if (j * kPartThreads + tid < left) {
-        const unsigned b = place[j] >> 16, to = at[b] + (place[j] & 0xffffu);
-        keys[to] = v[j];
-        ids[to] = (unsigned short)b;
+        keys[(at[place[j] >> 16] + place[j]) & 0xffffu] = v[j];
       }
     load(t0 + (long long)gridDim.x * TILE);
     __syncthreads();
+    // a warp's 32 places lie in one word: the runs that begin after the first place, counted
 #pragma unroll 4
-    for (int i = tid; i < left; i += kPartThreads) out[delta[ids[i]] + (unsigned)i] = keys[i];
+    for (int i = tid; i < left; i += kPartThreads) {
+      const uint2 w = runs[i >> 5];
+      out[delta[w.x + (unsigned)__popc(w.y & (0xffffffffu >> (31 - (i & 31))) & ~1u)] + (unsigned)i] = keys[i];
+    }
   }
 }
 
