@@ -473,7 +473,7 @@ template <bool SINGLE>
 __global__ void __launch_bounds__(kSortThreads, 2) sort_buckets_kernel(const unsigned* __restrict__ in, long long n, SortState* st,
                                                                        const unsigned* first, unsigned* x) {
   extern __shared__ __align__(16) unsigned sm[];
-  __shared__ unsigned part[kSortThreads / 32 + 1], lo_s[kSortThreads / 32], hi_s[kSortThreads / 32];
+  __shared__ unsigned part[kSortThreads / 32 + 1], lo_s[kSortThreads / 32], hi_s[kSortThreads / 32], most_s[kSortThreads / 32];
   unsigned* keys = sm;                              // [kCap + 16]
   unsigned* bins = sm + kCap + 16;                  // [kParts / 2] two 16-bit counts a word, then two first places
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -610,9 +610,10 @@ __global__ void __launch_bounds__(kSortThreads, 2) sort_buckets_kernel(const uns
     };
     if (value) count(by_value); else count(by_bits);
     most = exact ? 0u : __reduce_max_sync(0xffffffffu, most);
-    if (lane == 0) hi_s[warp] = most;
+    // (not hi_s: a warp without keys comes here while others still read that, no barrier lies between on the usual way)
+    if (lane == 0) most_s[warp] = most;
     __syncthreads();
-    most = __reduce_max_sync(0xffffffffu, hi_s[lane & (kSortThreads / 32 - 1)]);
+    most = __reduce_max_sync(0xffffffffu, most_s[lane & (kSortThreads / 32 - 1)]);
     const bool far = most >= 8, loose = most >= 1;       // parts of more than eight keys, of more than one
     {
       // first places: 32 parts a thread, read twice (their counts beside the keys and ranks would not fit the registers)

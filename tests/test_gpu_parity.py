@@ -1173,3 +1173,12 @@ def test_dbci_sort_of_large_arrays(n):
     w = torch.randn(n, generator=g, device="cuda") * 0.02
     r = lcd.dbci(w)
     assert torch.equal(r["sorted"], torch.sort(w).values)
+
+
+@pytest.mark.parametrize("n", [40, 700, 16384, 20_000, 100_003])
+def test_dbci_sort_of_buckets_that_leave_warps_without_keys(n):
+    # keys of one binary order of magnitude, none of them zero: a warp without keys runs ahead of the others as far as it can
+    w = np.random.default_rng(n).uniform(0.5, 1.0, n).astype(np.float32)
+    x, want = torch.from_numpy(w).cuda(), np.sort(w).view(np.int32)
+    for _ in range(20):
+        assert np.array_equal(lcd.dbci(x)["sorted"].cpu().numpy().view(np.int32), want)
