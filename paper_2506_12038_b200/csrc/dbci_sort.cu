@@ -526,7 +526,11 @@ __global__ void __launch_bounds__(kSortThreads, 2) sort_buckets_kernel(const uns
     if (!SINGLE) {
       at = at_next;
       cnt = (int)(end_next - at_next);
-      if (cnt < 2 || cnt > kCap) cnt = 0;             // nothing to sort: one key, or one value (see above)
+      if (cnt == 1 && tid == 0) {                     // nothing to sort, but it may be the only zero of its sign
+        const unsigned v = __ldcg(x + at);
+        if (value_of(v) == 0u) atomicOr(&st->zeros, v == 0u ? 1 : 2);
+      }
+      if (cnt < 2 || cnt > kCap) cnt = 0;             // one key, or one value (see above)
     }
     const unsigned* src = SINGLE ? in : x + at;
 #pragma unroll

@@ -1182,3 +1182,23 @@ def test_dbci_sort_of_buckets_that_leave_warps_without_keys(n):
     x, want = torch.from_numpy(w).cuda(), np.sort(w).view(np.int32)
     for _ in range(20):
         assert np.array_equal(lcd.dbci(x)["sorted"].cpu().numpy().view(np.int32), want)
+
+
+def _zeros_of_one_sign_alone():
+    one = np.zeros(16500)
+    one[16401:] = 1e-4 * np.arange(1, 100)
+    for at in (0, 1000, 16400):              # the smallest key, a bucket of its own; mirrored: the largest but for the tail's
+        w = one.copy()
+        w[at] = -0.0
+        yield w
+        yield -w
+    yield np.concatenate([[0.0], np.full(20000, -0.0), np.full(10, -1.0)])
+    yield np.concatenate([np.full(20000, 0.0), [-0.0], np.full(10, 1.0)])
+
+
+def test_dbci_sort_keeps_a_single_zero_of_either_sign_in_its_place():
+    # among many zeros of the other sign: it may be the one key of its bucket
+    for w in _zeros_of_one_sign_alone():
+        w = w.astype(np.float32)
+        r = lcd.dbci(torch.from_numpy(w).cuda())
+        assert np.array_equal(r["sorted"].cpu().numpy().view(np.int32), np.sort(w, kind="stable").view(np.int32))
