@@ -467,10 +467,11 @@ __device__ __noinline__ void sort_any(unsigned* keys, int cnt) {
   __syncthreads();
 }
 
-// SINGLE: the whole array is one bucket, read from `in`; otherwise the buckets of x,
+// SINGLE: the whole array is one bucket, read from `in` (the call's first kernel: no __restrict__, its loads may not become
+// non-coherent ones, as an earlier kernel may still be writing the weights while this one starts); otherwise the buckets of x,
 // in place, the next one's keys on their way while one is sorted.
 template <bool SINGLE>
-__global__ void __launch_bounds__(kSortThreads, 2) sort_buckets_kernel(const unsigned* __restrict__ in, long long n, SortState* st,
+__global__ void __launch_bounds__(kSortThreads, 2) sort_buckets_kernel(const unsigned* in, long long n, SortState* st,
                                                                        const unsigned* first, unsigned* x) {
   extern __shared__ __align__(16) unsigned sm[];
   __shared__ unsigned part[kSortThreads / 32 + 1], lo_s[kSortThreads / 32], hi_s[kSortThreads / 32], most_s[kSortThreads / 32];
@@ -535,7 +536,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) sort_buckets_kernel(const uns
     const unsigned* src = SINGLE ? in : x + at;
 #pragma unroll
     for (int j = 0; j < kSortItems; ++j)
-      if (j * kSortThreads + tid < cnt) k[j] = SINGLE ? src[j * kSortThreads + tid] : __ldcs(src + j * kSortThreads + tid);
+      if (j * kSortThreads + tid < cnt) k[j] = __ldcs(src + j * kSortThreads + tid);
   };
   look(blockIdx.x);
   load();
@@ -658,7 +659,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) sort_buckets_kernel(const uns
     // the network's groups are whole: what lies behind the last key stays there
     const int groups = (sorted + 15) / 16;
     if (tid < 24 && sorted + tid < groups * 16 + 8) keys[spread((unsigned)(sorted + tid))] = 0xffffffffu;
-    load();
+    if (!SINGLE) load();
     __syncthreads();
     if (loose) {
       for (int round = 0;; ++round) {

@@ -1202,3 +1202,14 @@ def test_dbci_sort_keeps_a_single_zero_of_either_sign_in_its_place():
         w = w.astype(np.float32)
         r = lcd.dbci(torch.from_numpy(w).cuda())
         assert np.array_equal(r["sorted"].cpu().numpy().view(np.int32), np.sort(w, kind="stable").view(np.int32))
+
+
+@pytest.mark.parametrize("n", [1000, 16384, 16385])
+def test_dbci_of_weights_that_the_kernel_before_writes(n):
+    # the same buffer written anew before every call, whose first kernel may start while the writing one ends
+    sources = [torch.from_numpy(np.random.default_rng(s).normal(0, 0.02, n).astype(np.float32)).cuda() for s in range(4)]
+    want = [torch.sort(s).values for s in sources]
+    w = torch.empty(n, device="cuda")
+    for i in range(24):
+        torch.mul(sources[i % 4], 1.0, out=w)
+        assert torch.equal(lcd.dbci(w)["sorted"], want[i % 4])
