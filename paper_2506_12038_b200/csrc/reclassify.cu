@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(kRcThreads) reclassify_kernel(const uint8_t* _
       if (kPacked && ++step == 16) { empty(); step = 1; }           // 240 weights since: no byte has overflowed
       const int64_t k = k0 + (int64_t)tid * 16;
       if (k >= K) continue;
-      if (!kAhead) load(k);
+      if (!kAhead || k0 > 0) load(k);
       const uint32_t iw[4] = {iv.x, iv.y, iv.z, iv.w};
       uint32_t ow[4];
 #pragma unroll
@@ -135,7 +135,6 @@ __global__ void __launch_bounds__(kRcThreads) reclassify_kernel(const uint8_t* _
         ow[q] = o;
       }
       *reinterpret_cast<uint4*>(outr + k) = make_uint4(ow[0], ow[1], ow[2], ow[3]);
-      if (kAhead) load(k + (int64_t)kRcThreads * 16);
     }
   } else {
     // rows at any alignment: kRun weights' loads in flight together (one after the other, with the counts' emptying in between,
