@@ -1213,3 +1213,20 @@ def test_dbci_of_weights_that_the_kernel_before_writes(n):
     for i in range(24):
         torch.mul(sources[i % 4], 1.0, out=w)
         assert torch.equal(lcd.dbci(w)["sorted"], want[i % 4])
+
+
+@pytest.mark.parametrize("n,seeds", [(40_000, 1024), (40_000, 1026), (100_003, 3000)])
+def test_dbci_with_many_points_to_a_core(n, seeds):
+    # MinPts on either side of what a tile's window holds (1024 places): tiles without a core point, with some and with nothing else
+    rng = np.random.default_rng(n + seeds)
+    eps = 0.35 / seeds                                       # (sigma is about 0.35: most weights lie within 0.5 of zero)
+    sizes = rng.integers(1, 6 * seeds, 60)
+    body = [c + rng.uniform(-1, 1, s) * eps * rng.choice([0.0, 0.4, 1.5, 6.0]) for c, s in zip(rng.uniform(-0.6, 0.6, 60), sizes)]
+    body = np.resize(rng.permutation(np.concatenate(body)), n - 2 * seeds)
+    w = np.concatenate([body, 2 + rng.uniform(-1e-3, 1e-3, seeds), -2 - rng.uniform(-1e-3, 1e-3, seeds)]).astype(np.float32)
+    r = lcd.dbci(torch.from_numpy(w).cuda())
+    ref = O.dbci_scan(w)
+    assert (r["sigma"], r["eps"], r["min_pts"]) == (ref["sigma"], ref["eps"], ref["min_pts"]) and ref["min_pts"] == seeds
+    assert np.array_equal(r["labels"].cpu().numpy().astype(np.int64), ref["labels"])
+    assert r["n_noise"] == int((ref["labels"] < 0).sum()) and n // 50 < r["n_noise"] < n - n // 50
+    assert np.array_equal(r["centroids"].cpu().numpy().astype(np.float64), ref["centroids"])
