@@ -570,6 +570,7 @@ __global__ void __launch_bounds__(32 * kTileWarps, 4) dbci_label_kernel(const fl
     }
     send();
     if (lane == 0 && noise) atomicAdd(&P->n_noise, noise);
+    __syncwarp();                         // word_of has been read
   }
 }
 

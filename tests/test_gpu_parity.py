@@ -1230,3 +1230,15 @@ def test_dbci_with_many_points_to_a_core(n, seeds):
     assert np.array_equal(r["labels"].cpu().numpy().astype(np.int64), ref["labels"])
     assert r["n_noise"] == int((ref["labels"] < 0).sum()) and n // 50 < r["n_noise"] < n - n // 50
     assert np.array_equal(r["centroids"].cpu().numpy().astype(np.float64), ref["centroids"])
+
+
+def test_dbci_labels_of_many_tiles_that_are_not_plain():
+    # a CTA labels several tiles one after the other: sparse weights without a core point and dense ones among them
+    rng = np.random.default_rng(8)
+    n, k = 12_000_000, 7200
+    w = np.concatenate([rng.uniform(-0.05, 0.05, n - 480_000 - 2 * k), np.repeat(rng.uniform(-0.05, 0.05, 30), 16_000), np.repeat([-0.5, 0.5], k)])
+    w = w.astype(np.float32)
+    r = lcd.dbci(torch.from_numpy(w).cuda())
+    ref = O.dbci_scan(w)
+    assert ref["min_pts"] == k and len(ref["centroids"]) > 25
+    assert np.array_equal(r["labels"].cpu().numpy().astype(np.int64), ref["labels"]) and r["n_noise"] == int((ref["labels"] < 0).sum())
