@@ -46,6 +46,7 @@ struct SortState {
   int large;                // there are fine bins of more than kCap keys
   int zeros;                // bit 0: there are positive zeros, bit 1: negative ones
   int general;              // the radix sort has to do it
+  int n_uneven;             // buckets for sort_uneven_kernel
 };
 
 __device__ __forceinline__ unsigned key_of(unsigned raw) { return raw ^ ((unsigned)((int)raw >> 31) | 0x80000000u); }
@@ -146,6 +147,7 @@ __global__ void __cluster_dims__(kPlanCtas, 1, 1) __launch_bounds__(1024) sort_p
     st->large = 0;
     st->zeros = 0;
     st->general = 0;
+    st->n_uneven = 0;
   }
 }
 
@@ -445,26 +447,64 @@ constexpr int kSortSmem = (kCap + 16) * 4 + kParts * 2;
 // that threads that read neighbouring groups do not meet in a bank.
 __device__ __forceinline__ unsigned spread(unsigned i) { return i ^ ((i >> 3) & 12u); }
 
-// Keys in shared memory in any order: bitonic merges of a power of two of them (60 us of a CTA for kCap keys; hardly a bucket
-// comes here).
-__device__ __noinline__ void sort_any(unsigned* keys, int cnt) {
-  int size = 32;
-  while (size < cnt) size *= 2;
-  for (int i = cnt + threadIdx.x; i < size; i += kSortThreads) keys[spread(i)] = 0xffffffffu;
-  for (int k = 2; k <= size; k *= 2)
-    for (int j = k / 2; j > 0; j /= 2) {
-      __syncthreads();
-      for (int i = threadIdx.x; i < size / 2; i += kSortThreads) {
-        const int a = 2 * i - (i & (j - 1)), b = a + j;
-        unsigned &p = keys[spread(a)], &q = keys[spread(b)];
-        const unsigned u = p, v = q;
-        if ((u > v) == ((a & k) == 0)) {
-          p = v;
-          q = u;
-        }
+// Sixteen neighbours at a time, twice, the second time half a step further: parts of up to eight keys are in order then, and no
+// key leaves its part.
+__device__ __forceinline__ void sort_small_parts(unsigned* keys, int cnt) {
+  const int groups = (cnt + 15) / 16;
+#pragma unroll
+  for (int half = 0; half < 2; ++half) {
+    for (int g = threadIdx.x; g < groups; g += kSortThreads) {
+      unsigned v[16];
+      const unsigned i0 = (unsigned)(g * 16 + half * 8);
+      if (half && (int)i0 + 8 >= cnt) break;                // nothing behind the half group
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint4 w = *reinterpret_cast<const uint4*>(keys + spread(i0 + 4 * q));
+        v[4 * q] = w.x; v[4 * q + 1] = w.y; v[4 * q + 2] = w.z; v[4 * q + 3] = w.w;
       }
+      network16(v);
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        *reinterpret_cast<uint4*>(keys + spread(i0 + 4 * q)) = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
     }
-  __syncthreads();
+    __syncthreads();
+  }
+}
+
+// cnt keys at `from` by one warp: bitonic merges whose comparisons all put the smaller key first, so that the places behind the
+// last key, up to a power of two, need not be there.
+__device__ void sort_by_warp(unsigned* keys, unsigned from, unsigned cnt) {
+  const unsigned lane = threadIdx.x & 31;
+  unsigned size = 16, lo = 0xffffffffu, hi = 0u;
+  for (unsigned i = lane; i < cnt; i += 32) {
+    lo = min(lo, keys[spread(from + i)]);
+    hi = max(hi, keys[spread(from + i)]);
+  }
+  if (__reduce_min_sync(0xffffffffu, lo) == __reduce_max_sync(0xffffffffu, hi)) return;        // one value
+  while (size < cnt) size *= 2;
+  auto order = [&](unsigned a, unsigned b) {
+    if (b >= cnt) return;
+    unsigned &p = keys[spread(from + a)], &q = keys[spread(from + b)];
+    const unsigned u = p, v = q;
+    if (u > v) {
+      p = v;
+      q = u;
+    }
+  };
+  for (unsigned k = 2; k <= size; k *= 2) {
+    for (unsigned t = lane; t < size / 2; t += 32) {
+      const unsigned block = t & ~(k / 2 - 1), off = t & (k / 2 - 1);
+      order(2 * block + off, 2 * block + k - 1 - off);
+    }
+    __syncwarp();
+    for (unsigned j = k / 4; j > 0; j /= 2) {
+      for (unsigned t = lane; t < size / 2; t += 32) {
+        const unsigned a = 2 * t - (t & (j - 1));
+        order(a, a + j);
+      }
+      __syncwarp();
+    }
+  }
 }
 
 // SINGLE: the whole array is one bucket, read from `in` (the call's first kernel: no __restrict__, its loads may not become
@@ -472,7 +512,7 @@ __device__ __noinline__ void sort_any(unsigned* keys, int cnt) {
 // in place, the next one's keys on their way while one is sorted.
 template <bool SINGLE>
 __global__ void __launch_bounds__(kSortThreads, 2) sort_buckets_kernel(const unsigned* in, long long n, SortState* st,
-                                                                       const unsigned* first, unsigned* x) {
+                                                                       const unsigned* first, unsigned* x, uint2* uneven) {
   extern __shared__ __align__(16) unsigned sm[];
   __shared__ unsigned part[kSortThreads / 32 + 1], lo_s[kSortThreads / 32], hi_s[kSortThreads / 32], most_s[kSortThreads / 32];
   unsigned* keys = sm;                              // [kCap + 16]
@@ -523,6 +563,12 @@ __global__ void __launch_bounds__(kSortThreads, 2) sort_buckets_kernel(const uns
       end_next = first[b + 1];
     }
   };
+  auto reload = [&]() {
+    const unsigned* src = SINGLE ? in : x + at;
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j)
+      if (j * kSortThreads + tid < cnt) k[j] = __ldcs(src + j * kSortThreads + tid);
+  };
   auto load = [&]() {
     if (!SINGLE) {
       at = at_next;
@@ -533,10 +579,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) sort_buckets_kernel(const uns
       }
       if (cnt < 2 || cnt > kCap) cnt = 0;             // one key, or one value (see above)
     }
-    const unsigned* src = SINGLE ? in : x + at;
-#pragma unroll
-    for (int j = 0; j < kSortItems; ++j)
-      if (j * kSortThreads + tid < cnt) k[j] = __ldcs(src + j * kSortThreads + tid);
+    reload();
   };
   look(blockIdx.x);
   load();
@@ -562,7 +605,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) sort_buckets_kernel(const uns
     __syncthreads();
     lo = __reduce_min_sync(0xffffffffu, lo_s[lane & (kSortThreads / 32 - 1)]);
     hi = __reduce_max_sync(0xffffffffu, hi_s[lane & (kSortThreads / 32 - 1)]);
-    if (SINGLE && tid == 0) st->general = 0;
+    if (SINGLE && tid == 0) st->general = st->n_uneven = 0;
     if (lo <= 0x80000000u && hi >= 0x7fffffffu) {
       int zeros = 0;
 #pragma unroll
@@ -657,48 +700,182 @@ __global__ void __launch_bounds__(kSortThreads, 2) sort_buckets_kernel(const uns
     const unsigned to0 = at;
     const int sorted = cnt;
     // the network's groups are whole: what lies behind the last key stays there
-    const int groups = (sorted + 15) / 16;
-    if (tid < 24 && sorted + tid < groups * 16 + 8) keys[spread((unsigned)(sorted + tid))] = 0xffffffffu;
+    if (tid < 24 && sorted + tid < (sorted + 15) / 16 * 16 + 8) keys[spread((unsigned)(sorted + tid))] = 0xffffffffu;
     if (!SINGLE) load();
     __syncthreads();
     if (loose) {
-      for (int round = 0;; ++round) {
-      // parts of more than eight keys: once more; if that is not enough, or if there are many more (one value repeated, in
-      // order as it is, or a few keys far from the others), whatever order they are in
-      if (far && (round > 0 || most >= 64)) {
-        bool bad = false;
-        for (int i = tid + 1; i < sorted; i += kSortThreads) bad = bad || keys[spread(i - 1)] > keys[spread(i)];
-        if (!__syncthreads_or(bad)) break;
-        if (round == 2 || most >= 64) {
-          sort_any(keys, sorted);
+      for (bool again = false;; again = true) {
+        // parts of more than eight keys; many in a part are often one value repeated, among others that are, in order as it is
+        if (far && (again || most >= 64)) {
+          bool bad = false;
+          for (int i = tid + 1; i < sorted; i += kSortThreads) {
+            const unsigned u = keys[spread(i - 1)], v = keys[spread(i)];
+            bad = bad || (u > v && (u != 0x80000000u || v != 0x7fffffffu));          // (zeros of either sign are equal)
+          }
+          if (!__syncthreads_or(bad)) break;
+          if (again) {
+            if (tid == 0) uneven[atomicAdd(&st->n_uneven, 1)] = make_uint2(to0, (unsigned)sorted);
+            break;
+          }
+        } else if (again) {
           break;
         }
-      } else if (round > 0) {
-        break;
-      }
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          for (int g = tid; g < groups; g += kSortThreads) {
-            unsigned v[16];
-            const unsigned i0 = (unsigned)(g * 16 + half * 8);
-            if (half && (int)i0 + 8 >= sorted) break;                // nothing behind the half group
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const uint4 w = *reinterpret_cast<const uint4*>(keys + spread(i0 + 4 * q));
-              v[4 * q] = w.x; v[4 * q + 1] = w.y; v[4 * q + 2] = w.z; v[4 * q + 3] = w.w;
-            }
-            network16(v);
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-              *reinterpret_cast<uint4*>(keys + spread(i0 + 4 * q)) = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-          }
-          __syncthreads();
-        }
+        sort_small_parts(keys, sorted);
       }
     }
 #pragma unroll 8
     for (int i = tid; i < sorted; i += kSortThreads) __stcg(x + to0 + i, raw_of(keys[spread(i)]));
   }
+}
+
+// A bucket that equal stretches of its range leave with too many keys in one of them (an infinity among ordinary weights, values
+// repeated in the tail of others): a run of keys is counted in kCoarse equal stretches of its range, these are divided into parts, as
+// many as their keys ask for, kParts in all, and the keys are placed by parts.  Up to eight keys of a part are left to the network, up
+// to kWarpKeys to a warp, more are a run of their own, of at most a 256th of the range: a key is placed three times at most, and of
+// 16384 keys at most 31 runs wait at any time.  (One bitonic sort of the bucket took 150 to 200 us: 925 K weights on 255 levels with
+// 10 % of others 349 us the whole call, 213 so; 4 M weights, 300 of them infinite 319, 239.)
+constexpr unsigned kWarpKeys = 512;
+constexpr int kCoarse = 512;
+static_assert(kCoarse == kSortThreads, "a thread has one coarse stretch");
+__device__ __forceinline__ void sort_uneven_bucket(unsigned* x, int cnt, SortState* st, unsigned* keys, unsigned* bins) {
+  __shared__ uint2 runs[kCap / kWarpKeys];          // first place, keys
+  __shared__ unsigned full[kCap / 9];               // parts for a warp: first place << 16 | keys
+  __shared__ int n_runs, n_full;
+  __shared__ unsigned part[kSortThreads / 32 + 1], lo_s[kSortThreads / 32], hi_s[kSortThreads / 32];
+  __shared__ unsigned table[kCoarse];               // keys of a coarse stretch, then its first part << 16 | its parts
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+#pragma unroll 8
+  for (int i = tid; i < cnt; i += kSortThreads) {
+    const unsigned v = __ldcg(x + i);
+    if (v == 0x80000000u) atomicOr(&st->zeros, 3);          // one value with positive zeros here: written again by the next kernel
+    keys[spread(i)] = key_of(value_of(v));
+  }
+  if (tid < 24 && cnt + tid < (cnt + 15) / 16 * 16 + 8) keys[spread((unsigned)(cnt + tid))] = 0xffffffffu;
+  if (tid == 0) {
+    runs[0] = make_uint2(0u, (unsigned)cnt);
+    n_runs = 1;
+  }
+  __syncthreads();
+  while (n_runs > 0) {
+    const uint2 run = runs[n_runs - 1];
+    const unsigned from = run.x, c = run.y;
+    unsigned k[kSortItems], lo = 0xffffffffu, hi = 0u;
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j)
+      if ((unsigned)(j * kSortThreads + tid) < c) {
+        k[j] = keys[spread(from + j * kSortThreads + tid)];
+        lo = min(lo, k[j]);
+        hi = max(hi, k[j]);
+      }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0) { lo_s[warp] = lo; hi_s[warp] = hi; }
+    table[tid] = 0u;
+#pragma unroll
+    for (int i = 0; i < kParts / 2 / kSortThreads; ++i) bins[i * kSortThreads + tid] = 0u;
+    __syncthreads();                                // (also: every thread has read the run)
+    if (tid == 0) {
+      --n_runs;
+      n_full = 0;
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo_s[lane & (kSortThreads / 32 - 1)]);
+    hi = __reduce_max_sync(0xffffffffu, hi_s[lane & (kSortThreads / 32 - 1)]);
+    const unsigned span = hi - lo;
+    if (span == 0) {
+      __syncthreads();
+      continue;
+    }
+    const bool exact = span < (unsigned)kParts;     // a part for every value
+    const int shift = exact ? 0 : 32 - __clz(span) - 9;
+    if (!exact) {
+#pragma unroll
+      for (int j = 0; j < kSortItems; ++j)
+        if ((unsigned)(j * kSortThreads + tid) < c) atomicAdd(&table[(k[j] - lo) >> shift], 1u);
+      __syncthreads();
+      const unsigned parts = min(1u + table[tid] * (unsigned)(kParts - kCoarse) / c, 1u << min(shift, 15));        // (16384 x 15872 fits)
+      const unsigned first = block_exclusive<kSortThreads / 32>(parts, part);
+      table[tid] = first << 16 | parts;
+      __syncthreads();
+    }
+    auto part_of = [&](unsigned key) {
+      const unsigned d = key - lo;
+      if (exact) return d;
+      const unsigned e = table[d >> shift];
+      return (e >> 16) + __umulhi(d << (32 - shift), e & 0xffffu);
+    };
+    // the next place of a key's part; a warp whose keys are of one part (a value repeated: the bucket comes in the order of its parts)
+    // asks once (11000 equal keys one by one take 20 us)
+    auto next_of = [&](unsigned key, bool in) {
+      const unsigned p = in ? part_of(key) : 0xffffffffu, s = (p & 1u) * 16u;
+      const unsigned p0 = __shfl_sync(0xffffffffu, p, 0);
+      unsigned v = 0;
+      if (__all_sync(0xffffffffu, in && p == p0)) {
+        if (lane == 0) v = atomicAdd(&bins[p >> 1], 32u << s);
+        return ((__shfl_sync(0xffffffffu, v, 0) >> s) & 0xffffu) + lane;
+      }
+      if (in) v = atomicAdd(&bins[p >> 1], 1u << s);
+      return (v >> s) & 0xffffu;
+    };
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j)
+      if ((unsigned)(j * kSortThreads + warp * 32) < c) next_of(k[j], (unsigned)(j * kSortThreads + tid) < c);
+    __syncthreads();
+    constexpr int Q = kParts / 8 / kSortThreads;
+    uint4* mine = reinterpret_cast<uint4*>(bins) + tid * Q;
+    unsigned sum = 0;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      const uint4 v = mine[i];
+      sum += v.x + v.y + v.z + v.w;
+    }
+    unsigned e = block_exclusive<kSortThreads / 32>((sum & 0xffffu) + (sum >> 16), part);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      uint4 v = mine[i];
+      auto place = [&](unsigned& w) {
+        const unsigned first = w & 0xffffu, second = w >> 16;
+        w = e | (e + first) << 16;
+        e += first + second;
+      };
+      place(v.x); place(v.y); place(v.z); place(v.w);
+      mine[i] = v;
+    }
+    __syncthreads();
+    // every key takes its part's next place: the word of a part then says where it ends
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j)
+      if ((unsigned)(j * kSortThreads + warp * 32) < c) {
+        const bool in = (unsigned)(j * kSortThreads + tid) < c;
+        const unsigned to = next_of(k[j], in);
+        if (in) keys[spread(from + to)] = k[j];
+      }
+    __syncthreads();
+    if (exact) continue;
+    for (int w = tid; w < kParts / 2; w += kSortThreads) {
+      const unsigned ends = bins[w], a = w ? bins[w - 1] >> 16 : 0u, b = ends & 0xffffu, z = ends >> 16;
+      auto look = [&](unsigned first, unsigned end) {
+        if (end - first > kWarpKeys) runs[atomicAdd(&n_runs, 1)] = make_uint2(from + first, end - first);
+        else if (end - first > 8) full[atomicAdd(&n_full, 1)] = (from + first) << 16 | (end - first);
+      };
+      look(a, b);
+      look(b, z);
+    }
+    __syncthreads();
+    for (int i = warp; i < n_full; i += kSortThreads / 32) sort_by_warp(keys, full[i] >> 16, full[i] & 0xffffu);
+    __syncthreads();
+  }
+  sort_small_parts(keys, cnt);
+#pragma unroll 8
+  for (int i = tid; i < cnt; i += kSortThreads) __stcg(x + i, raw_of(keys[spread(i)]));
+  __syncthreads();
+}
+
+__global__ void __launch_bounds__(kSortThreads, 2) sort_uneven_kernel(SortState* st, const uint2* uneven, unsigned* x) {
+  extern __shared__ __align__(16) unsigned sm[];
+  wait_for_last_kernel();
+  let_next_kernel_start();
+  const int n = st->n_uneven;
+  for (int i = blockIdx.x; i < n; i += gridDim.x) sort_uneven_bucket(x + uneven[i].x, (int)uneven[i].y, st, sm, sm + kCap + 16);
 }
 
 // ---- the general sort: four stable passes of eight bits ---------------------------------------------------
@@ -856,7 +1033,7 @@ __global__ void __launch_bounds__(kRadixThreads, 2) sort_general_kernel(const un
 
 size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
 struct Layout {
-  size_t state, samples, table, fine, begins, first, cursor, counts, tmp, total;
+  size_t state, samples, table, fine, begins, first, cursor, uneven, counts, tmp, total;
 };
 Layout layout(int64_t n) {
   Layout l;
@@ -868,6 +1045,7 @@ Layout layout(int64_t n) {
   l.begins = off; off += up256(kFineMax / 4);
   l.first = off; off += up256((kMaxBuckets + 1) * 4);
   l.cursor = off; off += up256(kMaxBuckets * 4);
+  l.uneven = off; off += up256(kMaxBuckets * 8);
   l.counts = off; off += up256(kRadixGridMax * 256 * 4);
   l.tmp = off; off += up256((size_t)n * 4);
   l.total = off;
@@ -898,16 +1076,17 @@ cudaError_t launch_dbci_sort(const float* weights, int64_t n, float* sorted, voi
   unsigned* begins = reinterpret_cast<unsigned*>(base + l.begins);
   unsigned* first = reinterpret_cast<unsigned*>(base + l.first);
   unsigned* cursor = reinterpret_cast<unsigned*>(base + l.cursor);
+  uint2* uneven = reinterpret_cast<uint2*>(base + l.uneven);
   unsigned* counts = reinterpret_cast<unsigned*>(base + l.counts);
   unsigned* tmp = reinterpret_cast<unsigned*>(base + l.tmp);
   const unsigned* in = reinterpret_cast<const unsigned*>(weights);
   unsigned* x = reinterpret_cast<unsigned*>(sorted);
-  static PerDeviceFlag f_count, f_part_l, f_part_s, f_sort, f_single;
+  static PerDeviceFlag f_count, f_part_l, f_part_s, f_sort, f_single, f_uneven;
   const int sms = current_sm_count();
   cudaError_t e;
   if (n <= kCap) {
     if ((e = opt_in(sort_buckets_kernel<true>, kSortSmem, f_single)) != cudaSuccess) return e;
-    e = launch_after(sort_buckets_kernel<true>, 1, kSortThreads, kSortSmem, s, in, (long long)n, st, (const unsigned*)first, x);
+    e = launch_after(sort_buckets_kernel<true>, 1, kSortThreads, kSortSmem, s, in, (long long)n, st, (const unsigned*)first, x, uneven);
   } else {
     constexpr int L = 24, S = 4;
     if ((e = opt_in(sort_count_kernel, kCountSmem, f_count)) != cudaSuccess) return e;
@@ -933,8 +1112,12 @@ cudaError_t launch_dbci_sort(const float* weights, int64_t n, float* sorted, voi
                      in, (long long)n, (const SortState*)st, (const unsigned*)table, (const unsigned*)begins, cursor, x);
     if (e != cudaSuccess) return e;
     const int64_t most = 2 * (n / target) + 2;
-    e = launch_after(sort_buckets_kernel<false>, (unsigned)(most < 2 * sms ? most : 2 * sms), kSortThreads, kSortSmem, s, in, (long long)n, st, (const unsigned*)first, x);
+    e = launch_after(sort_buckets_kernel<false>, (unsigned)(most < 2 * sms ? most : 2 * sms), kSortThreads, kSortSmem, s, in, (long long)n, st, (const unsigned*)first, x, uneven);
   }
+  if (e != cudaSuccess) return e;
+  if ((e = opt_in(sort_uneven_kernel, kSortSmem, f_uneven)) != cudaSuccess) return e;
+  const int64_t uneven_most = n / 256 + 1;
+  e = launch_after(sort_uneven_kernel, (unsigned)(n <= kCap ? 1 : uneven_most < 2 * sms ? uneven_most : 2 * sms), kSortThreads, kSortSmem, s, st, (const uint2*)uneven, x);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sort_general_kernel, kRadixThreads, 0)) != cudaSuccess) return e;

@@ -1242,3 +1242,33 @@ def test_dbci_labels_of_many_tiles_that_are_not_plain():
     ref = O.dbci_scan(w)
     assert ref["min_pts"] == k and len(ref["centroids"]) > 25
     assert np.array_equal(r["labels"].cpu().numpy().astype(np.int64), ref["labels"]) and r["n_noise"] == int((ref["labels"] < 0).sum())
+
+
+def _uneven(kind, n, rng):
+    ulps = lambda at, spread, size: (np.float32(at).view(np.int32) + rng.integers(0, spread, size)).astype(np.int32).view(np.float32)
+    if kind == "nested":                     # most of the keys in a small part of the range of the rest, again and again
+        few = [ulps(1.0, 1 << b, n // d) for b, d in ((29, 16), (24, 8), (18, 4), (14, 8))]
+        return np.concatenate(few + [ulps(1.0, 1 << 3, n - sum(map(len, few)))])
+    if kind == "runs":                       # runs of equal and of nearly equal keys at the sizes at which another way is taken
+        sizes = [1, 2, 8, 9, 16, 17, 511, 512, 513, 1024, 3000]
+        w = [np.full(s, v, np.float32) for s, v in zip(sizes, ulps(0.3, 1 << 20, len(sizes)))]
+        w += [ulps(v, 3 * s, s) for s, v in zip(sizes, ulps(0.2, 1 << 20, len(sizes)))]
+        w.append(rng.normal(0, 1e20, 50).astype(np.float32))
+        return np.resize(np.concatenate(w), n)
+    # zeros of either sign and subnormal numbers beside ordinary weights and infinities
+    w = rng.normal(0, 0.02, n).astype(np.float32)
+    w[::3] = 0.0
+    w[1::3] = -0.0
+    w[::50] = ulps(1e-42, 300, len(w[::50])) * (-1) ** np.arange(len(w[::50]))
+    w[7::500] = np.inf
+    return w
+
+
+@pytest.mark.parametrize("n", [100, 4097, 16384, 40_003, 300_000])
+@pytest.mark.parametrize("kind", ["nested", "runs", "zeros"])
+def test_dbci_sort_of_unevenly_spread_keys(kind, n):
+    # equal stretches of a bucket's range leave most of its keys in few of them
+    rng = np.random.default_rng(n)
+    w = rng.permutation(_uneven(kind, n, rng))
+    r = lcd.dbci(torch.from_numpy(w).cuda())
+    assert np.array_equal(r["sorted"].cpu().numpy().view(np.int32), np.sort(w, kind="stable").view(np.int32))
