@@ -6,20 +6,19 @@
 //             ask for ("fine bins", about 3 K keys of 45 M each; one more at either end for what
 //             lies at or beyond the sample's extremes, where clipped weights repeat one value);
 //   count     exact counts of the fine bins;
-//   map       one CTA: neighbouring fine bins become buckets of at most kCap keys, a larger fine bin a bucket of its own;
-//   partition every key to its bucket's place in the output, in no order;
+//   map       one CTA: neighbouring fine bins become buckets of at most kCap keys, a larger fine bin a segment of its own;
+//   partition every key to its bucket's or segment's place in the output, in no order;
+//   segments  nothing, unless there are some: those of one value stay as they are (weights in bf16, clipped or pruned ones), the
+//             others (narrow clumps, a value repeated among others) are divided by their own ranges into buckets;
 //   buckets   a CTA sorts a bucket where it lies: 16384 equal parts of its range, a place for every key by a counting pass
 //             (the shared-memory atomic's result), then sixteen neighbours at a time through a sorting network, twice, the
-//             second time half a step further, which puts parts of up to eight keys in order.  A larger bucket is right if
-//             it holds one value alone, and that is checked;
-//   general   nothing, unless one of these has found keys that it cannot take (narrow clumps or values repeated among others
-//             in one fine bin): then a radix sort of the input in four stable passes by one cooperative launch.  Zeros of either
-//             sign are equal and keep their order; if there are both, the same launch writes them again in that order.
-// 45 M Gaussian weights: 620 us (plan 6, count 55, map 18, partition 240, buckets 285), CUB's radix sort 1070; 925 K: 52 and 110.
-// Bytes are 0.9 GB, 140 us: what bounds the passes is shared memory at random addresses (three lookups or atomics and two stores
-// a key in the partition, an atomic, a lookup and a store in the buckets, each three to four bank conflicts a warp) and, where the
-// partition writes runs of six keys, the sectors that L2 takes.  Inputs that need the general sort: 1490 us after the count
-// (CUB 1070).
+//             second time half a step further, which puts parts of up to eight keys in order;
+//   finish    nothing, unless a bucket's keys lie too close together in places (it is divided again by their density) or
+//             there are zeros of either sign: they are equal and keep their order, so they are written again in the input's.
+// 45 M Gaussian weights: 570 us (plan 6, count 55, map 18, partition 220, buckets 275), CUB's radix sort 1070; 925 K: 55 and 110.
+// Bytes are 0.9 GB, 140 us: what bounds the passes is shared memory at random addresses (a key's three lookups or atomics, a store
+// and two loads in the partition, an atomic, a lookup and a store in the buckets, each three to four bank conflicts a warp) and, where the
+// partition writes runs of six keys, the sectors that L2 takes.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -36,24 +35,95 @@ constexpr int kSamples = 16384, kBins = 2048, kFineMax = 24576, kFineBudget = 14
 static_assert(kFineBudget + 5 * kBins + 2 <= kFineMax, "shares of the budget are rounded up, every bin has four parts at least");
 constexpr int kCap = 16384;                  // keys a CTA sorts
 constexpr int kTarget = 12288;               // keys of a bucket of a large array
+constexpr int kPartsOfChunk = 264;           // counters of a segment, for kCap of its keys: a part for 64 keys, two more and a margin
 constexpr int kMaxBuckets = 8192;
 constexpr int64_t kMostKeys = (int64_t)(kMaxBuckets / 2 - 1) * kTarget;
 
+// A stretch of the array with more keys than a bucket holds, by chunks of kCap keys.
+struct Segment {
+  unsigned from, keys;
+  unsigned chunk;           // its first one among those of its level
+  unsigned lo, hi;          // no key lies outside
+  unsigned pivot;           // a key of it, the one that repeats most where one does
+  unsigned mixed;           // it has other keys
+  unsigned equal, equal_to; // the pivot's places
+};
+constexpr int kLevels = 4;                   // 32 bits of a key, eight or more a level
+constexpr int kPhases = 4 * kLevels + 3;     // of the kernels whose CTAs wait for one another
 struct SortState {
+  unsigned long long segments[kLevels];      // number << 32 | chunks
+  unsigned ticket[kPhases], done[kPhases];
+  int mixed[kLevels];       // some segment is
   unsigned kmin, kmax;      // sample extremes
   int shift;                // bin of a key: (key - kmin) >> shift
   int n_fine, n_buckets;
-  int large;                // there are fine bins of more than kCap keys
+  int n_extra;              // buckets made from segments
   int zeros;                // bit 0: there are positive zeros, bit 1: negative ones
-  int general;              // the radix sort has to do it
-  int n_uneven;             // buckets for sort_uneven_kernel
+  int n_uneven;             // buckets to be divided again
 };
+constexpr size_t kStateBytes = 512;
+static_assert(sizeof(SortState) <= kStateBytes, "space for the state");
 
 __device__ __forceinline__ unsigned key_of(unsigned raw) { return raw ^ ((unsigned)((int)raw >> 31) | 0x80000000u); }
 __device__ __forceinline__ unsigned raw_of(unsigned key) { return key ^ (~(unsigned)((int)key >> 31) | 0x80000000u); }
 
 // The same for zeros of either sign, which are equal.
 __device__ __forceinline__ unsigned value_of(unsigned raw) { return raw == 0x80000000u ? 0u : raw; }
+
+// `items` pieces of work of one phase of a kernel, given out one by one to the CTAs that ask, then a wait until all are done.
+// Nothing says that the CTAs of a launch run at the same time, so none waits for another one to come: what is not done was taken by
+// a CTA that runs.  A CTA that has waited kPolls times (ten milliseconds or more) gets `false` and is to leave; the one that does the last
+// piece never waits, goes on, and takes what the others leave.  What one phase writes the next ones read past L1 (__ldcg).
+// ahead(i, slot): done by the first warp for a piece of work before its turn (slot: 0 and 1 in turn), the first one at once, the others
+// where work(i, slot, look_ahead) calls look_ahead, once in every case.
+constexpr int kPolls = 20000;
+template <typename Ahead, typename Work>
+__device__ __forceinline__ bool run_phase(SortState* st, int phase, unsigned items, Ahead ahead, Work work) {
+  __shared__ unsigned given;
+  if (items == 0) return true;
+  const bool first_warp = threadIdx.x < 32, first = threadIdx.x == 0;
+  unsigned mine = 0;
+  if (first_warp) {
+    if (first) mine = atomicAdd(&st->ticket[phase], 1u);
+    mine = __shfl_sync(0xffffffffu, mine, 0);
+    if (mine < items) ahead(mine, 0);
+  }
+  for (int slot = 0;; slot ^= 1) {
+    __syncthreads();                      // the last piece's shared memory has been read
+    if (first) given = mine;
+    __syncthreads();
+    const unsigned i = given;
+    if (i >= items) break;
+    if (first) mine = atomicAdd(&st->ticket[phase], 1u);          // (the next one, while this one is done)
+    work(i, slot, [&]() {
+      if (!first_warp) return;
+      mine = __shfl_sync(0xffffffffu, mine, 0);
+      if (mine < items) ahead(mine, slot ^ 1);
+    });
+    __syncthreads();
+    if (first) {
+      __threadfence();
+      atomicAdd(&st->done[phase], 1u);
+    }
+  }
+  bool all = false;
+  if (first) {
+    for (int t = 0; t < kPolls && !all; ++t) {
+      unsigned done;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(done) : "l"(&st->done[phase]) : "memory");
+      all = done >= items;
+      if (!all) __nanosleep(100);
+    }
+  }
+  return __syncthreads_or(all);
+}
+template <typename Work>
+__device__ __forceinline__ bool run_phase(SortState* st, int phase, unsigned items, Work work) {
+  return run_phase(st, phase, items, [](unsigned, int) {}, [&](unsigned i, int, auto look_ahead) {
+    look_ahead();
+    work(i);
+  });
+}
 
 // Exclusive sum over the 32 * WARPS threads of a CTA; part: WARPS + 1 words (the last: the total).
 template <int WARPS>
@@ -107,6 +177,7 @@ __global__ void __cluster_dims__(kPlanCtas, 1, 1) __launch_bounds__(1024) sort_p
   for (int i = blockIdx.x * 1024 + tid; i < kFineMax / 4; i += kPlanCtas * 1024) reinterpret_cast<uint4*>(fine)[i] = make_uint4(0u, 0u, 0u, 0u);
   cooperative_groups::this_cluster().sync();
   if (blockIdx.x != 0) return;
+  if (tid < (int)(sizeof(SortState) / 4)) reinterpret_cast<unsigned*>(st)[tid] = 0u;
   unsigned k[PER], lo = 0xffffffffu, hi = 0u;
 #pragma unroll
   for (int j = 0; j < PER / 4; ++j) {
@@ -143,11 +214,6 @@ __global__ void __cluster_dims__(kPlanCtas, 1, 1) __launch_bounds__(1024) sort_p
     st->kmax = hi;
     st->shift = shift;
     st->n_fine = (int)part[32] + 2;
-    st->n_buckets = 0;
-    st->large = 0;
-    st->zeros = 0;
-    st->general = 0;
-    st->n_uneven = 0;
   }
 }
 
@@ -161,6 +227,21 @@ struct FineMap {
     if (d - 1u >= kmax - kmin - 1u || kmax == kmin) return k <= kmin ? 0 : last;          // seldom
     const unsigned e = table[d >> shift];
     return (int)((e >> 16) + __umulhi(d << (32 - shift), e & 0xffffu));                   // (d below its bin) * parts >> shift
+  }
+  // the keys of a fine bin
+  __device__ void bounds(int f, const unsigned* table, unsigned& lo, unsigned& hi) const {
+    lo = 0u;
+    hi = 0xffffffffu;
+    if (f == 0) hi = kmin;
+    if (f == last) lo = kmax;
+    if (f == 0 || f == last) return;
+    int bin = 0;
+    for (int s = kBins / 2; s > 0; s /= 2)
+      if ((int)(table[bin + s] >> 16) <= f) bin += s;
+    const unsigned parts = table[bin] & 0xffffu;
+    const unsigned long long part = (unsigned)f - (table[bin] >> 16);
+    lo = kmin + ((unsigned)bin << shift) + (unsigned)(((part << shift) + parts - 1) / parts);
+    hi = kmin + ((unsigned)bin << shift) + (unsigned)((((part + 1) << shift) + parts - 1) / parts) - 1u;
   }
 };
 
@@ -198,17 +279,28 @@ __global__ void __launch_bounds__(kCountThreads, 2) sort_count_kernel(const unsi
   }
 }
 
+// Segments are numbered in the order of their chunks.
+__device__ __forceinline__ void add_segment(SortState* st, Segment* segments, int level, unsigned from, unsigned keys, unsigned lo, unsigned hi) {
+  const unsigned long long at = atomicAdd(&st->segments[level], 1ull << 32 | (keys + kCap - 1) / kCap);
+  Segment* s = segments + (at >> 32);
+  s->from = from;
+  s->keys = keys;
+  s->chunk = (unsigned)at;
+  s->lo = lo;
+  s->hi = hi;
+  s->mixed = 0;
+}
+
 // A bucket is a run of fine bins that begin between the same two multiples of `target` in the sorted order; a fine bin that ends
 // more than kCap keys after the first of the two begins another one.  So a bucket has at most kCap keys unless it is a fine bin of
 // more, and there are at most two for every `target` keys.  Empty fine bins begin none.
 // begins: a word for sixteen fine bins, a bit for each that begins a bucket under the number of buckets begun before, less one.
 constexpr int kMapThreads = kFineMax / 32, kMapWarps = kMapThreads / 32;
-__global__ void __launch_bounds__(kMapThreads) sort_map_kernel(long long n, int target, SortState* st, unsigned* fine, const unsigned* samples, const unsigned* table,
-                                                               unsigned* __restrict__ begins,
-                                                               unsigned* __restrict__ first, unsigned* __restrict__ cursor) {
+__global__ void __launch_bounds__(kMapThreads) sort_map_kernel(long long n, int target, SortState* st, const unsigned* fine, unsigned* __restrict__ begins,
+                                                               unsigned* __restrict__ first, unsigned* __restrict__ cursor, Segment* segments) {
   constexpr int PER = 32;
   __shared__ unsigned part[kMapWarps + 1];
-  __shared__ unsigned tail[kMapWarps], is_large[kMapThreads];
+  __shared__ unsigned tail[kMapWarps];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   wait_for_last_kernel();
   let_next_kernel_start();
@@ -218,14 +310,11 @@ __global__ void __launch_bounds__(kMapThreads) sort_map_kernel(long long n, int 
     const uint4 v = reinterpret_cast<const uint4*>(fine)[tid * (PER / 4) + j];
     c[4 * j] = v.x; c[4 * j + 1] = v.y; c[4 * j + 2] = v.z; c[4 * j + 3] = v.w;
   }
-  unsigned large = 0;
 #pragma unroll
   for (int j = 0; j < PER; ++j) {
     sum += c[j];
     last = c[j] ? c[j] : last;
-    large |= c[j] > (unsigned)kCap ? 1u << j : 0u;
   }
-  is_large[tid] = large;
   unsigned at = block_exclusive<kMapWarps>(sum, part);
   // the last non-empty fine bin before this thread's
   unsigned before = last;
@@ -258,6 +347,7 @@ __global__ void __launch_bounds__(kMapThreads) sort_map_kernel(long long n, int 
   unsigned id = block_exclusive<kMapWarps>((unsigned)__popc(starts), part);
   const int total = (int)part[kMapWarps];
   reinterpret_cast<uint2*>(begins)[tid] = make_uint2((id - 1u) << 16 | (starts & 0xffffu), (id - 1u + (unsigned)__popc(starts & 0xffffu)) << 16 | starts >> 16);
+  unsigned large = 0;
   p = at;
 #pragma unroll
   for (int j = 0; j < PER; ++j) {
@@ -266,32 +356,18 @@ __global__ void __launch_bounds__(kMapThreads) sort_map_kernel(long long n, int 
       cursor[id] = p;
       ++id;
     }
+    large |= c[j] > (unsigned)kCap ? 1u << j : 0u;
     p += c[j];
   }
-  // Fine bins of more than kCap keys: two different samples in one, and the work of the next two kernels would be in vain.
-  const bool any_large = __syncthreads_or(large != 0u);
-  bool mixed = false;
-  if (any_large) {
-    const FineMap map(st);
-#pragma unroll
-    for (int j = 0; j < PER; ++j)
-      if ((large >> j) & 1u) __stcg(fine + tid * PER + j, 0u);
-    __syncthreads();
-    for (int i = tid; i < kSamples; i += kMapThreads) {
-      const unsigned k = key_of(value_of(raw_of(samples[i])));
-      const int f = map.of(k, table);
-      if ((is_large[f >> 5] >> (f & 31)) & 1u) {
-        const unsigned other = atomicCAS(fine + f, 0u, k);
-        mixed = mixed || (other != 0u && other != k);
-      }
-    }
+  for (; large; large &= large - 1) {             // (their ranges: see the partition)
+    const int j = __ffs(large) - 1;
+    p = at;
+    for (int i = 0; i < j; ++i) p += fine[tid * PER + i];
+    add_segment(st, segments, 0, p, fine[tid * PER + j], (unsigned)(tid * PER + j), 0u);
   }
-  mixed = __syncthreads_or(mixed);
   if (tid == 0) {
     first[total] = (unsigned)n;
     st->n_buckets = total;
-    st->large = any_large;
-    st->general = mixed;
   }
 }
 
@@ -305,7 +381,7 @@ constexpr int partition_smem() { return kBins * 4 + kFineMax / 4 + kMaxBuckets *
 template <int ITEMS>
 __global__ void __launch_bounds__(kPartThreads, 1) sort_partition_kernel(const unsigned* __restrict__ in, long long n, const SortState* st,
                                                                          const unsigned* table_g, const unsigned* begins_g,
-                                                                         unsigned* cursor, unsigned* __restrict__ out) {
+                                                                         unsigned* cursor, unsigned* __restrict__ out, Segment* segments, unsigned* counters) {
   constexpr int TILE = kPartThreads * ITEMS, kLong = 128;
   extern __shared__ __align__(16) unsigned sm[];
   __shared__ unsigned part[kPartThreads / 32 + 1];
@@ -313,7 +389,6 @@ __global__ void __launch_bounds__(kPartThreads, 1) sort_partition_kernel(const u
   __shared__ int n_long;
   wait_for_last_kernel();
   let_next_kernel_start();
-  if (st->general) return;
   unsigned* at = sm;                                      // [kMaxBuckets] counts, then first place in the tile
   unsigned* delta = at + kMaxBuckets;                     // [kMaxBuckets] of the tile's runs: place in the output - place in the tile
   unsigned* table = delta + kMaxBuckets;                  // [kBins]
@@ -325,6 +400,18 @@ __global__ void __launch_bounds__(kPartThreads, 1) sort_partition_kernel(const u
   const bool many = st->n_buckets > kMaxBuckets / 2;
   for (int i = tid; i < kBins; i += kPartThreads) table[i] = table_g[i];
   for (int i = tid; i <= map.last / 16; i += kPartThreads) begins[i] = begins_g[i];
+  if (st->segments[0] != 0) {
+    // for the next kernel: ranges of the segments, given by their fine bins so far, and counters
+    __syncthreads();
+    const unsigned number = (unsigned)(st->segments[0] >> 32), all = (unsigned)st->segments[0] * kPartsOfChunk;
+    for (unsigned i = blockIdx.x * kPartThreads + tid; i < number; i += gridDim.x * kPartThreads) {
+      unsigned lo, hi;
+      map.bounds((int)segments[i].lo, table, lo, hi);
+      segments[i].lo = lo;
+      segments[i].hi = hi == 0x7fffffffu ? 0x80000000u : hi;          // (zeros of either sign count as positive ones there)
+    }
+    for (unsigned i = blockIdx.x * kPartThreads + tid; i < all; i += gridDim.x * kPartThreads) counters[i] = 0u;
+  }
   long long t0 = (long long)blockIdx.x * TILE;
   unsigned v[ITEMS];
   auto load = [&](long long t) {
@@ -471,16 +558,24 @@ __device__ __forceinline__ void sort_small_parts(unsigned* keys, int cnt) {
   }
 }
 
+__device__ __forceinline__ bool one_value(const unsigned* keys, unsigned from, unsigned cnt) {          // by a warp
+  unsigned lo = 0xffffffffu, hi = 0u;
+#pragma unroll 4
+  for (unsigned i = threadIdx.x & 31; i < cnt; i += 32) {
+    const unsigned k = keys[spread(from + i)];
+    lo = min(lo, k);
+    hi = max(hi, k);
+  }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  return lo == hi;
+}
+
 // cnt keys at `from` by one warp: bitonic merges whose comparisons all put the smaller key first, so that the places behind the
 // last key, up to a power of two, need not be there.
 __device__ void sort_by_warp(unsigned* keys, unsigned from, unsigned cnt) {
   const unsigned lane = threadIdx.x & 31;
-  unsigned size = 16, lo = 0xffffffffu, hi = 0u;
-  for (unsigned i = lane; i < cnt; i += 32) {
-    lo = min(lo, keys[spread(from + i)]);
-    hi = max(hi, keys[spread(from + i)]);
-  }
-  if (__reduce_min_sync(0xffffffffu, lo) == __reduce_max_sync(0xffffffffu, hi)) return;        // one value
+  unsigned size = 16;
   while (size < cnt) size *= 2;
   auto order = [&](unsigned a, unsigned b) {
     if (b >= cnt) return;
@@ -512,55 +607,31 @@ __device__ void sort_by_warp(unsigned* keys, unsigned from, unsigned cnt) {
 // in place, the next one's keys on their way while one is sorted.
 template <bool SINGLE>
 __global__ void __launch_bounds__(kSortThreads, 2) sort_buckets_kernel(const unsigned* in, long long n, SortState* st,
-                                                                       const unsigned* first, unsigned* x, uint2* uneven) {
+                                                                       const unsigned* first, const uint2* extra, unsigned* x, uint2* uneven) {
   extern __shared__ __align__(16) unsigned sm[];
   __shared__ unsigned part[kSortThreads / 32 + 1], lo_s[kSortThreads / 32], hi_s[kSortThreads / 32], most_s[kSortThreads / 32];
   unsigned* keys = sm;                              // [kCap + 16]
   unsigned* bins = sm + kCap + 16;                  // [kParts / 2] two 16-bit counts a word, then two first places
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  int nb = 1;
   wait_for_last_kernel();
   let_next_kernel_start();
-  if (!SINGLE) {
-    if (__syncthreads_or(tid == 0 && st->general)) return;        // (asked once: another CTA may be setting it)
-    nb = st->n_buckets;
-    if (st->large) {
-      // Every CTA takes a stretch of the array and compares what lies in buckets of more than kCap keys with their first one.
-      const unsigned a = (unsigned)(n * blockIdx.x / gridDim.x), e = (unsigned)(n * (blockIdx.x + 1) / gridDim.x);
-      int l = 0, h = nb - 1;                        // the bucket of place a
-      while (l < h) {
-        const int m = (l + h + 1) >> 1;
-        if (first[m] <= a) l = m; else h = m - 1;
-      }
-      bool same = true;
-      for (; l < nb && first[l] < e; ++l) {
-        const unsigned f0 = first[l], f1 = first[l + 1];
-        if (f1 - f0 <= (unsigned)kCap) continue;
-        const unsigned want = value_of(__ldcg(x + f0)), to = min(f1, e);
-        unsigned ones = 0xffffffffu, any = 0u;
-#pragma unroll 4
-        for (unsigned i = max(f0, a) + tid; i < to; i += kSortThreads) {
-          const unsigned v = __ldcg(x + i);
-          ones &= v;
-          any |= v;
-          same = same && value_of(v) == want;
-        }
-        if (want == 0u && ones <= any) {                  // (some were read)
-          const int zeros = (ones == 0u ? 1 : 0) | (any != 0u ? 2 : 0);
-          if (~st->zeros & zeros) atomicOr(&st->zeros, zeros);
-        }
-      }
-      if (!same) st->general = 1;
-    }
+  const int nf = SINGLE ? 1 : st->n_buckets, nb = SINGLE ? 1 : nf + st->n_extra;
+  if (SINGLE) {
+    if (tid < (int)(sizeof(SortState) / 4)) reinterpret_cast<unsigned*>(st)[tid] = 0u;
+    __syncthreads();
   }
   unsigned k[kSortItems], at = 0;
   int cnt = (int)n;
   unsigned at_next = 0, end_next = 0;               // of the bucket to be loaded next
   auto look = [&](int b) {
     at_next = end_next = 0;
-    if (!SINGLE && b < nb) {
+    if (!SINGLE && b < nf) {
       at_next = first[b];
       end_next = first[b + 1];
+    } else if (!SINGLE && b < nb) {
+      const uint2 e = extra[b - nf];
+      at_next = e.x;
+      end_next = e.x + e.y;
     }
   };
   auto reload = [&]() {
@@ -577,7 +648,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) sort_buckets_kernel(const uns
         const unsigned v = __ldcg(x + at);
         if (value_of(v) == 0u) atomicOr(&st->zeros, v == 0u ? 1 : 2);
       }
-      if (cnt < 2 || cnt > kCap) cnt = 0;             // one key, or one value (see above)
+      if (cnt < 2 || cnt > kCap) cnt = 0;             // one key, or a segment
     }
     reload();
   };
@@ -605,7 +676,6 @@ __global__ void __launch_bounds__(kSortThreads, 2) sort_buckets_kernel(const uns
     __syncthreads();
     lo = __reduce_min_sync(0xffffffffu, lo_s[lane & (kSortThreads / 32 - 1)]);
     hi = __reduce_max_sync(0xffffffffu, hi_s[lane & (kSortThreads / 32 - 1)]);
-    if (SINGLE && tid == 0) st->general = st->n_uneven = 0;
     if (lo <= 0x80000000u && hi >= 0x7fffffffu) {
       int zeros = 0;
 #pragma unroll
@@ -613,9 +683,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) sort_buckets_kernel(const uns
         if (j * kSortThreads + tid < cnt && k[j] - 0x7fffffffu <= 1u) zeros |= k[j] == 0x80000000u ? 1 : 2;
       const int pos = __syncthreads_or(zeros & 1), neg = __syncthreads_or(zeros & 2);
       zeros = (pos ? 1 : 0) | (neg ? 2 : 0);
-      if (tid == 0) { if (SINGLE) st->zeros = zeros; else atomicOr(&st->zeros, zeros); }
-    } else if (SINGLE && tid == 0) {
-      st->zeros = 0;
+      if (tid == 0) atomicOr(&st->zeros, zeros);
     }
     // The part of a key, monotone in the key: one value each if there are enough parts for the range, else equal stretches of
     // the range of the keys' values, over which they are spread smoothly (the bits of one binary order of magnitude have half the
@@ -733,64 +801,60 @@ __global__ void __launch_bounds__(kSortThreads, 2) sort_buckets_kernel(const uns
 // many as their keys ask for, kParts in all, and the keys are placed by parts.  Up to eight keys of a part are left to the network, up
 // to kWarpKeys to a warp, more are a run of their own, of at most a 256th of the range: a key is placed three times at most, and of
 // 16384 keys at most 31 runs wait at any time.  (One bitonic sort of the bucket took 150 to 200 us: 925 K weights on 255 levels with
-// 10 % of others 349 us the whole call, 213 so; 4 M weights, 300 of them infinite 319, 239.)
+// 10 % of others 349 us the whole call, 188 so; 4 M weights, 300 of them infinite 319, 225.)
 constexpr unsigned kWarpKeys = 512;
 constexpr int kCoarse = 512;
 static_assert(kCoarse == kSortThreads, "a thread has one coarse stretch");
-__device__ __forceinline__ void sort_uneven_bucket(unsigned* x, int cnt, SortState* st, unsigned* keys, unsigned* bins) {
+__device__ __forceinline__ void sort_uneven_bucket(unsigned* x, int cnt, SortState* st, unsigned* keys, unsigned* bins, unsigned* source) {
   __shared__ uint2 runs[kCap / kWarpKeys];          // first place, keys
-  __shared__ unsigned full[kCap / 9];               // parts for a warp: first place << 16 | keys
+  __shared__ unsigned full[kCap / 9];               // parts of more than eight keys: first place << 16 | keys
   __shared__ int n_runs, n_full;
-  __shared__ unsigned part[kSortThreads / 32 + 1], lo_s[kSortThreads / 32], hi_s[kSortThreads / 32];
+  __shared__ unsigned part[kSortThreads / 32 + 1], lo_s, hi_s;
   __shared__ unsigned table[kCoarse];               // keys of a coarse stretch, then its first part << 16 | its parts
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  bool negative = false;
 #pragma unroll 8
   for (int i = tid; i < cnt; i += kSortThreads) {
     const unsigned v = __ldcg(x + i);
-    if (v == 0x80000000u) atomicOr(&st->zeros, 3);          // one value with positive zeros here: written again by the next kernel
-    keys[spread(i)] = key_of(value_of(v));
+    negative = negative || v == 0x80000000u;
+    source[i] = key_of(value_of(v));
   }
+  if (negative) atomicOr(&st->zeros, 3);            // one value with positive zeros here: written again by the next phase
   if (tid < 24 && cnt + tid < (cnt + 15) / 16 * 16 + 8) keys[spread((unsigned)(cnt + tid))] = 0xffffffffu;
-  if (tid == 0) {
-    runs[0] = make_uint2(0u, (unsigned)cnt);
-    n_runs = 1;
-  }
-  __syncthreads();
-  while (n_runs > 0) {
-    const uint2 run = runs[n_runs - 1];
-    const unsigned from = run.x, c = run.y;
-    unsigned k[kSortItems], lo = 0xffffffffu, hi = 0u;
-#pragma unroll
-    for (int j = 0; j < kSortItems; ++j)
-      if ((unsigned)(j * kSortThreads + tid) < c) {
-        k[j] = keys[spread(from + j * kSortThreads + tid)];
-        lo = min(lo, k[j]);
-        hi = max(hi, k[j]);
-      }
-    lo = __reduce_min_sync(0xffffffffu, lo);
-    hi = __reduce_max_sync(0xffffffffu, hi);
-    if (lane == 0) { lo_s[warp] = lo; hi_s[warp] = hi; }
-    table[tid] = 0u;
-#pragma unroll
-    for (int i = 0; i < kParts / 2 / kSortThreads; ++i) bins[i * kSortThreads + tid] = 0u;
-    __syncthreads();                                // (also: every thread has read the run)
+  unsigned from = 0, c = (unsigned)cnt;
+  if (tid == 0) n_runs = 0;
+  for (;;) {
     if (tid == 0) {
-      --n_runs;
+      lo_s = 0xffffffffu;
+      hi_s = 0u;
       n_full = 0;
     }
-    lo = __reduce_min_sync(0xffffffffu, lo_s[lane & (kSortThreads / 32 - 1)]);
-    hi = __reduce_max_sync(0xffffffffu, hi_s[lane & (kSortThreads / 32 - 1)]);
-    const unsigned span = hi - lo;
-    if (span == 0) {
-      __syncthreads();
-      continue;
+    table[tid] = 0u;
+#pragma unroll
+    for (int i = 0; i < kParts / 8 / kSortThreads; ++i) reinterpret_cast<uint4*>(bins)[i * kSortThreads + tid] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    unsigned lo = 0xffffffffu, hi = 0u;
+#pragma unroll 4
+    for (unsigned i = tid; i < c; i += kSortThreads) {
+      const unsigned k = source[i];
+      lo = min(lo, k);
+      hi = max(hi, k);
     }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0) {
+      atomicMin(&lo_s, lo);
+      atomicMax(&hi_s, hi);
+    }
+    __syncthreads();
+    lo = lo_s;
+    hi = hi_s;
+    const unsigned span = hi - lo;
     const bool exact = span < (unsigned)kParts;     // a part for every value
     const int shift = exact ? 0 : 32 - __clz(span) - 9;
     if (!exact) {
-#pragma unroll
-      for (int j = 0; j < kSortItems; ++j)
-        if ((unsigned)(j * kSortThreads + tid) < c) atomicAdd(&table[(k[j] - lo) >> shift], 1u);
+#pragma unroll 4
+      for (unsigned i = tid; i < c; i += kSortThreads) atomicAdd(&table[(source[i] - lo) >> shift], 1u);
       __syncthreads();
       const unsigned parts = min(1u + table[tid] * (unsigned)(kParts - kCoarse) / c, 1u << min(shift, 15));        // (16384 x 15872 fits)
       const unsigned first = block_exclusive<kSortThreads / 32>(parts, part);
@@ -804,21 +868,17 @@ __device__ __forceinline__ void sort_uneven_bucket(unsigned* x, int cnt, SortSta
       return (e >> 16) + __umulhi(d << (32 - shift), e & 0xffffu);
     };
     // the next place of a key's part; a warp whose keys are of one part (a value repeated: the bucket comes in the order of its parts)
-    // asks once (11000 equal keys one by one take 20 us)
-    auto next_of = [&](unsigned key, bool in) {
-      const unsigned p = in ? part_of(key) : 0xffffffffu, s = (p & 1u) * 16u;
-      const unsigned p0 = __shfl_sync(0xffffffffu, p, 0);
+    // asks once
+    auto next_of = [&](unsigned p, bool in) {
+      const unsigned s = (p & 1u) * 16u, p0 = __shfl_sync(0xffffffffu, p, 0);
+      const bool one = __all_sync(0xffffffffu, in && p == p0);
       unsigned v = 0;
-      if (__all_sync(0xffffffffu, in && p == p0)) {
-        if (lane == 0) v = atomicAdd(&bins[p >> 1], 32u << s);
-        return ((__shfl_sync(0xffffffffu, v, 0) >> s) & 0xffffu) + lane;
-      }
-      if (in) v = atomicAdd(&bins[p >> 1], 1u << s);
-      return (v >> s) & 0xffffu;
+      if (one ? lane == 0 : in) v = atomicAdd(&bins[p >> 1], (one ? 32u : 1u) << s);
+      const unsigned v0 = __shfl_sync(0xffffffffu, v, 0);
+      return one ? ((v0 >> s) & 0xffffu) + lane : (v >> s) & 0xffffu;
     };
-#pragma unroll
-    for (int j = 0; j < kSortItems; ++j)
-      if ((unsigned)(j * kSortThreads + warp * 32) < c) next_of(k[j], (unsigned)(j * kSortThreads + tid) < c);
+#pragma unroll 2
+    for (unsigned i = tid; i - lane < c; i += kSortThreads) next_of(i < c ? part_of(source[i]) : 0xffffffffu, i < c);
     __syncthreads();
     constexpr int Q = kParts / 8 / kSortThreads;
     uint4* mine = reinterpret_cast<uint4*>(bins) + tid * Q;
@@ -842,27 +902,33 @@ __device__ __forceinline__ void sort_uneven_bucket(unsigned* x, int cnt, SortSta
     }
     __syncthreads();
     // every key takes its part's next place: the word of a part then says where it ends
-#pragma unroll
-    for (int j = 0; j < kSortItems; ++j)
-      if ((unsigned)(j * kSortThreads + warp * 32) < c) {
-        const bool in = (unsigned)(j * kSortThreads + tid) < c;
-        const unsigned to = next_of(k[j], in);
-        if (in) keys[spread(from + to)] = k[j];
-      }
-    __syncthreads();
-    if (exact) continue;
-    for (int w = tid; w < kParts / 2; w += kSortThreads) {
-      const unsigned ends = bins[w], a = w ? bins[w - 1] >> 16 : 0u, b = ends & 0xffffu, z = ends >> 16;
-      auto look = [&](unsigned first, unsigned end) {
-        if (end - first > kWarpKeys) runs[atomicAdd(&n_runs, 1)] = make_uint2(from + first, end - first);
-        else if (end - first > 8) full[atomicAdd(&n_full, 1)] = (from + first) << 16 | (end - first);
-      };
-      look(a, b);
-      look(b, z);
+#pragma unroll 2
+    for (unsigned i = tid; i - lane < c; i += kSortThreads) {
+      const unsigned k = i < c ? source[i] : 0u, to = next_of(i < c ? part_of(k) : 0xffffffffu, i < c);
+      if (i < c) keys[spread(from + to)] = k;
     }
     __syncthreads();
-    for (int i = warp; i < n_full; i += kSortThreads / 32) sort_by_warp(keys, full[i] >> 16, full[i] & 0xffffu);
+    if (!exact) {
+      for (int w = tid; w < kParts / 2; w += kSortThreads) {
+        const unsigned ends = bins[w], a = w ? bins[w - 1] >> 16 : 0u, b = ends & 0xffffu, z = ends >> 16;
+        if (b - a > 8) full[atomicAdd(&n_full, 1)] = (from + a) << 16 | (b - a);
+        if (z - b > 8) full[atomicAdd(&n_full, 1)] = (from + b) << 16 | (z - b);
+      }
+      __syncthreads();
+      for (int i = warp; i < n_full; i += kSortThreads / 32) {
+        const unsigned at = full[i] >> 16, of = full[i] & 0xffffu;
+        if (one_value(keys, at, of)) continue;
+        if (of <= kWarpKeys) sort_by_warp(keys, at, of);
+        else if (lane == 0) runs[atomicAdd(&n_runs, 1)] = make_uint2(at, of);
+      }
+      __syncthreads();
+    }
+    if (n_runs == 0) break;
+    from = runs[n_runs - 1].x;
+    c = runs[n_runs - 1].y;
+    for (unsigned i = tid; i < c; i += kSortThreads) source[i] = keys[spread(from + i)];
     __syncthreads();
+    if (tid == 0) --n_runs;
   }
   sort_small_parts(keys, cnt);
 #pragma unroll 8
@@ -870,183 +936,400 @@ __device__ __forceinline__ void sort_uneven_bucket(unsigned* x, int cnt, SortSta
   __syncthreads();
 }
 
-__global__ void __launch_bounds__(kSortThreads, 2) sort_uneven_kernel(SortState* st, const uint2* uneven, unsigned* x) {
+// After the buckets: those left to be divided again, then the order of the zeros where there are some of either sign.  They are
+// equal and belong in the order of the input: by chunks their number and their signs (a bit each), then their place in the sorted
+// array, where they are written again.
+constexpr int kSignWords = kCap / 32;
+constexpr int kFinishSmem = kSortSmem + kCap * 4;
+__global__ void __launch_bounds__(kSortThreads, 1) sort_finish_kernel(const unsigned* in, long long n, SortState* st, const uint2* uneven, unsigned* counts,
+                                                                      unsigned* all_signs, unsigned* x) {
   extern __shared__ __align__(16) unsigned sm[];
+  __shared__ unsigned of_warp[kSortThreads / 32], begin_s;
   wait_for_last_kernel();
   let_next_kernel_start();
-  const int n = st->n_uneven;
-  for (int i = blockIdx.x; i < n; i += gridDim.x) sort_uneven_bucket(x + uneven[i].x, (int)uneven[i].y, st, sm, sm + kCap + 16);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (!run_phase(st, 4 * kLevels, (unsigned)st->n_uneven, [&](unsigned i) { sort_uneven_bucket(x + uneven[i].x, (int)uneven[i].y, st, sm, sm + kCap + 16, sm + kSortSmem / 4); })) return;
+  if (__ldcg(&st->zeros) != 3) return;
+  constexpr int kRows = kCap / kSortThreads;
+  static_assert(kRows == 32 && kSignWords == kSortThreads, "a lane keeps a row's word, a thread writes one");
+  const unsigned chunks = (unsigned)((n + kCap - 1) / kCap);
+  if (!run_phase(st, 4 * kLevels + 1, chunks, [&](unsigned chunk) {
+        sm[tid] = 0u;
+        // a warp has 32 rows of 32 neighbouring weights
+        const long long i0 = (long long)chunk * kCap + warp * (32 * kRows) + lane;
+        unsigned zeros = 0, negative = 0;              // zeros of the lane's row; the lane's own negative ones, a bit a row
+#pragma unroll
+        for (int j = 0; j < kRows; ++j) {
+          const unsigned v = i0 + 32 * j < n ? __ldcg(in + i0 + 32 * j) : 1u;
+          const unsigned row = __ballot_sync(0xffffffffu, value_of(v) == 0u);
+          if (lane == j) zeros = row;
+          negative |= v == 0x80000000u ? 1u << j : 0u;
+        }
+        const unsigned mine = __reduce_add_sync(0xffffffffu, (unsigned)__popc(zeros));
+        if (lane == 0) of_warp[warp] = mine;
+        __syncthreads();
+        const unsigned of = lane < kSortThreads / 32 ? of_warp[lane] : 0u;
+        unsigned at = __reduce_add_sync(0xffffffffu, lane < warp ? of : 0u);
+        const unsigned all = __reduce_add_sync(0xffffffffu, of);
+#pragma unroll
+        for (int j = 0; j < kRows; ++j) {
+          const unsigned row = __shfl_sync(0xffffffffu, zeros, j);
+          if ((negative >> j) & 1u) {
+            const unsigned i = at + (unsigned)__popc(row & ((1u << lane) - 1u));
+            atomicOr(&sm[i >> 5], 1u << (i & 31u));
+          }
+          at += (unsigned)__popc(row);
+        }
+        __syncthreads();
+        if (32u * tid < all) __stcg(all_signs + (size_t)chunk * kSignWords + tid, sm[tid]);
+        if (tid == 0) __stcg(counts + chunk, all);
+      }))
+    return;
+  if (warp == 0) {
+    long long l = 0, h = n;                       // the first place of x that does not lie before the zeros
+    while (l < h) {
+      const long long step = (h - l + 31) / 32, at = l + lane * step;
+      const bool before = at < h && key_of(value_of(__ldcg(x + at))) < 0x80000000u;
+      const int c = 32 - __clz(__ballot_sync(0xffffffffu, before));
+      if (c == 0) break;
+      l += (c - 1) * step + 1;
+      h = min(h, l + step - 1);
+    }
+    if (lane == 0) begin_s = (unsigned)l;
+  }
+  run_phase(st, 4 * kLevels + 2, chunks, [&](unsigned chunk) {
+    const unsigned all = __ldcg(counts + chunk);
+    if (all == 0u) return;
+    unsigned before = 0;
+    for (unsigned i = tid; i < chunk; i += kSortThreads) before += __ldcg(counts + i);
+    before = __reduce_add_sync(0xffffffffu, before);
+    if (lane == 0) of_warp[warp] = before;
+    if (32u * tid < all) sm[tid] = __ldcg(all_signs + (size_t)chunk * kSignWords + tid);
+    __syncthreads();
+    unsigned* to = x + (begin_s + __reduce_add_sync(0xffffffffu, lane < kSortThreads / 32 ? of_warp[lane] : 0u));
+#pragma unroll 4
+    for (unsigned i = tid; i < all; i += kSortThreads) __stcg(to + i, (sm[i >> 5] >> (i & 31u)) << 31);
+  });
 }
 
-// ---- the general sort: four stable passes of eight bits ---------------------------------------------------
-constexpr int kRadixThreads = 512, kRadixWarps = kRadixThreads / 32, kRadixRows = 16, kRadixTile = kRadixThreads * kRadixRows;
-constexpr int kRadixGridMax = 512;
-__device__ __forceinline__ unsigned digit_of(unsigned raw, int shift) { return (key_of(value_of(raw)) >> shift) & 255u; }
+// ---- segments: more keys in one fine bin than a bucket holds ---------------------------------------------------
+// A value repeated so often, by itself or among others, or a narrow clump.  Level by level: the segment's range is divided into 256 to
+// 2048 equal parts, and the pivot, the median of 32 of its keys, has a part of its own between the smaller and the larger keys of the
+// part it lies in.  A segment without other keys is left as it is.  Parts of one value each are written from their counts; otherwise
+// the other keys are partitioned (and the pivot's written), parts of few keys become buckets together, and a part of more keys than
+// a bucket holds is a segment of the next level, whose range has eight bits less at least.
+// 45 M weights, the whole call: 255 levels with 10 % of other weights 990 us, eight clumps of 0.1 % width 1430 (a radix
+// sort of the whole array in four passes 1785 and 2037; CUB's 1270 and, with the marking of before, 2775); eight levels: 76 us here.
+constexpr int kSegThreads = 512, kSegTile = 8192, kSegItems = kSegTile / kSegThreads, kSegPartsLog = 11;
+constexpr int kSegPer = 5, kSegSlots = kSegThreads * kSegPer;       // parts of a thread; of a segment: at most 2048 and two more
+constexpr int kSegSmem = (2 * kSegSlots + 4 + kSegTile) * 4;
+static_assert((1 << kSegPartsLog) + 2 <= kSegSlots && kCap % kSegTile == 0 && kCap / 64 + 2 <= kPartsOfChunk && kCap >= 64 << 8, "sizes of a segment's parts");
 
-__global__ void __launch_bounds__(kRadixThreads, 2) sort_general_kernel(const unsigned* __restrict__ in, long long n, const SortState* __restrict__ st,
-                                                                        unsigned* x, unsigned* tmp, unsigned* counts) {
-  namespace cg = cooperative_groups;
-  if (!st->general && st->zeros != 3) return;
-  __shared__ unsigned keys[kRadixTile];
-  __shared__ unsigned short warp_cnt[kRadixWarps][256];
-  __shared__ unsigned run[256], delta[256], part[kRadixWarps + 1];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, G = gridDim.x;
-  const long long tiles = (n + kRadixTile - 1) / kRadixTile;
-  const long long tile0 = tiles * blockIdx.x / G, tile1 = tiles * (blockIdx.x + 1) / G;
-  const long long from = tile0 * kRadixTile, to = min(n, tile1 * kRadixTile);
-  if (!st->general) {
-    // Sorted but for the zeros, which belong in the order of the input: count them, find their place, write them again.
-    const int full = (int)((to - from + kRadixThreads - 1) / kRadixThreads);
-    int mine = 0;
-#pragma unroll 8
-    for (int j = 0; j < full; ++j) {
-      const long long i = from + (long long)j * kRadixThreads + tid;
-      if (i < to) mine += value_of(in[i]) == 0u;
-    }
-    mine = (int)__reduce_add_sync(0xffffffffu, (unsigned)mine);
-    if (tid == 0) run[0] = 0u;
-    __syncthreads();
-    if (lane == 0) atomicAdd(&run[0], (unsigned)mine);
-    __syncthreads();
-    if (tid == 0) __stcg(counts + blockIdx.x, run[0]);
-    cg::this_grid().sync();
-    if (run[0] == 0u) return;
-    unsigned place = 0;
-    if (warp == 0) {
-      for (int c = lane; c < (int)blockIdx.x; c += 32) place += __ldcg(counts + c);
-      place = __reduce_add_sync(0xffffffffu, place);
-      long long l = 0, h = n;                       // first place of x that does not lie before the zeros
-      while (l < h) {
-        const long long step = (h - l + 31) / 32, at = l + lane * step;
-        const bool before = at < h && key_of(value_of(__ldcg(x + at))) < 0x80000000u;
-        const int c = 32 - __clz(__ballot_sync(0xffffffffu, before));
-        if (c == 0) break;
-        l += (c - 1) * step + 1;
-        h = min(h, l + step - 1);
-      }
-      if (lane == 0) run[1] = (unsigned)l + place;
-    }
-    __syncthreads();
-    unsigned next = run[1];
-    for (int j = 0; j < full; ++j) {
-      const long long i = from + (long long)j * kRadixThreads + tid;
-      const unsigned v = i < to ? in[i] : 1u;
-      const bool zero = value_of(v) == 0u;
-      if (!__syncthreads_or(zero)) continue;
-      const unsigned e = block_exclusive<kRadixWarps>(zero ? 1u : 0u, part);
-      if (zero) __stcg(x + next + e, v);
-      next += part[kRadixWarps];
-      __syncthreads();
-    }
-    return;
-  }
-  for (int pass = 0; pass < 4; ++pass) {
-    const unsigned* src = pass == 0 ? in : (pass & 1) ? tmp : x;
-    unsigned* dst = (pass & 1) ? x : tmp;
-    const int shift = 8 * pass;
-    if (tid < 256) run[tid] = 0u;
-    __syncthreads();
-    for (long long i0 = from; i0 < to; i0 += 8 * kRadixThreads) {
-      unsigned v[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j)
-        if (i0 + j * kRadixThreads + tid < to) v[j] = __ldcg(src + i0 + j * kRadixThreads + tid);
-#pragma unroll
-      for (int j = 0; j < 8; ++j)
-        if (i0 + j * kRadixThreads + tid < to) atomicAdd(&run[digit_of(v[j], shift)], 1u);
-    }
-    __syncthreads();
-    if (tid < 256) __stcg(counts + blockIdx.x * 256 + tid, run[tid]);
-    cg::this_grid().sync();
-    // where this CTA's keys of every digit go: after all smaller digits, and after the CTAs before it
-    unsigned mine = 0, all = 0;
-    if (tid < 256) {
-#pragma unroll 8
-      for (int c = 0; c < G; ++c) {
-        const unsigned v = __ldcg(counts + c * 256 + tid);
-        all += v;
-        mine += c < (int)blockIdx.x ? v : 0u;
-      }
-    }
-    const unsigned smaller = block_exclusive<kRadixWarps>(all, part);
-    if (tid < 256) run[tid] = smaller + mine;
-    for (long long t = tile0; t < tile1; ++t) {
-      const long long base = t * kRadixTile;
-      const int left = (int)min((long long)kRadixTile, n - base);
-      __syncthreads();
-      for (int i = lane; i < 128; i += 32) reinterpret_cast<unsigned*>(warp_cnt[warp])[i] = 0u;
+__global__ void __launch_bounds__(kSegThreads, 2) sort_segments_kernel(SortState* st, Segment* all_segments, int per_level, unsigned* all_counters,
+                                                                       uint2* extra, unsigned* x, unsigned* tmp) {
+  extern __shared__ __align__(16) unsigned sm[];
+  unsigned *count = sm, *delta = sm + kSegSlots + 4, *keys = delta + kSegSlots;          // [kSegSlots + 1], [kSegSlots], [kSegTile]
+  __shared__ unsigned part[kSegThreads / 32 + 1], tail[kSegThreads / 32], numbers[2];
+  __shared__ Segment fetched[2];
+  wait_for_last_kernel();
+  let_next_kernel_start();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int level = 0; level < kLevels; ++level) {
+    const unsigned long long number = __ldcg(&st->segments[level]);
+    const unsigned n_segments = (unsigned)(number >> 32), n_chunks = (unsigned)number;
+    if (n_segments == 0) return;
+    Segment* segments = all_segments + level * per_level;
+    auto fetch = [&](unsigned i, int slot) {
+      if (lane == 0) numbers[slot] = i;
+      if (lane < (int)(sizeof(Segment) / 4)) reinterpret_cast<unsigned*>(&fetched[slot])[lane] = __ldcg(reinterpret_cast<const unsigned*>(segments + i) + lane);
       __syncwarp();
-      // a warp has 512 neighbouring keys, 32 at a time in order
-      unsigned v[kRadixRows];
-      unsigned rank[kRadixRows];
-#pragma unroll
-      for (int j = 0; j < kRadixRows; ++j) {
-        const int i = warp * (32 * kRadixRows) + 32 * j + lane;
-        v[j] = i < left ? __ldcg(src + base + i) : 0u;
+    };
+    // the segment of a chunk: the last one whose first chunk does not come after it
+    auto find = [&](unsigned chunk, int slot) {
+      unsigned l = 0, h = n_segments;           // in [l, h)
+      while (h - l > 1) {
+        const unsigned step = (h - l + 31) / 32, at = l + lane * step;
+        const bool not_after = at < h && __ldcg(&segments[at].chunk) <= chunk;
+        l += (unsigned)(__popc(__ballot_sync(0xffffffffu, not_after)) - 1) * step;
+        h = min(h, l + step);
       }
+      fetch(l, slot);
+    };
+    // a chunk's places in the array
+    auto places = [&](const Segment& seg, unsigned chunk, unsigned& begin, unsigned& end) {
+      begin = seg.from + (chunk - seg.chunk) * kCap;
+      end = min(begin + kCap, seg.from + seg.keys);
+    };
+    // equal parts of 2^shift keys each, of one value if it is 0; part_of: the number of a key's part, with the pivot's
+    auto shift_of = [&](const Segment& seg) { return max(32 - __clz(seg.hi - seg.lo) - min(31 - __clz(seg.keys / 64), kSegPartsLog), 0); };
+    auto key_at = [&](const unsigned* p) { return key_of(value_of(__ldcg(p))); };
+    auto part_of = [&](const Segment& seg, unsigned key, int shift) { return ((key - seg.lo) >> shift) + (key > seg.pivot ? 2u : key == seg.pivot ? 1u : 0u); };
+    auto parts_of = [&](const Segment& seg, int shift) { return (int)((seg.hi - seg.lo) >> shift) + 3; };
+
+    bool go = run_phase(
+        st, 4 * level, n_chunks,
+        [&](unsigned chunk, int slot) {
+          find(chunk, slot);
+          Segment& seg = fetched[slot];
+          const unsigned k = key_at(x + seg.from + (unsigned)((unsigned long long)(seg.keys - 1) * lane / 31));
+          int less = 0, equal = 0;
 #pragma unroll
-      for (int j = 0; j < kRadixRows; ++j) {
-        const bool in_tile = warp * (32 * kRadixRows) + 32 * j + lane < left;
-        const unsigned d = digit_of(v[j], shift);
-        unsigned same = __ballot_sync(0xffffffffu, in_tile);
+          for (int l = 0; l < 32; ++l) {
+            const unsigned other = __shfl_sync(0xffffffffu, k, l);
+            less += other < k;
+            equal += other == k;
+          }
+          const unsigned middle = __ballot_sync(0xffffffffu, less <= 16 && less + equal > 16);
+          const unsigned pivot = __shfl_sync(0xffffffffu, k, __ffs(middle) - 1);
+          if (lane == 0) {
+            seg.pivot = pivot;
+            if (chunk == seg.chunk) __stcg(&segments[numbers[slot]].pivot, pivot);
+          }
+        },
+        [&](unsigned chunk, int slot, auto look_ahead) {
+          constexpr int kBatch = 16;                // (more would not stay in registers)
+          const Segment& seg = fetched[slot];
+          unsigned begin, end, v[kBatch];
+          places(seg, chunk, begin, end);
+          auto load = [&]() {
 #pragma unroll
-        for (int b = 0; b < 8; ++b) {
-          const unsigned w = __ballot_sync(0xffffffffu, (d >> b) & 1u);
-          same &= ((d >> b) & 1u) ? w : ~w;
+            for (int j = 0; j < kBatch; ++j)
+              if (begin + j * kSegThreads + tid < end) v[j] = __ldcg(x + begin + j * kSegThreads + tid);
+          };
+          load();
+          for (int d = tid; d < kSegSlots; d += kSegThreads) count[d] = 0u;
+          look_ahead();
+          __syncthreads();
+          const unsigned pivot = seg.pivot, keys_of = end - begin;
+          const int shift = shift_of(seg);
+          unsigned others = 0, signs = 0;
+          for (;;) {
+#pragma unroll
+            for (int j = 0; j < kBatch; ++j)
+              if (begin + j * kSegThreads + tid < end) {
+                const unsigned k = key_of(value_of(v[j]));
+                signs |= k != 0x80000000u ? 0u : v[j] == 0u ? 1u : 2u;
+                if (k != pivot) {
+                  ++others;
+                  atomicAdd(&count[part_of(seg, k, shift)], 1u);
+                }
+              }
+            begin += kBatch * kSegThreads;
+            if (begin >= end) break;
+            load();
+          }
+          signs = __reduce_or_sync(0xffffffffu, signs);
+          others = __reduce_add_sync(0xffffffffu, others);
+          if (lane == 0 && signs) atomicOr(&st->zeros, (int)signs);
+          unsigned& of_pivot = count[part_of(seg, pivot, shift)];
+          if (lane == 0 && others) atomicSub(&of_pivot, others);
+          if (tid == 0) atomicAdd(&of_pivot, keys_of);
+          const bool mixed = __syncthreads_or(others != 0);
+          unsigned* counters = all_counters + seg.chunk * kPartsOfChunk;
+          if (!mixed) {
+            if (tid == 0) atomicAdd(counters + part_of(seg, pivot, shift), keys_of);
+            return;
+          }
+          for (int d = tid; d < kSegSlots; d += kSegThreads) {
+            const unsigned c = count[d];
+            if (c) atomicAdd(counters + d, c);
+          }
+          if (tid == 0) {
+            segments[numbers[slot]].mixed = 1u;
+            st->mixed[level] = 1;
+          }
+        });
+    if (!go || __ldcg(&st->mixed[level]) == 0) return;
+
+    // Where the parts begin.  Parts of up to half a bucket that begin between the same multiples of half a bucket form one together.
+    go = run_phase(st, 4 * level + 1, n_segments, [&](unsigned i) {
+      constexpr unsigned kHalf = kCap / 2;
+      if (warp == 0) fetch(i, 0);
+      __syncthreads();
+      const Segment seg = fetched[0];
+      if (!seg.mixed) return;
+      const int shift = shift_of(seg), parts = parts_of(seg, shift), of_pivot = (int)part_of(seg, seg.pivot, shift);
+      unsigned* counters = all_counters + seg.chunk * kPartsOfChunk;
+      unsigned c[kSegPer], sum = 0, last = 0;            // last: keys of the last part that has any (the pivot's: more than any)
+#pragma unroll
+      for (int q = 0; q < kSegPer; ++q) {
+        const int d = tid * kSegPer + q;
+        c[q] = d < parts ? __ldcg(counters + d) : 0u;
+        sum += c[q];
+        if (c[q]) last = d == of_pivot ? 0xffffffffu : c[q];
+      }
+      const unsigned at = block_exclusive<kSegThreads / 32>(sum, part);
+      unsigned p = at;
+#pragma unroll
+      for (int q = 0; q < kSegPer; ++q) {
+        const int d = tid * kSegPer + q;
+        if (d < parts) __stcg(counters + d, seg.from + p);
+        if (d == of_pivot) {
+          __stcg(&segments[i].equal, seg.from + p);
+          __stcg(&segments[i].equal_to, seg.from + p + c[q]);
         }
-        const unsigned before = in_tile ? warp_cnt[warp][d] : 0u, below = __popc(same & ((1u << lane) - 1u));
-        rank[j] = before + below;
-        __syncwarp();
-        if (in_tile && below == 0) warp_cnt[warp][d] = (unsigned short)(before + __popc(same));
-        __syncwarp();
+        p += c[q];
       }
-      __syncthreads();
-      unsigned cnt = 0;
-      if (tid < 256) {
+      if (shift == 0) return;
+      unsigned before = last;                   // the same of the threads before
 #pragma unroll
-        for (int w = 0; w < kRadixWarps; ++w) {
-          const unsigned c = warp_cnt[w][tid];
-          warp_cnt[w][tid] = (unsigned short)cnt;
-          cnt += c;
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned u = __shfl_up_sync(0xffffffffu, before, o);
+        if (lane >= o && before == 0) before = u;
+      }
+      if (lane == 31) tail[warp] = before;
+      before = __shfl_up_sync(0xffffffffu, before, 1);
+      if (lane == 0) before = 0;
+      __syncthreads();
+      for (int w = warp - 1; w >= 0 && before == 0; --w) before = tail[w];
+      unsigned starts = 0;
+      p = at;
+#pragma unroll
+      for (int q = 0; q < kSegPer; ++q)
+        if (c[q]) {
+          const bool is_pivot = tid * kSegPer + q == of_pivot;
+          if (before == 0 || before > kHalf || c[q] > kHalf || is_pivot || (p - before) / kHalf != p / kHalf) starts |= 1u << q;
+          before = is_pivot ? 0xffffffffu : c[q];
+          p += c[q];
+        }
+      unsigned to = block_exclusive<kSegThreads / 32>((unsigned)__popc(starts), part);
+      const unsigned total = part[kSegThreads / 32];
+      p = at;
+#pragma unroll
+      for (int q = 0; q < kSegPer; ++q) {
+        if ((starts >> q) & 1u) {
+          count[to] = p;
+          delta[to++] = (unsigned)(tid * kSegPer + q);
+        }
+        p += c[q];
+      }
+      if (tid == 0) count[total] = seg.keys;
+      __syncthreads();
+      for (unsigned b = tid; b < total; b += kSegThreads) {
+        const unsigned from = seg.from + count[b], of = count[b + 1] - count[b];
+        const int d = (int)delta[b];
+        if (d == of_pivot) continue;
+        if (of > (unsigned)kCap) {              // (never at the last level, whose parts are of one value)
+          unsigned lo = seg.lo + ((unsigned)(d < of_pivot ? d : d - 2) << shift), hi = lo + min((1u << shift) - 1u, seg.hi - lo);
+          if (d == of_pivot - 1) hi = seg.pivot - 1u;
+          if (d == of_pivot + 1) lo = seg.pivot + 1u;
+          add_segment(st, all_segments + (level + 1) * per_level, level + 1, from, of, lo, hi);
+        } else {
+          extra[atomicAdd(&st->n_extra, 1)] = make_uint2(from, of);
         }
       }
-      const unsigned start = block_exclusive<kRadixWarps>(cnt, part);
-      if (tid < 256) {
-        delta[tid] = run[tid] - start;
-        run[tid] += cnt;
+    });
+    if (!go) return;
+
+    go = run_phase(st, 4 * level + 2, n_chunks, find, [&](unsigned chunk, int slot, auto look_ahead) {
+      const Segment seg = fetched[slot];
+      look_ahead();
+      if (!seg.mixed) return;
+      unsigned begin, end;
+      places(seg, chunk, begin, end);
+      const int shift = shift_of(seg), parts = parts_of(seg, shift);
+      const unsigned pivot = seg.pivot;
+      unsigned* counters = all_counters + seg.chunk * kPartsOfChunk;
+      if (shift == 0) {                         // written from the parts' beginnings
+        const int of_pivot = (int)part_of(seg, pivot, 0);
+        for (int d = tid; d < parts; d += kSegThreads) count[d] = __ldcg(counters + d);
+        __syncthreads();
+#pragma unroll 4
+        for (unsigned i = begin + tid; i < end; i += kSegThreads) {
+          int d = 0;
 #pragma unroll
-        for (int w = 0; w < kRadixWarps; ++w) warp_cnt[w][tid] = (unsigned short)(warp_cnt[w][tid] + start);
+          for (int s = 1 << kSegPartsLog; s > 0; s /= 2)
+            if (d + s < parts && count[d + s] <= i) d += s;
+          __stcg(x + i, raw_of(d == of_pivot ? pivot : seg.lo + (unsigned)(d < of_pivot ? d : d - 2)));
+        }
+        // zeros have become positive: if there are others, all are written again at the end
+        if (tid == 0 && seg.lo <= 0x80000000u && seg.hi >= 0x80000000u && (__ldcg(&st->zeros) & 2)) atomicOr(&st->zeros, 3);
+        return;
       }
-      __syncthreads();
+      for (; begin < end; begin += kSegTile) {
+        const int left = (int)min((unsigned)kSegTile, end - begin);
+        unsigned v[kSegItems], rank[kSegItems / 2];          // ranks of 16 bits
 #pragma unroll
-      for (int j = 0; j < kRadixRows; ++j)
-        if (warp * (32 * kRadixRows) + 32 * j + lane < left) keys[warp_cnt[warp][digit_of(v[j], shift)] + rank[j]] = v[j];
-      __syncthreads();
-      for (int i = tid; i < left; i += kRadixThreads) {
-        const unsigned v1 = keys[i];
-        __stcg(dst + delta[digit_of(v1, shift)] + i, v1);
+        for (int j = 0; j < kSegItems; ++j)
+          v[j] = j * kSegThreads + tid < left ? key_at(x + begin + j * kSegThreads + tid) : pivot;
+        for (int d = tid; d < kSegSlots; d += kSegThreads) count[d] = 0u;
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kSegItems; ++j) {
+          const unsigned r = v[j] != pivot ? atomicAdd(&count[part_of(seg, v[j], shift)], 1u) : 0u;
+          rank[j / 2] = (j & 1) ? rank[j / 2] | r << 16 : r;
+        }
+        __syncthreads();
+        unsigned c[kSegPer], g[kSegPer], sum = 0;
+#pragma unroll
+        for (int q = 0; q < kSegPer; ++q) {
+          c[q] = count[tid * kSegPer + q];
+          g[q] = c[q] ? atomicAdd(counters + tid * kSegPer + q, c[q]) : 0u;
+          sum += c[q];
+        }
+        unsigned e = block_exclusive<kSegThreads / 32>(sum, part);
+        const int others = (int)part[kSegThreads / 32];
+#pragma unroll
+        for (int q = 0; q < kSegPer; ++q) {
+          count[tid * kSegPer + q] = e;
+          delta[tid * kSegPer + q] = g[q] - e;
+          e += c[q];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kSegItems; ++j)
+          if (v[j] != pivot) keys[count[part_of(seg, v[j], shift)] + ((rank[j / 2] >> ((j & 1) * 16)) & 0xffffu)] = v[j];
+        __syncthreads();
+#pragma unroll 4
+        for (int i = tid; i < others; i += kSegThreads) {
+          const unsigned k = keys[i];
+          __stcg(tmp + (delta[part_of(seg, k, shift)] + (unsigned)i), raw_of(k));
+        }
       }
-    }
-    cg::this_grid().sync();
+      if (tid == 0 && seg.lo <= 0x80000000u && seg.hi >= 0x80000000u && (__ldcg(&st->zeros) & 2)) atomicOr(&st->zeros, 3);
+    });
+    if (!go) return;
+
+    // back into the array, and the next level's counters cleared
+    const unsigned next_chunks = level + 1 < kLevels ? (unsigned)__ldcg(&st->segments[level + 1]) : 0u;
+    go = run_phase(st, 4 * level + 3, n_chunks, find, [&](unsigned chunk, int slot, auto look_ahead) {
+      const Segment seg = fetched[slot];
+      look_ahead();
+      for (unsigned c = chunk; c < next_chunks; c += n_chunks)
+        if (tid < kPartsOfChunk) __stcg(all_counters + c * kPartsOfChunk + tid, 0u);
+      if (!seg.mixed || shift_of(seg) == 0) return;
+      unsigned begin, end;
+      places(seg, chunk, begin, end);
+      const unsigned pivot = raw_of(seg.pivot);
+#pragma unroll 16
+      for (unsigned i = begin + tid; i < end; i += kSegThreads) __stcg(x + i, i >= seg.equal && i < seg.equal_to ? pivot : __ldcg(tmp + i));
+    });
+    if (!go) return;
   }
 }
 
 size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
+// Segments of a level: more than kCap keys each.  Their chunks: at most two for every kCap keys.  Buckets made from a segment: a part of
+// more than half a bucket, or what begins between two multiples of half a bucket; twice where the pivot lies between.
+int64_t most_segments(int64_t n) { return n / kCap + 1; }
+int64_t most_extra(int64_t n) { return kLevels * 7 * (n / kCap + 1); }
 struct Layout {
-  size_t state, samples, table, fine, begins, first, cursor, uneven, counts, tmp, total;
+  size_t state, samples, table, fine, begins, first, cursor, uneven, segments, counters, extra, tmp, total;
 };
 Layout layout(int64_t n) {
   Layout l;
   size_t off = 0;
-  l.state = off; off += 256;
+  l.state = off; off += kStateBytes;
   l.samples = off; off += up256(kSamples * 4);
   l.table = off; off += up256(kBins * 4);
   l.fine = off; off += up256(kFineMax * 4);
   l.begins = off; off += up256(kFineMax / 4);
   l.first = off; off += up256((kMaxBuckets + 1) * 4);
   l.cursor = off; off += up256(kMaxBuckets * 4);
-  l.uneven = off; off += up256(kMaxBuckets * 8);
-  l.counts = off; off += up256(kRadixGridMax * 256 * 4);
+  l.uneven = off; off += up256((kMaxBuckets + most_extra(n)) * sizeof(uint2));
+  l.segments = off; off += up256(kLevels * most_segments(n) * sizeof(Segment));
+  l.counters = off; off += up256(2 * most_segments(n) * kPartsOfChunk * 4);
+  l.extra = off; off += up256(most_extra(n) * sizeof(uint2));
   l.tmp = off; off += up256((size_t)n * 4);
   l.total = off;
   return l;
@@ -1077,16 +1360,18 @@ cudaError_t launch_dbci_sort(const float* weights, int64_t n, float* sorted, voi
   unsigned* first = reinterpret_cast<unsigned*>(base + l.first);
   unsigned* cursor = reinterpret_cast<unsigned*>(base + l.cursor);
   uint2* uneven = reinterpret_cast<uint2*>(base + l.uneven);
-  unsigned* counts = reinterpret_cast<unsigned*>(base + l.counts);
+  Segment* segments = reinterpret_cast<Segment*>(base + l.segments);
+  unsigned* counters = reinterpret_cast<unsigned*>(base + l.counters);
+  uint2* extra = reinterpret_cast<uint2*>(base + l.extra);
   unsigned* tmp = reinterpret_cast<unsigned*>(base + l.tmp);
   const unsigned* in = reinterpret_cast<const unsigned*>(weights);
   unsigned* x = reinterpret_cast<unsigned*>(sorted);
-  static PerDeviceFlag f_count, f_part_l, f_part_s, f_sort, f_single, f_uneven;
+  static PerDeviceFlag f_count, f_part_l, f_part_s, f_sort, f_single, f_segments, f_finish;
   const int sms = current_sm_count();
   cudaError_t e;
   if (n <= kCap) {
     if ((e = opt_in(sort_buckets_kernel<true>, kSortSmem, f_single)) != cudaSuccess) return e;
-    e = launch_after(sort_buckets_kernel<true>, 1, kSortThreads, kSortSmem, s, in, (long long)n, st, (const unsigned*)first, x, uneven);
+    e = launch_after(sort_buckets_kernel<true>, 1, kSortThreads, kSortSmem, s, in, (long long)n, st, (const unsigned*)first, (const uint2*)extra, x, uneven);
   } else {
     constexpr int L = 24, S = 4;
     if ((e = opt_in(sort_count_kernel, kCountSmem, f_count)) != cudaSuccess) return e;
@@ -1103,32 +1388,27 @@ cudaError_t launch_dbci_sort(const float* weights, int64_t n, float* sorted, voi
     e = launch_after(sort_count_kernel, (unsigned)(count_tiles < 2 * sms ? count_tiles : 2 * sms), kCountThreads, kCountSmem, s, in, (long long)n, st,
                      (const unsigned*)table, fine);
     if (e != cudaSuccess) return e;
-    e = launch_after(sort_map_kernel, 1, kMapThreads, 0, s, (long long)n, target, st, fine, (const unsigned*)samples, (const unsigned*)table, begins, first, cursor);
+    e = launch_after(sort_map_kernel, 1, kMapThreads, 0, s, (long long)n, target, st, (const unsigned*)fine, begins, first, cursor, segments);
     if (e != cudaSuccess) return e;
     const bool large = n >= (int64_t)kPartThreads * L * sms;
     const int64_t tile = kPartThreads * (large ? L : S), tiles = (n + tile - 1) / tile;
     const unsigned grid = (unsigned)(tiles < sms ? tiles : sms);
     e = launch_after(large ? sort_partition_kernel<L> : sort_partition_kernel<S>, grid, kPartThreads, large ? partition_smem<L>() : partition_smem<S>(), s,
-                     in, (long long)n, (const SortState*)st, (const unsigned*)table, (const unsigned*)begins, cursor, x);
+                     in, (long long)n, (const SortState*)st, (const unsigned*)table, (const unsigned*)begins, cursor, x, segments, counters);
+    if (e != cudaSuccess) return e;
+    if ((e = opt_in(sort_segments_kernel, kSegSmem, f_segments)) != cudaSuccess) return e;
+    const int64_t chunks = 2 * most_segments(n);
+    e = launch_after(sort_segments_kernel, (unsigned)(chunks < 2 * sms ? chunks : 2 * sms), kSegThreads, kSegSmem, s, st, segments, (int)most_segments(n), counters,
+                     extra, x, tmp);
     if (e != cudaSuccess) return e;
     const int64_t most = 2 * (n / target) + 2;
-    e = launch_after(sort_buckets_kernel<false>, (unsigned)(most < 2 * sms ? most : 2 * sms), kSortThreads, kSortSmem, s, in, (long long)n, st, (const unsigned*)first, x, uneven);
+    e = launch_after(sort_buckets_kernel<false>, (unsigned)(most < 2 * sms ? most : 2 * sms), kSortThreads, kSortSmem, s, in, (long long)n, st, (const unsigned*)first, (const uint2*)extra, x, uneven);
   }
   if (e != cudaSuccess) return e;
-  if ((e = opt_in(sort_uneven_kernel, kSortSmem, f_uneven)) != cudaSuccess) return e;
-  const int64_t uneven_most = n / 256 + 1;
-  e = launch_after(sort_uneven_kernel, (unsigned)(n <= kCap ? 1 : uneven_most < 2 * sms ? uneven_most : 2 * sms), kSortThreads, kSortSmem, s, st, (const uint2*)uneven, x);
-  if (e != cudaSuccess) return e;
-  int per_sm = 0;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sort_general_kernel, kRadixThreads, 0)) != cudaSuccess) return e;
-  const int64_t radix_tiles = (n + kRadixTile - 1) / kRadixTile;
-  int64_t grid = (int64_t)per_sm * sms;
-  grid = grid < kRadixGridMax ? grid : kRadixGridMax;
-  grid = grid < radix_tiles ? grid : radix_tiles;
-  long long n_arg = n;
-  const SortState* st_arg = st;
-  void* args[] = {(void*)&in, (void*)&n_arg, (void*)&st_arg, (void*)&x, (void*)&tmp, (void*)&counts};
-  return cudaLaunchCooperativeKernel((const void*)sort_general_kernel, dim3((unsigned)grid), dim3(kRadixThreads), args, 0, s);
+  if ((e = opt_in(sort_finish_kernel, kFinishSmem, f_finish)) != cudaSuccess) return e;
+  const int64_t pieces = n / 256 + 1;                    // buckets of an array of that size, and more
+  return launch_after(sort_finish_kernel, (unsigned)(n <= kCap ? 1 : pieces < sms ? pieces : sms), kSortThreads, kFinishSmem, s, in, (long long)n, st,
+                      (const uint2*)uneven, counters, tmp, x);
 }
 
 }  // namespace lcd

@@ -1272,3 +1272,85 @@ def test_dbci_sort_of_unevenly_spread_keys(kind, n):
     w = rng.permutation(_uneven(kind, n, rng))
     r = lcd.dbci(torch.from_numpy(w).cuda())
     assert np.array_equal(r["sorted"].cpu().numpy().view(np.int32), np.sort(w, kind="stable").view(np.int32))
+
+
+def _dense_places(kind, n, rng):
+    ulps = lambda at, spread, size: (np.float32(at).view(np.int32) + rng.integers(0, spread, size)).astype(np.int32).view(np.float32)
+    w = rng.normal(0, 0.02, n).astype(np.float32)
+    if kind == "levels":                     # values repeated among others
+        at = rng.uniform(0, 1, n) < 0.9
+        w[at] = np.round(w[at] / np.float32(0.007)) * np.float32(0.007)
+    elif kind == "one":                      # one value, and a few keys of its fine bin that hardly any sample shows
+        w[:] = 0.25
+        w[rng.integers(0, n, 7)] = ulps(0.25, 40, 7)
+    elif kind == "nested":                   # clumps within clumps: several levels of segments
+        for b, share in ((20, 0.9), (12, 0.7), (4, 0.5)):
+            at = rng.uniform(0, 1, n) < share
+            w[at] = ulps(0.03125, 1 << b, at.sum())
+    elif kind == "ends":                     # the extreme values repeated, and what no sample shows beyond them
+        w = np.clip(w, -0.03, 0.03)
+        w[rng.integers(0, n, 5)] = [-np.inf, -1e30, 1e-30, 3.0, np.inf]
+        w[rng.integers(0, n, 3)] = ulps(0.03, 300, 3)
+    elif kind == "zeros":                    # zeros of either sign, subnormal numbers between and around them
+        at = rng.uniform(0, 1, n) < 0.7
+        w[at] = rng.choice(np.array([0.0, -0.0], np.float32), at.sum())
+        few = rng.integers(0, n, n // 100)
+        w[few] = ulps(1e-44, 1 << 12, len(few)) * rng.choice(np.array([-1, 1], np.float32), len(few))
+    else:                                    # "negative zeros" alone, and others
+        w[::2] = -0.0
+    return w
+
+
+@pytest.mark.parametrize("n", [20_000, 131_077, 700_001])
+@pytest.mark.parametrize("kind", ["levels", "one", "nested", "ends", "zeros", "negative zeros"])
+def test_dbci_sort_of_more_keys_in_one_place_than_a_bucket_holds(kind, n):
+    rng = np.random.default_rng(n)
+    w = rng.permutation(_dense_places(kind, n, rng))
+    r = lcd.dbci(torch.from_numpy(w).cuda())
+    assert np.array_equal(r["sorted"].cpu().numpy().view(np.int32), np.sort(w, kind="stable").view(np.int32))
+
+
+def _captured_dbci(w, n_words):
+    # the C call into a graph: (graph, its buffers)
+    from ctypes import byref, c_size_t, c_void_p
+    lib = lcd.binding.lib
+    need = c_size_t(0)
+    assert lib.lcd_dbci_workspace_bytes(w.numel(), 4096, byref(need)) == 0
+    buffers = [torch.empty(need.value, dtype=torch.uint8, device="cuda"), torch.empty(4096, device="cuda"),
+               torch.empty(n_words, dtype=torch.int32, device="cuda"), torch.empty(w.numel(), device="cuda"), torch.empty(64, dtype=torch.uint8, device="cuda")]
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g):
+        assert lib.lcd_dbci(c_void_p(w.data_ptr()), w.numel(), c_void_p(buffers[0].data_ptr()), need.value, c_void_p(buffers[1].data_ptr()), 4096,
+                            c_void_p(buffers[2].data_ptr()), c_void_p(buffers[3].data_ptr()), c_void_p(buffers[4].data_ptr()),
+                            c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
+    return g, buffers
+
+
+@pytest.mark.parametrize("n", [10_000, 200_000])
+def test_dbci_in_a_graph(n):
+    # no kernel needs all of its CTAs on the GPU at once (a cooperative launch waits for other streams' kernels to leave, and fails where
+    # a process has only some of the multiprocessors), and a replay takes what the weights have become
+    from cuda.bindings import driver
+    w = torch.empty(n, device="cuda")
+    g, (_, _, labels, srt, _) = _captured_dbci(w, n)
+    graph = driver.CUgraph(g.raw_cuda_graph())
+    err, _, count = driver.cuGraphGetNodes(graph)
+    err, nodes, _ = driver.cuGraphGetNodes(graph, count)
+    kernels = 0
+    for node in nodes:
+        err, kind = driver.cuGraphNodeGetType(node)
+        if kind != driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            continue
+        kernels += 1
+        err, value = driver.cuGraphKernelNodeGetAttribute(node, driver.CUlaunchAttributeID.CU_LAUNCH_ATTRIBUTE_COOPERATIVE)
+        assert err == driver.CUresult.CUDA_SUCCESS and not value.cooperative
+    assert kernels >= 6
+    g.instantiate()
+    rng = np.random.default_rng(n)
+    for kind in ("gauss", "levels", "zeros", "one"):
+        x = rng.permutation(_dense_places(kind, n, rng)) if kind != "gauss" else rng.normal(0, 0.02, n).astype(np.float32)
+        w.copy_(torch.from_numpy(x))
+        g.replay()
+        torch.cuda.synchronize()
+        assert np.array_equal(srt.cpu().numpy().view(np.int32), np.sort(x, kind="stable").view(np.int32))
+        assert torch.equal(labels, lcd.dbci(w)["labels"])
