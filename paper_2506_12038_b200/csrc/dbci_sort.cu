@@ -228,16 +228,17 @@ struct FineMap {
     const unsigned e = table[d >> shift];
     return (int)((e >> 16) + __umulhi(d << (32 - shift), e & 0xffffu));                   // (d below its bin) * parts >> shift
   }
-  // the keys of a fine bin
-  __device__ void bounds(int f, const unsigned* table, unsigned& lo, unsigned& hi) const {
+  // The keys of a fine bin.  bin: where to look for it, 0 or what an earlier fine bin left there.
+  __device__ void bounds(int f, const unsigned* table, int& bin, unsigned& lo, unsigned& hi) const {
     lo = 0u;
     hi = 0xffffffffu;
     if (f == 0) hi = kmin;
     if (f == last) lo = kmax;
     if (f == 0 || f == last) return;
-    int bin = 0;
-    for (int s = kBins / 2; s > 0; s /= 2)
-      if ((int)(table[bin + s] >> 16) <= f) bin += s;
+    if (bin == 0)
+      for (int s = kBins / 2; s > 0; s /= 2)
+        if ((int)(table[bin + s] >> 16) <= f) bin += s;
+    while (bin + 1 < kBins && (int)(table[bin + 1] >> 16) <= f) ++bin;
     const unsigned parts = table[bin] & 0xffffu;
     const unsigned long long part = (unsigned)f - (table[bin] >> 16);
     lo = kmin + ((unsigned)bin << shift) + (unsigned)(((part << shift) + parts - 1) / parts);
@@ -296,7 +297,7 @@ __device__ __forceinline__ void add_segment(SortState* st, Segment* segments, in
 // more, and there are at most two for every `target` keys.  Empty fine bins begin none.
 // begins: a word for sixteen fine bins, a bit for each that begins a bucket under the number of buckets begun before, less one.
 constexpr int kMapThreads = kFineMax / 32, kMapWarps = kMapThreads / 32;
-__global__ void __launch_bounds__(kMapThreads) sort_map_kernel(long long n, int target, SortState* st, const unsigned* fine, unsigned* __restrict__ begins,
+__global__ void __launch_bounds__(kMapThreads) sort_map_kernel(long long n, int target, SortState* st, const unsigned* fine, const unsigned* table, unsigned* __restrict__ begins,
                                                                unsigned* __restrict__ first, unsigned* __restrict__ cursor, Segment* segments) {
   constexpr int PER = 32;
   __shared__ unsigned part[kMapWarps + 1];
@@ -359,11 +360,15 @@ __global__ void __launch_bounds__(kMapThreads) sort_map_kernel(long long n, int 
     large |= c[j] > (unsigned)kCap ? 1u << j : 0u;
     p += c[j];
   }
-  for (; large; large &= large - 1) {             // (their ranges: see the partition)
+  int bin = 0;
+  for (; large; large &= large - 1) {
     const int j = __ffs(large) - 1;
+    unsigned lo, hi;
+    FineMap(st).bounds(tid * PER + j, table, bin, lo, hi);
+    if (hi == 0x7fffffffu) hi = 0x80000000u;          // (in a segment zeros of either sign count as positive ones)
     p = at;
     for (int i = 0; i < j; ++i) p += fine[tid * PER + i];
-    add_segment(st, segments, 0, p, fine[tid * PER + j], (unsigned)(tid * PER + j), 0u);
+    add_segment(st, segments, 0, p, fine[tid * PER + j], lo, hi);
   }
   if (tid == 0) {
     first[total] = (unsigned)n;
@@ -381,7 +386,7 @@ constexpr int partition_smem() { return kBins * 4 + kFineMax / 4 + kMaxBuckets *
 template <int ITEMS>
 __global__ void __launch_bounds__(kPartThreads, 1) sort_partition_kernel(const unsigned* __restrict__ in, long long n, const SortState* st,
                                                                          const unsigned* table_g, const unsigned* begins_g,
-                                                                         unsigned* cursor, unsigned* __restrict__ out, Segment* segments, unsigned* counters) {
+                                                                         unsigned* cursor, unsigned* __restrict__ out, unsigned* counters) {
   constexpr int TILE = kPartThreads * ITEMS, kLong = 128;
   extern __shared__ __align__(16) unsigned sm[];
   __shared__ unsigned part[kPartThreads / 32 + 1];
@@ -400,16 +405,8 @@ __global__ void __launch_bounds__(kPartThreads, 1) sort_partition_kernel(const u
   const bool many = st->n_buckets > kMaxBuckets / 2;
   for (int i = tid; i < kBins; i += kPartThreads) table[i] = table_g[i];
   for (int i = tid; i <= map.last / 16; i += kPartThreads) begins[i] = begins_g[i];
-  if (st->segments[0] != 0) {
-    // for the next kernel: ranges of the segments, given by their fine bins so far, and counters
-    __syncthreads();
-    const unsigned number = (unsigned)(st->segments[0] >> 32), all = (unsigned)st->segments[0] * kPartsOfChunk;
-    for (unsigned i = blockIdx.x * kPartThreads + tid; i < number; i += gridDim.x * kPartThreads) {
-      unsigned lo, hi;
-      map.bounds((int)segments[i].lo, table, lo, hi);
-      segments[i].lo = lo;
-      segments[i].hi = hi == 0x7fffffffu ? 0x80000000u : hi;          // (zeros of either sign count as positive ones there)
-    }
+  if (st->segments[0] != 0) {                             // the next kernel's counters
+    const unsigned all = (unsigned)st->segments[0] * kPartsOfChunk;
     for (unsigned i = blockIdx.x * kPartThreads + tid; i < all; i += gridDim.x * kPartThreads) counters[i] = 0u;
   }
   long long t0 = (long long)blockIdx.x * TILE;
@@ -772,20 +769,21 @@ __global__ void __launch_bounds__(kSortThreads, 2) sort_buckets_kernel(const uns
     if (!SINGLE) load();
     __syncthreads();
     if (loose) {
-      for (bool again = false;; again = true) {
-        // parts of more than eight keys; many in a part are often one value repeated, among others that are, in order as it is
-        if (far && (again || most >= 64)) {
+      for (int round = 0;; ++round) {
+        // parts of more than eight keys: up to three times where they are not many more (of 45 M Gaussian weights a few buckets have
+        // such a part); many in a part are often one value repeated, among others that are, in order as it is
+        if (far && (round > 0 || most >= 64)) {
           bool bad = false;
           for (int i = tid + 1; i < sorted; i += kSortThreads) {
             const unsigned u = keys[spread(i - 1)], v = keys[spread(i)];
             bad = bad || (u > v && (u != 0x80000000u || v != 0x7fffffffu));          // (zeros of either sign are equal)
           }
           if (!__syncthreads_or(bad)) break;
-          if (again) {
+          if (round == 3 || (round == 1 && most >= 64)) {
             if (tid == 0) uneven[atomicAdd(&st->n_uneven, 1)] = make_uint2(to0, (unsigned)sorted);
             break;
           }
-        } else if (again) {
+        } else if (round > 0) {
           break;
         }
         sort_small_parts(keys, sorted);
@@ -1388,13 +1386,13 @@ cudaError_t launch_dbci_sort(const float* weights, int64_t n, float* sorted, voi
     e = launch_after(sort_count_kernel, (unsigned)(count_tiles < 2 * sms ? count_tiles : 2 * sms), kCountThreads, kCountSmem, s, in, (long long)n, st,
                      (const unsigned*)table, fine);
     if (e != cudaSuccess) return e;
-    e = launch_after(sort_map_kernel, 1, kMapThreads, 0, s, (long long)n, target, st, (const unsigned*)fine, begins, first, cursor, segments);
+    e = launch_after(sort_map_kernel, 1, kMapThreads, 0, s, (long long)n, target, st, (const unsigned*)fine, (const unsigned*)table, begins, first, cursor, segments);
     if (e != cudaSuccess) return e;
     const bool large = n >= (int64_t)kPartThreads * L * sms;
     const int64_t tile = kPartThreads * (large ? L : S), tiles = (n + tile - 1) / tile;
     const unsigned grid = (unsigned)(tiles < sms ? tiles : sms);
     e = launch_after(large ? sort_partition_kernel<L> : sort_partition_kernel<S>, grid, kPartThreads, large ? partition_smem<L>() : partition_smem<S>(), s,
-                     in, (long long)n, (const SortState*)st, (const unsigned*)table, (const unsigned*)begins, cursor, x, segments, counters);
+                     in, (long long)n, (const SortState*)st, (const unsigned*)table, (const unsigned*)begins, cursor, x, counters);
     if (e != cudaSuccess) return e;
     if ((e = opt_in(sort_segments_kernel, kSegSmem, f_segments)) != cudaSuccess) return e;
     const int64_t chunks = 2 * most_segments(n);
