@@ -1310,6 +1310,64 @@ def test_dbci_sort_of_more_keys_in_one_place_than_a_bucket_holds(kind, n):
     assert np.array_equal(r["sorted"].cpu().numpy().view(np.int32), np.sort(w, kind="stable").view(np.int32))
 
 
+@pytest.mark.parametrize("kind", ["sorted", "reversed", "constant", "bf16", "levels", "pruned"])
+def test_dbci_sort_of_4_million_weights(kind):
+    # the partition's wide tiles: runs of a bucket as long as the tile, buckets and segments of one value
+    n = 4_000_003
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    w = torch.randn(n, generator=g, device="cuda") * 0.02
+    if kind in ("sorted", "reversed"):
+        w = torch.sort(w, descending=kind == "reversed").values
+    elif kind == "constant":
+        w = torch.full((n,), -0.75, device="cuda")
+    elif kind == "bf16":
+        w = w.bfloat16().float()
+    elif kind == "levels":                   # nine of ten on a grid
+        w = torch.where(torch.rand(n, generator=g, device="cuda") < 0.9, torch.round(w / 0.0007) * 0.0007, w)
+    else:
+        w = w * (torch.rand(n, generator=g, device="cuda") < 0.4)
+    r = lcd.dbci(w)
+    assert torch.equal(r["sorted"], torch.sort(w).values)
+    assert (r["sorted"].view(torch.int32) < 0).sum() == (w.view(torch.int32) < 0).sum()          # signs of zeros, too
+
+
+def test_dbci_sort_into_more_than_4096_buckets():
+    # 3068 values, each a little less often than a bucket holds, and smooth stretches of 100 keys between them: by the plan's and the
+    # map's rules 6137 buckets, of an array just within what the sort takes
+    at = torch.arange(3068, dtype=torch.int32, device="cuda") * 2734 + 0x3f800000
+    between = (at[:, None] + 1200 + 3 * torch.arange(100, dtype=torch.int32, device="cuda")).reshape(-1)
+    w = torch.cat([at.repeat_interleave(16300), between])
+    g = torch.Generator(device="cuda")
+    g.manual_seed(1)
+    w = w[torch.randperm(w.numel(), generator=g, device="cuda")]
+    r = lcd.dbci(w.view(torch.float32), want_labels=False)
+    assert torch.equal(r["sorted"].view(torch.int32), torch.sort(w).values)
+
+
+@pytest.mark.parametrize("n,outliers", [(9000, 3), (300_001, 40)])
+def test_dbci_at_odd_addresses(n, outliers):
+    # weights, labels and sorted weights that begin on four bytes
+    from ctypes import byref, c_size_t, c_void_p
+    rng = np.random.default_rng(n)
+    w = rng.normal(0, 0.02, n).astype(np.float32)
+    w[:outliers], w[outliers:2 * outliers] = 0.3, -0.3
+    ref = O.dbci_scan(w)
+    need = c_size_t(0)
+    assert lcd.binding.lib.lcd_dbci_workspace_bytes(n, 64, byref(need)) == 0
+    ws, cents = torch.empty(need.value, dtype=torch.uint8, device="cuda"), torch.empty(64, device="cuda")
+    res = torch.empty(64, dtype=torch.uint8, device="cuda")
+    for off in (1, 2, 3):
+        x, labels, srt = (torch.full((n + 8,), 77, dtype=t, device="cuda") for t in (torch.float32, torch.int32, torch.float32))
+        x[off:off + n] = torch.from_numpy(w)
+        assert lcd.binding.lib.lcd_dbci(c_void_p(x.data_ptr() + 4 * off), n, c_void_p(ws.data_ptr()), need.value, c_void_p(cents.data_ptr()), 64,
+                                        c_void_p(labels.data_ptr() + 4 * off), c_void_p(srt.data_ptr() + 4 * off), c_void_p(res.data_ptr()),
+                                        c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
+        assert np.array_equal(labels[off:off + n].cpu().numpy(), ref["labels"]) and np.array_equal(srt[off:off + n].cpu().numpy(), ref["sorted"])
+        for t in (labels, srt):
+            assert (t[:off] == 77).all() and (t[off + n:] == 77).all()
+
+
 def _captured_dbci(w, n_words):
     # the C call into a graph: (graph, its buffers)
     from ctypes import byref, c_size_t, c_void_p
