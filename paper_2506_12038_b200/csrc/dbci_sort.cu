@@ -15,7 +15,7 @@
 //             second time half a step further, which puts parts of up to eight keys in order;
 //   finish    nothing, unless a bucket's keys lie too close together in places (it is divided again by their density) or
 //             there are zeros of either sign: they are equal and keep their order, so they are written again in the input's.
-// 45 M Gaussian weights: 570 us (plan 6, count 55, map 18, partition 220, buckets 275), CUB's radix sort 1070; 925 K: 55 and 110.
+// 45 M Gaussian weights: 560 us (plan 6, count 55, map 15, partition 220, buckets 265), CUB's radix sort 1070; 925 K: 53 and 110.
 // Bytes are 0.9 GB, 140 us: what bounds the passes is shared memory at random addresses (a key's three lookups or atomics, a store
 // and two loads in the partition, an atomic, a lookup and a store in the buckets, each three to four bank conflicts a warp) and, where the
 // partition writes runs of six keys, the sectors that L2 takes.
@@ -799,7 +799,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) sort_buckets_kernel(const uns
 // many as their keys ask for, kParts in all, and the keys are placed by parts.  Up to eight keys of a part are left to the network, up
 // to kWarpKeys to a warp, more are a run of their own, of at most a 256th of the range: a key is placed three times at most, and of
 // 16384 keys at most 31 runs wait at any time.  (One bitonic sort of the bucket took 150 to 200 us: 925 K weights on 255 levels with
-// 10 % of others 349 us the whole call, 188 so; 4 M weights, 300 of them infinite 319, 225.)
+// 10 % of others 349 us the whole call, 181 so; 4 M weights, 300 of them infinite 319, 227.)
 constexpr unsigned kWarpKeys = 512;
 constexpr int kCoarse = 512;
 static_assert(kCoarse == kSortThreads, "a thread has one coarse stretch");
@@ -1016,7 +1016,7 @@ __global__ void __launch_bounds__(kSortThreads, 1) sort_finish_kernel(const unsi
 // part it lies in.  A segment without other keys is left as it is.  Parts of one value each are written from their counts; otherwise
 // the other keys are partitioned (and the pivot's written), parts of few keys become buckets together, and a part of more keys than
 // a bucket holds is a segment of the next level, whose range has eight bits less at least.
-// 45 M weights, the whole call: 255 levels with 10 % of other weights 990 us, eight clumps of 0.1 % width 1430 (a radix
+// 45 M weights, the whole call: 255 levels with 10 % of other weights 1003 us, eight clumps of 0.1 % width 1444 (a radix
 // sort of the whole array in four passes 1785 and 2037; CUB's 1270 and, with the marking of before, 2775); eight levels: 76 us here.
 constexpr int kSegThreads = 512, kSegTile = 8192, kSegItems = kSegTile / kSegThreads, kSegPartsLog = 11;
 constexpr int kSegPer = 5, kSegSlots = kSegThreads * kSegPer;       // parts of a thread; of a segment: at most 2048 and two more

@@ -59,10 +59,11 @@ __global__ void __launch_bounds__(256) smoothing_factors_kernel(const __half* x,
 // partial[g][t] = sum_k (x - level * s_q * s)^2 of token t under candidate g, kTokens tokens a CTA (a factor is loaded and
 // widened once for all of them); the CTA that arrives last averages, picks the first smallest candidate and writes its
 // factors.  Per element and candidate two multiplications, rounding by one addition, one conversion and four binary64
-// operations, 22 instructions in all with the pass that finds the tokens' maxima.  What bounds it is issue and the half-rate
-// integer and minimum pipe: 128 tokens, 4096 columns, 21 candidates, 11 M of them: 22.1 us for the whole search (24.1 with a clip, two
-// minimum operations, and an integer addition more; 512 x 14336 x 33: 205 and 236), of which the factors' kernel takes 6 and
-// starting, the last CTA's means and the copy of the winner's factors 5.
+// operations, 22 instructions in all with the pass that finds the tokens' maxima.  128 tokens, 4096 columns, 21 candidates: 11 M of
+// them are 6.5 us of issue, of 22.1 for the whole search.  No pipe is full: the factors' kernel takes 6 (a chain of binary64 powers in
+// less than a CTA an SM), this one's elements 11, with half of the issue slots and half of the warps' places used and the loads
+// as the longest stall, starting, the last CTA's means and the copy of the winner's factors 5.  (24.1 with a clip, two
+// minimum operations, and an integer addition more; 512 x 14336 x 33: 205 and 236.)
 constexpr int kTokens = 4;
 // PER_SM: CTAs that an SM must hold.  Four leave all the registers the compiler wants; a grid that does not fit four times
 // into the SMs is faster with five (512 tokens x 14336 columns x 33 candidates 221 -> 205 us, six 208; 128 x 4096 x 21: 24.4, 22.1
