@@ -17,7 +17,8 @@ namespace {
 constexpr int kRcThreads = 256;
 constexpr int kRcMaxC = 16;
 
-template <int CMAX>
+// AHEAD: the first step's loads are on their way before the thresholds are made.
+template <int CMAX, bool AHEAD>
 __global__ void __launch_bounds__(kRcThreads) reclassify_kernel(const uint8_t* __restrict__ idx, const uint16_t* __restrict__ codebook,
                                                                 const float* __restrict__ delta_w, int64_t K, int64_t ldw, int C,
                                                                 uint8_t* __restrict__ new_idx, double* __restrict__ delta_c,
@@ -31,11 +32,7 @@ __global__ void __launch_bounds__(kRcThreads) reclassify_kernel(const uint8_t* _
   const uint8_t* ir = idx + n * K;
   const float* dr = delta_w + n * ldw;
   uint8_t* outr = new_idx + n * K;
-  // 16 weights per thread and step: one 16-byte index load, four 16-byte update loads, one 16-byte store.  Above eight clusters,
-  // where shared memory holds few CTAs an SM, the first step's loads are on their way before the thresholds are made (4096 x 4096,
-  // 10 / 16 clusters 55.0 / 59.4 -> 51.0 / 55.4 us, 777 x 8192, 10 clusters 24.7 -> 21.9); with fewer the registers that
-  // takes cost as much (8192 x 8192, 4 clusters 99.2 -> 102.5).
-  constexpr bool kAhead = CMAX > 8;
+  // 16 weights per thread and step: one 16-byte index load, four 16-byte update loads, one 16-byte store
   uint4 iv = make_uint4(0u, 0u, 0u, 0u);
   float4 d[4];
   auto load = [&](int64_t k) {
@@ -44,7 +41,7 @@ __global__ void __launch_bounds__(kRcThreads) reclassify_kernel(const uint8_t* _
 #pragma unroll
     for (int q = 0; q < 4; ++q) d[q] = __ldg(reinterpret_cast<const float4*>(dr + k + 4 * q));
   };
-  if (kAhead && vec) load((int64_t)tid * 16);
+  if (AHEAD && vec) load((int64_t)tid * 16);
   if (tid < 12) s_total[tid >> 2][tid & 3] = 0;
   if (tid < C) s_c[tid] = __half2float(__ushort_as_half(codebook[n * C + tid]));
   __syncthreads();
@@ -123,7 +120,7 @@ __global__ void __launch_bounds__(kRcThreads) reclassify_kernel(const uint8_t* _
       if (kPacked && ++step == 16) { empty(); step = 1; }           // 240 weights since: no byte has overflowed
       const int64_t k = k0 + (int64_t)tid * 16;
       if (k >= K) continue;
-      if (!kAhead || k0 > 0) load(k);
+      if (!AHEAD || k0 > 0) load(k);
       const uint32_t iw[4] = {iv.x, iv.y, iv.z, iv.w};
       uint32_t ow[4];
 #pragma unroll
@@ -197,10 +194,10 @@ __global__ void __launch_bounds__(kRcThreads) reclassify_kernel(const uint8_t* _
   }
 }
 
-template <int CMAX>
+template <int CMAX, bool AHEAD = false>
 lcd_status launch_rows(const uint8_t* idx, const uint16_t* codebook, const float* delta_w, int64_t N, int64_t K, int64_t ldw, int C,
                        uint8_t* new_idx, double* delta_c, int32_t* counts, bool vec, cudaStream_t s) {
-  auto kern = reclassify_kernel<CMAX>;
+  auto kern = reclassify_kernel<CMAX, AHEAD>;
   constexpr int smem = CMAX * kRcThreads * (CMAX <= 4 ? 8 : CMAX <= 8 ? 20 : 12);
   if (smem > 40 * 1024) {             // (with the static tables more than the 48 KB that need no opt-in)
     static PerDeviceFlag attr_set;    // needs the opt-in, on every device
@@ -226,6 +223,11 @@ lcd_status launch_reclassify(const uint8_t* idx, const uint16_t* codebook, const
   const bool vec = K % 16 == 0 && ldw % 4 == 0 && al16(idx) && al16(delta_w) && al16(new_idx);
   if (C <= 4) return launch_rows<4>(idx, codebook, delta_w, N, K, ldw, C, new_idx, delta_c, counts, vec, s);
   if (C <= 8) return launch_rows<8>(idx, codebook, delta_w, N, K, ldw, C, new_idx, delta_c, counts, vec, s);
+  // Above eight clusters shared memory holds few CTAs an SM: the loads go ahead (4096 x 4096, 10 / 16 clusters 55.3 / 59.4 -> 51.0 /
+  // 55.4 us, 777 x 8192, 10 clusters 24.6 -> 22.2), but on short rows, of which a part of the CTA takes one step, the registers for it
+  // cost more (512 x 512 / 1024, 16 clusters 6.7 / 7.6 -> 7.2 / 8.2; 512 x 2048 8.2 either way), as they do with fewer clusters (8192
+  // x 8192, 4 clusters 99.2 -> 102.5).
+  if (K >= 2048) return launch_rows<kRcMaxC, true>(idx, codebook, delta_w, N, K, ldw, C, new_idx, delta_c, counts, vec, s);
   return launch_rows<kRcMaxC>(idx, codebook, delta_w, N, K, ldw, C, new_idx, delta_c, counts, vec, s);
 }
 

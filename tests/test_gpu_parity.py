@@ -1127,6 +1127,12 @@ def test_reclassify_rows_at_any_alignment(N, K, C, ld_extra):
     test_reclassify_matches_oracle(N, K, C, ld_extra)
 
 
+@pytest.mark.parametrize("K", [16, 2032, 2048, 4096, 4112, 8208])
+def test_reclassify_ten_clusters_on_either_side_of_the_loads_that_go_ahead(K):
+    # rows on 16 bytes; one step and parts of it, steps after the first
+    test_reclassify_matches_oracle(3, K, 10, 0)
+
+
 @pytest.mark.parametrize("act_bits,name", [(4, "lcd_lut_linear:"), (8, "lcd_lut_linear_act8:")])
 def test_lookup_errors_name_the_call(act_bits, name):
     L = gen.random_case(seed=1, N=16, K=300, bits=2, M=20)
