@@ -572,7 +572,20 @@ __device__ __forceinline__ bool one_value(const unsigned* keys, unsigned from, u
 // last key, up to a power of two, need not be there.
 __device__ void sort_by_warp(unsigned* keys, unsigned from, unsigned cnt) {
   const unsigned lane = threadIdx.x & 31;
-  unsigned size = 16;
+  if (cnt <= 32) {                        // a key a lane
+    unsigned v = lane < cnt ? keys[spread(from + lane)] : 0xffffffffu;
+#pragma unroll
+    for (unsigned k = 2; k <= 32; k *= 2)
+#pragma unroll
+      for (unsigned j = k / 2; j > 0; j /= 2) {
+        const unsigned o = __shfl_xor_sync(0xffffffffu, v, j == k / 2 ? k - 1 : j);
+        v = (lane & j) ? max(v, o) : min(v, o);
+      }
+    if (lane < cnt) keys[spread(from + lane)] = v;
+    __syncwarp();
+    return;
+  }
+  unsigned size = 64;
   while (size < cnt) size *= 2;
   auto order = [&](unsigned a, unsigned b) {
     if (b >= cnt) return;
@@ -797,18 +810,19 @@ __global__ void __launch_bounds__(kSortThreads, 2) sort_buckets_kernel(const uns
 // A bucket that equal stretches of its range leave with too many keys in one of them (an infinity among ordinary weights, values
 // repeated in the tail of others): a run of keys is counted in kCoarse equal stretches of its range, these are divided into parts, as
 // many as their keys ask for, kParts in all, and the keys are placed by parts.  Up to eight keys of a part are left to the network, up
-// to kWarpKeys to a warp, more are a run of their own, of at most a 256th of the range: a key is placed three times at most, and of
+// to kWarpKeys to a warp, more are a run of their own, of at most a 1024th of the range: a key is placed three times at most, and of
 // 16384 keys at most 31 runs wait at any time.  (One bitonic sort of the bucket took 150 to 200 us: 925 K weights on 255 levels with
-// 10 % of others 349 us the whole call, 181 so; 4 M weights, 300 of them infinite 319, 227.)
+// 10 % of others 349 us the whole call, 178 so; 4 M weights, 300 of them infinite 319, 228.)
 constexpr unsigned kWarpKeys = 512;
-constexpr int kCoarse = 512;
-static_assert(kCoarse == kSortThreads, "a thread has one coarse stretch");
+constexpr int kCoarseLog = 11, kCoarse = 1 << kCoarseLog;
+static_assert(kCoarse == 4 * kSortThreads, "a thread has four coarse stretches");
 __device__ __forceinline__ void sort_uneven_bucket(unsigned* x, int cnt, SortState* st, unsigned* keys, unsigned* bins, unsigned* source) {
   __shared__ uint2 runs[kCap / kWarpKeys];          // first place, keys
   __shared__ unsigned full[kCap / 9];               // parts of more than eight keys: first place << 16 | keys
   __shared__ int n_runs, n_full;
   __shared__ unsigned part[kSortThreads / 32 + 1], lo_s, hi_s;
-  __shared__ unsigned table[kCoarse];               // keys of a coarse stretch, then its first part << 16 | its parts
+  __shared__ uint4 table4[kSortThreads];
+  unsigned* table = reinterpret_cast<unsigned*>(table4);          // [kCoarse] keys of a coarse stretch, then its first part << 16 | its parts
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   bool negative = false;
 #pragma unroll 8
@@ -827,7 +841,7 @@ __device__ __forceinline__ void sort_uneven_bucket(unsigned* x, int cnt, SortSta
       hi_s = 0u;
       n_full = 0;
     }
-    table[tid] = 0u;
+    table4[tid] = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
     for (int i = 0; i < kParts / 8 / kSortThreads; ++i) reinterpret_cast<uint4*>(bins)[i * kSortThreads + tid] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
@@ -849,14 +863,22 @@ __device__ __forceinline__ void sort_uneven_bucket(unsigned* x, int cnt, SortSta
     hi = hi_s;
     const unsigned span = hi - lo;
     const bool exact = span < (unsigned)kParts;     // a part for every value
-    const int shift = exact ? 0 : 32 - __clz(span) - 9;
+    const int shift = exact ? 0 : 32 - __clz(span) - kCoarseLog;
     if (!exact) {
 #pragma unroll 4
       for (unsigned i = tid; i < c; i += kSortThreads) atomicAdd(&table[(source[i] - lo) >> shift], 1u);
       __syncthreads();
-      const unsigned parts = min(1u + table[tid] * (unsigned)(kParts - kCoarse) / c, 1u << min(shift, 15));        // (16384 x 15872 fits)
-      const unsigned first = block_exclusive<kSortThreads / 32>(parts, part);
-      table[tid] = first << 16 | parts;
+      uint4 v = table4[tid];
+      auto parts = [&](unsigned& w) { w = min(1u + w * (unsigned)(kParts - kCoarse) / c, 1u << min(shift, 15)); };        // (16384 x 14336 fits)
+      parts(v.x); parts(v.y); parts(v.z); parts(v.w);
+      unsigned first = block_exclusive<kSortThreads / 32>(v.x + v.y + v.z + v.w, part);
+      auto entry = [&](unsigned& w) {
+        const unsigned of = w;
+        w |= first << 16;
+        first += of;
+      };
+      entry(v.x); entry(v.y); entry(v.z); entry(v.w);
+      table4[tid] = v;
       __syncthreads();
     }
     auto part_of = [&](unsigned key) {
@@ -1016,7 +1038,7 @@ __global__ void __launch_bounds__(kSortThreads, 1) sort_finish_kernel(const unsi
 // part it lies in.  A segment without other keys is left as it is.  Parts of one value each are written from their counts; otherwise
 // the other keys are partitioned (and the pivot's written), parts of few keys become buckets together, and a part of more keys than
 // a bucket holds is a segment of the next level, whose range has eight bits less at least.
-// 45 M weights, the whole call: 255 levels with 10 % of other weights 1003 us, eight clumps of 0.1 % width 1444 (a radix
+// 45 M weights, the whole call: 255 levels with 10 % of other weights 992 us, eight clumps of 0.1 % width 1440 (a radix
 // sort of the whole array in four passes 1785 and 2037; CUB's 1270 and, with the marking of before, 2775); eight levels: 76 us here.
 constexpr int kSegThreads = 512, kSegTile = 8192, kSegItems = kSegTile / kSegThreads, kSegPartsLog = 11;
 constexpr int kSegPer = 5, kSegSlots = kSegThreads * kSegPer;       // parts of a thread; of a segment: at most 2048 and two more
